@@ -33,6 +33,7 @@ struct paac_ctx {
   // second iteration (the two frame buffers alternate), so after two plain iterations each parity is captured
   // once into a CUDA graph and replayed from then on.  Anything that changes the sequence drops the graphs.
   bool graphs_on;          // option: allow recording
+  cudaStream_t record_st;  // where sequences are recorded when st is the legacy default stream (made on first use)
   // recorded launch sequences: kind 0 = rollout, 1 = update, 2 + 2 t + v = step t of the external-environment mode
   // (v = 1: with the frame stack built on the device), each for both parities of the frame buffers
   static constexpr int GRAPH_KINDS = 2 + 2 * 65;
@@ -214,13 +215,21 @@ template <class F> void run_recorded(paac_ctx* c, int kind, int parity, F enqueu
   }
   if (allowed && c->plain_calls[kind][parity] >= 1) {
     cudaGraph_t g = nullptr;
-    if (cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    // The legacy default stream cannot be captured, but a graph can be launched into it: the sequence is recorded on a
+    // stream of the context's own (nothing runs there).  Default-stream contexts replay like all others from then on.
+    const bool legacy = c->st == nullptr || c->st == cudaStreamLegacy;
+    if (legacy && c->record_st == nullptr && cudaStreamCreateWithFlags(&c->record_st, cudaStreamNonBlocking) != cudaSuccess)
+      c->record_st = nullptr;
+    const cudaStream_t rec = legacy && c->record_st != nullptr ? c->record_st : c->st;
+    if (cudaStreamBeginCapture(rec, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       const uint64_t before = c->lc.count;
       c->lc.serialize_next = true;
+      c->lc.st = rec;
       enqueue();
+      c->lc.st = c->st;
       const uint64_t launched = c->lc.count - before;
       cudaGraphExec_t exec = nullptr;
-      if (cudaStreamEndCapture(c->st, &g) == cudaSuccess && g != nullptr &&
+      if (cudaStreamEndCapture(rec, &g) == cudaSuccess && g != nullptr &&
           cudaGraphInstantiate(&exec, g, 0) == cudaSuccess) {
         cudaGraphDestroy(g);
         c->graph[kind][parity] = exec;
@@ -469,6 +478,7 @@ int paac_destroy(paac_ctx* c) {
   cudaStreamSynchronize(c->st);
   drop_graphs(c);
   c->lc.release();
+  if (c->record_st) cudaStreamDestroy(c->record_st);
   if (c->owns_workspace) cudaFree(c->ws);
   cudaGetLastError();
   delete c;
