@@ -159,9 +159,11 @@ void refresh_weight_copies(paac_ctx* c, bool cast) {
 
 // network + heads on the n_e states of `frames`, activations into slot `slot`.  With `tail` the caller is about
 // to step the synthetic environments and can take the actions there: if the forward pass left the heads as partial
-// sums (see HeadsTail), no sampling kernel is launched, *tail describes what is left, and the result is true.
+// sums (see HeadsTail), no sampling kernel is launched, *tail describes what is left, and the result is true.  With `env`
+// the CUDA-core path steps the environments itself (*advanced says so); without sampling *advanced says whether the
+// environments' step index has been moved on.
 bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, HeadsTail* tail = nullptr,
-                  bool* advanced = nullptr) {
+                  bool* advanced = nullptr, const EnvStepArgs* env = nullptr) {
   void* act[MAX_LAYERS];
   for (int l = 0; l <= c->nd.n_conv; ++l)
     act[l] = (char*)c->act[l] + (size_t)slot * c->n_e * c->nd.layer[l].out_size * c->elt;
@@ -185,14 +187,17 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
     if (advanced) *advanced = splits == 0 && !sample;      // the sampling kernel has moved the step index on
     return false;
   }
+  float* scratch = c->scratch + c->simt_scratch_off;
+  int splits = 0;
   if (use_tc(c))
     tc_forward(c->lc, c->arch, c->nd, c->theta, c->theta16, c->w_images, frames, c->n_e, act, c->scratch,
                &c->stats->error_word);
   else
-    simt_forward(c->lc, c->arch, c->prec, c->nd, c->theta, c->theta16, frames, c->n_e, act, c->scratch + c->simt_scratch_off);
-  launch_heads(c->lc, c->prec, c->nd, c->theta, c->theta16, act[c->nd.n_conv], c->n_e,
-               c->logits + row * c->A, c->values + row, c->seed, c->step_dev, (uint32_t)slot, forced, actions, sampled,
-               uniforms, head_mode(c));
+    splits = simt_forward(c->lc, c->arch, c->prec, c->nd, c->theta, c->theta16, frames, c->n_e, act, scratch);
+  launch_simt_tail(c->lc, c->prec, c->nd, c->theta, c->theta16, scratch, splits, act[c->nd.n_conv], c->n_e, c->logits + row * c->A,
+                   c->values + row, c->seed, c->step_dev, (uint32_t)slot, forced, actions, sampled, uniforms, head_mode(c),
+                   sample ? env : nullptr, advanced && !sample ? c->step_dev : nullptr, (uint32_t)c->t_max);
+  if (advanced) *advanced = sample ? env != nullptr : true;
   return false;
 }
 
@@ -325,9 +330,12 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
   run_recorded(c, 0, c->cur, [&]() {
     for (int t = 0; t < c->t_max; ++t) {
       HeadsTail tail;
-      const bool deferred = forward_slot(c, fr + t * fstep, t, true, &tail);
       uint8_t* dst = t + 1 < c->t_max ? fr + (t + 1) * fstep : nxt;
       const size_t row = (size_t)t * c->n_e;
+      const EnvStepArgs env{c->hp.term_denom, dst, c->rewards + row, c->terminals + row, c->counters, pattern_actions(c)};
+      bool stepped = false;
+      const bool deferred = forward_slot(c, fr + t * fstep, t, true, &tail, &stepped, &env);
+      if (stepped) continue;
       if (deferred)
         launch_env_step_sampling(c->lc, c->seed, c->n_e, c->step_dev, (uint32_t)t, c->hp.term_denom, dst, c->rewards + row,
                                  c->terminals + row, c->counters, tail, pattern_actions(c));
@@ -362,7 +370,7 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
                         c->scratch, &c->grad_segs);
     else
       heads_backward(c->lc, c->prec, c->nd, c->theta, c->theta16, c->act[L], c->B, c->dz, c->dV, c->gact[L],
-                     c->grad, c->scratch + c->simt_scratch_off);
+                     c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs);
     uint32_t* err = &c->stats->error_word;
     c->gact0_scale = 1.f;
     const bool chunked = use_tc(c) && c->update_chunks > 1 && (c->tc_wgrad_mask & 3) == 3;
@@ -394,12 +402,11 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
       }
       if (!wgrad_done || (l > 0 && !dgrad_done))
         simt_backward_layer(c->lc, c->arch, c->prec, c->nd, c->theta, c->theta16, c->frames[c->cur], c->B, c->act,
-                            c->gact, c->grad, c->scratch + c->simt_scratch_off, l, !wgrad_done, l > 0 && !dgrad_done);
+                            c->gact, c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, !wgrad_done, l > 0 && !dgrad_done);
     }
     // when every gradient goes through the finishing kernel, it also delivers the squared norm
-    const bool all_finished = use_tc(c) && c->tc_wgrad_mask == 0xF && tc_heads_backward_supported(c->nd);
-    int ready = 0;
-    if (use_tc(c)) ready = tc_backward_finish(c->lc, &c->grad_segs, all_finished ? c->norm_partials : nullptr);
+    const bool all_finished = !c->lc.fp32_tensor_cores || (use_tc(c) && c->tc_wgrad_mask == 0xF && tc_heads_backward_supported(c->nd));
+    const int ready = finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials : nullptr);
     launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad,
                         c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
                         c->norm_partials, c->stats, all_finished ? ready : 0);

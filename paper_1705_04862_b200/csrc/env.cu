@@ -1,4 +1,5 @@
 // Parameter initialisation and the synthetic hashed environment.
+#include "env_device.cuh"
 #include "kernels.h"
 
 namespace paac {
@@ -55,7 +56,6 @@ void launch_cast_bf16(LaunchCtx& lc, const float* src, bf16* dst, size_t n) {
 // write the 84x84x4 frame of the state reached, one hashed 32-bit word per pixel (its bytes,
 // little endian, are the four channels), as 16-byte stores.
 constexpr int ENV_THREADS = 256;
-constexpr int FRAME_WORDS = FRAME_H * FRAME_W;   // 7056, a multiple of 4
 
 // With SAMPLE the block's first warp also takes the action first: it finishes the heads of its environment from the
 // two partial dot products hp[half][e][k] the fully connected kernel left (k < A policy rows, k = A value row;
@@ -67,20 +67,15 @@ env_step_kernel(uint64_t seed, int n_e, const uint64_t* __restrict__ step_base, 
                 const int32_t* actions, uint32_t term_denom,
                 uint8_t* __restrict__ next_frames, int8_t* __restrict__ rewards, uint8_t* __restrict__ terminals,
                 int32_t* __restrict__ counters, HeadsTail ht, int pattern_actions) {
-  // pattern_actions > 0: the learnable environment.  The state at step k of environment e has the goal
-  // hash(e, k, 'GOAL') mod A; its frame is the hashed frame with every byte reduced to its low six bits (a dim
-  // texture) and rows [band goal, band (goal + 1)), band = 84 / A, set to 255; an action pays 1 if it is the current
-  // state's goal and 0 otherwise.
   // Two roles run side by side until the action is known: the first warp takes it (SAMPLE), and the first thread of
   // the second warp prepares everything of the transition that does not depend on it -- the hash chains of this step
   // and the next up to the point where the action enters, and the environment's counters, whose loads would otherwise
   // be waited for after the draw.  One hash step, the reward / terminal bits and the frame's base remain.
-  __shared__ uint32_t s_base, s_band_lo, s_band_hi;
+  __shared__ EnvFrame s_frame;
   __shared__ int32_t s_action;
   const uint32_t e = blockIdx.x;
   const bool stepping = SAMPLE || actions != nullptr;          // else: the start frames (step 0, tag 0)
-  uint32_t pre_step = 0u, pre_next = 0u, step = 0u;
-  int32_t len = 0, ret = 0, episodes = 0;
+  EnvPrep prep{};
   if (SAMPLE && threadIdx.x < 32) {
     const int lane = threadIdx.x, A = ht.A;
     const float bias = lane < A ? __ldg(ht.bpi + lane) : (lane == A ? __ldg(ht.bv) : 0.f);   // older than the previous kernel
@@ -95,63 +90,22 @@ env_step_kernel(uint64_t seed, int n_e, const uint64_t* __restrict__ step_base, 
     pdl_entry();
     if (threadIdx.x == 32) {
       if (stepping) {
-        step = (uint32_t)(*step_base) + t;                      // global step index of this transition
-        pre_step = env_hash_prefix(seed, e, step);
-        pre_next = env_hash_prefix(seed, e, step + 1u);
-        len = counters[e]; ret = counters[n_e + e]; episodes = counters[2 * n_e + e];
+        prep = env_prepare(seed, e, n_e, (uint32_t)(*step_base) + t, counters);     // global step index of this transition
         if (!SAMPLE) s_action = actions[e];
       } else {
-        pre_next = env_hash_prefix(seed, e, 0u);
+        prep.pre_next = env_hash_prefix(seed, e, 0u);
       }
     }
   }
   __syncthreads();
-  bool term = false;
-  int r = 0;
+  EnvOutcome o{0, false, 0u};
   if (threadIdx.x == 32) {
-    uint32_t tag = 0u;
-    if (stepping) {
-      const int32_t a = s_action;
-      const uint32_t base = hash_mix(pre_step ^ ((uint32_t)a + 1u));
-      const uint32_t hr = hash_mix(base ^ HASH_TAG_REWARD) & 15u;
-      r = hr == 0u ? 1 : (hr == 1u ? -1 : 0);
-      if (pattern_actions > 0)
-        r = (uint32_t)a == hash_mix(hash_mix(pre_step) ^ HASH_TAG_GOAL) % (uint32_t)pattern_actions ? 1 : 0;
-      const uint32_t hterm = hash_mix(base ^ HASH_TAG_TERMINAL);
-      term = (uint32_t)(((uint64_t)hterm * term_denom) >> 32) == 0u;
-      tag = term ? 0u : (uint32_t)a + 1u;
-    }
-    s_base = hash_mix(pre_next ^ tag);
-    s_band_lo = s_band_hi = 0u;
-    if (pattern_actions > 0) {
-      const uint32_t goal = hash_mix(hash_mix(pre_next) ^ HASH_TAG_GOAL) % (uint32_t)pattern_actions;
-      const uint32_t band = (uint32_t)(FRAME_H / pattern_actions);
-      s_band_lo = band * goal * FRAME_W;                  // in pixel words; a row is 84 words, so four words never straddle it
-      s_band_hi = s_band_lo + band * FRAME_W;
-    }
+    if (stepping) o = env_outcome(prep, s_action, term_denom, pattern_actions);
+    s_frame = env_frame_of(prep.pre_next, o.tag, pattern_actions);
   }
   __syncthreads();
-  if (threadIdx.x == 32 && stepping) {
-    rewards[e] = (int8_t)r;
-    terminals[e] = term ? 1 : 0;
-    len += 1; ret += r;
-    if (term) { counters[2 * n_e + e] = episodes + 1; len = 0; ret = 0; }
-    counters[e] = len; counters[n_e + e] = ret;
-  }
-  const uint32_t base = s_base, band_lo = s_band_lo, band_hi = s_band_hi;
-  const uint32_t keep = pattern_actions > 0 ? 0x3F3F3F3Fu : 0xFFFFFFFFu;
-  uint4* out = reinterpret_cast<uint4*>(next_frames + (size_t)e * FRAME_BYTES);
-  for (int q = threadIdx.x; q < FRAME_WORDS / 4; q += ENV_THREADS) {
-    const uint32_t p = (uint32_t)q * 4u + 1u;
-    uint4 v;
-    v.x = hash_mix(base + HASH_K0 * p);
-    v.y = hash_mix(base + HASH_K0 * (p + 1u));
-    v.z = hash_mix(base + HASH_K0 * (p + 2u));
-    v.w = hash_mix(base + HASH_K0 * (p + 3u));
-    v.x &= keep; v.y &= keep; v.z &= keep; v.w &= keep;
-    if ((uint32_t)q * 4u >= band_lo && (uint32_t)q * 4u < band_hi) v = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-    out[q] = v;
-  }
+  if (threadIdx.x == 32 && stepping) env_record(prep, o, e, n_e, rewards, terminals, counters);
+  env_write_frame<ENV_THREADS>(s_frame, next_frames + (size_t)e * FRAME_BYTES, pattern_actions);
 }
 
 void launch_env_step(LaunchCtx& lc, uint64_t seed, int n_e, const uint64_t* step_base, uint32_t t,

@@ -1,0 +1,74 @@
+// The synthetic environments' transition and frame, shared by the kernels that step them (one block per environment).
+#pragma once
+#include "common.cuh"
+
+namespace paac {
+
+constexpr int FRAME_WORDS = FRAME_H * FRAME_W;   // 7056, a multiple of 4
+
+// what of a transition does not depend on the action: prepared by one thread while the action is being found
+struct EnvPrep { uint32_t pre_step, pre_next; int32_t len, ret, episodes; };
+__device__ __forceinline__ EnvPrep env_prepare(uint64_t seed, uint32_t e, int n_e, uint32_t step, const int32_t* counters) {
+  EnvPrep p;
+  p.pre_step = env_hash_prefix(seed, e, step);
+  p.pre_next = env_hash_prefix(seed, e, step + 1u);
+  p.len = counters[e]; p.ret = counters[n_e + e]; p.episodes = counters[2 * n_e + e];
+  return p;
+}
+// the frame of a state: its hash base, and the band of the learnable environment in pixel words (empty otherwise)
+struct EnvFrame { uint32_t base, band_lo, band_hi; };
+// pattern_actions > 0: the learnable environment.  The state at step k of environment e has the goal
+// hash(e, k, 'GOAL') mod A; its frame is the hashed frame with every byte reduced to its low six bits (a dim
+// texture) and rows [band goal, band (goal + 1)), band = 84 / A, set to 255; an action pays 1 if it is the current
+// state's goal and 0 otherwise.
+__device__ __forceinline__ EnvFrame env_frame_of(uint32_t pre_next, uint32_t tag, int pattern_actions) {
+  EnvFrame f{hash_mix(pre_next ^ tag), 0u, 0u};
+  if (pattern_actions > 0) {
+    const uint32_t goal = hash_mix(hash_mix(pre_next) ^ HASH_TAG_GOAL) % (uint32_t)pattern_actions;
+    const uint32_t band = (uint32_t)(FRAME_H / pattern_actions);
+    f.band_lo = band * goal * FRAME_W;                  // a row is 84 words, so four words never straddle it
+    f.band_hi = f.band_lo + band * FRAME_W;
+  }
+  return f;
+}
+struct EnvOutcome { int reward; bool terminal; uint32_t tag; };
+__device__ __forceinline__ EnvOutcome env_outcome(const EnvPrep& p, int32_t a, uint32_t term_denom, int pattern_actions) {
+  EnvOutcome o;
+  const uint32_t base = hash_mix(p.pre_step ^ ((uint32_t)a + 1u));
+  const uint32_t hr = hash_mix(base ^ HASH_TAG_REWARD) & 15u;
+  o.reward = hr == 0u ? 1 : (hr == 1u ? -1 : 0);
+  if (pattern_actions > 0)
+    o.reward = (uint32_t)a == hash_mix(hash_mix(p.pre_step) ^ HASH_TAG_GOAL) % (uint32_t)pattern_actions ? 1 : 0;
+  const uint32_t hterm = hash_mix(base ^ HASH_TAG_TERMINAL);
+  o.terminal = (uint32_t)(((uint64_t)hterm * term_denom) >> 32) == 0u;
+  o.tag = o.terminal ? 0u : (uint32_t)a + 1u;
+  return o;
+}
+__device__ __forceinline__ void env_record(const EnvPrep& p, const EnvOutcome& o, uint32_t e, int n_e, int8_t* rewards,
+                                           uint8_t* terminals, int32_t* counters) {
+  rewards[e] = (int8_t)o.reward;
+  terminals[e] = o.terminal ? 1 : 0;
+  if (o.terminal) counters[2 * n_e + e] = p.episodes + 1;
+  counters[e] = o.terminal ? 0 : p.len + 1;
+  counters[n_e + e] = o.terminal ? 0 : p.ret + o.reward;
+}
+// the whole block writes the 84 x 84 x 4 frame, one hashed 32-bit word per pixel (its bytes, little endian, are the
+// four channels), as 16-byte stores
+template <int THREADS>
+__device__ __forceinline__ void env_write_frame(const EnvFrame f, uint8_t* frame, int pattern_actions) {
+  const uint32_t keep = pattern_actions > 0 ? 0x3F3F3F3Fu : 0xFFFFFFFFu;
+  uint4* out = reinterpret_cast<uint4*>(frame);
+  for (int q = threadIdx.x; q < FRAME_WORDS / 4; q += THREADS) {
+    const uint32_t p = (uint32_t)q * 4u + 1u;
+    uint4 v;
+    v.x = hash_mix(f.base + HASH_K0 * p);
+    v.y = hash_mix(f.base + HASH_K0 * (p + 1u));
+    v.z = hash_mix(f.base + HASH_K0 * (p + 2u));
+    v.w = hash_mix(f.base + HASH_K0 * (p + 3u));
+    v.x &= keep; v.y &= keep; v.z &= keep; v.w &= keep;
+    if ((uint32_t)q * 4u >= f.band_lo && (uint32_t)q * 4u < f.band_hi) v = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    out[q] = v;
+  }
+}
+
+}  // namespace paac

@@ -1,4 +1,4 @@
-// The same generic contraction as gemm_simt.cuh on the tensor cores, accurate to float level:
+// The generic contraction of the float path on the tensor cores, accurate to float level:
 //   C(m, n) = sum_k A(m, k) * B(n, k)
 // with every float operand split into two TF32 pieces, x = hi + lo (hi = tf32(x), lo = tf32(x - hi), round to nearest,
 // together 22 significant bits), and three tcgen05 passes (kind::tf32) per block of 32 k into a float accumulator in
@@ -6,8 +6,8 @@
 //   hi*hi + hi*lo + lo*hi      (the dropped lo*lo term and the rounding of lo are below 2^-21 of a product).
 // Two bfloat16 pieces (16 bits) are not enough here: errors of 1e-5 flip about one ReLU unit per update of the small
 // network and the free-running trajectories leave the float tolerance within three updates.
-// Operands come from the same index functors and results go to the same epilogue functors as the CUDA-core
-// kernel, so every layer of the float path (forward, data and weight gradients, split-k included) can run through it.
+// Operands come from the index functors and results go to epilogue functors (gemm_ops.cuh),
+// so every layer of the float path (forward, data and weight gradients, split-k included) can run through it.
 // One CTA per 128 x 64 output tile and k split; 544 threads:
 //   warps 0-15 producers: per block of 32 k a thread evaluates two 16-byte chunks (four k of one row) of A and one of B,
 //              splits them, and writes them into the hi and the lo image (128-byte rows, 128-byte swizzle); then the
@@ -22,7 +22,7 @@
 // Every wait is bounded.  The contractions of the float configurations are small (4 to 160 rows in the fully connected
 // layers), so most of a 128-row tile is padding there: this path exists for its arithmetic, not for speed.
 #pragma once
-#include "gemm_simt.cuh"
+#include "gemm_ops.cuh"
 #include "tc_common.cuh"
 
 namespace paac {
@@ -227,7 +227,7 @@ gemm_tc3_kernel(int M, int N, int K, int k_per_split, LA la, LB lb, EP ep, uint3
   }
 }
 
-// same split geometry as gemm_simt (the callers size their partial-sum scratch and their reductions by it)
+// split geometry of gemm_k_splits (the callers size their partial-sum scratch and their reductions by it)
 template <class LA, class LB, class EP>
 inline void gemm_tc3(LaunchCtx& lc, int kid, int M, int N, int K, int splits, LA la, LB lb, EP ep) {
   if (M <= 0 || N <= 0 || K <= 0) return;
@@ -244,11 +244,5 @@ inline void gemm_tc3(LaunchCtx& lc, int kid, int M, int N, int K, int splits, LA
   launch_kernel(lc, kern, grid, T3_THREADS, T3_SMEM, M, N, K, kps, la, lb, ep, lc.error_word);
 }
 
-// the float path's contractions: on the CUDA cores, or (option) through the three-pass tensor-core kernel
-template <class LA, class LB, class EP>
-inline void gemm_f32(LaunchCtx& lc, int kid, int M, int N, int K, int splits, LA la, LB lb, EP ep) {
-  if (lc.fp32_tensor_cores && lc.error_word != nullptr) gemm_tc3(lc, kid, M, N, K, splits, la, lb, ep);
-  else gemm_simt(lc, kid, M, N, K, splits, la, lb, ep);
-}
 
 }  // namespace paac

@@ -1,5 +1,6 @@
 // Policy / value heads with softmax, entropy and Philox inverse-CDF sampling; the reverse
 // scan for n-step returns; the loss gradient at the heads.
+#include "env_device.cuh"
 #include "kernels.h"
 
 namespace paac {
@@ -15,60 +16,128 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// EPL consecutive elements of a row as floats (EPL = 8 or 16; 16-byte loads)
-template <int EPL> __device__ __forceinline__ void load_row_slice(const float* p, float (&v)[EPL]) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-#pragma unroll
-  for (int i = 0; i < EPL / 4; ++i) { const float4 t = __ldg(q + i); v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w; }
-}
-template <int EPL> __device__ __forceinline__ void load_row_slice(const bf16* p, float (&v)[EPL]) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-  for (int i = 0; i < EPL / 8; ++i) {
-    const uint4 t = __ldg(q + i);
-    const uint32_t w[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { v[8 * i + 2 * j] = __uint_as_float(w[j] << 16); v[8 * i + 2 * j + 1] = __uint_as_float(w[j] & 0xFFFF0000u); }
-  }
-}
-
-// One warp per state; lane l holds elements [l*EPL, (l+1)*EPL) of the fc activation (F = 32*EPL) and of
-// each head row.  Lane k ends up holding logit k (A <= 32).  If `actions` is given, the warp also draws
-// a_t: u from Philox counter (env, step_lo, step_hi, ACTION stream), then the smallest k with
-// u < p_0 + ... + p_k, the running sum taken serially in float in index order.
-template <class T, class TW, int EPL>
-__global__ void __launch_bounds__(128)
-heads_kernel(const T* __restrict__ h, const TW* __restrict__ wpi, const float* __restrict__ bpi,
-             const TW* __restrict__ wv, const float* __restrict__ bv, int n, int A,
-             float* __restrict__ logits, float* __restrict__ values, uint64_t seed, const uint64_t* __restrict__ step_base, uint32_t t,
-             const int32_t* __restrict__ forced, int32_t* __restrict__ actions, int32_t* __restrict__ sampled,
-             float* __restrict__ uniforms, HeadMode mode) {
+// The end of a forward pass on the CUDA cores, one block per state: the fully connected layer's split-k partial sums are
+// added (in double: the pre-activation then differs from an exactly rounded one only by the error inside each short
+// partial sum, and fewer units near zero end up on the other side of the ReLU), bias and ReLU give h, each warp takes
+// the dot products of every eighth head output, the first warp finishes the heads (softmax and draw), and in a rollout
+// the block goes on to step its environment: transition by one thread, frame by all.  One launch and a few block-wide
+// barriers where three kernels in a row each waited for the one before (finish 11-19 us, heads 8-22 us, environment
+// 3-4 us a step by themselves, about 6 us together at 4 to 128 states).  A few microseconds of latency: the head
+// weights are staged before the wait on the previous kernel, which does not write them.
+// 2 F threads: two per hidden unit share its partial sums, all loads of which are in flight together.
+struct TailArgs {
+  const float* part; int splits;                 // [splits][n][F]; splits == 0: h is complete
+  const float* fc_bias;
+  int n, A;
+  float* logits; float* values;
+  uint64_t seed; const uint64_t* step_base; uint32_t t;
+  const int32_t* forced; int32_t* actions; int32_t* sampled; float* uniforms; HeadMode mode;
+  uint64_t* advance_step; uint32_t advance_by;
+};
+template <class T, class TW, int F, bool STEP>
+__global__ void __launch_bounds__(2 * F)
+simt_tail_kernel(TailArgs q, T* h, const TW* wpi, const float* bpi, const TW* wv, const float* bv, EnvStepArgs env) {
+  constexpr int TAIL_THREADS = 2 * F, WARPS = TAIL_THREADS / 32, BATCH = 24;
+  extern __shared__ __align__(16) float wsh[];   // [A + 1][F]
+  __shared__ float xs[F], zs[33];
+  __shared__ double upper[F];                    // the sums of the second half of the splits
+  __shared__ EnvFrame s_frame;
+  __shared__ int32_t s_action;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, A = q.A;
+  const size_t e = blockIdx.x;
+  for (int i = threadIdx.x; i < (A + 1) * F; i += TAIL_THREADS) wsh[i] = i < A * F ? to_f(wpi[i]) : to_f(wv[i - A * F]);
   pdl_entry();
-  constexpr int F = 32 * EPL;
-  const int lane = threadIdx.x & 31;
-  const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (e >= n) return;
-  float x[EPL], w[EPL];
-  load_row_slice<EPL>(h + (size_t)e * F + lane * EPL, x);
-  float z = -INFINITY;
-  for (int k = 0; k < A; ++k) {
-    load_row_slice<EPL>(wpi + (size_t)k * F + lane * EPL, w);
+  // the last kernel of a rollout also moves the environments' step index on (nothing in that launch reads it)
+  if (q.advance_step != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *q.advance_step += q.advance_by;
+  const int unit = threadIdx.x % F, part_half = threadIdx.x / F;
+  double sum = 0.0;
+  {
+    const int half = (q.splits + 1) / 2, p1 = part_half ? q.splits : half;
+    const float* src = q.part + e * F + unit;
+    const size_t stride = (size_t)q.n * F;
+    for (int p = part_half * half; p < p1; p += BATCH) {
+      float v[BATCH];
+#pragma unroll
+      for (int j = 0; j < BATCH; ++j) v[j] = p + j < p1 ? src[(size_t)(p + j) * stride] : 0.f;
+#pragma unroll
+      for (int j = 0; j < BATCH; ++j) sum += (double)v[j];
+    }
+    if (part_half) upper[unit] = sum;
+  }
+  EnvPrep prep{};
+  if (STEP && threadIdx.x == 32) prep = env_prepare(q.seed, (uint32_t)e, q.n, (uint32_t)(*q.step_base) + q.t, env.counters);
+  __syncthreads();
+  if (part_half == 0) {
+    if (q.splits == 0) {
+      xs[unit] = to_f(h[e * F + unit]);
+    } else {
+      const T x = from_f<T>(fmaxf((float)((sum + upper[unit]) + (double)q.fc_bias[unit]), 0.f));
+      h[e * F + unit] = x;
+      xs[unit] = to_f(x);
+    }
+  }
+  __syncthreads();
+  for (int k = warp; k <= A; k += WARPS) {
     float acc = 0.f;
 #pragma unroll
-    for (int i = 0; i < EPL; ++i) acc = fmaf(w[i], x[i], acc);
-    acc = warp_sum(acc) + bpi[k];
-    if (lane == k) z = acc;
+    for (int i = 0; i < F / 32; ++i) acc = fmaf(wsh[k * F + lane + 32 * i], xs[lane + 32 * i], acc);
+    acc = warp_sum(acc);
+    if (lane == 0) zs[k] = acc + (k < A ? bpi[k] : bv[0]);
   }
-  // the value row follows the policy biases in the parameter vector, so it is not 16-byte aligned
-  float v = 0.f;
-#pragma unroll
-  for (int i = 0; i < EPL; ++i) v = fmaf(to_f(wv[lane * EPL + i]), x[i], v);
-  v = warp_sum(v) + bv[0];
-  warp_finish_heads(mode, z, v, lane, A, (size_t)e, logits, values, actions != nullptr, seed,
-                    actions != nullptr ? *step_base + t : 0ull, forced, actions, sampled, uniforms);
+  __syncthreads();
+  if (warp == 0) {
+    const int32_t a = warp_finish_heads(q.mode, lane < A ? zs[lane] : -INFINITY, zs[A], lane, A, e, q.logits, q.values, q.actions != nullptr,
+                                        q.seed, q.actions != nullptr ? *q.step_base + q.t : 0ull, q.forced, q.actions, q.sampled, q.uniforms);
+    if (STEP && lane == 0) s_action = a;
+  }
+  if constexpr (STEP) {
+    __syncthreads();
+    EnvOutcome o{0, false, 0u};
+    if (threadIdx.x == 32) {
+      o = env_outcome(prep, s_action, env.term_denom, env.pattern_actions);
+      s_frame = env_frame_of(prep.pre_next, o.tag, env.pattern_actions);
+    }
+    __syncthreads();
+    if (threadIdx.x == 32) env_record(prep, o, (uint32_t)e, q.n, env.rewards, env.terminals, env.counters);
+    env_write_frame<TAIL_THREADS>(s_frame, env.next_frames + e * FRAME_BYTES, env.pattern_actions);
+  }
 }
 
-// The same, fused with the end of the fully connected layer of the tensor-core path: the warp first finishes
+template <class T, class TW, int F>
+static void tail_launch(LaunchCtx& lc, const TailArgs& q, T* h, const TW* wpi, const float* bpi, const TW* wv, const float* bv,
+                        const EnvStepArgs* env) {
+  const size_t smem = (size_t)(q.A + 1) * F * sizeof(float);
+  auto go = [&](auto kern) {
+    if (smem + 4096 > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      lc.host_failure = true;
+    // few blocks: they may set up while the previous kernel drains; many small blocks would pile up on the first free SMs
+    if (q.n <= 148) launch_kernel_overlapped(lc, kern, dim3(q.n), dim3(2 * F), smem, q, h, wpi, bpi, wv, bv, env ? *env : EnvStepArgs{});
+    else launch_kernel(lc, kern, dim3(q.n), dim3(2 * F), smem, q, h, wpi, bpi, wv, bv, env ? *env : EnvStepArgs{});
+  };
+  if (env) go(simt_tail_kernel<T, TW, F, true>); else go(simt_tail_kernel<T, TW, F, false>);
+}
+
+void launch_simt_tail(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const float* part, int splits,
+                      void* h, int n, float* logits, float* values, uint64_t seed, const uint64_t* step_base, uint32_t t,
+                      const int32_t* forced, int32_t* actions, int32_t* sampled, float* uniforms, HeadMode mode,
+                      const EnvStepArgs* env, uint64_t* advance_step, uint32_t advance_by) {
+  KernelScope scope(lc, env ? KID_ENV_STEP : KID_HEADS_FWD);
+  TailArgs q{part, splits, theta + nd.layer[nd.n_conv].b_off, n, nd.A, logits, values, seed, step_base, t, forced, actions, sampled,
+             uniforms, mode, advance_step, advance_by};
+  const float* bpi = theta + nd.pi_b; const float* bv = theta + nd.v_b;
+  if (prec == PAAC_BF16) {
+    if (nd.F == 512) tail_launch<bf16, bf16, 512>(lc, q, (bf16*)h, theta16 + nd.pi_w, bpi, theta16 + nd.v_w, bv, env);
+    else tail_launch<bf16, bf16, 256>(lc, q, (bf16*)h, theta16 + nd.pi_w, bpi, theta16 + nd.v_w, bv, env);
+  } else {
+    if (nd.F == 512) tail_launch<float, float, 512>(lc, q, (float*)h, theta + nd.pi_w, bpi, theta + nd.v_w, bv, env);
+    else tail_launch<float, float, 256>(lc, q, (float*)h, theta + nd.pi_w, bpi, theta + nd.v_w, bv, env);
+  }
+}
+
+// The heads fused with the end of the fully connected layer of the tensor-core path, one warp per state, lane k ending up
+// with output k (A <= 32).  If `actions` is given, the warp also draws a_t: u from Philox counter (env, step_lo, step_hi,
+// ACTION stream), then the smallest k with u < p_0 + ... + p_k, the running sum taken serially in float in index order.  The
+// warp first finishes
 // its state's 512 hidden units from the split-k partial sums, h = bf16(relu(sum_s part[s][e][:] + bias)), the
 // splits added in order, stores them for the backward pass and goes on with the rounded values.  The A dot
 // products are reduced together: every lane keeps one partial sum per action, and a butterfly that halves the
@@ -177,7 +246,7 @@ heads_fused_kernel(const float* __restrict__ part, int splits, const float* __re
 
 // The tail of the heads for the cluster path of the fully connected layer, which has already taken the head dot
 // products over each half of the hidden units: hp[half][e][k], k < A the policy rows, k = A the value row, rows
-// HS_LD floats apart.  One warp per state, lane k holds logit k; softmax and sampling as in heads_kernel.
+// HS_LD floats apart.  One warp per state, lane k holds logit k; softmax and sampling as above.
 constexpr int HS_LD = 32, HS_WARPS = 4;
 __global__ void __launch_bounds__(HS_WARPS * 32)
 heads_sample_kernel(const float* __restrict__ hp, const float* __restrict__ bpi, const float* __restrict__ bv, int n, int A,
@@ -215,61 +284,6 @@ void launch_heads_fused(LaunchCtx& lc, const NetDims& nd, const float* theta, co
   launch_kernel(lc, heads_fused_kernel, (n + HF_WARPS - 1) / HF_WARPS, HF_WARPS * 32, 0, part, splits, theta + nd.layer[nd.n_conv].b_off, h_out,
                 theta16 + nd.pi_w, theta + nd.pi_b, theta16 + nd.v_w, theta + nd.v_b, n, nd.A, logits, values, seed,
                 step_base, t, forced, actions, sampled, uniforms, mode);
-}
-
-// Element-wise variant of the heads kernel for layouts without 16-byte alignment and for float storage.
-// One warp per state.  Lane k ends up holding logit k (A <= 32).  If `actions` is given,
-// the warp also draws a_t: u from Philox counter (env, step_lo, step_hi, ACTION stream), then the
-// smallest k with u < p_0 + ... + p_k, the running sum taken serially in float in index order.
-template <class T, class TW>
-__global__ void __launch_bounds__(128)
-heads_slow_kernel(const T* __restrict__ h, const TW* __restrict__ wpi, const float* __restrict__ bpi,
-             const TW* __restrict__ wv, const float* __restrict__ bv, int n, int F, int A,
-             float* __restrict__ logits, float* __restrict__ values, uint64_t seed, const uint64_t* __restrict__ step_base, uint32_t t,
-             const int32_t* __restrict__ forced, int32_t* __restrict__ actions, int32_t* __restrict__ sampled,
-             float* __restrict__ uniforms, HeadMode mode) {
-  pdl_entry();
-  const int lane = threadIdx.x & 31;
-  const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (e >= n) return;
-  const T* x = h + (size_t)e * F;
-  float z = -INFINITY;
-  for (int k = 0; k < A; ++k) {
-    float acc = 0.f;
-    for (int i = lane; i < F; i += 32) acc = fmaf(to_f(wpi[(size_t)k * F + i]), to_f(x[i]), acc);
-    acc = warp_sum(acc) + bpi[k];
-    if (lane == k) z = acc;
-  }
-  float v = 0.f;
-  for (int i = lane; i < F; i += 32) v = fmaf(to_f(wv[i]), to_f(x[i]), v);
-  v = warp_sum(v) + bv[0];
-  warp_finish_heads(mode, z, v, lane, A, (size_t)e, logits, values, actions != nullptr, seed,
-                    actions != nullptr ? *step_base + t : 0ull, forced, actions, sampled, uniforms);
-}
-
-void launch_heads(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta,
-                  const bf16* theta16, const void* h, int n, float* logits, float* values, uint64_t seed,
-                  const uint64_t* step_base, uint32_t t, const int32_t* forced, int32_t* actions, int32_t* sampled,
-                  float* uniforms, HeadMode mode) {
-  const int blocks = (n + 3) / 4;
-  KernelScope scope(lc, KID_HEADS_FWD);
-  cudaStream_t st = lc.st;
-  const float* bpi = theta + nd.pi_b; const float* bv = theta + nd.v_b;
-  const bool aligned = nd.pi_w % 8 == 0;      // 16-byte loads of the policy rows
-  if (prec == PAAC_BF16 && nd.F == 512 && aligned)
-    launch_kernel(lc, heads_kernel<bf16, bf16, 16>, blocks, 128, 0, (const bf16*)h, theta16 + nd.pi_w, bpi, theta16 + nd.v_w, bv, n,
-                                                         nd.A, logits, values, seed, step_base, t, forced, actions, sampled, uniforms, mode);
-  else if (prec == PAAC_BF16 && nd.F == 256 && aligned)
-    launch_kernel(lc, heads_kernel<bf16, bf16, 8>, blocks, 128, 0, (const bf16*)h, theta16 + nd.pi_w, bpi, theta16 + nd.v_w, bv, n,
-                                                        nd.A, logits, values, seed, step_base, t, forced, actions, sampled, uniforms, mode);
-  else if (prec == PAAC_BF16)
-    launch_kernel(lc, heads_slow_kernel<bf16, bf16>, blocks, 128, 0, (const bf16*)h, theta16 + nd.pi_w, bpi, theta16 + nd.v_w, bv,
-                                                          n, nd.F, nd.A, logits, values, seed, step_base, t, forced, actions,
-                                                          sampled, uniforms, mode);
-  else
-    launch_kernel(lc, heads_slow_kernel<float, float>, blocks, 128, 0, (const float*)h, theta + nd.pi_w, bpi, theta + nd.v_w, bv,
-                                                            n, nd.F, nd.A, logits, values, seed, step_base, t, forced, actions,
-                                                            sampled, uniforms, mode);
 }
 
 // One warp per experience i = (t, e).  Lane 0 first walks the environment's transitions backwards from the bootstrap

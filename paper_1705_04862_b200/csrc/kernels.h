@@ -28,16 +28,24 @@ void launch_env_step_sampling(LaunchCtx& lc, uint64_t seed, int n_e, const uint6
 
 void launch_advance_step(LaunchCtx& lc, uint64_t* step_base, uint32_t by);
 
+// ---- weight gradients as split-k partial sums --------------------------------------------
+// The weight-gradient kernels leave partial sums part[split][J][CO] (J = 1 for biases) in scratch regions of their own
+// and note them in a GradSegments list; finish_gradients() adds them up, splits in a fixed order, into the gradient
+// vector (dst[co * J + j], times scale) with one launch and empties the list.
+struct GradSegment { const float* part; float* dst; int splits, J, CO; float scale; int first_group, groups, wide; };
+struct GradSegments { GradSegment seg[12]; int n; int total_groups; };
+bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale);   // false: list full
+// sumsq_partials != nullptr: every block also leaves the sum of squares of the gradient values it wrote in
+// sumsq_partials[block]; returns the number of blocks launched
+int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials);
+
 // ---- network on the CUDA cores (net_simt.cu) --------------------------------------------
-// act[l]: stored activation of layer l for the n states, storage float (PAAC_FP32) or bf16
-// scratch: simt_scratch_floats() floats for the split-k partial sums of the fully connected layer (nullptr: no split)
-void simt_forward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta,
-                  const bf16* theta16, const uint8_t* frames, int n, void* const act[], float* scratch);
-// from gact[fc] (gradient at the fc pre-activation) down to conv1; fills grad for conv and fc layers
-void simt_backward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta,
-                   const bf16* theta16, const uint8_t* frames, int n, void* const act[], void* const gact[],
-                   float* grad, float* scratch);
-// scratch floats simt_backward / heads_backward (n states) and simt_forward (n_fwd states) need for split-k partials
+// act[l]: stored activation of layer l for the n states, storage float (PAAC_FP32) or bf16.  Returns the number of split-k
+// partial sums [split][n][F] the fully connected layer was left as in scratch (simt_scratch_floats() floats), for
+// launch_simt_tail to finish; 0: the layer is complete.
+int simt_forward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta,
+                 const bf16* theta16, const uint8_t* frames, int n, void* const act[], float* scratch);
+// scratch floats simt_backward_layer / heads_backward (n states) and simt_forward (n_fwd states) need for split-k partials
 size_t simt_scratch_floats(int arch, const NetDims& nd, int n, int n_fwd);
 
 // ---- network on the tensor cores (net_tc.cu): Nature CNN, bf16 ------------------------------
@@ -65,11 +73,8 @@ void tc_backward_dgrad_conv3(LaunchCtx& lc, const bf16* images, int n, void* con
 void tc_backward_dgrad_conv2(LaunchCtx& lc, const bf16* images, int n, void* const act[], void* const gact[], uint32_t* err,
                              float out_scale);
 float tc_conv1_grad_scale();
-// weight + bias gradient of one layer (0 = conv1 .. 3 = fc) as split-k partial sums in its own region of a
-// scratch of tc_scratch_floats(B) floats; the regions are noted in a GradSegments list, and
-// tc_backward_finish() adds them up into the gradient vector with one launch and empties the list
-struct GradSegment { const float* part; float* dst; int splits, J, CO; float scale; int first_group, groups, wide; };
-struct GradSegments { GradSegment seg[12]; int n; int total_groups; };
+// weight + bias gradients of one layer (0 = conv1 .. 3 = fc) as partial sums in the layer's own region of a scratch of
+// tc_scratch_floats(B) floats, noted in the GradSegments list
 size_t tc_scratch_floats(int n);
 // frame stack: out = (three newest channels of prev, newest plane), or four copies of the plane where restart[e] != 0
 void launch_stack_push(LaunchCtx& lc, const uint8_t* prev, const uint8_t* newest, const uint8_t* restart /* nullable */,
@@ -82,11 +87,8 @@ void tc_backward_conv2d_conv1w_chunked(LaunchCtx& lc, const NetDims& nd, const b
                                        GradSegments* segs, uint32_t* err);
 void tc_backward_wgrad(LaunchCtx& lc, const NetDims& nd, const uint8_t* frames, int n, void* const act[],
                        void* const gact[], float* grad, float* scratch, int layer, GradSegments* segs, uint32_t* err);
-// sumsq_partials != nullptr: every block also leaves the sum of squares of the gradient values it wrote in
-// sumsq_partials[block]; returns the number of blocks launched
-int tc_backward_finish(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials);
 // both heads in one kernel: gradient at the fc pre-activation into g_fc, the heads' parameter gradients as one more
-// set of partial sums for tc_backward_finish()
+// set of partial sums for finish_gradients()
 bool tc_heads_backward_supported(const NetDims& nd);
 void tc_heads_backward(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, const bf16* h, int n, const float* dz,
                        const float* dV, bf16* g_fc, float* grad, float* scratch, GradSegments* segs);
@@ -94,14 +96,19 @@ void tc_heads_backward(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, co
 // kernel of its own yet)
 void simt_backward_layer(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta, const bf16* theta16,
                          const uint8_t* frames, int n, void* const act[], void* const gact[], float* grad,
-                         float* scratch, int layer, bool wgrad, bool dgrad);
+                         float* scratch, GradSegments* segs, int layer, bool wgrad, bool dgrad);
 
 // ---- heads, sampling, returns, loss gradient (heads.cu) -----------------------------------
-// logits/values of n states from the fc activation; if actions != nullptr also samples
-void launch_heads(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta,
-                  const bf16* theta16, const void* h, int n, float* logits, float* values, uint64_t seed,
-                  const uint64_t* step_base /* device */, uint32_t t, const int32_t* forced, int32_t* actions, int32_t* sampled /* action before forcing */,
-                  float* uniforms, HeadMode mode);
+// The end of a forward pass on the CUDA cores (see simt_forward): logits / values of n states from the fully connected
+// layer's partial sums (splits > 0; h is then written too) or from h; if actions != nullptr also samples; with `env` (and
+// sampling) also steps the synthetic environments with the sampled actions.  advance_step: as in launch_heads_fused.
+struct EnvStepArgs {
+  uint32_t term_denom; uint8_t* next_frames; int8_t* rewards; uint8_t* terminals; int32_t* counters; int pattern_actions;
+};
+void launch_simt_tail(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const float* part, int splits,
+                      void* h, int n, float* logits, float* values, uint64_t seed, const uint64_t* step_base, uint32_t t,
+                      const int32_t* forced, int32_t* actions, int32_t* sampled /* action before forcing */, float* uniforms,
+                      HeadMode mode, const EnvStepArgs* env, uint64_t* advance_step, uint32_t advance_by);
 // the same for the tensor-core path, which leaves the fully connected layer as split-k partial sums
 // part[split][n][F]: finishes h (sum, bias, ReLU, bf16) into h_out on the way
 bool heads_fused_supported(const NetDims& nd);
@@ -120,7 +127,7 @@ void launch_returns_head_grad(LaunchCtx& lc, HeadMode mode, int n_e, int t_max, 
 // gradient of the two heads' parameters and of the fc pre-activation
 void heads_backward(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta,
                     const bf16* theta16, const void* h, int n, const float* dz, const float* dV, void* gact_fc,
-                    float* grad, float* scratch);
+                    float* grad, float* scratch, GradSegments* segs);
 
 // ---- optimiser (optim.cu) -------------------------------------------------------------------
 constexpr int NORM_BLOCKS = 1184;

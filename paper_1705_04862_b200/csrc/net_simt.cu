@@ -1,10 +1,14 @@
 // The network's layers as contractions on the CUDA cores (float accumulate):
 // forward with fused bias + ReLU, data gradients with the ReLU mask of the layer
 // below fused, weight gradients as split-k partial sums reduced in a fixed order.
+#include "gemm_ffma.cuh"
 #include "gemm_tc3.cuh"
 #include "kernels.h"
 
 namespace paac {
+
+// the three-pass tensor-core kernel instead of the CUDA cores (an option)
+static bool use_tc3(const LaunchCtx& lc) { return lc.fp32_tensor_cores && lc.error_word != nullptr; }
 
 static int pick_splits(int M, int N, int K) {
   const int blocks = ((M + SG_BM - 1) / SG_BM) * ((N + SG_BN - 1) / SG_BN);
@@ -13,7 +17,7 @@ static int pick_splits(int M, int N, int K) {
   if (s > by_k) s = by_k;
   if (s > 512) s = 512;
   if (s < 1) s = 1;
-  return gemm_simt_splits(K, s);
+  return gemm_k_splits(K, s);
 }
 
 static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_rows, int row0,
@@ -25,99 +29,169 @@ static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_
   launch_kernel(lc, wgrad_reduce_kernel, blocks, 256, 0, part, splits, part_rows, row0, rows, cols, scale, gw, gb);
 }
 
+// Tiles of the CUDA-core contraction for N columns (16, 32, 64 or many): four warps of 32 x 8 TN outputs each.  With
+// enough rows for two CTAs per SM they cover 128 (N <= 32) or 64 rows; with fewer rows two or all four of them share a
+// tile and split every k block between them, so that a batch of a few states still gives every SM its warps; below one
+// CTA per SM eight warps do, and the k blocks are as many times longer: such a launch is a chain of load latencies, one
+// per block.
+constexpr int FF_SMS = 148;
+static size_t ff_heads_scratch_floats(const NetDims& nd, int n);
+template <int N, class LA, class LB, class EP>
+static void ff_rows(LaunchCtx& lc, int kid, int M, int n_cols, int K, int classes, LA la, LB lb, EP ep) {
+  const int cols = (n_cols + N - 1) / N * classes;
+  if constexpr (N <= 32) {
+    constexpr int TN = N / 8;
+    if ((M + 127) / 128 * cols >= 2 * FF_SMS) gemm_ffma<4, 1, TN, 1>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+    else if ((M + 63) / 64 * cols >= FF_SMS) gemm_ffma<2, 1, TN, 2>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+    else if ((M + 31) / 32 * cols >= FF_SMS) gemm_ffma<1, 1, TN, 4>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+    else gemm_ffma<1, 1, TN, 8>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+  } else {
+    if ((M + 63) / 64 * cols >= 2 * FF_SMS) gemm_ffma<2, 2, 4, 1>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+    else if ((M + 31) / 32 * cols >= FF_SMS) gemm_ffma<1, 2, 4, 2>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+    else gemm_ffma<1, 2, 4, 4>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+  }
+}
+
+// Weight gradients: C(j, co) = sum over output positions of window(j) * gradient(co), one run of positions per split;
+// the splits' sums (and the bias gradient's, the column sums of the second operand) are added by finish_gradients().
+struct FfWgradPlan { int splits, kps; size_t part, total; };      // floats: the weights' partial sums, and all of them
+static int ff_wgrad_tiles(int J, int CO) { return CO <= 32 ? (J + 127) / 128 : ((J + 63) / 64) * ((CO + 63) / 64); }
+static FfWgradPlan ff_wgrad_plan(int J, int CO, int K) {
+  int s = 2 * FF_SMS / ff_wgrad_tiles(J, CO);
+  const int by_k = (K + 63) / 64;
+  if (s > by_k) s = by_k;
+  if (s < 1) s = 1;
+  FfWgradPlan p;
+  p.kps = ffma_k_per_split(K, s, 16);
+  p.splits = (K + p.kps - 1) / p.kps;
+  p.part = (size_t)p.splits * J * CO;
+  p.total = (p.part + (size_t)p.splits * CO + 63) / 64 * 64;
+  return p;
+}
+template <int CO_TILE, class LA, class LB>
+static void ff_wgrad(LaunchCtx& lc, int kid, int J, int CO, int K, LA window, LB grad_rows, float scale, float* gw, float* gb,
+                     float* scratch, GradSegments* segs) {
+  const FfWgradPlan p = ff_wgrad_plan(J, CO, K);
+  FfPartialColsum ep;
+  ep.part = scratch; ep.M = J; ep.N = CO; ep.colpart = scratch + p.part;
+  if constexpr (CO_TILE <= 32) gemm_ffma<4, 1, CO_TILE / 8, 1>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else gemm_ffma<2, 2, 4, 1>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  if (!add_grad_segment(segs, scratch, gw, p.splits, J, CO, scale) || !add_grad_segment(segs, ep.colpart, gb, p.splits, 1, CO, 1.f))
+    lc.host_failure = true;
+}
+
 template <class G, class TIn, class T, class TW>
 static void conv_fwd(LaunchCtx& lc, int kid, const TIn* x, const TW* w, const float* bias, T* out, int n,
                      float scale) {
-  gemm_f32(lc, kid, n * G::OH * G::OW, G::CO, G::KK, 1, ConvWindowOp<G, TIn>{x}, RowMajorOp<TW>{w, G::KK},
-            BiasReluEp<T>{out, bias, G::CO, scale});
+  if (use_tc3(lc))
+    gemm_tc3(lc, kid, n * G::OH * G::OW, G::CO, G::KK, 1, ConvWindowOp<G, TIn>{x}, RowMajorOp<TW>{w, G::KK}, BiasReluEp<T>{out, bias, G::CO, scale});
+  else
+    ff_rows<G::CO>(lc, kid, n * G::OH * G::OW, G::CO, G::KK, 1, FfWindow<G, TIn>{x}, FfRows<TW>{w, G::KK}, FfBiasRelu<T>{out, bias, G::CO, scale});
 }
-// out[m][n] = relu(sum over splits (in order) of part[split][m][n] + bias[n])
-template <class T>
-static __global__ void fc_finish_simt_kernel(const float* __restrict__ part, int splits, int M, int N,
-                                             const float* __restrict__ bias, T* __restrict__ out) {
-  pdl_entry();
-  const size_t total = (size_t)M * N;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    // the partial sums are added in double: the pre-activation then differs from an exactly rounded one only by the
-    // error inside each short partial sum, and fewer units near zero end up on the other side of the ReLU
-    double s = 0.0;
-    for (int p = 0; p < splits; ++p) s += (double)part[(size_t)p * total + i];
-    out[i] = from_f<T>(fmaxf((float)(s + (double)bias[i % N]), 0.f));
-  }
+// With few states the fully connected layer is a handful of tiles over a reduction of thousands: the reduction is then
+// split over many blocks (partial sums in scratch, added by launch_simt_tail) so that the weight matrix is streamed by
+// the whole device instead of by four blocks.  Returns the number of splits left in scratch (0: the layer is complete).
+static int fc_fwd_splits(int n, int F, int IN, int* kps) {
+  // as many splits as give every SM four CTAs, each at least 64 long
+  int s = 4 * FF_SMS / (((n + 31) / 32) * ((F + 63) / 64));
+  if (s > (IN + 63) / 64) s = (IN + 63) / 64;
+  if (s < 1) s = 1;
+  *kps = ffma_k_per_split(IN, s, 32);
+  return (IN + *kps - 1) / *kps;
 }
-// With few states the fully connected layer is a handful of 64 x 64 tiles over a reduction of thousands: the
-// reduction is then split over many blocks (partial sums in scratch, added in a fixed order by a finishing kernel)
-// so that the weight matrix is streamed by the whole device instead of by four blocks.
 template <class T, class TW>
-static void fc_fwd(LaunchCtx& lc, int kid, const T* x, const TW* w, const float* bias, T* out, int n,
+static int fc_fwd(LaunchCtx& lc, int kid, const T* x, const TW* w, const float* bias, T* out, int n,
                    int IN, int F, float* scratch) {
-  const int splits = scratch != nullptr ? pick_splits(n, F, IN) : 1;
-  if (splits <= 1) {
-    gemm_f32(lc, kid, n, F, IN, 1, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, BiasReluEp<T>{out, bias, F, 1.f});
-    return;
+  int splits = 1;
+  if (use_tc3(lc)) {
+    splits = pick_splits(n, F, IN);
+    if (splits <= 1) {
+      gemm_tc3(lc, kid, n, F, IN, 1, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, BiasReluEp<T>{out, bias, F, 1.f});
+      return 0;
+    }
+    gemm_tc3(lc, kid, n, F, IN, splits, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, PartialEp{scratch, n, F});
+  } else {
+    int kps = IN;
+    splits = fc_fwd_splits(n, F, IN, &kps);
+    if (splits <= 1) {
+      gemm_ffma<2, 2, 4, 1>(lc, kid, n, F, IN, IN, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfBiasRelu<T>{out, bias, F, 1.f});
+      return 0;
+    }
+    gemm_ffma<1, 2, 4, 2>(lc, kid, n, F, IN, kps, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfPartial{scratch, n, F});
   }
-  gemm_f32(lc, kid, n, F, IN, splits, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, PartialEp{scratch, n, F});
-  KernelScope scope(lc, kid);
-  int blocks = (n * F + 255) / 256;
-  if (blocks > 1184) blocks = 1184;
-  launch_kernel(lc, fc_finish_simt_kernel<T>, blocks, 256, 0, scratch, splits, n, F, bias, out);
+  return splits;
 }
 template <class G, class T, class TW>
 static void conv_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T* act_in, T* gin, int n) {
   if constexpr (G::S == 2 && G::K == 4 && G::H % 2 == 0 && G::W % 2 == 0) {
     // four parity classes, each a dense contraction over its own four taps (a quarter of the multiply-adds)
-    for (int z = 0; z < 4; ++z)
-      gemm_f32(lc, kid, n * (G::H / 2) * (G::W / 2), G::C, 4 * G::CO, 1, ConvDgradClassOp<G, T>{g, z >> 1, z & 1},
-                ConvWeightClassOp<G, TW>{w, z >> 1, z & 1}, ReluMaskClassEp<G, T>{gin, act_in, z >> 1, z & 1});
+    const int M = n * (G::H / 2) * (G::W / 2), K = 4 * G::CO;
+    if (use_tc3(lc))
+      for (int z = 0; z < 4; ++z)
+        gemm_tc3(lc, kid, M, G::C, K, 1, ConvDgradClassOp<G, T>{g, z >> 1, z & 1}, ConvWeightClassOp<G, TW>{w, z >> 1, z & 1},
+                 ReluMaskClassEp<G, T>{gin, act_in, z >> 1, z & 1});
+    else
+      ff_rows<G::C>(lc, kid, M, G::C, K, 4, FfDgradClass<G, T>{g}, FfWeightClass<G, TW>{w, 0}, FfReluMaskClass<G, T>{gin, act_in, 0});
     return;
   }
-  gemm_f32(lc, kid, n * G::H * G::W, G::C, G::K * G::K * G::CO, 1, ConvDgradOp<G, T>{g}, ConvWeightTOp<G, TW>{w},
-            ReluMaskEp<T>{gin, act_in, G::C});
+  const int M = n * G::H * G::W, K = G::K * G::K * G::CO;
+  if (use_tc3(lc)) gemm_tc3(lc, kid, M, G::C, K, 1, ConvDgradOp<G, T>{g}, ConvWeightTOp<G, TW>{w}, ReluMaskEp<T>{gin, act_in, G::C});
+  else ff_rows<G::C>(lc, kid, M, G::C, K, 1, FfDgradWindow<G, T>{g}, FfWeightT<G, TW>{w}, FfReluMask<T>{gin, act_in, G::C});
 }
 template <class G, class TIn, class T>
 static void conv_wgrad(LaunchCtx& lc, int kid, const T* g, const TIn* x, int n, float scale, float* gw,
-                       float* gb, float* scratch) {
-  const int M = G::CO, N = G::KK + 1, K = n * G::OH * G::OW;
+                       float* gb, float* scratch, GradSegments* segs) {
+  const int K = n * G::OH * G::OW;
+  if (!use_tc3(lc)) {
+    ff_wgrad<G::CO>(lc, kid, G::KK, G::CO, K, FfWindowT<G, TIn>{x}, FfCols<T>{g, G::CO}, scale, gw, gb, scratch, segs);
+    return;
+  }
+  const int M = G::CO, N = G::KK + 1;
   const int splits = pick_splits(M, N, K);
-  gemm_f32(lc, kid, M, N, K, splits, ColMajorOp<T>{g, G::CO}, ConvWindowTOp<G, TIn>{x}, PartialEp{scratch, M, N});
+  gemm_tc3(lc, kid, M, N, K, splits, ColMajorOp<T>{g, G::CO}, ConvWindowTOp<G, TIn>{x}, PartialEp{scratch, M, N});
   reduce_wgrad(lc, scratch, splits, M, 0, M, G::KK, scale, gw, gb);
 }
 template <class T, class TW>
 static void fc_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T* act_in, T* gin, int n,
                      int IN, int F) {
-  gemm_f32(lc, kid, n, IN, F, 1, RowMajorOp<T>{g, F}, ColMajorOp<TW>{w, IN}, ReluMaskEp<T>{gin, act_in, IN});
+  if (use_tc3(lc)) gemm_tc3(lc, kid, n, IN, F, 1, RowMajorOp<T>{g, F}, ColMajorOp<TW>{w, IN}, ReluMaskEp<T>{gin, act_in, IN});
+  else ff_rows<64>(lc, kid, n, IN, F, 1, FfRows<T>{g, F}, FfCols<TW>{w, IN}, FfReluMask<T>{gin, act_in, IN});
 }
 template <class T>
 static void fc_wgrad(LaunchCtx& lc, int kid, const T* g, const T* x, int n, int IN, int F, float* gw,
-                     float* gb, float* scratch) {
+                     float* gb, float* scratch, GradSegments* segs) {
+  if (!use_tc3(lc)) {
+    ff_wgrad<64>(lc, kid, IN, F, n, FfCols<T>{x, IN}, FfCols<T>{g, F}, 1.f, gw, gb, scratch, segs);
+    return;
+  }
   const int M = F, N = IN + 1, K = n;
   const int splits = pick_splits(M, N, K);
-  gemm_f32(lc, kid, M, N, K, splits, ColMajorOp<T>{g, F}, ColMajorOnesOp<T>{x, IN, IN}, PartialEp{scratch, M, N});
+  gemm_tc3(lc, kid, M, N, K, splits, ColMajorOp<T>{g, F}, ColMajorOnesOp<T>{x, IN, IN}, PartialEp{scratch, M, N});
   reduce_wgrad(lc, scratch, splits, M, 0, M, IN, 1.f, gw, gb);
 }
 
 template <class T, class TW>
-static void forward_t(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, const TW* w,
+static int forward_t(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, const TW* w,
                       const uint8_t* frames, int n, void* const act[], float* scratch) {
   const LayerDims* d = nd.layer;
   const float s255 = 1.0f / 255.0f;
   if (arch == PAAC_ARCH_NIPS) {
     conv_fwd<NipsConv1, uint8_t, T, TW>(lc, KID_CONV1_FWD, frames, w + d[0].w_off, theta + d[0].b_off, (T*)act[0], n, s255);
     conv_fwd<NipsConv2, T, T, TW>(lc, KID_CONV2_FWD, (const T*)act[0], w + d[1].w_off, theta + d[1].b_off, (T*)act[1], n, 1.f);
-    fc_fwd<T, TW>(lc, KID_FC_FWD, (const T*)act[1], w + d[2].w_off, theta + d[2].b_off, (T*)act[2], n, 2592, 256, scratch);
+    return fc_fwd<T, TW>(lc, KID_FC_FWD, (const T*)act[1], w + d[2].w_off, theta + d[2].b_off, (T*)act[2], n, 2592, 256, scratch);
   } else {
     conv_fwd<NatConv1, uint8_t, T, TW>(lc, KID_CONV1_FWD, frames, w + d[0].w_off, theta + d[0].b_off, (T*)act[0], n, s255);
     conv_fwd<NatConv2, T, T, TW>(lc, KID_CONV2_FWD, (const T*)act[0], w + d[1].w_off, theta + d[1].b_off, (T*)act[1], n, 1.f);
     conv_fwd<NatConv3, T, T, TW>(lc, KID_CONV3_FWD, (const T*)act[1], w + d[2].w_off, theta + d[2].b_off, (T*)act[2], n, 1.f);
-    fc_fwd<T, TW>(lc, KID_FC_FWD, (const T*)act[2], w + d[3].w_off, theta + d[3].b_off, (T*)act[3], n, 3136, 512, scratch);
+    return fc_fwd<T, TW>(lc, KID_FC_FWD, (const T*)act[2], w + d[3].w_off, theta + d[3].b_off, (T*)act[3], n, 3136, 512, scratch);
   }
 }
 
 // one layer of the backward pass: its weight gradient and/or the data gradient handed to the layer below
 template <class T, class TW>
 static void backward_layer_t(LaunchCtx& lc, int arch, const NetDims& nd, const TW* w, const uint8_t* frames, int n,
-                             void* const act[], void* const gact[], float* grad, float* scratch, int l, bool wg,
-                             bool dg) {
+                             void* const act[], void* const gact[], float* grad, float* scratch, GradSegments* segs, int l,
+                             bool wg, bool dg) {
   const LayerDims* d = nd.layer;
   const float s255 = 1.0f / 255.0f;
   const T* g = (const T*)gact[l];
@@ -127,54 +201,62 @@ static void backward_layer_t(LaunchCtx& lc, int arch, const NetDims& nd, const T
   const TW* wl = w + d[l].w_off;
   if (arch == PAAC_ARCH_NIPS) {
     if (l == 2) {
-      if (wg) fc_wgrad<T>(lc, KID_FC_WGRAD, g, x, n, 2592, 256, gw, gb, scratch);
+      if (wg) fc_wgrad<T>(lc, KID_FC_WGRAD, g, x, n, 2592, 256, gw, gb, scratch, segs);
       if (dg) fc_dgrad<T, TW>(lc, KID_FC_DGRAD, g, wl, x, gin, n, 2592, 256);
     } else if (l == 1) {
-      if (wg) conv_wgrad<NipsConv2, T, T>(lc, KID_CONV2_WGRAD, g, x, n, 1.f, gw, gb, scratch);
+      if (wg) conv_wgrad<NipsConv2, T, T>(lc, KID_CONV2_WGRAD, g, x, n, 1.f, gw, gb, scratch, segs);
       if (dg) conv_dgrad<NipsConv2, T, TW>(lc, KID_CONV2_DGRAD, g, wl, x, gin, n);
     } else if (wg) {
-      conv_wgrad<NipsConv1, uint8_t, T>(lc, KID_CONV1_WGRAD, g, frames, n, s255, gw, gb, scratch);
+      conv_wgrad<NipsConv1, uint8_t, T>(lc, KID_CONV1_WGRAD, g, frames, n, s255, gw, gb, scratch, segs);
     }
   } else {
     if (l == 3) {
-      if (wg) fc_wgrad<T>(lc, KID_FC_WGRAD, g, x, n, 3136, 512, gw, gb, scratch);
+      if (wg) fc_wgrad<T>(lc, KID_FC_WGRAD, g, x, n, 3136, 512, gw, gb, scratch, segs);
       if (dg) fc_dgrad<T, TW>(lc, KID_FC_DGRAD, g, wl, x, gin, n, 3136, 512);
     } else if (l == 2) {
-      if (wg) conv_wgrad<NatConv3, T, T>(lc, KID_CONV3_WGRAD, g, x, n, 1.f, gw, gb, scratch);
+      if (wg) conv_wgrad<NatConv3, T, T>(lc, KID_CONV3_WGRAD, g, x, n, 1.f, gw, gb, scratch, segs);
       if (dg) conv_dgrad<NatConv3, T, TW>(lc, KID_CONV3_DGRAD, g, wl, x, gin, n);
     } else if (l == 1) {
-      if (wg) conv_wgrad<NatConv2, T, T>(lc, KID_CONV2_WGRAD, g, x, n, 1.f, gw, gb, scratch);
+      if (wg) conv_wgrad<NatConv2, T, T>(lc, KID_CONV2_WGRAD, g, x, n, 1.f, gw, gb, scratch, segs);
       if (dg) conv_dgrad<NatConv2, T, TW>(lc, KID_CONV2_DGRAD, g, wl, x, gin, n);
     } else if (wg) {
-      conv_wgrad<NatConv1, uint8_t, T>(lc, KID_CONV1_WGRAD, g, frames, n, s255, gw, gb, scratch);
+      conv_wgrad<NatConv1, uint8_t, T>(lc, KID_CONV1_WGRAD, g, frames, n, s255, gw, gb, scratch, segs);
     }
   }
 }
 
+// Where layer l's partial sums start in the update's scratch (a region of its own for every layer, since they are kept
+// until finish_gradients() has run); l = number of layers: the heads' region; one more: the end.
+static size_t ff_scratch_offset(const NetDims& nd, int n, int l) {
+  size_t off = 0;
+  for (int q = 0; q < l && q <= nd.n_conv; ++q) {
+    const LayerDims& d = nd.layer[q];
+    off += ff_wgrad_plan(q < nd.n_conv ? d.K * d.K * d.C : d.H * d.W * d.C, d.CO, n * d.OH * d.OW).total;
+  }
+  if (l > nd.n_conv + 1) off += ff_heads_scratch_floats(nd, n);
+  return off;
+}
+
 void simt_backward_layer(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta, const bf16* theta16,
                          const uint8_t* frames, int n, void* const act[], void* const gact[], float* grad,
-                         float* scratch, int layer, bool wgrad, bool dgrad) {
+                         float* scratch, GradSegments* segs, int layer, bool wgrad, bool dgrad) {
+  float* sc = use_tc3(lc) ? scratch : scratch + ff_scratch_offset(nd, n, layer);
   if (prec == PAAC_BF16)
-    backward_layer_t<bf16, bf16>(lc, arch, nd, theta16, frames, n, act, gact, grad, scratch, layer, wgrad, dgrad);
+    backward_layer_t<bf16, bf16>(lc, arch, nd, theta16, frames, n, act, gact, grad, sc, segs, layer, wgrad, dgrad);
   else
-    backward_layer_t<float, float>(lc, arch, nd, theta, frames, n, act, gact, grad, scratch, layer, wgrad, dgrad);
+    backward_layer_t<float, float>(lc, arch, nd, theta, frames, n, act, gact, grad, sc, segs, layer, wgrad, dgrad);
 }
 
-void simt_forward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta,
-                  const bf16* theta16, const uint8_t* frames, int n, void* const act[], float* scratch) {
-  if (prec == PAAC_BF16) forward_t<bf16, bf16>(lc, arch, nd, theta, theta16, frames, n, act, scratch);
-  else forward_t<float, float>(lc, arch, nd, theta, theta, frames, n, act, scratch);
-}
-
-void simt_backward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta,
-                   const bf16* theta16, const uint8_t* frames, int n, void* const act[], void* const gact[],
-                   float* grad, float* scratch) {
-  for (int l = nd.n_conv; l >= 0; --l)
-    simt_backward_layer(lc, arch, prec, nd, theta, theta16, frames, n, act, gact, grad, scratch, l, true, l > 0);
+int simt_forward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta,
+                 const bf16* theta16, const uint8_t* frames, int n, void* const act[], float* scratch) {
+  if (prec == PAAC_BF16) return forward_t<bf16, bf16>(lc, arch, nd, theta, theta16, frames, n, act, scratch);
+  return forward_t<float, float>(lc, arch, nd, theta, theta, frames, n, act, scratch);
 }
 
 size_t simt_scratch_floats(int arch, const NetDims& nd, int n, int n_fwd) {
-  size_t best = 0;
+  (void)arch;
+  // an update on the CUDA cores keeps all its partial sums; one through the three-pass kernel finishes layer by layer
+  size_t best = ff_scratch_offset(nd, n, nd.n_conv + 2);
   for (int l = 0; l <= nd.n_conv; ++l) {
     const LayerDims& d = nd.layer[l];
     const int M = d.CO;
@@ -184,11 +266,14 @@ size_t simt_scratch_floats(int arch, const NetDims& nd, int n, int n_fwd) {
     if (need > best) best = need;
   }
   const size_t heads = (size_t)pick_splits(nd.A + 1, nd.F + 1, n) * (nd.A + 1) * (nd.F + 1);
-  (void)arch;
   if (heads > best) best = heads;
   // split-k partial sums of the fully connected layer's forward pass, which only ever sees n_fwd states at a time
   const LayerDims& f = nd.layer[nd.n_conv];
-  const size_t fwd = (size_t)pick_splits(n_fwd, nd.F, f.H * f.W * f.C) * n_fwd * nd.F;
+  const int IN = f.H * f.W * f.C;
+  int kps = 0, fs = fc_fwd_splits(n_fwd, nd.F, IN, &kps);
+  const int t3 = pick_splits(n_fwd, nd.F, IN);
+  if (t3 > fs) fs = t3;
+  const size_t fwd = (size_t)fs * n_fwd * nd.F;
   return best > fwd ? best : fwd;
 }
 
@@ -211,26 +296,132 @@ template <class TW> struct HeadWeightOp {   // row = fc unit i, k = head unit
   }
 };
 
+// Both heads in one kernel, for either storage type and either hidden size (the tensor-core path has one of its own for
+// 512 bf16 units): with dz[b][k] the loss gradient at output k of row b (the value is row k = A of the combined matrix),
+//   g_fc[b][i] = (h[b][i] > 0) * sum_k dz[b][k] W[k][i],   dW[k][i] = sum_b dz[b][k] h[b][i],   db[k] = sum_b dz[b][k].
+// A thread owns hidden units tid, tid + 256; their weights and gradient sums stay in registers, so a row costs it one
+// load of h per unit and 2 NK multiply-adds.  A block walks FH_ROWS or more rows (few enough blocks that their partial
+// sums, one set each, do not outweigh the gradient) and fetches all rows of a group before it uses them.
+constexpr int FH_THREADS = 256, FH_ROWS = 8, FH_MAX_BLOCKS = 148;
+template <class T, class TW, int F, int NK>
+__global__ void __launch_bounds__(FH_THREADS, 1)
+heads_backward_kernel(const T* h, const float* dz, const float* dV, const TW* wpi, const TW* wv, int n, int A, int rows_per,
+                      T* g_fc, float* part_w, float* part_b, float* part_vw, float* part_vb) {
+  constexpr int U = F / FH_THREADS;
+  __shared__ __align__(16) float dzs[FH_ROWS][NK];
+  const int tid = threadIdx.x;
+  pdl_entry();
+  float w[NK][U], acc[NK][U], accb = 0.f;
+#pragma unroll
+  for (int k = 0; k < NK; ++k)
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int col = tid + u * FH_THREADS;
+      acc[k][u] = 0.f;
+      w[k][u] = k < A ? to_f(wpi[(size_t)k * F + col]) : (k == A ? to_f(wv[col]) : 0.f);
+    }
+  const int r0 = blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
+  for (int rb = r0; rb < r1; rb += FH_ROWS) {
+    float hv[FH_ROWS][U];
+#pragma unroll
+    for (int j = 0; j < FH_ROWS; ++j)
+#pragma unroll
+      for (int u = 0; u < U; ++u) hv[j][u] = rb + j < r1 ? to_f(h[(size_t)(rb + j) * F + tid + u * FH_THREADS]) : 0.f;
+    __syncthreads();
+    for (int i = tid; i < FH_ROWS * NK; i += FH_THREADS) {
+      const int r = rb + i / NK, k = i % NK;
+      dzs[i / NK][k] = r < r1 ? (k < A ? dz[(size_t)r * A + k] : (k == A ? dV[r] : 0.f)) : 0.f;
+    }
+    __syncthreads();
+    if (tid <= A)
+#pragma unroll
+      for (int j = 0; j < FH_ROWS; ++j) accb += dzs[j][tid];          // rows past the end hold zeros
+#pragma unroll
+    for (int j = 0; j < FH_ROWS; ++j) {
+      if (rb + j >= r1) break;
+      float g[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) g[u] = 0.f;
+#pragma unroll
+      for (int k = 0; k < NK; ++k) {
+        const float d = dzs[j][k];
+#pragma unroll
+        for (int u = 0; u < U; ++u) { g[u] = fmaf(d, w[k][u], g[u]); acc[k][u] = fmaf(d, hv[j][u], acc[k][u]); }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        g_fc[(size_t)(rb + j) * F + tid + u * FH_THREADS] = from_f<T>(hv[j][u] > 0.f ? g[u] : 0.f);
+    }
+  }
+  const size_t cta = blockIdx.x;
+#pragma unroll
+  for (int k = 0; k < NK; ++k)
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int col = tid + u * FH_THREADS;
+      if (k < A) part_w[(cta * A + k) * F + col] = acc[k][u];
+      else if (k == A) part_vw[cta * F + col] = acc[k][u];
+    }
+  if (tid < A) part_b[cta * A + tid] = accb;
+  else if (tid == A) part_vb[cta] = accb;
+}
+static int ff_heads_blocks(int n, int* rows_per) {
+  int blocks = (n + FH_ROWS - 1) / FH_ROWS;
+  if (blocks > FH_MAX_BLOCKS) blocks = FH_MAX_BLOCKS;
+  *rows_per = (n + blocks - 1) / blocks;
+  return (n + *rows_per - 1) / *rows_per;
+}
+static size_t ff_heads_scratch_floats(const NetDims& nd, int n) {
+  int rows = 0;
+  return (size_t)ff_heads_blocks(n, &rows) * (nd.A + 1) * (nd.F + 1) + 8;
+}
+
 template <class T, class TW>
 static void heads_backward_t(LaunchCtx& lc, const NetDims& nd, const TW* w, const T* h, int n,
-                             const float* dz, const float* dV, T* gact_fc, float* grad, float* scratch) {
+                             const float* dz, const float* dV, T* gact_fc, float* grad, float* scratch, GradSegments* segs) {
   const int A = nd.A, F = nd.F;
-  gemm_f32(lc, KID_HEADS_BWD, n, F, A + 1, 1, HeadGradOp{dz, dV, A}, HeadWeightOp<TW>{w + nd.pi_w, w + nd.v_w, F, A},
-            ReluMaskEp<T>{gact_fc, h, F});
-  const int splits = pick_splits(A + 1, F + 1, n);
-  gemm_f32(lc, KID_HEADS_BWD, A + 1, F + 1, n, splits, HeadGradTOp{dz, dV, A}, ColMajorOnesOp<T>{h, F, F},
-            PartialEp{scratch, A + 1, F + 1});
-  reduce_wgrad(lc, scratch, splits, A + 1, 0, A, F, 1.f, grad + nd.pi_w, grad + nd.pi_b);
-  reduce_wgrad(lc, scratch, splits, A + 1, A, 1, F, 1.f, grad + nd.v_w, grad + nd.v_b);
+  if (use_tc3(lc)) {
+    gemm_tc3(lc, KID_HEADS_BWD, n, F, A + 1, 1, HeadGradOp{dz, dV, A}, HeadWeightOp<TW>{w + nd.pi_w, w + nd.v_w, F, A},
+              ReluMaskEp<T>{gact_fc, h, F});
+    const int splits = pick_splits(A + 1, F + 1, n);
+    gemm_tc3(lc, KID_HEADS_BWD, A + 1, F + 1, n, splits, HeadGradTOp{dz, dV, A}, ColMajorOnesOp<T>{h, F, F},
+              PartialEp{scratch, A + 1, F + 1});
+    reduce_wgrad(lc, scratch, splits, A + 1, 0, A, F, 1.f, grad + nd.pi_w, grad + nd.pi_b);
+    reduce_wgrad(lc, scratch, splits, A + 1, A, 1, F, 1.f, grad + nd.v_w, grad + nd.v_b);
+    return;
+  }
+  int rows_per = 0;
+  const int blocks = ff_heads_blocks(n, &rows_per);
+  float* part_w = scratch + ff_scratch_offset(nd, n, nd.n_conv + 1);
+  float* part_b = part_w + (size_t)blocks * A * F;
+  float* part_vw = part_b + (size_t)blocks * A;
+  float* part_vb = part_vw + (size_t)blocks * F;
+  auto launch = [&](auto kern) {
+    KernelScope scope(lc, KID_HEADS_BWD);
+    launch_kernel_overlapped(lc, kern, dim3(blocks), dim3(FH_THREADS), 0, h, dz, dV, w + nd.pi_w, w + nd.v_w, n, A, rows_per,
+                             gact_fc, part_w, part_b, part_vw, part_vb);
+  };
+  if (F == 256) {
+    if (A < 8) launch(heads_backward_kernel<T, TW, 256, 8>);
+    else if (A < 20) launch(heads_backward_kernel<T, TW, 256, 20>);
+    else launch(heads_backward_kernel<T, TW, 256, 33>);
+  } else {
+    if (A < 8) launch(heads_backward_kernel<T, TW, 512, 8>);
+    else if (A < 20) launch(heads_backward_kernel<T, TW, 512, 20>);
+    else launch(heads_backward_kernel<T, TW, 512, 33>);
+  }
+  if (!add_grad_segment(segs, part_w, grad + nd.pi_w, blocks, 1, F * A, 1.f) || !add_grad_segment(segs, part_b, grad + nd.pi_b, blocks, 1, A, 1.f) ||
+      !add_grad_segment(segs, part_vw, grad + nd.v_w, blocks, 1, F, 1.f) || !add_grad_segment(segs, part_vb, grad + nd.v_b, blocks, 1, 1, 1.f))
+    lc.host_failure = true;
 }
 
 void heads_backward(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta,
                     const bf16* theta16, const void* h, int n, const float* dz, const float* dV, void* gact_fc,
-                    float* grad, float* scratch) {
+                    float* grad, float* scratch, GradSegments* segs) {
   if (prec == PAAC_BF16)
-    heads_backward_t<bf16, bf16>(lc, nd, theta16, (const bf16*)h, n, dz, dV, (bf16*)gact_fc, grad, scratch);
+    heads_backward_t<bf16, bf16>(lc, nd, theta16, (const bf16*)h, n, dz, dV, (bf16*)gact_fc, grad, scratch, segs);
   else
-    heads_backward_t<float, float>(lc, nd, theta, (const float*)h, n, dz, dV, (float*)gact_fc, grad, scratch);
+    heads_backward_t<float, float>(lc, nd, theta, (const float*)h, n, dz, dV, (float*)gact_fc, grad, scratch, segs);
 }
 
 }  // namespace paac

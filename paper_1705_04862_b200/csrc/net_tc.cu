@@ -2604,7 +2604,7 @@ __global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments seg
   }
 }
 
-static bool add_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale) {
+bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale) {
   if (segs->n >= (int)(sizeof(segs->seg) / sizeof(segs->seg[0]))) return false;      // the caller reports a host failure
   GradSegment& g = segs->seg[segs->n++];
   g.part = part; g.dst = dst; g.splits = splits; g.J = J; g.CO = CO; g.scale = scale;
@@ -2651,7 +2651,7 @@ static void tc_wgrad(LaunchCtx& lc, int kid, XSrc xs, GSrc gs, int rows, int n_a
   KernelScope scope(lc, kid);
   launch_kernel_overlapped(lc, kern, dim3(splits, gy, gz), TC_THREADS, smem, *tm_x, *tm_g, xs, gs, scratch, bias_part, n_atoms, J, CO,
                            num_blocks, bps, err);
-  if (!add_segment(segs, scratch, gw, splits, J, CO, scale) || !add_segment(segs, bias_part, gb, splits, 1, CO, 1.f))
+  if (!add_grad_segment(segs, scratch, gw, splits, J, CO, scale) || !add_grad_segment(segs, bias_part, gb, splits, 1, CO, 1.f))
     lc.host_failure = true;
 }
 
@@ -2867,7 +2867,7 @@ static void tc_shift_wgrad(LaunchCtx& lc, int kid, Cfg cfg, const bf16* g, int s
   float* bias_part = scratch + (size_t)splits * J * 64;
   KernelScope scope(lc, kid);
   launch_kernel_overlapped(lc, kern, splits, SWG_THREADS, smem, cfg, g, states, scratch, bias_part, tiles, per, err);
-  if (!add_segment(segs, scratch, gw, splits, J, 64, 1.f) || !add_segment(segs, bias_part, gb, splits, 1, 64, 1.f))
+  if (!add_grad_segment(segs, scratch, gw, splits, J, 64, 1.f) || !add_grad_segment(segs, bias_part, gb, splits, 1, 64, 1.f))
     lc.host_failure = true;
 }
 
@@ -3186,8 +3186,8 @@ static void tc_conv1_wgrad(LaunchCtx& lc, const uint8_t* frames, const bf16* g, 
   float* bias_part = scratch + (size_t)tc_conv1_wgrad_splits(n_states) * 256 * 32;
   const int splits = tc_conv1_wgrad_launch<G>(lc, frames, g, n_states, scratch, bias_part, err);
   // the gradient rows arrive multiplied by C1_GRAD_SCALE (see tc_backward_dgrad_conv2), the pixels as n * 2^-133
-  if (!add_segment(segs, scratch, gw, splits, 256, 32, C1_WGRAD_OUTPUT_SCALE) ||
-      !add_segment(segs, bias_part, gb, 2 * splits, 1, 32, C1_BIAS_OUTPUT_SCALE))      // two bias warps per CTA, a row each
+  if (!add_grad_segment(segs, scratch, gw, splits, 256, 32, C1_WGRAD_OUTPUT_SCALE) ||
+      !add_grad_segment(segs, bias_part, gb, 2 * splits, 1, 32, C1_BIAS_OUTPUT_SCALE))      // two bias warps per CTA, a row each
     lc.host_failure = true;
 }
 
@@ -3210,8 +3210,8 @@ static size_t tc_heads_scratch_floats();
 size_t tc_scratch_floats(int n) { return tc_layer_scratch_offset(n, 4) + tc_heads_scratch_floats(); }
 
 // Enqueues the weight-gradient kernel of `layer` (0 = conv1 .. 3 = fc) and notes in *segs where its partial
-// sums are; tc_backward_finish() then turns all noted partial sums into the gradient vector in one launch.
-int tc_backward_finish(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials) {
+// sums are; finish_gradients() then turns all noted partial sums into the gradient vector in one launch.
+int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials) {
   int blocks = 0;
   if (segs->n > 0) {
     KernelScope scope(lc, KID_WGRAD_REDUCE);
@@ -3350,8 +3350,8 @@ void tc_heads_backward(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, co
     launch_kernel_overlapped(lc, heads_backward_kernel<20>, splits, HB_THREADS, 0, h, dz, dV, theta16 + nd.pi_w, theta16 + nd.v_w, n, A,
                   rows_per, g_fc, part_w, part_b, part_vw, part_vb);
   // already in parameter order: plain sums
-  if (!add_segment(segs, part_w, grad + nd.pi_w, splits, 1, 512 * A, 1.f) || !add_segment(segs, part_b, grad + nd.pi_b, splits, 1, A, 1.f) ||
-      !add_segment(segs, part_vw, grad + nd.v_w, splits, 1, 512, 1.f) || !add_segment(segs, part_vb, grad + nd.v_b, splits, 1, 1, 1.f))
+  if (!add_grad_segment(segs, part_w, grad + nd.pi_w, splits, 1, 512 * A, 1.f) || !add_grad_segment(segs, part_b, grad + nd.pi_b, splits, 1, A, 1.f) ||
+      !add_grad_segment(segs, part_vw, grad + nd.v_w, splits, 1, 512, 1.f) || !add_grad_segment(segs, part_vb, grad + nd.v_b, splits, 1, 1, 1.f))
     lc.host_failure = true;
 }
 
@@ -3481,8 +3481,8 @@ void tc_backward_conv2d_conv1w_chunked(LaunchCtx& lc, const NetDims& nd, const b
                                       bias_part + (size_t)done * 2 * 32, err);
   }
   const LayerDims* d = nd.layer;
-  if (!add_segment(segs, part, grad + d[0].w_off, total_splits, 256, 32, C1_WGRAD_OUTPUT_SCALE) ||
-      !add_segment(segs, bias_part, grad + d[0].b_off, 2 * total_splits, 1, 32, C1_BIAS_OUTPUT_SCALE))
+  if (!add_grad_segment(segs, part, grad + d[0].w_off, total_splits, 256, 32, C1_WGRAD_OUTPUT_SCALE) ||
+      !add_grad_segment(segs, bias_part, grad + d[0].b_off, 2 * total_splits, 1, 32, C1_BIAS_OUTPUT_SCALE))
     lc.host_failure = true;
 }
 
