@@ -136,30 +136,29 @@ def _host_ptr(a):
     return a.data_ptr()
 
 
+def _addr(x):
+    """Device address of a torch CUDA tensor or a raw address; None stays None."""
+    return x if x is None or isinstance(x, int) else x.data_ptr()
+
+
 def clip_rmsprop_noalloc(theta, rms, grad, n, lr, rms_decay, rms_eps, clip_norm, theta_bf16=None,
                          norm_and_scale=None, stream=None):
     """Optimiser step on caller-owned device arrays for hosts that may not allocate device memory (see
     paac_clip_rmsprop_noalloc in include/paac.h).  Arguments are torch CUDA tensors (or raw device
     addresses); returns the library status without raising, so callers can test for ERR_LIMIT."""
-    def addr(x):
-        return None if x is None else (x if isinstance(x, int) else x.data_ptr())
-    return int(lib().paac_clip_rmsprop_noalloc(addr(theta), addr(rms), addr(grad), addr(theta_bf16), n, lr, rms_decay,
-                                               rms_eps, clip_norm, addr(norm_and_scale), addr(stream)))
+    return int(lib().paac_clip_rmsprop_noalloc(_addr(theta), _addr(rms), _addr(grad), _addr(theta_bf16), n, lr, rms_decay,
+                                               rms_eps, clip_norm, _addr(norm_and_scale), _addr(stream)))
 
 
 def preprocess(raw_prev, raw_last, state_in, state_out, n, stream=None):
     """Section 5.1 pre-processing on device buffers (torch CUDA uint8 tensors or raw addresses): see paac_preprocess
     in include/paac.h.  Returns the library status."""
-    def addr(x):
-        return None if x is None else (x if isinstance(x, int) else x.data_ptr())
-    return int(lib().paac_preprocess(addr(raw_prev), addr(raw_last), addr(state_in), addr(state_out), n, addr(stream)))
+    return int(lib().paac_preprocess(_addr(raw_prev), _addr(raw_last), _addr(state_in), _addr(state_out), n, _addr(stream)))
 
 
 def stack_push(state_in, newest, restart, state_out, n, stream=None):
     """The four-frame stack on device buffers: see paac_stack_push in include/paac.h.  Returns the library status."""
-    def addr(x):
-        return None if x is None else (x if isinstance(x, int) else x.data_ptr())
-    return int(lib().paac_stack_push(addr(state_in), addr(newest), addr(restart), addr(state_out), n, addr(stream)))
+    return int(lib().paac_stack_push(_addr(state_in), _addr(newest), _addr(restart), _addr(state_out), n, _addr(stream)))
 
 
 class Paac:

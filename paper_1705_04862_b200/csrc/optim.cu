@@ -38,26 +38,34 @@ sumsq_kernel(const float* __restrict__ g, size_t P, float* __restrict__ partials
 // and refreshes the bf16 copy.  A non-finite norm leaves theta and m untouched, and so does a device error
 // left by any earlier kernel (a bounded wait that gave up means some tile or partial sum of this update is
 // garbage): the status then names the error.
-__global__ void __launch_bounds__(OPT_THREADS)
-clip_rmsprop_kernel(size_t P, float* __restrict__ theta, float* __restrict__ rms, const float* __restrict__ g,
+// One wave of two blocks per SM, launched so that it may start while the finishing kernel drains: a thread's first
+// UPD_AHEAD groups of parameters and state (all of them, up to 1.8 M parameters) are fetched before the wait, the
+// gradients right after it, together with the partial sums of the norm.
+constexpr int UPD_THREADS = 512, UPD_BLOCKS = 296, UPD_AHEAD = 3;
+__global__ void __launch_bounds__(UPD_THREADS, 2)
+clip_rmsprop_kernel(size_t P, float* theta, float* rms, const float* g,
                     bf16* __restrict__ theta16, float lr, float rho, float eps, float clip,
-                    const float* __restrict__ partials, int n_partials, DeviceStats* stats) {
-  pdl_entry();
-  __shared__ float sh[OPT_THREADS / 32];
+                    const float* partials, int n_partials, DeviceStats* stats) {
+  __shared__ float sh[UPD_THREADS / 32];
   __shared__ float s_scale;
-  // this thread's first elements do not depend on the norm: fetch them before the norm is known
-  const size_t n4 = P / 4;
+  const size_t n4 = P / 4, stride = (size_t)gridDim.x * UPD_THREADS;
   float4* t4 = reinterpret_cast<float4*>(theta);
   float4* m4 = reinterpret_cast<float4*>(rms);
   const float4* g4 = reinterpret_cast<const float4*>(g);
-  const size_t i0 = blockIdx.x * (size_t)OPT_THREADS + threadIdx.x;
-  float4 gv0 = make_float4(0.f, 0.f, 0.f, 0.f), mv0 = gv0, tv0 = gv0;
-  if (i0 < n4) { gv0 = g4[i0]; mv0 = m4[i0]; tv0 = t4[i0]; }
+  const size_t i0 = blockIdx.x * (size_t)UPD_THREADS + threadIdx.x;
+  float4 gv0[UPD_AHEAD], mv0[UPD_AHEAD], tv0[UPD_AHEAD];
+#pragma unroll
+  for (int u = 0; u < UPD_AHEAD; ++u)
+    if (i0 + u * stride < n4) { mv0[u] = m4[i0 + u * stride]; tv0[u] = t4[i0 + u * stride]; }
+  pdl_entry();
+#pragma unroll
+  for (int u = 0; u < UPD_AHEAD; ++u)
+    if (i0 + u * stride < n4) gv0[u] = g4[i0 + u * stride];
   // the device error word, fetched now so that its latency hides behind the sum of the partials
   uint32_t dev_err = 0u;
   if (threadIdx.x == 0) dev_err = *reinterpret_cast<const volatile uint32_t*>(&stats->error_word);
   float acc = 0.f;
-  for (int i = threadIdx.x; i < n_partials; i += OPT_THREADS) acc += partials[i];
+  for (int i = threadIdx.x; i < n_partials; i += UPD_THREADS) acc += partials[i];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -65,7 +73,7 @@ clip_rmsprop_kernel(size_t P, float* __restrict__ theta, float* __restrict__ rms
   if (threadIdx.x == 0) {
     float total = 0.f;
 #pragma unroll
-    for (int w = 0; w < OPT_THREADS / 32; ++w) total += sh[w];
+    for (int w = 0; w < UPD_THREADS / 32; ++w) total += sh[w];
     const float norm = sqrtf(total);
     float scale = 1.f;
     const bool ok = isfinite(norm) && dev_err == 0u;
@@ -83,11 +91,8 @@ clip_rmsprop_kernel(size_t P, float* __restrict__ theta, float* __restrict__ rms
   const float scale = s_scale;
   if (scale < 0.f) return;
   const float one_m_rho = 1.f - rho;
-  for (size_t i = i0; i < n4; i += (size_t)gridDim.x * OPT_THREADS) {
-    float4 gv, mv, tv;
-    if (i == i0) { gv = gv0; mv = mv0; tv = tv0; }
-    else { gv = g4[i]; mv = m4[i]; tv = t4[i]; }
-    float* gp = &gv.x; float* mp = &mv.x; float* tp = &tv.x;
+  auto apply = [&](size_t i, float4& tv, float4& mv, const float4& gv) {
+    const float* gp = &gv.x; float* mp = &mv.x; float* tp = &tv.x;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float gs = scale * gp[j];
@@ -101,9 +106,16 @@ clip_rmsprop_kernel(size_t P, float* __restrict__ theta, float* __restrict__ rms
       pk.x = *reinterpret_cast<uint32_t*>(&lo); pk.y = *reinterpret_cast<uint32_t*>(&hi);
       reinterpret_cast<uint2*>(theta16)[i] = pk;
     }
+  };
+#pragma unroll
+  for (int u = 0; u < UPD_AHEAD; ++u)
+    if (i0 + u * stride < n4) apply(i0 + u * stride, tv0[u], mv0[u], gv0[u]);
+  for (size_t i = i0 + UPD_AHEAD * stride; i < n4; i += stride) {
+    float4 tv = t4[i], mv = m4[i];
+    apply(i, tv, mv, g4[i]);
   }
   if (blockIdx.x == 0) {
-    for (size_t i = n4 * 4 + threadIdx.x; i < P; i += OPT_THREADS) {
+    for (size_t i = n4 * 4 + threadIdx.x; i < P; i += UPD_THREADS) {
       const float gs = scale * g[i];
       const float m = fmaf(rho, rms[i], one_m_rho * gs * gs);
       rms[i] = m;
@@ -124,7 +136,7 @@ void launch_clip_rmsprop(LaunchCtx& lc, size_t P, float* theta, float* rms, cons
     n_partials = NORM_BLOCKS;
   }
   KernelScope scope(lc, KID_CLIP_RMSPROP);
-  launch_kernel(lc, clip_rmsprop_kernel, NORM_BLOCKS, OPT_THREADS, 0, P, theta, rms, grad, theta16, lr, rho, eps, clip,
+  launch_kernel_overlapped(lc, clip_rmsprop_kernel, UPD_BLOCKS, UPD_THREADS, 0, P, theta, rms, grad, theta16, lr, rho, eps, clip,
                                                               norm_partials, n_partials, stats);
 }
 

@@ -79,3 +79,28 @@ def test_noalloc_rejects_sizes_beyond_its_scratch_and_bad_arguments():
     assert pb.clip_rmsprop_noalloc(th, m, gr, 5000, 0.01, 0.99, 0.1, 40.0, norm_and_scale=out) == pb.OK
     torch.cuda.synchronize()
     assert torch.all(th == 1) and torch.all(m == 2) and out[1].item() == 0.0
+
+
+@pytest.mark.parametrize("n,shift", [(1, 0), (1023, 0), (8192, 0), (8193, 0), (8195, 1), (100001, 3), (2000003, 0)])
+def test_noalloc_sizes_and_alignments(n, shift):
+    """One block, two launches with 16-byte accesses and with 4-byte ones, remainders, more than the prefetched groups."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    th, m, gr = (torch.randn(n + 4, device="cuda", generator=gen) for _ in range(3))
+    m = m.abs()
+    half = torch.zeros(n + 4, dtype=torch.bfloat16, device="cuda")
+    view = [x[shift:shift + n] for x in (th, m, gr, half)]
+    before = [x.clone() for x in (th, m)]
+    g64, scale = view[2].double(), 0.5
+    norm = float(g64.norm())
+    want_m = 0.99 * view[1].double() + 0.01 * (scale * g64) ** 2
+    want_t = view[0].double() - 0.02 * scale * g64 / (want_m + 0.1).sqrt()
+    out = torch.zeros(2, device="cuda")
+    assert pb.clip_rmsprop_noalloc(view[0], view[1], view[2], n, 0.02, 0.99, 0.1, scale * norm, theta_bf16=view[3],
+                                   norm_and_scale=out) == pb.OK
+    torch.cuda.synchronize()
+    assert abs(float(out[0]) - norm) <= 1e-5 * norm and abs(float(out[1]) - scale) <= 1e-5
+    assert rel(view[0].cpu(), want_t.cpu()) <= 1e-5 and rel(view[1].cpu(), want_m.cpu()) <= 1e-5
+    assert torch.equal(view[3], view[0].to(torch.bfloat16))
+    for x, b in ((th, before[0]), (m, before[1])):          # nothing outside the n elements
+        assert torch.equal(x[:shift], b[:shift]) and torch.equal(x[shift + n:], b[shift + n:])
