@@ -7,6 +7,17 @@
 
 using namespace paac;
 
+// Pinned memory both sides see.  Results the host waits for are stored there by the kernel that ends a launch sequence
+// and picked up by polling a flag: no copy engine, no stream synchronisation.  The pointers let a recorded sequence
+// read buffers that differ from call to call.
+struct HostBox {
+  volatile uint32_t done;                       // set by the device when actions and values are there
+  HostPlanes planes;                            // the newest frames and the restart flags of the step in flight
+  DeviceStats stats;
+  int32_t* actions; float* values; uint8_t* restart;      // [n_e] each, behind this struct
+  uint8_t* outcomes;                            // rewards and terminal flags, laid out as on the device (outcome_bytes())
+};
+
 struct paac_ctx {
   int arch, n_e, t_max, A, prec, B;
   paac_hparams hp;
@@ -21,7 +32,9 @@ struct paac_ctx {
   uint64_t N;              // timesteps consumed by updates
   uint64_t env_step;       // global step index of the environments (same for all)
   bool rollout_fresh;      // a rollout has completed since the last update
-  uint8_t* newest;         // staging for paac_act_host_newest: [n_e][84][84] planes, then [n_e] restart flags
+  uint8_t* newest;         // staging for paac_act_host_newest with pageable planes: [n_e][84][84]
+  HostBox* box;            // pinned, device-visible: what host and device hand each other (made on first use)
+  bool observed;           // outcomes of this rollout wait in the box for their copy to the device
   int host_t;              // external-environment mode: next expected step
   int update_chunks;       // > 1: conv2 data gradient and conv1 weight gradient alternate over this many groups of states
   bool host_next_valid;    // the bootstrap state of the last host-mode rollout sits where step 0 of the next one goes
@@ -98,7 +111,7 @@ size_t carve(paac_ctx* c, char* base) {
   c->w_images = k.take<bf16>(tc_supported(c->arch, c->prec) ? tc_weight_image_elems() : 0);
   c->frames[0] = k.take<uint8_t>(T * n_e * FRAME_BYTES);
   c->frames[1] = k.take<uint8_t>(T * n_e * FRAME_BYTES);
-  c->newest = k.take<uint8_t>(n_e * (FRAME_H * FRAME_W + 4));          // newest planes from the host, then restart flags
+  c->newest = k.take<uint8_t>(n_e * FRAME_H * FRAME_W);
   for (int l = 0; l <= nd.n_conv; ++l) {
     c->act[l] = k.take<char>((T + 1) * n_e * nd.layer[l].out_size * c->elt);
     c->gact[l] = k.take<char>(B * nd.layer[l].out_size * c->elt);
@@ -199,6 +212,29 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
                    sample ? env : nullptr, advanced && !sample ? c->step_dev : nullptr, (uint32_t)c->t_max);
   if (advanced) *advanced = sample ? env != nullptr : true;
   return false;
+}
+
+size_t outcome_bytes(const paac_ctx* c) { return (size_t)((const char*)c->terminals - (const char*)c->rewards) + c->B; }
+bool host_box(paac_ctx* c) {
+  if (c->box) return true;
+  const size_t n = c->n_e, head = (sizeof(HostBox) + 255) / 256 * 256;
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, head + n * 9 + outcome_bytes(c), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError(); return false;
+  }
+  c->box = new (p) HostBox{};
+  char* q = (char*)p + head;
+  c->box->actions = (int32_t*)q; c->box->values = (float*)(q + 4 * n);
+  c->box->restart = (uint8_t*)(q + 8 * n); c->box->outcomes = (uint8_t*)(q + 9 * n);
+  return true;
+}
+// the rollout's outcomes, gathered by paac_observe_host, to the device in one copy
+int send_outcomes(paac_ctx* c) {
+  if (!c->observed) return PAAC_OK;
+  c->observed = false;
+  if (cudaMemcpyAsync(c->rewards, c->box->outcomes, outcome_bytes(c), cudaMemcpyHostToDevice, c->st) == cudaSuccess) return PAAC_OK;
+  cudaGetLastError();
+  return PAAC_ERR_CUDA;
 }
 
 void drop_graphs(paac_ctx* c) {
@@ -416,7 +452,8 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
   c->rollout_fresh = false;
   if (cuda_status(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (stats) {
-    DeviceStats ds;
+    if (!host_box(c)) return PAAC_ERR_CUDA;
+    DeviceStats& ds = c->box->stats;
     if (cudaMemcpyAsync(&ds, c->stats, sizeof(ds), cudaMemcpyDeviceToHost, c->st) != cudaSuccess ||
         cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
     stats->policy_loss = ds.policy_loss; stats->value_loss = ds.value_loss; stats->entropy = ds.entropy;
@@ -485,6 +522,7 @@ int paac_destroy(paac_ctx* c) {
   cudaStreamSynchronize(c->st);
   drop_graphs(c);
   c->lc.release();
+  if (c->box) cudaFreeHost(c->box);
   if (c->record_st) cudaStreamDestroy(c->record_st);
   if (c->owns_workspace) cudaFree(c->ws);
   cudaGetLastError();
@@ -554,23 +592,31 @@ int paac_profile_read(paac_ctx* c, int max_entries, const char** names, double* 
 }
 
 // ---- external-environment mode ------------------------------------------------------------------
-// Step t of an external-environment rollout once the host's bytes are on their way: (the frame stack,) the network on
-// the state at `dst` -- a recorded sequence from the second time on --, results to the host, bookkeeping.
+// The network on the state at `dst`, with `prev` after the frame stack has built that state, and the results into the
+// box: one launch sequence, recorded from the second time on.
 static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, uint8_t* dst, int32_t* actions, float* values) {
   const bool sample = t < c->t_max;
-  const size_t plane = (size_t)c->n_e * FRAME_H * FRAME_W;
-  run_recorded(c, 2 + 2 * t + (prev ? 1 : 0), c->cur, [&]() {
-    if (prev) launch_stack_push(c->lc, prev, c->newest, c->newest + plane, dst, c->n_e);
-    forward_slot(c, dst, t, sample);
-  });
   const size_t row = (size_t)t * c->n_e;
-  if (sample) cudaMemcpyAsync(actions, c->actions + row, c->n_e * sizeof(int32_t), cudaMemcpyDeviceToHost, c->st);
-  if (values) cudaMemcpyAsync(values, c->values + row, c->n_e * sizeof(float), cudaMemcpyDeviceToHost, c->st);
-  if (cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
-  if (t == c->t_max) {
-    launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
-    c->host_t = 0; c->env_step += c->t_max; c->rollout_fresh = true; c->host_next_valid = true;
+  HostBox* box = c->box;
+  box->done = 0u;
+  run_recorded(c, 2 + 2 * t + (prev ? 1 : 0), c->cur, [&]() {
+    if (prev) launch_stack_pull(c->lc, prev, &box->planes, dst, c->n_e);
+    bool advanced = false;
+    forward_slot(c, dst, t, sample, nullptr, sample ? nullptr : &advanced);
+    if (!sample && !advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
+    launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
+  });
+  // the flag is set by the sequence's last kernel; a failed launch or kernel shows in the stream's status instead
+  for (uint32_t polls = 1; !box->done; ++polls) {
+    if (polls & 0x3FFFu) continue;
+    const cudaError_t st = cudaStreamQuery(c->st);
+    if (st == cudaErrorNotReady) continue;
+    if (st != cudaSuccess || !box->done) { cudaGetLastError(); return PAAC_ERR_CUDA; }
   }
+  __atomic_thread_fence(__ATOMIC_ACQUIRE);
+  if (sample) memcpy(actions, box->actions, c->n_e * sizeof(int32_t));
+  if (values) memcpy(values, box->values, c->n_e * sizeof(float));
+  if (t == c->t_max) { c->host_t = 0; c->env_step += c->t_max; c->rollout_fresh = true; c->host_next_valid = true; }
   else c->host_t = t + 1;
   return cuda_status(c);
 }
@@ -581,28 +627,42 @@ int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, f
   if (t != c->host_t) return PAAC_ERR_STATE;
   // s_0 of a rollout is s_{t_max} of the one before (Algorithm 1): those frames are on the device already
   if (!frames && !(t == 0 && c->host_next_valid)) return PAAC_ERR_ARG;
+  if (!host_box(c)) return PAAC_ERR_CUDA;
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
   if (t == 0) c->cur ^= 1;
   uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
   if (frames && cudaMemcpyAsync(dst, frames, fstep, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
+  if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   return act_host_finish(c, t, nullptr, dst, actions, values);
+}
+
+// the device's view of pinned host memory, nullptr for anything else
+static const uint8_t* pinned_view(const uint8_t* p) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  return a.type == cudaMemoryTypeHost ? (const uint8_t*)a.devicePointer : nullptr;
 }
 
 int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_t* restart, int32_t* actions, float* values) {
   if (c) c->lc.serialize_next = true;
   if (!c || !newest || t < 1 || t > c->t_max || (t < c->t_max && !actions)) return PAAC_ERR_ARG;
   if (t != c->host_t) return PAAC_ERR_STATE;
+  if (!host_box(c)) return PAAC_ERR_CUDA;
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES, plane = (size_t)c->n_e * FRAME_H * FRAME_W;
   const uint8_t* prev = c->frames[c->cur] + (size_t)(t - 1) * fstep;
   uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
-  // the restart flags always live on the device (all zero when the host has none), so that the recorded sequence
-  // is the same either way
-  const cudaError_t e1 = cudaMemcpyAsync(c->newest, newest, plane, cudaMemcpyHostToDevice, c->st);
-  const cudaError_t e2 = restart ? cudaMemcpyAsync(c->newest + plane, restart, c->n_e, cudaMemcpyHostToDevice, c->st)
-                                 : cudaMemsetAsync(c->newest + plane, 0, c->n_e, c->st);
-  if (e1 != cudaSuccess || e2 != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
+  // Pinned planes (16-byte aligned) are read over the link by the kernel that builds the states, which saves the copy's
+  // set-up, its hand-over to the first kernel and a round trip through device memory; others are copied first.
+  const uint8_t* view = ((uintptr_t)newest & 15u) == 0 ? pinned_view(newest) : nullptr;
+  c->box->planes.newest = view ? view : c->newest;
+  c->box->planes.restart = restart ? c->box->restart : nullptr;
+  if (restart) memcpy(c->box->restart, restart, c->n_e);
+  if (!view && cudaMemcpyAsync(c->newest, newest, plane, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
+    cudaGetLastError(); return PAAC_ERR_CUDA;
+  }
+  if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   return act_host_finish(c, t, prev, dst, actions, values);
 }
 
@@ -610,11 +670,11 @@ int paac_observe_host(paac_ctx* c, int t, const int8_t* rewards, const uint8_t* 
   if (c) c->lc.serialize_next = true;
   if (!c || !rewards || !terminals || t < 0 || t >= c->t_max) return PAAC_ERR_ARG;
   if (t + 1 != c->host_t) return PAAC_ERR_STATE;
+  if (!host_box(c)) return PAAC_ERR_CUDA;
   const size_t row = (size_t)t * c->n_e;
-  if (cudaMemcpyAsync(c->rewards + row, rewards, c->n_e, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
-      cudaMemcpyAsync(c->terminals + row, terminals, c->n_e, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
-    cudaGetLastError(); return PAAC_ERR_CUDA;
-  }
+  memcpy(c->box->outcomes + row, rewards, c->n_e);
+  memcpy(c->box->outcomes + (outcome_bytes(c) - c->B) + row, terminals, c->n_e);
+  c->observed = true;
   return PAAC_OK;
 }
 
@@ -665,6 +725,7 @@ int paac_debug_read(paac_ctx* c, int which, void* dst, size_t bytes) {
   size_t b = 0;
   void* p = debug_ptr(c, which, &b);
   if (!p || b != bytes) return PAAC_ERR_ARG;
+  if (send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (cudaMemcpyAsync(dst, p, b, cudaMemcpyDeviceToHost, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
   if (which == PAAC_DBG_GACT0 && c->prec == PAAC_BF16 && c->gact0_scale != 1.f) {
@@ -689,6 +750,7 @@ int paac_debug_write(paac_ctx* c, int which, const void* src, size_t bytes) {
   size_t b = 0;
   void* p = debug_ptr(c, which, &b);
   if (!p || b != bytes) return PAAC_ERR_ARG;
+  if (send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (cudaMemcpyAsync(p, src, b, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
   return PAAC_OK;

@@ -26,6 +26,16 @@ void launch_env_step_sampling(LaunchCtx& lc, uint64_t seed, int n_e, const uint6
                               uint8_t* next_frames, int8_t* rewards, uint8_t* terminals, int32_t* counters,
                               const HeadsTail& ht, int pattern_actions = 0);
 
+// ---- external-environment mode (preprocess.cu) --------------------------------------------
+// The newest plane of every environment, [n][84][84] at a 16-byte aligned address, and restart flags [n] (nullable): both
+// may be pinned host memory.  The struct itself is read by the kernel too, so a recorded launch can be pointed elsewhere.
+struct HostPlanes { const uint8_t* newest; const uint8_t* restart; };
+// frame stack: out = (three newest channels of prev, newest plane), or four copies of the plane where restart[e] != 0
+void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const HostPlanes* planes, uint8_t* out, int n);
+// actions (nullable) and values of n environments to pinned host memory, then *done = 1
+void launch_publish(LaunchCtx& lc, const int32_t* actions, const float* values, int n, int32_t* host_actions, float* host_values,
+                    volatile uint32_t* done);
+
 void launch_advance_step(LaunchCtx& lc, uint64_t* step_base, uint32_t by);
 
 // ---- weight gradients as split-k partial sums --------------------------------------------
@@ -76,9 +86,6 @@ float tc_conv1_grad_scale();
 // weight + bias gradients of one layer (0 = conv1 .. 3 = fc) as partial sums in the layer's own region of a scratch of
 // tc_scratch_floats(B) floats, noted in the GradSegments list
 size_t tc_scratch_floats(int n);
-// frame stack: out = (three newest channels of prev, newest plane), or four copies of the plane where restart[e] != 0
-void launch_stack_push(LaunchCtx& lc, const uint8_t* prev, const uint8_t* newest, const uint8_t* restart /* nullable */,
-                       uint8_t* out, int n);
 // the same data gradient followed by the first layer's weight gradient, alternating over `chunks` (at most
 // TC_MAX_UPDATE_CHUNKS) groups of states; notes the weight gradient's partial sums in *segs
 constexpr int TC_MAX_UPDATE_CHUNKS = 4;

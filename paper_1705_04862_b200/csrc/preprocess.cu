@@ -149,9 +149,76 @@ stack_push_kernel(const uint8_t* prev, const uint8_t* __restrict__ newest, const
   }
 }
 
-void launch_stack_push(LaunchCtx& lc, const uint8_t* prev, const uint8_t* newest, const uint8_t* restart, uint8_t* out, int n) {
+// The same for the external-environment mode, sixteen pixels per thread and all of a thread's plane words asked for before
+// any is used: they come over the host link, whose latency is a microsecond or two and whose bandwidth (about 50 GB/s) is
+// what bounds the kernel from a few dozen environments on.
+constexpr int PULL_ITEMS = FRAME_H * FRAME_W / 16, PULL_AHEAD = 3, PULL_BLOCKS = 592;
+static_assert(PULL_ITEMS * 16 == FRAME_H * FRAME_W, "whole 16-byte words");
+__global__ void __launch_bounds__(SP_THREADS)
+stack_pull_kernel(const uint8_t* prev, const HostPlanes* planes, uint8_t* out, int n) {
+  __shared__ HostPlanes from;
+  pdl_entry();
+  if (threadIdx.x == 0) from = *planes;
+  __syncthreads();
+  const uint32_t items = (uint32_t)n * PULL_ITEMS, stride = gridDim.x * SP_THREADS;
+  const uint4* newest = reinterpret_cast<const uint4*>(from.newest);
+  for (uint32_t base = blockIdx.x * SP_THREADS + threadIdx.x; base < items; base += PULL_AHEAD * stride) {
+    uint4 v[PULL_AHEAD];
+    bool fresh[PULL_AHEAD];
+#pragma unroll
+    for (int u = 0; u < PULL_AHEAD; ++u) {
+      const uint32_t i = base + u * stride;
+      if (i < items) {
+        v[u] = newest[i];
+        fresh[u] = from.restart != nullptr && from.restart[i / PULL_ITEMS] != 0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < PULL_AHEAD; ++u) {
+      const uint32_t i = base + u * stride;
+      if (i >= items) break;
+      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+      const uint4* src = reinterpret_cast<const uint4*>(prev) + (size_t)i * 4;
+      uint4* dst = reinterpret_cast<uint4*>(out) + (size_t)i * 4;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint4 o;
+        if (fresh[u]) {
+          o = make_uint4((w[q] & 0xFFu) * 0x01010101u, ((w[q] >> 8) & 0xFFu) * 0x01010101u, ((w[q] >> 16) & 0xFFu) * 0x01010101u,
+                         (w[q] >> 24) * 0x01010101u);
+        } else {
+          const uint4 p = src[q];
+          o = make_uint4((p.x >> 8) | (w[q] << 24), (p.y >> 8) | ((w[q] >> 8) << 24), (p.z >> 8) | ((w[q] >> 16) << 24),
+                         (p.w >> 8) | ((w[q] >> 24) << 24));
+        }
+        dst[q] = o;
+      }
+    }
+  }
+}
+void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const HostPlanes* planes, uint8_t* out, int n) {
+  const size_t blocks = ((size_t)n * PULL_ITEMS + SP_THREADS - 1) / SP_THREADS;
   KernelScope scope(lc, KID_ENV_STEP);
-  launch_kernel(lc, stack_push_kernel, dim3(2, n), SP_THREADS, 0, prev, newest, restart, out);
+  launch_kernel(lc, stack_pull_kernel, dim3(blocks < PULL_BLOCKS ? (unsigned)blocks : PULL_BLOCKS), dim3(SP_THREADS), 0, prev, planes, out, n);
+}
+
+// one block: a few kilobytes of posted writes over the host link, made visible before the flag
+constexpr int PUB_THREADS = 512;
+__global__ void __launch_bounds__(PUB_THREADS)
+publish_kernel(const int32_t* actions, const float* values, int n, int32_t* host_actions, float* host_values, volatile uint32_t* done) {
+  pdl_entry();
+  for (int i = threadIdx.x; i < n; i += PUB_THREADS) {
+    if (actions != nullptr) host_actions[i] = actions[i];
+    host_values[i] = values[i];
+  }
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) *done = 1u;
+}
+void launch_publish(LaunchCtx& lc, const int32_t* actions, const float* values, int n, int32_t* host_actions, float* host_values,
+                    volatile uint32_t* done) {
+  KernelScope scope(lc, KID_HEADS_FWD);
+  launch_kernel_overlapped(lc, publish_kernel, dim3(1), dim3(PUB_THREADS), 0, actions, values, n, host_actions, host_values, done);
 }
 
 }  // namespace paac
