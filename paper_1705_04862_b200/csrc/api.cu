@@ -46,6 +46,8 @@ struct paac_ctx {
   // second iteration (the two frame buffers alternate), so after two plain iterations each parity is captured
   // once into a CUDA graph and replayed from then on.  Anything that changes the sequence drops the graphs.
   bool graphs_on;          // option: allow recording
+  cudaStream_t side_st;    // weight gradients run here, next to the chain of data gradients (see SideBranch)
+  cudaEvent_t side_ev[MAX_LAYERS + 1];
   cudaStream_t record_st;  // where sequences are recorded when st is the legacy default stream (made on first use)
   // recorded launch sequences: kind 0 = rollout, 1 = update, 2 + 2 t + v = step t of the external-environment mode
   // (v = 1: with the frame stack built on the device), each for both parities of the frame buffers
@@ -292,6 +294,36 @@ template <class F> void run_recorded(paac_ctx* c, int kind, int parity, F enqueu
   ++c->plain_calls[kind][parity];
 }
 
+// A second stream beside the context's, for launches that nothing on the main one waits for until the join.  Off (all
+// launches stay on the main stream) while kernels are being timed one by one, or if the stream cannot be had.
+struct SideBranch {
+  paac_ctx* c; cudaStream_t main; bool on, forked; int used;
+  explicit SideBranch(paac_ctx* ctx) : c(ctx), main(ctx->lc.st), on(!ctx->lc.profiling), forked(false), used(0) {
+    if (on && !c->side_st) {
+      on = cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking) == cudaSuccess;
+      for (int i = 0; on && i <= MAX_LAYERS; ++i) on = cudaEventCreateWithFlags(&c->side_ev[i], cudaEventDisableTiming) == cudaSuccess;
+      if (!on) cudaGetLastError();
+    }
+  }
+  // `enqueue` runs on the side stream, after everything the main one holds so far and after the side's own launches
+  template <class F> void run(F enqueue) {
+    if (!on || used >= MAX_LAYERS) { enqueue(); return; }
+    cudaEventRecord(c->side_ev[used], main);
+    cudaStreamWaitEvent(c->side_st, c->side_ev[used], 0);
+    ++used; forked = true;
+    const bool keep = c->lc.serialize_next;
+    c->lc.st = c->side_st; c->lc.serialize_next = true;
+    enqueue();
+    c->lc.st = main; c->lc.serialize_next = keep;
+  }
+  void join() {
+    if (!forked) return;
+    cudaEventRecord(c->side_ev[MAX_LAYERS], c->side_st);
+    cudaStreamWaitEvent(main, c->side_ev[MAX_LAYERS], 0);
+    c->lc.serialize_next = true;
+  }
+};
+
 }  // namespace
 
 extern "C" {
@@ -410,36 +442,42 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
     uint32_t* err = &c->stats->error_word;
     c->gact0_scale = 1.f;
     const bool chunked = use_tc(c) && c->update_chunks > 1 && (c->tc_wgrad_mask & 3) == 3;
+    // The data gradients are a chain, and the first layer's weight gradient ends it; the other layers' weight gradients
+    // only need their own layer's gradient and run beside the chain.
+    SideBranch side(c);
     for (int l = L; l >= 0; --l) {
       // tensor-core kernels where they exist, the CUDA-core contraction otherwise
+      const bool tc_wgrad = use_tc(c) && (c->tc_wgrad_mask >> l) & 1;
+      auto wgrad = [&]() {
+        if (tc_wgrad)
+          tc_backward_wgrad(c->lc, c->nd, c->frames[c->cur], c->B, c->act, c->gact, c->grad, c->scratch, l, &c->grad_segs, err);
+        else
+          simt_backward_layer(c->lc, c->arch, c->prec, c->nd, c->theta, c->theta16, c->frames[c->cur], c->B, c->act, c->gact,
+                              c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, true, false);
+      };
+      if (l > 0) side.run(wgrad); else wgrad();
       if (chunked && l == 1) {
-        // the layer's own weight gradient first, then data gradient and first-layer weight gradient group by group
-        tc_backward_wgrad(c->lc, c->nd, c->frames[c->cur], c->B, c->act, c->gact, c->grad, c->scratch, 1, &c->grad_segs, err);
+        // data gradient and first-layer weight gradient group by group
         c->gact0_scale = tc_conv1_grad_scale();
         tc_backward_conv2d_conv1w_chunked(c->lc, c->nd, c->w_images, c->frames[c->cur], c->B, c->act, c->gact, c->grad,
                                           c->scratch, c->update_chunks, &c->grad_segs, err);
         break;
       }
-      bool dgrad_done = false;
+      if (l == 0) break;
       if (use_tc(c)) {
-        if (l == 3) { tc_backward_dgrad_fc(c->lc, c->w_images, c->B, c->act, c->gact, err); dgrad_done = true; }
-        if (l == 2) { tc_backward_dgrad_conv3(c->lc, c->w_images, c->B, c->act, c->gact, err); dgrad_done = true; }
+        if (l == 3) tc_backward_dgrad_fc(c->lc, c->w_images, c->B, c->act, c->gact, err);
+        if (l == 2) tc_backward_dgrad_conv3(c->lc, c->w_images, c->B, c->act, c->gact, err);
         if (l == 1) {
           // the first layer's tensor-core weight gradient takes its gradient operand times a power of two
           c->gact0_scale = (c->tc_wgrad_mask & 1) ? tc_conv1_grad_scale() : 1.f;
           tc_backward_dgrad_conv2(c->lc, c->w_images, c->B, c->act, c->gact, err, c->gact0_scale);
-          dgrad_done = true;
         }
+      } else {
+        simt_backward_layer(c->lc, c->arch, c->prec, c->nd, c->theta, c->theta16, c->frames[c->cur], c->B, c->act, c->gact,
+                            c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, false, true);
       }
-      bool wgrad_done = false;
-      if (use_tc(c) && (c->tc_wgrad_mask >> l) & 1) {
-        tc_backward_wgrad(c->lc, c->nd, c->frames[c->cur], c->B, c->act, c->gact, c->grad, c->scratch, l, &c->grad_segs, err);
-        wgrad_done = true;
-      }
-      if (!wgrad_done || (l > 0 && !dgrad_done))
-        simt_backward_layer(c->lc, c->arch, c->prec, c->nd, c->theta, c->theta16, c->frames[c->cur], c->B, c->act,
-                            c->gact, c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, !wgrad_done, l > 0 && !dgrad_done);
     }
+    side.join();
     // when every gradient goes through the finishing kernel, it also delivers the squared norm
     const bool all_finished = !c->lc.fp32_tensor_cores || (use_tc(c) && c->tc_wgrad_mask == 0xF && tc_heads_backward_supported(c->nd));
     const int ready = finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials : nullptr);
@@ -523,6 +561,8 @@ int paac_destroy(paac_ctx* c) {
   drop_graphs(c);
   c->lc.release();
   if (c->box) cudaFreeHost(c->box);
+  if (c->side_st) cudaStreamDestroy(c->side_st);
+  for (cudaEvent_t e : c->side_ev) if (e) cudaEventDestroy(e);
   if (c->record_st) cudaStreamDestroy(c->record_st);
   if (c->owns_workspace) cudaFree(c->ws);
   cudaGetLastError();
