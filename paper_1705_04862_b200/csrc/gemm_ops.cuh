@@ -10,12 +10,12 @@ namespace paac {
 
 constexpr int SG_BM = 64, SG_BN = 64, SG_BK = 16;
 
-// number of k splits that are really launched for a requested count
-inline int gemm_k_splits(int K, int splits) {
-  int kps = (K + splits - 1) / splits;
-  kps = (kps + SG_BK - 1) / SG_BK * SG_BK;
-  return (K + kps - 1) / kps;
+// k per split for a requested number of splits, and how many splits that gives
+inline int gemm_k_per_split(int K, int splits) {
+  const int kps = (K + splits - 1) / splits;
+  return (kps + SG_BK - 1) / SG_BK * SG_BK;
 }
+inline int gemm_k_splits(int K, int splits) { const int kps = gemm_k_per_split(K, splits); return (K + kps - 1) / kps; }
 
 // ---- operand functors ----------------------------------------------------------------
 // x[row][k], rows ld apart

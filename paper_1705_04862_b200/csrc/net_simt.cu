@@ -29,40 +29,57 @@ static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_
   launch_kernel(lc, wgrad_reduce_kernel, blocks, 256, 0, part, splits, part_rows, row0, rows, cols, scale, gw, gb);
 }
 
-// Tiles of the CUDA-core contraction for N columns (16, 32, 64 or many): four warps of 32 x 8 TN outputs each.  With
-// enough rows for two CTAs per SM they cover 128 (N <= 32) or 64 rows; with fewer rows two or all four of them share a
-// tile and split every k block between them, so that a batch of a few states still gives every SM its warps; below one
-// CTA per SM eight warps do, and the k blocks are as many times longer: such a launch is a chain of load latencies, one
-// per block.
+// Shapes of the CUDA-core contraction for N columns (16, 32, or 64 and more).  Measured at 128 states forward and 640
+// backward on the larger network (TMAC/s, of 36 the multiply-add pipe could do; every shape ends near 20, at 75 % of the
+// issue slots): the wide shape (8 x 8 per lane for 64 columns, 8 x 4 below, where 8 x 8 leaves tiles of too many rows) wins
+// from two warps per scheduler on (1184 of them; 19.8 against 18.4), below that 4 x 4 (18.4 against 12.2 with one and a half),
+// and 2 x 4 where even that leaves a scheduler without a warp (592).
 constexpr int FF_SMS = 148;
 static size_t ff_heads_scratch_floats(const NetDims& nd, int n);
-template <int N, class LA, class LB, class EP>
-static void ff_rows(LaunchCtx& lc, int kid, int M, int n_cols, int K, int classes, LA la, LB lb, EP ep) {
-  const int cols = (n_cols + N - 1) / N * classes;
-  if constexpr (N <= 32) {
-    constexpr int TN = N / 8;
-    if ((M + 127) / 128 * cols >= 2 * FF_SMS) gemm_ffma<4, 1, TN, 1>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
-    else if ((M + 63) / 64 * cols >= FF_SMS) gemm_ffma<2, 1, TN, 2>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
-    else if ((M + 31) / 32 * cols >= FF_SMS) gemm_ffma<1, 1, TN, 4>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
-    else gemm_ffma<1, 1, TN, 8>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+static int ff_shape(int N, long long outputs) {              // outputs of all classes and splits
+  if (outputs >= 1184LL * 32 * 8 * (N >= 64 ? 8 : 4)) return 2;
+  return outputs >= 592LL * 32 * 16 ? 1 : 0;
+}
+template <int N, int SHAPE, class LA, class LB, class EP>
+static void ff_launch(LaunchCtx& lc, int kid, int M, int n_cols, int K, int kps, int classes, LA la, LB lb, EP ep) {
+  constexpr int WIDE_BK = sizeof(typename LA::Elem) == 1 ? 32 : 16;       // bytes pass through registers, one block ahead
+  if constexpr (N == 16) {
+    if constexpr (SHAPE == 2) gemm_ffma<8, 8, 4, 4, 1, WIDE_BK>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else if constexpr (SHAPE == 1) gemm_ffma<8, 4, 4, 4, 1, 32>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else gemm_ffma<8, 2, 4, 4, 1, 64>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+  } else if constexpr (N == 32) {
+    if constexpr (SHAPE == 2) gemm_ffma<4, 8, 4, 4, 1, WIDE_BK>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else if constexpr (SHAPE == 1) gemm_ffma<4, 4, 4, 4, 1, 32>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else gemm_ffma<4, 2, 4, 4, 1, 64>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
   } else {
-    if ((M + 63) / 64 * cols >= 2 * FF_SMS) gemm_ffma<2, 2, 4, 1>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
-    else if ((M + 31) / 32 * cols >= FF_SMS) gemm_ffma<1, 2, 4, 2>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
-    else gemm_ffma<1, 2, 4, 4>(lc, kid, M, n_cols, K, K, classes, la, lb, ep);
+    if constexpr (SHAPE == 2) gemm_ffma<4, 8, 8, 4, 1, 16>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else if constexpr (SHAPE == 1) gemm_ffma<4, 4, 4, 2, 2, 32>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else gemm_ffma<4, 2, 4, 2, 2, 64>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
   }
+}
+template <int N, class LA, class LB, class EP>
+static void ff_rows(LaunchCtx& lc, int kid, int M, int n_cols, int K, int kps, int classes, LA la, LB lb, EP ep) {
+  const int shape = ff_shape(N, (long long)M * n_cols * classes * ((K + kps - 1) / kps));
+  if (shape == 2) ff_launch<N, 2>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+  else if (shape == 1) ff_launch<N, 1>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+  else ff_launch<N, 0>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
 }
 
 // Weight gradients: C(j, co) = sum over output positions of window(j) * gradient(co), one run of positions per split;
 // the splits' sums (and the bias gradient's, the column sums of the second operand) are added by finish_gradients().
-struct FfWgradPlan { int splits, kps; size_t part, total; };      // floats: the weights' partial sums, and all of them
-static int ff_wgrad_tiles(int J, int CO) { return CO <= 32 ? (J + 127) / 128 : ((J + 63) / 64) * ((CO + 63) / 64); }
+struct FfWgradPlan { int splits, kps; bool full; size_t part, total; };      // floats: the weights' partial sums, and all of them
 static FfWgradPlan ff_wgrad_plan(int J, int CO, int K) {
-  int s = 2 * FF_SMS / ff_wgrad_tiles(J, CO);
+  // tiles of 4096 outputs, 8 x 8 per lane, two warps; as many splits as fill the device once (six resident blocks per SM,
+  // three with 16 columns, whose tile is 256 rows high): a second, partly filled round costs as much as a full one
+  const int rows = CO == 16 ? 256 : (CO == 32 ? 128 : 64), cols = CO < 64 ? CO : 64;
+  const int tiles = ((J + rows - 1) / rows) * ((CO + cols - 1) / cols);
+  int s = (CO == 16 ? 3 : 6) * FF_SMS / tiles;
   const int by_k = (K + 63) / 64;
+  FfWgradPlan p;
+  p.full = s <= by_k;                                    // enough positions to fill the device that way
   if (s > by_k) s = by_k;
   if (s < 1) s = 1;
-  FfWgradPlan p;
-  p.kps = ffma_k_per_split(K, s, 16);
+  p.kps = ((K + s - 1) / s + 15) / 16 * 16;
   p.splits = (K + p.kps - 1) / p.kps;
   p.part = (size_t)p.splits * J * CO;
   p.total = (p.part + (size_t)p.splits * CO + 63) / 64 * 64;
@@ -74,8 +91,10 @@ static void ff_wgrad(LaunchCtx& lc, int kid, int J, int CO, int K, LA window, LB
   const FfWgradPlan p = ff_wgrad_plan(J, CO, K);
   FfPartialColsum ep;
   ep.part = scratch; ep.M = J; ep.N = CO; ep.colpart = scratch + p.part;
-  if constexpr (CO_TILE <= 32) gemm_ffma<4, 1, CO_TILE / 8, 1>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
-  else gemm_ffma<2, 2, 4, 1>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  if (!p.full) ff_rows<CO_TILE>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else if constexpr (CO_TILE == 16) gemm_ffma<16, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else if constexpr (CO_TILE == 32) gemm_ffma<8, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else gemm_ffma<4, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
   if (!add_grad_segment(segs, scratch, gw, p.splits, J, CO, scale) || !add_grad_segment(segs, ep.colpart, gb, p.splits, 1, CO, 1.f))
     lc.host_failure = true;
 }
@@ -86,40 +105,24 @@ static void conv_fwd(LaunchCtx& lc, int kid, const TIn* x, const TW* w, const fl
   if (use_tc3(lc))
     gemm_tc3(lc, kid, n * G::OH * G::OW, G::CO, G::KK, 1, ConvWindowOp<G, TIn>{x}, RowMajorOp<TW>{w, G::KK}, BiasReluEp<T>{out, bias, G::CO, scale});
   else
-    ff_rows<G::CO>(lc, kid, n * G::OH * G::OW, G::CO, G::KK, 1, FfWindow<G, TIn>{x}, FfRows<TW>{w, G::KK}, FfBiasRelu<T>{out, bias, G::CO, scale});
+    ff_rows<G::CO>(lc, kid, n * G::OH * G::OW, G::CO, G::KK, G::KK, 1, FfWindow<G, TIn>{x}, FfRows<TW>{w, G::KK}, FfBiasRelu<T>{out, bias, G::CO, scale});
 }
 // With few states the fully connected layer is a handful of tiles over a reduction of thousands: the reduction is then
 // split over many blocks (partial sums in scratch, added by launch_simt_tail) so that the weight matrix is streamed by
 // the whole device instead of by four blocks.  Returns the number of splits left in scratch (0: the layer is complete).
-static int fc_fwd_splits(int n, int F, int IN, int* kps) {
-  // as many splits as give every SM four CTAs, each at least 64 long
-  int s = 4 * FF_SMS / (((n + 31) / 32) * ((F + 63) / 64));
-  if (s > (IN + 63) / 64) s = (IN + 63) / 64;
-  if (s < 1) s = 1;
-  *kps = ffma_k_per_split(IN, s, 32);
-  return (IN + *kps - 1) / *kps;
-}
 template <class T, class TW>
 static int fc_fwd(LaunchCtx& lc, int kid, const T* x, const TW* w, const float* bias, T* out, int n,
                    int IN, int F, float* scratch) {
-  int splits = 1;
+  const int splits = pick_splits(n, F, IN);
   if (use_tc3(lc)) {
-    splits = pick_splits(n, F, IN);
-    if (splits <= 1) {
-      gemm_tc3(lc, kid, n, F, IN, 1, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, BiasReluEp<T>{out, bias, F, 1.f});
-      return 0;
-    }
-    gemm_tc3(lc, kid, n, F, IN, splits, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, PartialEp{scratch, n, F});
+    if (splits <= 1) gemm_tc3(lc, kid, n, F, IN, 1, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, BiasReluEp<T>{out, bias, F, 1.f});
+    else gemm_tc3(lc, kid, n, F, IN, splits, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, PartialEp{scratch, n, F});
+  } else if (splits <= 1) {
+    ff_rows<64>(lc, kid, n, F, IN, IN, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfBiasRelu<T>{out, bias, F, 1.f});
   } else {
-    int kps = IN;
-    splits = fc_fwd_splits(n, F, IN, &kps);
-    if (splits <= 1) {
-      gemm_ffma<2, 2, 4, 1>(lc, kid, n, F, IN, IN, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfBiasRelu<T>{out, bias, F, 1.f});
-      return 0;
-    }
-    gemm_ffma<1, 2, 4, 2>(lc, kid, n, F, IN, kps, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfPartial{scratch, n, F});
+    ff_rows<64>(lc, kid, n, F, IN, gemm_k_per_split(IN, splits), 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfPartial{scratch, n, F});
   }
-  return splits;
+  return splits <= 1 ? 0 : splits;
 }
 template <class G, class T, class TW>
 static void conv_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T* act_in, T* gin, int n) {
@@ -131,12 +134,12 @@ static void conv_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T*
         gemm_tc3(lc, kid, M, G::C, K, 1, ConvDgradClassOp<G, T>{g, z >> 1, z & 1}, ConvWeightClassOp<G, TW>{w, z >> 1, z & 1},
                  ReluMaskClassEp<G, T>{gin, act_in, z >> 1, z & 1});
     else
-      ff_rows<G::C>(lc, kid, M, G::C, K, 4, FfDgradClass<G, T>{g}, FfWeightClass<G, TW>{w, 0}, FfReluMaskClass<G, T>{gin, act_in, 0});
+      ff_rows<G::C>(lc, kid, M, G::C, K, K, 4, FfDgradClass<G, T>{g}, FfWeightClass<G, TW>{w, 0}, FfReluMaskClass<G, T>{gin, act_in, 0});
     return;
   }
   const int M = n * G::H * G::W, K = G::K * G::K * G::CO;
   if (use_tc3(lc)) gemm_tc3(lc, kid, M, G::C, K, 1, ConvDgradOp<G, T>{g}, ConvWeightTOp<G, TW>{w}, ReluMaskEp<T>{gin, act_in, G::C});
-  else ff_rows<G::C>(lc, kid, M, G::C, K, 1, FfDgradWindow<G, T>{g}, FfWeightT<G, TW>{w}, FfReluMask<T>{gin, act_in, G::C});
+  else ff_rows<G::C>(lc, kid, M, G::C, K, K, 1, FfDgradWindow<G, T>{g}, FfWeightT<G, TW>{w}, FfReluMask<T>{gin, act_in, G::C});
 }
 template <class G, class TIn, class T>
 static void conv_wgrad(LaunchCtx& lc, int kid, const T* g, const TIn* x, int n, float scale, float* gw,
@@ -155,7 +158,7 @@ template <class T, class TW>
 static void fc_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T* act_in, T* gin, int n,
                      int IN, int F) {
   if (use_tc3(lc)) gemm_tc3(lc, kid, n, IN, F, 1, RowMajorOp<T>{g, F}, ColMajorOp<TW>{w, IN}, ReluMaskEp<T>{gin, act_in, IN});
-  else ff_rows<64>(lc, kid, n, IN, F, 1, FfRows<T>{g, F}, FfCols<TW>{w, IN}, FfReluMask<T>{gin, act_in, IN});
+  else ff_rows<64>(lc, kid, n, IN, F, F, 1, FfRows<T>{g, F}, FfCols<TW>{w, IN}, FfReluMask<T>{gin, act_in, IN});
 }
 template <class T>
 static void fc_wgrad(LaunchCtx& lc, int kid, const T* g, const T* x, int n, int IN, int F, float* gw,
@@ -270,10 +273,7 @@ size_t simt_scratch_floats(int arch, const NetDims& nd, int n, int n_fwd) {
   // split-k partial sums of the fully connected layer's forward pass, which only ever sees n_fwd states at a time
   const LayerDims& f = nd.layer[nd.n_conv];
   const int IN = f.H * f.W * f.C;
-  int kps = 0, fs = fc_fwd_splits(n_fwd, nd.F, IN, &kps);
-  const int t3 = pick_splits(n_fwd, nd.F, IN);
-  if (t3 > fs) fs = t3;
-  const size_t fwd = (size_t)fs * n_fwd * nd.F;
+  const size_t fwd = (size_t)pick_splits(n_fwd, nd.F, IN) * n_fwd * nd.F;
   return best > fwd ? best : fwd;
 }
 

@@ -628,3 +628,16 @@ def test_pattern_environment_matches_the_oracle_and_can_be_learned(orc):
         last = mean_reward(20)
         assert last > 0.8 and last > first + 0.2, (first, last)
         g.close()
+
+
+@pytest.mark.parametrize("arch,n_e,t_max,A", [("nips", 1, 1, 2), ("nips", 49, 1, 32), ("nips", 97, 1, 7), ("nature", 3, 2, 20),
+                                              ("nature", 66, 1, 6)])
+def test_float_contraction_shapes(orc, arch, n_e, t_max, A):
+    """The CUDA-core contraction in each of its tile shapes, with remainders in every dimension, and the kernel that ends a
+    forward step with few and many head outputs: one update each, both passes from identical tensors."""
+    cfg = dict(arch=arch, precision="fp32", n_e=n_e, t_max=t_max, n_actions=A, lr=0.0028, term_denom=3)
+    o, g = make_pair(orc, cfg)
+    check_rollout(orc, o, g, TOL["fp32"])
+    check_update(orc, o, g, TOL["fp32"], inject=True)
+    assert g.error_word() == 0
+    g.close()
