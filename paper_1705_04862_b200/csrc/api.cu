@@ -316,6 +316,14 @@ struct SideBranch {
     enqueue();
     c->lc.st = main; c->lc.serialize_next = keep;
   }
+  // runs on the side stream after the side's own launches (and what those waited for) only
+  template <class F> void append(F enqueue) {
+    if (!forked) { enqueue(); return; }
+    const bool keep = c->lc.serialize_next;
+    c->lc.st = c->side_st; c->lc.serialize_next = true;
+    enqueue();
+    c->lc.st = main; c->lc.serialize_next = keep;
+  }
   void join() {
     if (!forked) return;
     cudaEventRecord(c->side_ev[MAX_LAYERS], c->side_st);
@@ -445,6 +453,9 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
     // The data gradients are a chain, and the first layer's weight gradient ends it; the other layers' weight gradients
     // only need their own layer's gradient and run beside the chain.
     SideBranch side(c);
+    // when every gradient goes through the finishing kernel, it also delivers the squared norm
+    const bool all_finished = !c->lc.fp32_tensor_cores || (use_tc(c) && c->tc_wgrad_mask == 0xF && tc_heads_backward_supported(c->nd));
+    int ready = 0;
     for (int l = L; l >= 0; --l) {
       // tensor-core kernels where they exist, the CUDA-core contraction otherwise
       const bool tc_wgrad = use_tc(c) && (c->tc_wgrad_mask >> l) & 1;
@@ -456,6 +467,12 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
                               c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, true, false);
       };
       if (l > 0) side.run(wgrad); else wgrad();
+      if (l == 2 && all_finished) {
+        // what has piled up so far (the heads, the fully connected layer, the third convolution) is most of the gradient:
+        // finished beside the rest of the chain
+        auto finish = [&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2, nullptr); };
+        if (side.on) side.append(finish);
+      }
       if (chunked && l == 1) {
         // data gradient and first-layer weight gradient group by group
         c->gact0_scale = tc_conv1_grad_scale();
@@ -478,13 +495,16 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
       }
     }
     side.join();
-    // when every gradient goes through the finishing kernel, it also delivers the squared norm
-    const bool all_finished = !c->lc.fp32_tensor_cores || (use_tc(c) && c->tc_wgrad_mask == 0xF && tc_heads_backward_supported(c->nd));
-    const int ready = finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials : nullptr);
-    launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad,
-                        c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
-                        c->norm_partials, c->stats, all_finished ? ready : 0);
-    if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
+    ready += finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials + ready : nullptr, NORM_BLOCKS - ready, c->stats);
+    if (all_finished && tc_supported(c->arch, c->prec)) {
+      tc_close_update(c->lc, c->nd, c->theta, c->rms, c->grad, c->theta16, c->w_images, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
+                      c->norm_partials, ready, c->stats);
+    } else {
+      launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad,
+                          c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
+                          c->norm_partials, c->stats, all_finished ? ready : 0);
+      if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
+    }
   });
   c->N += (uint64_t)c->B;
   c->rollout_fresh = false;

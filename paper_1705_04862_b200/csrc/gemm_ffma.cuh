@@ -163,9 +163,7 @@ gemm_ffma_kernel(int M, int N, int K, int k_per_split, int splits, LA la, LB lb,
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
   FfLoader<LA, BM, BK, NT> fa;
   FfLoader<LB, BN, BK, NT> fb;
-  // column sums: BN / 4 threads abreast take every (NT / (BN / 4))-th k of a block
-  constexpr int CS_COLS = BN / 4, CS_STEP = NT / CS_COLS;
-  float4 colsum = make_float4(0.f, 0.f, 0.f, 0.f);
+  float colsum = 0.f;              // thread n < BN of the first tile row: the sum over k of column n, in order
   fa.init(la, m0, M);
   fb.init(lb, n0, N);
   auto stage_of = [&](int block) { return ff_smem + (block % FF_STAGES) * C::STAGE; };
@@ -204,12 +202,10 @@ gemm_ffma_kernel(int M, int N, int K, int k_per_split, int splits, LA la, LB lb,
           for (int y = 0; y < TN; ++y) acc[x][y] = fmaf(a[q][x], b[q][y], acc[x][y]);
     }
     if constexpr (EP::COLSUM) {
-      static_assert(!LB::K_CONTIG && CS_STEP * CS_COLS == NT, "weight gradients");
-      if (blockIdx.x == 0)
-        for (int k = threadIdx.x / CS_COLS; k < BK; k += CS_STEP) {
-          const float4 v = *reinterpret_cast<const float4*>(tb + k * FfTile<LB, BN, BK>::LD + (threadIdx.x % CS_COLS) * 4);
-          colsum.x += v.x; colsum.y += v.y; colsum.z += v.z; colsum.w += v.w;
-        }
+      static_assert(!LB::K_CONTIG && BN <= NT, "weight gradients");
+      if (blockIdx.x == 0 && threadIdx.x < BN)
+#pragma unroll
+        for (int k = 0; k < BK; ++k) colsum += tb[k * FfTile<LB, BN, BK>::LD + threadIdx.x];
     }
     if (!fa.ASYNC && i + 1 < blocks) fa.store(stage_of(i + 1));
     if (!fb.ASYNC && i + 1 < blocks) fb.store(stage_of(i + 1) + C::A_FLOATS);
@@ -233,21 +229,7 @@ gemm_ffma_kernel(int M, int N, int K, int k_per_split, int splits, LA la, LB lb,
     }
   }
   if constexpr (EP::COLSUM) {
-    if (blockIdx.x == 0) {
-      float4* sh = reinterpret_cast<float4*>(ff_smem);
-      __syncthreads();
-      sh[threadIdx.x] = colsum;
-      __syncthreads();
-      if (threadIdx.x < CS_COLS) {
-        float4 t = sh[threadIdx.x];
-        for (int q = 1; q < CS_STEP; ++q) {
-          const float4 v = sh[q * CS_COLS + threadIdx.x];
-          t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
-        }
-        const int n = n0 + threadIdx.x * 4;
-        if (n < N) ep.colsum(n, t, split);
-      }
-    }
+    if (blockIdx.x == 0 && threadIdx.x < BN && n0 + threadIdx.x < N) ep.colsum(n0 + threadIdx.x, colsum, split);
   }
 }
 
@@ -432,7 +414,7 @@ struct FfPartial {                                           // part[split][m][n
 struct FfPartialColsum : FfPartial {                         // and the sum over k of B's rows: colpart[split][n]
   static constexpr bool COLSUM = true;
   float* colpart;
-  __device__ __forceinline__ void colsum(int n, float4 v, int split) const { store4(colpart + (size_t)split * N + n, v); }
+  __device__ __forceinline__ void colsum(int n, float v, int split) const { colpart[(size_t)split * N + n] = v; }
 };
 
 }  // namespace paac

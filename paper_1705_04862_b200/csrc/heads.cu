@@ -80,7 +80,10 @@ simt_tail_kernel(TailArgs q, T* h, const TW* wpi, const float* bpi, const TW* wv
   for (int k = warp; k <= A; k += WARPS) {
     float acc = 0.f;
 #pragma unroll
-    for (int i = 0; i < F / 32; ++i) acc = fmaf(wsh[k * F + lane + 32 * i], xs[lane + 32 * i], acc);
+    for (int i = 0; i < F / 32; ++i) {
+      const int at = sizeof(T) == 2 ? lane * (F / 32) + i : lane + 32 * i;      // (bf16 rows have always been dealt out in runs)
+      acc = fmaf(wsh[k * F + at], xs[at], acc);
+    }
     acc = warp_sum(acc);
     if (lane == 0) zs[k] = acc + (k < A ? bpi[k] : bv[0]);
   }

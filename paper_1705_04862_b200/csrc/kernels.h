@@ -42,12 +42,15 @@ void launch_advance_step(LaunchCtx& lc, uint64_t* step_base, uint32_t by);
 // The weight-gradient kernels leave partial sums part[split][J][CO] (J = 1 for biases) in scratch regions of their own
 // and note them in a GradSegments list; finish_gradients() adds them up, splits in a fixed order, into the gradient
 // vector (dst[co * J + j], times scale) with one launch and empties the list.
-struct GradSegment { const float* part; float* dst; int splits, J, CO; float scale; int first_group, groups, wide; };
+struct GradSegment { const float* part; float* dst; int splits, J, CO; float scale; int first_group, groups, mode; };
 struct GradSegments { GradSegment seg[12]; int n; int total_groups; };
-bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale);   // false: list full
+// in_order: one running sum over the splits (the float path's); otherwise eight interleaved ones where there are many.
+// false: list full
+bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale, bool in_order = false);
 // sumsq_partials != nullptr: every block also leaves the sum of squares of the gradient values it wrote in
-// sumsq_partials[block]; returns the number of blocks launched
-int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials);
+// sumsq_partials[block]; returns the number of blocks launched (at most max_blocks).  stats != nullptr: the error word is
+// taken down for the kernel that closes the update.
+int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, int max_blocks, DeviceStats* stats);
 
 // ---- network on the CUDA cores (net_simt.cu) --------------------------------------------
 // act[l]: stored activation of layer l for the n states, storage float (PAAC_FP32) or bf16.  Returns the number of split-k
@@ -73,7 +76,12 @@ void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, 
 // parameter change), and the data-gradient kernels that use them
 size_t tc_weight_image_elems();
 // (a first-layer weight whose fp16 image would overflow raises DEV_ERR_RANGE in *error_word)
+// (afterwards tc_close_update() keeps them up to date)
 void tc_relayout_weights(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, bf16* images, uint32_t* error_word);
+// The end of a tensor-core update: clipping and RMSProp as launch_clip_rmsprop, and in the same pass the bf16 copy and the
+// weight images.  norm_partials[0 .. n_partials) hold the squared norm, stats->error_taken the error word (finish_gradients).
+void tc_close_update(LaunchCtx& lc, const NetDims& nd, float* theta, float* rms, const float* grad, bf16* theta16, bf16* images,
+                     float lr, float rho, float eps, float clip, const float* norm_partials, int n_partials, DeviceStats* stats);
 // one block waits at most max_polls polls on a barrier nobody signals, then records the time-out in *error_word
 void launch_wait_probe(LaunchCtx& lc, uint32_t max_polls, uint32_t* error_word);
 void tc_backward_dgrad_fc(LaunchCtx& lc, const bf16* images, int n, void* const act[], void* const gact[], uint32_t* err);

@@ -66,21 +66,13 @@ static void ff_rows(LaunchCtx& lc, int kid, int M, int n_cols, int K, int kps, i
 }
 
 // Weight gradients: C(j, co) = sum over output positions of window(j) * gradient(co), one run of positions per split;
-// the splits' sums (and the bias gradient's, the column sums of the second operand) are added by finish_gradients().
-struct FfWgradPlan { int splits, kps; bool full; size_t part, total; };      // floats: the weights' partial sums, and all of them
+// the splits' sums (and the bias gradient's, the column sums of the second operand) are added, in split order, by
+// finish_gradients().  The runs are those of the three-pass path (pick_splits).
+struct FfWgradPlan { int splits, kps; size_t part, total; };      // floats: the weights' partial sums, and all of them
 static FfWgradPlan ff_wgrad_plan(int J, int CO, int K) {
-  // tiles of 4096 outputs, 8 x 8 per lane, two warps; as many splits as fill the device once (six resident blocks per SM,
-  // three with 16 columns, whose tile is 256 rows high): a second, partly filled round costs as much as a full one
-  const int rows = CO == 16 ? 256 : (CO == 32 ? 128 : 64), cols = CO < 64 ? CO : 64;
-  const int tiles = ((J + rows - 1) / rows) * ((CO + cols - 1) / cols);
-  int s = (CO == 16 ? 3 : 6) * FF_SMS / tiles;
-  const int by_k = (K + 63) / 64;
   FfWgradPlan p;
-  p.full = s <= by_k;                                    // enough positions to fill the device that way
-  if (s > by_k) s = by_k;
-  if (s < 1) s = 1;
-  p.kps = ((K + s - 1) / s + 15) / 16 * 16;
-  p.splits = (K + p.kps - 1) / p.kps;
+  p.splits = pick_splits(CO, J + 1, K);
+  p.kps = gemm_k_per_split(K, p.splits);
   p.part = (size_t)p.splits * J * CO;
   p.total = (p.part + (size_t)p.splits * CO + 63) / 64 * 64;
   return p;
@@ -91,11 +83,14 @@ static void ff_wgrad(LaunchCtx& lc, int kid, int J, int CO, int K, LA window, LB
   const FfWgradPlan p = ff_wgrad_plan(J, CO, K);
   FfPartialColsum ep;
   ep.part = scratch; ep.M = J; ep.N = CO; ep.colpart = scratch + p.part;
-  if (!p.full) ff_rows<CO_TILE>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
-  else if constexpr (CO_TILE == 16) gemm_ffma<16, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
-  else if constexpr (CO_TILE == 32) gemm_ffma<8, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
-  else gemm_ffma<4, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
-  if (!add_grad_segment(segs, scratch, gw, p.splits, J, CO, scale) || !add_grad_segment(segs, ep.colpart, gb, p.splits, 1, CO, 1.f))
+  // 64 x 64 tiles of 8 x 8 per lane where they give every SM three blocks, 128 x 32 of 8 x 4 where those give it one
+  if (CO_TILE == 64 && (J + 63) / 64 * ((CO + 63) / 64) * p.splits >= 3 * FF_SMS)
+    gemm_ffma<4, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else if (CO_TILE == 32 && (J + 127) / 128 * p.splits >= FF_SMS)
+    gemm_ffma<4, 8, 4, 4, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else
+    ff_rows<CO_TILE>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  if (!add_grad_segment(segs, scratch, gw, p.splits, J, CO, scale, true) || !add_grad_segment(segs, ep.colpart, gb, p.splits, 1, CO, 1.f, true))
     lc.host_failure = true;
 }
 
@@ -299,81 +294,76 @@ template <class TW> struct HeadWeightOp {   // row = fc unit i, k = head unit
 // Both heads in one kernel, for either storage type and either hidden size (the tensor-core path has one of its own for
 // 512 bf16 units): with dz[b][k] the loss gradient at output k of row b (the value is row k = A of the combined matrix),
 //   g_fc[b][i] = (h[b][i] > 0) * sum_k dz[b][k] W[k][i],   dW[k][i] = sum_b dz[b][k] h[b][i],   db[k] = sum_b dz[b][k].
-// A thread owns hidden units tid, tid + 256; their weights and gradient sums stay in registers, so a row costs it one
-// load of h per unit and 2 NK multiply-adds.  A block walks FH_ROWS or more rows (few enough blocks that their partial
-// sums, one set each, do not outweigh the gradient) and fetches all rows of a group before it uses them.
-constexpr int FH_THREADS = 256, FH_ROWS = 8, FH_MAX_BLOCKS = 148;
-template <class T, class TW, int F, int NK>
-__global__ void __launch_bounds__(FH_THREADS, 1)
-heads_backward_kernel(const T* h, const float* dz, const float* dV, const TW* wpi, const TW* wv, int n, int A, int rows_per,
+// A thread owns one hidden unit; its weights and gradient sums stay in registers, so a row costs it one load of h and
+// 2 NK multiply-adds.  A block takes 64 units and the rows of one split (at most about 128), FH_ROWS at a time, the next
+// ones on their way while these are used: a chain of some microseconds whatever the batch.
+constexpr int FH_THREADS = 64, FH_ROWS = 8;
+template <class T, class TW, int NK>
+__global__ void __launch_bounds__(FH_THREADS)
+heads_backward_kernel(const T* h, const float* dz, const float* dV, const TW* wpi, const TW* wv, int n, int F, int A, int rows_per,
                       T* g_fc, float* part_w, float* part_b, float* part_vw, float* part_vb) {
-  constexpr int U = F / FH_THREADS;
-  __shared__ __align__(16) float dzs[FH_ROWS][NK];
-  const int tid = threadIdx.x;
+  __shared__ float dzs[FH_ROWS][NK];
+  const int tid = threadIdx.x, col = blockIdx.y * FH_THREADS + tid;
   pdl_entry();
-  float w[NK][U], acc[NK][U], accb = 0.f;
+  float w[NK], acc[NK], accb = 0.f;
 #pragma unroll
-  for (int k = 0; k < NK; ++k)
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int col = tid + u * FH_THREADS;
-      acc[k][u] = 0.f;
-      w[k][u] = k < A ? to_f(wpi[(size_t)k * F + col]) : (k == A ? to_f(wv[col]) : 0.f);
-    }
+  for (int k = 0; k < NK; ++k) {
+    acc[k] = 0.f;
+    w[k] = k < A ? to_f(wpi[(size_t)k * F + col]) : (k == A ? to_f(wv[col]) : 0.f);
+  }
   const int r0 = blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
+  constexpr int DZ = (FH_ROWS * NK + FH_THREADS - 1) / FH_THREADS;
+  float hv[FH_ROWS], dv[DZ];
+  auto fetch = [&](int rb) {
+#pragma unroll
+    for (int j = 0; j < FH_ROWS; ++j) hv[j] = rb + j < r1 ? to_f(h[(size_t)(rb + j) * F + col]) : 0.f;
+#pragma unroll
+    for (int q = 0; q < DZ; ++q) {
+      const int i = tid + q * FH_THREADS, r = rb + i / NK, k = i % NK;
+      dv[q] = i < FH_ROWS * NK && r < r1 ? (k < A ? dz[(size_t)r * A + k] : (k == A ? dV[r] : 0.f)) : 0.f;
+    }
+  };
+  fetch(r0);
   for (int rb = r0; rb < r1; rb += FH_ROWS) {
-    float hv[FH_ROWS][U];
+    float hc[FH_ROWS];
 #pragma unroll
-    for (int j = 0; j < FH_ROWS; ++j)
-#pragma unroll
-      for (int u = 0; u < U; ++u) hv[j][u] = rb + j < r1 ? to_f(h[(size_t)(rb + j) * F + tid + u * FH_THREADS]) : 0.f;
+    for (int j = 0; j < FH_ROWS; ++j) hc[j] = hv[j];
     __syncthreads();
-    for (int i = tid; i < FH_ROWS * NK; i += FH_THREADS) {
-      const int r = rb + i / NK, k = i % NK;
-      dzs[i / NK][k] = r < r1 ? (k < A ? dz[(size_t)r * A + k] : (k == A ? dV[r] : 0.f)) : 0.f;
+#pragma unroll
+    for (int q = 0; q < DZ; ++q) {
+      const int i = tid + q * FH_THREADS;
+      if (i < FH_ROWS * NK) dzs[i / NK][i % NK] = dv[q];
     }
     __syncthreads();
+    if (rb + FH_ROWS < r1) fetch(rb + FH_ROWS);
     if (tid <= A)
 #pragma unroll
       for (int j = 0; j < FH_ROWS; ++j) accb += dzs[j][tid];          // rows past the end hold zeros
 #pragma unroll
     for (int j = 0; j < FH_ROWS; ++j) {
-      if (rb + j >= r1) break;
-      float g[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) g[u] = 0.f;
+      float g = 0.f;
 #pragma unroll
       for (int k = 0; k < NK; ++k) {
         const float d = dzs[j][k];
-#pragma unroll
-        for (int u = 0; u < U; ++u) { g[u] = fmaf(d, w[k][u], g[u]); acc[k][u] = fmaf(d, hv[j][u], acc[k][u]); }
+        g = fmaf(d, w[k], g);
+        acc[k] = fmaf(d, hc[j], acc[k]);
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        g_fc[(size_t)(rb + j) * F + tid + u * FH_THREADS] = from_f<T>(hv[j][u] > 0.f ? g[u] : 0.f);
+      if (rb + j < r1) g_fc[(size_t)(rb + j) * F + col] = from_f<T>(hc[j] > 0.f ? g : 0.f);
     }
   }
-  const size_t cta = blockIdx.x;
+  const size_t split = blockIdx.x;
 #pragma unroll
-  for (int k = 0; k < NK; ++k)
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int col = tid + u * FH_THREADS;
-      if (k < A) part_w[(cta * A + k) * F + col] = acc[k][u];
-      else if (k == A) part_vw[cta * F + col] = acc[k][u];
-    }
-  if (tid < A) part_b[cta * A + tid] = accb;
-  else if (tid == A) part_vb[cta] = accb;
-}
-static int ff_heads_blocks(int n, int* rows_per) {
-  int blocks = (n + FH_ROWS - 1) / FH_ROWS;
-  if (blocks > FH_MAX_BLOCKS) blocks = FH_MAX_BLOCKS;
-  *rows_per = (n + blocks - 1) / blocks;
-  return (n + *rows_per - 1) / *rows_per;
+  for (int k = 0; k < NK; ++k) {
+    if (k < A) part_w[(split * A + k) * F + col] = acc[k];
+    else if (k == A) part_vw[split * F + col] = acc[k];
+  }
+  if (blockIdx.y == 0) {
+    if (tid < A) part_b[split * A + tid] = accb;
+    else if (tid == A) part_vb[split] = accb;
+  }
 }
 static size_t ff_heads_scratch_floats(const NetDims& nd, int n) {
-  int rows = 0;
-  return (size_t)ff_heads_blocks(n, &rows) * (nd.A + 1) * (nd.F + 1) + 8;
+  return (size_t)pick_splits(nd.A + 1, nd.F + 1, n) * (nd.A + 1) * (nd.F + 1) + 8;
 }
 
 template <class T, class TW>
@@ -390,28 +380,21 @@ static void heads_backward_t(LaunchCtx& lc, const NetDims& nd, const TW* w, cons
     reduce_wgrad(lc, scratch, splits, A + 1, A, 1, F, 1.f, grad + nd.v_w, grad + nd.v_b);
     return;
   }
-  int rows_per = 0;
-  const int blocks = ff_heads_blocks(n, &rows_per);
+  const int splits = pick_splits(A + 1, F + 1, n), rows_per = gemm_k_per_split(n, splits);
   float* part_w = scratch + ff_scratch_offset(nd, n, nd.n_conv + 1);
-  float* part_b = part_w + (size_t)blocks * A * F;
-  float* part_vw = part_b + (size_t)blocks * A;
-  float* part_vb = part_vw + (size_t)blocks * F;
+  float* part_b = part_w + (size_t)splits * A * F;
+  float* part_vw = part_b + (size_t)splits * A;
+  float* part_vb = part_vw + (size_t)splits * F;
   auto launch = [&](auto kern) {
     KernelScope scope(lc, KID_HEADS_BWD);
-    launch_kernel_overlapped(lc, kern, dim3(blocks), dim3(FH_THREADS), 0, h, dz, dV, w + nd.pi_w, w + nd.v_w, n, A, rows_per,
-                             gact_fc, part_w, part_b, part_vw, part_vb);
+    launch_kernel_overlapped(lc, kern, dim3(splits, F / FH_THREADS), dim3(FH_THREADS), 0, h, dz, dV, w + nd.pi_w, w + nd.v_w, n, F, A,
+                             rows_per, gact_fc, part_w, part_b, part_vw, part_vb);
   };
-  if (F == 256) {
-    if (A < 8) launch(heads_backward_kernel<T, TW, 256, 8>);
-    else if (A < 20) launch(heads_backward_kernel<T, TW, 256, 20>);
-    else launch(heads_backward_kernel<T, TW, 256, 33>);
-  } else {
-    if (A < 8) launch(heads_backward_kernel<T, TW, 512, 8>);
-    else if (A < 20) launch(heads_backward_kernel<T, TW, 512, 20>);
-    else launch(heads_backward_kernel<T, TW, 512, 33>);
-  }
-  if (!add_grad_segment(segs, part_w, grad + nd.pi_w, blocks, 1, F * A, 1.f) || !add_grad_segment(segs, part_b, grad + nd.pi_b, blocks, 1, A, 1.f) ||
-      !add_grad_segment(segs, part_vw, grad + nd.v_w, blocks, 1, F, 1.f) || !add_grad_segment(segs, part_vb, grad + nd.v_b, blocks, 1, 1, 1.f))
+  if (A < 8) launch(heads_backward_kernel<T, TW, 8>);
+  else if (A < 20) launch(heads_backward_kernel<T, TW, 20>);
+  else launch(heads_backward_kernel<T, TW, 33>);
+  if (!add_grad_segment(segs, part_w, grad + nd.pi_w, splits, 1, F * A, 1.f, true) || !add_grad_segment(segs, part_b, grad + nd.pi_b, splits, 1, A, 1.f, true) ||
+      !add_grad_segment(segs, part_vw, grad + nd.v_w, splits, 1, F, 1.f, true) || !add_grad_segment(segs, part_vb, grad + nd.v_b, splits, 1, 1, 1.f, true))
     lc.host_failure = true;
 }
 

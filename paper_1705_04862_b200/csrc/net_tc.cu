@@ -17,6 +17,7 @@
 #include <cuda.h>          // CUtensorMap and its enums only; the encoder is looked up at run time, nothing links to libcuda
 
 #include "kernels.h"
+#include "optim_device.cuh"
 #include "tc_common.cuh"
 
 namespace paac {
@@ -2514,10 +2515,15 @@ __global__ void tc_bias_final_kernel(const float* __restrict__ part, int blocks,
 //   many splits: a group is FG_J j x 32 co; warp w adds the splits w, w + 8, ... for these j, the eight warps' sums
 //                are then added in warp order;
 //   few splits:  a group is 32 j x 32 co; warp w adds all splits, in order, for rows w, w + 8, w + 16, w + 24.
+//   many splits, in order (the float path): the warps bring FG_CHUNK splits of a group into shared memory and one thread
+//                per output adds them up one after the other.
 constexpr int FG_J = 2;          // rows of j per group of a many-split segment
-__global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments segs, float* __restrict__ sumsq_partials) {
+constexpr int FG_CHUNK = 128;    // splits at a time of a segment added in order
+enum { FG_FEW = 0, FG_MANY = 1, FG_IN_ORDER = 2 };
+__global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments segs, float* __restrict__ sumsq_partials, DeviceStats* stats) {
   pdl_entry();
-  __shared__ float sh[8 * 8 * 33];
+  if (stats != nullptr && blockIdx.x == 0 && threadIdx.x == 0) stats->error_taken = *reinterpret_cast<const volatile uint32_t*>(&stats->error_word);
+  __shared__ float sh[FG_CHUNK * FG_J * 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float ss = 0.f;                       // sum of squares of the gradient values this thread writes
   for (int grp = blockIdx.x; grp < segs.total_groups; grp += gridDim.x) {
@@ -2528,7 +2534,42 @@ __global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments seg
     const int co0 = (local % co_tiles) * 32, J = sg.J, CO = sg.CO;
     const size_t total = (size_t)J * CO;
     const bool co_ok = co0 + lane < CO;
-    if (sg.wide) {
+    if (sg.mode == FG_IN_ORDER) {
+      const int j0 = (local / co_tiles) * FG_J, j = j0 + (int)threadIdx.x / 32;
+      const float* src = sg.part + (size_t)j0 * CO + co0 + lane;
+      float t = 0.f;
+      for (int p0 = 0; p0 < sg.splits; p0 += FG_CHUNK) {
+        const int count = min(FG_CHUNK, sg.splits - p0);
+        __syncthreads();
+        constexpr int PER = FG_CHUNK / 8;
+        float v[PER][FG_J];
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+#pragma unroll
+          for (int q = 0; q < FG_J; ++q)
+            v[u][q] = (co_ok && j0 + q < J && warp + 8 * u < count) ? __ldg(src + (size_t)(p0 + warp + 8 * u) * total + (size_t)q * CO) : 0.f;
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+#pragma unroll
+          for (int q = 0; q < FG_J; ++q) sh[((warp + 8 * u) * FG_J + q) * 32 + lane] = v[u][q];
+        __syncthreads();
+        if (threadIdx.x < FG_J * 32) {
+          const float* column = sh + threadIdx.x;
+          int p = 0;
+          for (; p + 16 <= count; p += 16) {
+#pragma unroll
+            for (int u = 0; u < 16; ++u) t += column[(p + u) * FG_J * 32];
+          }
+          for (; p < count; ++p) t += column[p * FG_J * 32];
+        }
+      }
+      if (threadIdx.x < FG_J * 32 && co_ok && j < J) {
+        const float v = t * sg.scale;
+        sg.dst[(size_t)(co0 + lane) * J + j] = v;
+        ss = fmaf(v, v, ss);
+      }
+      __syncthreads();
+    } else if (sg.mode == FG_MANY) {
       // a group is FG_J j x 32 co: small, so that the many-split layers spread over all blocks of the grid; warp w
       // adds the splits w, w + 8, ... with 32 loads in flight per thread (its latency, not the bandwidth, sets the
       // pace of a group); the additions keep their order
@@ -2604,13 +2645,14 @@ __global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments seg
   }
 }
 
-bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale) {
+bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale, bool in_order) {
   if (segs->n >= (int)(sizeof(segs->seg) / sizeof(segs->seg[0]))) return false;      // the caller reports a host failure
   GradSegment& g = segs->seg[segs->n++];
   g.part = part; g.dst = dst; g.splits = splits; g.J = J; g.CO = CO; g.scale = scale;
-  g.wide = splits > 8;
+  g.mode = splits <= 8 ? FG_FEW : (in_order ? FG_IN_ORDER : FG_MANY);
   g.first_group = segs->total_groups;
-  g.groups = ((J + (g.wide ? FG_J : 32) - 1) / (g.wide ? FG_J : 32)) * ((CO + 31) / 32);
+  const int rows = g.mode == FG_FEW ? 32 : FG_J;
+  g.groups = ((J + rows - 1) / rows) * ((CO + 31) / 32);
   segs->total_groups += g.groups;
   return true;
 }
@@ -3211,12 +3253,12 @@ size_t tc_scratch_floats(int n) { return tc_layer_scratch_offset(n, 4) + tc_head
 
 // Enqueues the weight-gradient kernel of `layer` (0 = conv1 .. 3 = fc) and notes in *segs where its partial
 // sums are; finish_gradients() then turns all noted partial sums into the gradient vector in one launch.
-int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials) {
+int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, int max_blocks, DeviceStats* stats) {
   int blocks = 0;
   if (segs->n > 0) {
     KernelScope scope(lc, KID_WGRAD_REDUCE);
-    blocks = segs->total_groups < NORM_BLOCKS ? segs->total_groups : NORM_BLOCKS;
-    launch_kernel(lc, tc_finalize_grads_kernel, blocks, 256, 0, *segs, sumsq_partials);
+    blocks = segs->total_groups < max_blocks ? segs->total_groups : max_blocks;
+    launch_kernel(lc, tc_finalize_grads_kernel, blocks, 256, 0, *segs, sumsq_partials, stats);
   }
   segs->n = 0; segs->total_groups = 0;
   return blocks;
@@ -3418,6 +3460,107 @@ void tc_relayout_weights(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, 
   launch_kernel(lc, relayout_weights_kernel, RL_FC_TILES + RL_SMALL_BLOCKS, 256, 0, theta16 + d[0].w_off, theta16 + d[1].w_off, theta16 + d[2].w_off,
                                                   theta16 + d[3].w_off, images + TC_IMG_W2, images + TC_IMG_W3,
                                                   images + TC_IMG_WFC, images + TC_IMG_W1, error_word);
+}
+
+// The end of an update in one launch: clipping, RMSProp, the bf16 copy and the weight images.  Blocks 0 .. RL_FC_TILES - 1
+// take a 64 x 64 tile of the fully connected matrix each and write its transposed bf16 tile through shared memory; the
+// others take 4096 of the remaining parameters each and scatter the bf16 values of the convolution weights into their
+// images.  Parameters and RMSProp state are fetched before the wait on the finishing kernel, gradients after it.  A launch
+// of its own for the images (5.6 us, and its wait for the optimiser kernel) is what this saves; what bounds the rest is
+// latency: 37 MB, most of it in L2, over 414 blocks.
+constexpr int CU_THREADS = 256, CU_PER = 4;                       // float4 per thread
+constexpr size_t CU_CHUNK = (size_t)CU_THREADS * CU_PER * 4;
+__global__ void __launch_bounds__(CU_THREADS, 3)
+tc_close_update_kernel(size_t P, size_t w1_off, size_t w2_off, size_t w3_off, size_t wfc_off, float* theta, float* rms, const float* grad,
+                       bf16* theta16, bf16* w2_d, bf16* w3_d, bf16* wfc_t, bf16* w1_b, float lr, float rho, float eps, float clip,
+                       const float* partials, int n_partials, DeviceStats* stats) {
+  typedef NatConv1 C1; typedef NatConv2 C2; typedef NatConv3 C3;
+  constexpr size_t NF = 3136 * 512;
+  __shared__ uint16_t tile[64][66];                              // row pitch of 33 words: column reads spread over the banks
+  const bool fc = blockIdx.x < RL_FC_TILES;
+  const int o0 = (blockIdx.x % 8) * 64, in0 = (blockIdx.x / 8) * 64, r = threadIdx.x >> 2, c = threadIdx.x & 3;
+  const size_t rest = P - NF;                                    // everything else, the fully connected matrix cut out
+  size_t at[CU_PER];                                             // first parameter of each group of four (P: none)
+#pragma unroll
+  for (int j = 0; j < CU_PER; ++j) {
+    if (fc) {
+      at[j] = wfc_off + (size_t)(o0 + r) * 3136 + in0 + 4 * c + 16 * j;
+    } else {
+      const size_t q = (blockIdx.x - RL_FC_TILES) * CU_CHUNK + ((size_t)j * CU_THREADS + threadIdx.x) * 4;
+      at[j] = q >= rest ? P : (q < wfc_off ? q : q + NF);
+    }
+  }
+  float4 t4[CU_PER], m4[CU_PER], g4[CU_PER];
+  auto load = [&](const float* p, size_t i) {
+    if (i + 4 <= P) return *reinterpret_cast<const float4*>(p + i);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < P) v.x = p[i];
+    if (i + 1 < P) v.y = p[i + 1];
+    if (i + 2 < P) v.z = p[i + 2];
+    return v;
+  };
+#pragma unroll
+  for (int j = 0; j < CU_PER; ++j) { t4[j] = load(theta, at[j]); m4[j] = load(rms, at[j]); }
+  pdl_entry();
+#pragma unroll
+  for (int j = 0; j < CU_PER; ++j) g4[j] = load(grad, at[j]);
+  const RmsStep step{lr, rho, eps, clip_scale_of<CU_THREADS>(partials, n_partials, clip, stats->error_taken, stats)};
+  if (step.scale < 0.f) return;
+#pragma unroll
+  for (int j = 0; j < CU_PER; ++j) {
+    const size_t i = at[j];
+    if (i >= P) continue;
+    float* t = &t4[j].x; float* m = &m4[j].x; const float* g = &g4[j].x;
+    uint16_t h[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { step(t[e], m[e], g[e]); h[e] = __bfloat16_as_ushort(__float2bfloat16_rn(t[e])); }
+    const uint2 packed = make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
+    if (i + 4 <= P) {
+      *reinterpret_cast<float4*>(theta + i) = t4[j]; *reinterpret_cast<float4*>(rms + i) = m4[j];
+      *reinterpret_cast<uint2*>(theta16 + i) = packed;
+    } else {
+      for (int e = 0; e < 4 && i + e < P; ++e) { theta[i + e] = t[e]; rms[i + e] = m[e]; reinterpret_cast<uint16_t*>(theta16)[i + e] = h[e]; }
+    }
+    if (fc) {
+      *reinterpret_cast<uint32_t*>(&tile[r][4 * c + 16 * j]) = packed.x;
+      *reinterpret_cast<uint32_t*>(&tile[r][4 * c + 16 * j + 2]) = packed.y;
+    } else if (i >= w3_off && i < w3_off + C3::CO * C3::KK) {     // four neighbours share all but the input channel
+      const int k = (int)(i - w3_off), ci = k % 64, tap = (k / 64) % 9, co = k / 576;
+      for (int e = 0; e < 4; ++e) reinterpret_cast<uint16_t*>(w3_d)[((ci + e) * 9 + tap) * 64 + co] = h[e];
+    } else if (i >= w2_off && i < w2_off + C2::CO * C2::KK) {
+      const int k = (int)(i - w2_off), ci = k % 32, s = (k / 32) % 4, rr = (k / 128) % 4, co = k / 512;
+      const int z = 2 * (rr & 1) + (s & 1), tap = 2 * (rr >> 1) + (s >> 1);
+      for (int e = 0; e < 4; ++e) reinterpret_cast<uint16_t*>(w2_d)[((z * 32 + ci + e) * 4 + tap) * 64 + co] = h[e];
+    } else if (i >= w1_off && i < w1_off + C1::CO * C1::KK) {
+      const int k = (int)(i - w1_off), s = (k / 4) % 8, rr = (k / 32) % 8, co = k / 256;
+      const int to = ((co * 4 + 2 * (rr >> 2) + (s >> 2)) * 4 + (rr & 3)) * 16 + (s & 3) * 4;
+      for (int e = 0; e < 4; ++e) {
+        // the forward kernel's copy of the first layer is fp16, scaled by 2^8 (see u8x4_to_f16x4)
+        const float scaled = __bfloat162float(__ushort_as_bfloat16(h[e])) * C1_F16_WEIGHT_SCALE;
+        if (!(fabsf(scaled) <= 65504.f)) atomicOr(&stats->error_word, DEV_ERR_RANGE);      // beyond fp16 (or not a number)
+        reinterpret_cast<__half*>(w1_b)[to + e] = __float2half_rn(scaled);
+      }
+    }
+  }
+  if (!fc) return;
+  __syncthreads();
+  uint32_t v[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    v[e] = (uint32_t)tile[16 * c + 2 * e][r] | ((uint32_t)tile[16 * c + 2 * e + 1][r] << 16);
+  uint4* dst = reinterpret_cast<uint4*>(wfc_t + (size_t)(in0 + r) * 512 + o0 + 16 * c);
+  dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+  dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+}
+
+void tc_close_update(LaunchCtx& lc, const NetDims& nd, float* theta, float* rms, const float* grad, bf16* theta16, bf16* images,
+                     float lr, float rho, float eps, float clip, const float* norm_partials, int n_partials, DeviceStats* stats) {
+  const LayerDims* d = nd.layer;
+  const size_t rest = nd.P - (size_t)3136 * 512;
+  KernelScope scope(lc, KID_CLIP_RMSPROP);
+  launch_kernel_overlapped(lc, tc_close_update_kernel, RL_FC_TILES + (int)((rest + CU_CHUNK - 1) / CU_CHUNK), CU_THREADS, 0, nd.P, d[0].w_off,
+                           d[1].w_off, d[2].w_off, d[3].w_off, theta, rms, grad, theta16, images + TC_IMG_W2, images + TC_IMG_W3,
+                           images + TC_IMG_WFC, images + TC_IMG_W1, lr, rho, eps, clip, norm_partials, n_partials, stats);
 }
 
 // ---- failure-path probe: a bounded wait that is made to run out ------------------------------------------------

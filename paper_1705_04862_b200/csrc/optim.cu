@@ -1,5 +1,6 @@
 // Global-norm clipping fused with RMSProp.
 #include "kernels.h"
+#include "optim_device.cuh"
 
 namespace paac {
 
@@ -32,12 +33,7 @@ sumsq_kernel(const float* __restrict__ g, size_t P, float* __restrict__ partials
   if (threadIdx.x == 0) partials[blockIdx.x] = sh[0];
 }
 
-// pass 2: every block re-adds the partials in the same order (so all agree bit for bit),
-// forms scale = min(1, clip / norm) and applies
-//   m <- rho m + (1 - rho) (scale g)^2,  theta <- theta - lr (scale g) / sqrt(m + eps)
-// and refreshes the bf16 copy.  A non-finite norm leaves theta and m untouched, and so does a device error
-// left by any earlier kernel (a bounded wait that gave up means some tile or partial sum of this update is
-// garbage): the status then names the error.
+// pass 2: norm, clipping factor, RMSProp and the refreshed bf16 copy (see optim_device.cuh).
 // One wave of two blocks per SM, launched so that it may start while the finishing kernel drains: a thread's first
 // UPD_AHEAD groups of parameters and state (all of them, up to 1.8 M parameters) are fetched before the wait, the
 // gradients right after it, together with the partial sums of the norm.
@@ -46,8 +42,6 @@ __global__ void __launch_bounds__(UPD_THREADS, 2)
 clip_rmsprop_kernel(size_t P, float* theta, float* rms, const float* g,
                     bf16* __restrict__ theta16, float lr, float rho, float eps, float clip,
                     const float* partials, int n_partials, DeviceStats* stats) {
-  __shared__ float sh[UPD_THREADS / 32];
-  __shared__ float s_scale;
   const size_t n4 = P / 4, stride = (size_t)gridDim.x * UPD_THREADS;
   float4* t4 = reinterpret_cast<float4*>(theta);
   float4* m4 = reinterpret_cast<float4*>(rms);
@@ -61,44 +55,12 @@ clip_rmsprop_kernel(size_t P, float* theta, float* rms, const float* g,
 #pragma unroll
   for (int u = 0; u < UPD_AHEAD; ++u)
     if (i0 + u * stride < n4) gv0[u] = g4[i0 + u * stride];
-  // the device error word, fetched now so that its latency hides behind the sum of the partials
-  uint32_t dev_err = 0u;
-  if (threadIdx.x == 0) dev_err = *reinterpret_cast<const volatile uint32_t*>(&stats->error_word);
-  float acc = 0.f;
-  for (int i = threadIdx.x; i < n_partials; i += UPD_THREADS) acc += partials[i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float total = 0.f;
-#pragma unroll
-    for (int w = 0; w < UPD_THREADS / 32; ++w) total += sh[w];
-    const float norm = sqrtf(total);
-    float scale = 1.f;
-    const bool ok = isfinite(norm) && dev_err == 0u;
-    if (ok && clip > 0.f && norm > clip) scale = clip / norm;
-    s_scale = ok ? scale : -1.f;
-    if (blockIdx.x == 0) {
-      stats->grad_norm = norm;
-      stats->clip_scale = ok ? scale : 0.f;
-      stats->status = ok ? PAAC_OK
-                         : ((dev_err & DEV_ERR_WAIT_MASK) ? PAAC_ERR_TIMEOUT
-                                                           : ((dev_err & DEV_ERR_RANGE) ? PAAC_ERR_RANGE : PAAC_ERR_NONFINITE));
-    }
-  }
-  __syncthreads();
-  const float scale = s_scale;
-  if (scale < 0.f) return;
-  const float one_m_rho = 1.f - rho;
+  const RmsStep step{lr, rho, eps, clip_scale_of<UPD_THREADS>(partials, n_partials, clip, stats->error_word, stats)};
+  if (step.scale < 0.f) return;
   auto apply = [&](size_t i, float4& tv, float4& mv, const float4& gv) {
     const float* gp = &gv.x; float* mp = &mv.x; float* tp = &tv.x;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float gs = scale * gp[j];
-      mp[j] = fmaf(rho, mp[j], one_m_rho * gs * gs);
-      tp[j] = tp[j] - lr * gs / sqrtf(mp[j] + eps);
-    }
+    for (int j = 0; j < 4; ++j) step(tp[j], mp[j], gp[j]);
     m4[i] = mv; t4[i] = tv;
     if (theta16 != nullptr) {
       __nv_bfloat162 lo = __floats2bfloat162_rn(tv.x, tv.y), hi = __floats2bfloat162_rn(tv.z, tv.w);
@@ -116,11 +78,9 @@ clip_rmsprop_kernel(size_t P, float* theta, float* rms, const float* g,
   }
   if (blockIdx.x == 0) {
     for (size_t i = n4 * 4 + threadIdx.x; i < P; i += UPD_THREADS) {
-      const float gs = scale * g[i];
-      const float m = fmaf(rho, rms[i], one_m_rho * gs * gs);
-      rms[i] = m;
-      const float t = theta[i] - lr * gs / sqrtf(m + eps);
-      theta[i] = t;
+      float t = theta[i], m = rms[i];
+      step(t, m, g[i]);
+      rms[i] = m; theta[i] = t;
       if (theta16 != nullptr) theta16[i] = __float2bfloat16_rn(t);
     }
   }
