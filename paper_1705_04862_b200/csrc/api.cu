@@ -11,7 +11,7 @@ using namespace paac;
 // and picked up by polling a flag: no copy engine, no stream synchronisation.  The pointers let a recorded sequence
 // read buffers that differ from call to call.
 struct HostBox {
-  volatile uint32_t done;                       // set by the device when actions and values are there
+  volatile uint32_t done;                       // set by the device when actions and values (or the statistics) are there
   HostPlanes planes;                            // the newest frames and the restart flags of the step in flight
   DeviceStats stats;
   int32_t* actions; float* values; uint8_t* restart;      // [n_e] each, behind this struct
@@ -49,9 +49,9 @@ struct paac_ctx {
   cudaStream_t side_st;    // weight gradients run here, next to the chain of data gradients (see SideBranch)
   cudaEvent_t side_ev[MAX_LAYERS + 1];
   cudaStream_t record_st;  // where sequences are recorded when st is the legacy default stream (made on first use)
-  // recorded launch sequences: kind 0 = rollout, 1 = update, 2 + 2 t + v = step t of the external-environment mode
+  // recorded launch sequences: kind 0 = rollout, 1 = update, 2 = update that reports, 3 + 2 t + v = step t of the external-environment mode
   // (v = 1: with the frame stack built on the device), each for both parities of the frame buffers
-  static constexpr int GRAPH_KINDS = 2 + 2 * 65;
+  static constexpr int GRAPH_KINDS = 3 + 2 * 65;
   int plain_calls[GRAPH_KINDS][2];   // calls made with plain launches
   cudaGraphExec_t graph[GRAPH_KINDS][2];
   uint64_t graph_launches[GRAPH_KINDS][2];
@@ -228,6 +228,18 @@ bool host_box(paac_ctx* c) {
   char* q = (char*)p + head;
   c->box->actions = (int32_t*)q; c->box->values = (float*)(q + 4 * n);
   c->box->restart = (uint8_t*)(q + 8 * n); c->box->outcomes = (uint8_t*)(q + 9 * n);
+  return true;
+}
+// Waits for the flag that the last kernel of a launch sequence sets; a failed launch or kernel shows in the stream's
+// status instead.
+bool await_box(paac_ctx* c) {
+  for (uint32_t polls = 1; !c->box->done; ++polls) {
+    if (polls & 0x3FFFu) continue;
+    const cudaError_t st = cudaStreamQuery(c->st);
+    if (st == cudaErrorNotReady) continue;
+    if (st != cudaSuccess || !c->box->done) { cudaGetLastError(); return false; }
+  }
+  __atomic_thread_fence(__ATOMIC_ACQUIRE);
   return true;
 }
 // the rollout's outcomes, gathered by paac_observe_host, to the device in one copy
@@ -435,8 +447,10 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
 int paac_update(paac_ctx* c, paac_update_stats* stats) {
   if (!c) return PAAC_ERR_ARG;
   if (!c->rollout_fresh) return PAAC_ERR_STATE;
+  if (stats && !host_box(c)) return PAAC_ERR_CUDA;
+  if (stats) c->box->done = 0u;
   const paac_hparams& hp = c->hp;
-  run_recorded(c, 1, c->cur, [&]() {
+  run_recorded(c, stats ? 2 : 1, c->cur, [&]() {
     launch_returns_head_grad(c->lc, head_mode(c), c->n_e, c->t_max, c->A, hp.gamma, hp.entropy_beta, hp.value_coef, c->rewards,
                              c->terminals, c->logits, c->values, c->actions, c->R, c->adv, c->dz, c->dV, c->loss_terms,
                              c->stats);
@@ -505,15 +519,14 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
                           c->norm_partials, c->stats, all_finished ? ready : 0);
       if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
     }
+    if (stats) launch_publish_stats(c->lc, c->stats, &c->box->stats, &c->box->done);
   });
   c->N += (uint64_t)c->B;
   c->rollout_fresh = false;
   if (cuda_status(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (stats) {
-    if (!host_box(c)) return PAAC_ERR_CUDA;
-    DeviceStats& ds = c->box->stats;
-    if (cudaMemcpyAsync(&ds, c->stats, sizeof(ds), cudaMemcpyDeviceToHost, c->st) != cudaSuccess ||
-        cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
+    if (!await_box(c)) return PAAC_ERR_CUDA;
+    const DeviceStats& ds = c->box->stats;
     stats->policy_loss = ds.policy_loss; stats->value_loss = ds.value_loss; stats->entropy = ds.entropy;
     stats->grad_norm = ds.grad_norm; stats->clip_scale = ds.clip_scale; stats->status = ds.status;
     stats->timesteps = c->N;
@@ -659,21 +672,14 @@ static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, uint8_t* dst
   const size_t row = (size_t)t * c->n_e;
   HostBox* box = c->box;
   box->done = 0u;
-  run_recorded(c, 2 + 2 * t + (prev ? 1 : 0), c->cur, [&]() {
+  run_recorded(c, 3 + 2 * t + (prev ? 1 : 0), c->cur, [&]() {
     if (prev) launch_stack_pull(c->lc, prev, &box->planes, dst, c->n_e);
     bool advanced = false;
     forward_slot(c, dst, t, sample, nullptr, sample ? nullptr : &advanced);
     if (!sample && !advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
     launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
   });
-  // the flag is set by the sequence's last kernel; a failed launch or kernel shows in the stream's status instead
-  for (uint32_t polls = 1; !box->done; ++polls) {
-    if (polls & 0x3FFFu) continue;
-    const cudaError_t st = cudaStreamQuery(c->st);
-    if (st == cudaErrorNotReady) continue;
-    if (st != cudaSuccess || !box->done) { cudaGetLastError(); return PAAC_ERR_CUDA; }
-  }
-  __atomic_thread_fence(__ATOMIC_ACQUIRE);
+  if (!await_box(c)) return PAAC_ERR_CUDA;
   if (sample) memcpy(actions, box->actions, c->n_e * sizeof(int32_t));
   if (values) memcpy(values, box->values, c->n_e * sizeof(float));
   if (t == c->t_max) { c->host_t = 0; c->env_step += c->t_max; c->rollout_fresh = true; c->host_next_valid = true; }

@@ -36,6 +36,9 @@ void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const HostPlanes* pla
 void launch_publish(LaunchCtx& lc, const int32_t* actions, const float* values, int n, int32_t* host_actions, float* host_values,
                     volatile uint32_t* done);
 
+// the statistics of an update to pinned host memory, then *done = 1
+void launch_publish_stats(LaunchCtx& lc, const DeviceStats* stats, DeviceStats* host_stats, volatile uint32_t* done);
+
 void launch_advance_step(LaunchCtx& lc, uint64_t* step_base, uint32_t by);
 
 // ---- weight gradients as split-k partial sums --------------------------------------------

@@ -297,11 +297,12 @@ template <class TW> struct HeadWeightOp {   // row = fc unit i, k = head unit
 // A thread owns one hidden unit; its weights and gradient sums stay in registers, so a row costs it one load of h and
 // 2 NK multiply-adds.  A block takes 64 units and the rows of one split (at most about 128), FH_ROWS at a time, the next
 // ones on their way while these are used: a chain of some microseconds whatever the batch.
-constexpr int FH_THREADS = 64, FH_ROWS = 8;
+constexpr int FH_THREADS = 64;
 template <class T, class TW, int NK>
 __global__ void __launch_bounds__(FH_THREADS)
 heads_backward_kernel(const T* h, const float* dz, const float* dV, const TW* wpi, const TW* wv, int n, int F, int A, int rows_per,
                       T* g_fc, float* part_w, float* part_b, float* part_vw, float* part_vb) {
+  constexpr int FH_ROWS = NK <= 20 ? 32 : 16;
   __shared__ float dzs[FH_ROWS][NK];
   const int tid = threadIdx.x, col = blockIdx.y * FH_THREADS + tid;
   pdl_entry();

@@ -221,6 +221,20 @@ void launch_publish(LaunchCtx& lc, const int32_t* actions, const float* values, 
   launch_kernel_overlapped(lc, publish_kernel, dim3(1), dim3(PUB_THREADS), 0, actions, values, n, host_actions, host_values, done);
 }
 
+__global__ void __launch_bounds__(32) publish_stats_kernel(const DeviceStats* stats, DeviceStats* host_stats, volatile uint32_t* done) {
+  constexpr int WORDS = sizeof(DeviceStats) / 4;
+  static_assert(WORDS <= 32, "one word per lane");
+  pdl_entry();
+  if (threadIdx.x < WORDS) reinterpret_cast<uint32_t*>(host_stats)[threadIdx.x] = reinterpret_cast<const uint32_t*>(stats)[threadIdx.x];
+  __threadfence_system();
+  __syncwarp();
+  if (threadIdx.x == 0) *done = 1u;
+}
+void launch_publish_stats(LaunchCtx& lc, const DeviceStats* stats, DeviceStats* host_stats, volatile uint32_t* done) {
+  KernelScope scope(lc, KID_CLIP_RMSPROP);
+  launch_kernel_overlapped(lc, publish_stats_kernel, dim3(1), dim3(32), 0, stats, host_stats, done);
+}
+
 }  // namespace paac
 
 extern "C" int paac_stack_push(const uint8_t* state_in, const uint8_t* newest, const uint8_t* restart, uint8_t* state_out,
