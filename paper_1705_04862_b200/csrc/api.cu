@@ -73,6 +73,7 @@ struct paac_ctx {
   int8_t* rewards;
   uint8_t* terminals;
   DeviceStats* stats;
+  uint32_t* barriers;      // of the one-launch rollout
   size_t elt;              // bytes of one stored activation element
 };
 
@@ -136,6 +137,7 @@ size_t carve(paac_ctx* c, char* base) {
       sc += c->simt_scratch_off;
       if (tc_fc_scratch_floats((int)n_e) > sc) sc = tc_fc_scratch_floats((int)n_e);
     }
+    if (c->arch == PAAC_ARCH_NIPS && rollout_small_part_floats((int)n_e) > sc) sc = rollout_small_part_floats((int)n_e);
     c->scratch = k.take<float>(sc);
   }
   c->norm_partials = k.take<float>(NORM_BLOCKS);
@@ -147,6 +149,7 @@ size_t carve(paac_ctx* c, char* base) {
   c->terminals = k.take<uint8_t>(B);
   c->stats = k.take<DeviceStats>(1);
   c->step_dev = k.take<uint64_t>(1);
+  c->barriers = k.take<uint32_t>(rollout_small_barrier_words((int)n_e));
   return (k.off + 255) & ~(size_t)255;
 }
 
@@ -172,6 +175,23 @@ void refresh_weight_copies(paac_ctx* c, bool cast) {
   if (tc_supported(c->arch, c->prec)) tc_relayout_weights(c->lc, c->nd, c->theta16, c->w_images, &c->stats->error_word);
 }
 
+// `steps` forward passes from slot t0 on in one launch (rollout_small_supported()); a rollout with `env`, else one pass
+void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sample_steps, const EnvStepArgs* env, bool advance) {
+  void* act[MAX_LAYERS];
+  for (int l = 0; l <= c->nd.n_conv; ++l)
+    act[l] = (char*)c->act[l] + (size_t)t0 * c->n_e * c->nd.layer[l].out_size * c->elt;
+  const size_t row = (size_t)t0 * c->n_e;
+  SmallRollout r{};
+  r.n = c->n_e; r.steps = steps; r.sample_steps = sample_steps; r.t0 = (uint32_t)t0; r.step_env = env != nullptr;
+  r.frames = frames; r.frame_step = (size_t)c->n_e * FRAME_BYTES; r.act = act; r.part = c->scratch; r.barriers = c->barriers;
+  r.logits = c->logits + row * c->A; r.values = c->values + row; r.uniforms = c->uniforms + row; r.actions = c->actions + row;
+  r.sampled = c->sampled + row; r.forced = c->forced_on ? c->forced + row : nullptr;
+  r.seed = c->seed; r.step_base = c->step_dev; r.advance = advance ? (uint32_t)c->t_max : 0u;
+  r.mode = head_mode(c); r.error_word = &c->stats->error_word;
+  if (env) r.env = *env;
+  launch_rollout_small(c->lc, c->prec, c->nd, c->theta, c->theta16, r);
+}
+
 // network + heads on the n_e states of `frames`, activations into slot `slot`.  With `tail` the caller is about
 // to step the synthetic environments and can take the actions there: if the forward pass left the heads as partial
 // sums (see HeadsTail), no sampling kernel is launched, *tail describes what is left, and the result is true.  With `env`
@@ -183,6 +203,11 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
   for (int l = 0; l <= c->nd.n_conv; ++l)
     act[l] = (char*)c->act[l] + (size_t)slot * c->n_e * c->nd.layer[l].out_size * c->elt;
   const size_t row = (size_t)slot * c->n_e;
+  if (rollout_small_supported(c->lc, c->arch, c->n_e)) {
+    small_rollout(c, frames, slot, 1, sample ? 1 : 0, nullptr, advanced && !sample);
+    if (advanced) *advanced = !sample;
+    return false;
+  }
   const int32_t* forced = sample && c->forced_on ? c->forced + row : nullptr;
   int32_t* actions = sample ? c->actions + row : nullptr;
   int32_t* sampled = sample ? c->sampled + row : nullptr;
@@ -416,6 +441,11 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
   uint8_t* nxt = c->frames[c->cur ^ 1];
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
   run_recorded(c, 0, c->cur, [&]() {
+    if (rollout_small_supported(c->lc, c->arch, c->n_e)) {
+      const EnvStepArgs env{c->hp.term_denom, nxt, c->rewards, c->terminals, c->counters, pattern_actions(c)};
+      small_rollout(c, fr, 0, c->t_max + 1, c->t_max, &env, true);
+      return;
+    }
     for (int t = 0; t < c->t_max; ++t) {
       HeadsTail tail;
       uint8_t* dst = t + 1 < c->t_max ? fr + (t + 1) * fstep : nxt;
@@ -819,6 +849,11 @@ int paac_debug_write(paac_ctx* c, int which, const void* src, size_t bytes) {
   if (send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (cudaMemcpyAsync(p, src, b, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
+  // a wait that gave up may have left the one-launch rollout's barriers half full: clearing the error word resets them
+  if (which == PAAC_DBG_ERROR_WORD &&
+      cudaMemsetAsync(c->barriers, 0, rollout_small_barrier_words(c->n_e) * sizeof(uint32_t), c->st) != cudaSuccess) {
+    cudaGetLastError(); return PAAC_ERR_CUDA;
+  }
   return PAAC_OK;
 }
 

@@ -52,23 +52,18 @@ __device__ __forceinline__ void env_record(const EnvPrep& p, const EnvOutcome& o
   counters[e] = o.terminal ? 0 : p.len + 1;
   counters[n_e + e] = o.terminal ? 0 : p.ret + o.reward;
 }
-// the whole block writes the 84 x 84 x 4 frame, one hashed 32-bit word per pixel (its bytes, little endian, are the
-// four channels), as 16-byte stores
+// sixteen bytes of a frame: one hashed 32-bit word per pixel (its bytes, little endian, are the four channels)
+__device__ __forceinline__ uint4 env_frame_quad(const EnvFrame f, uint32_t q, int pattern_actions) {
+  const uint32_t keep = pattern_actions > 0 ? 0x3F3F3F3Fu : 0xFFFFFFFFu, p = q * 4u + 1u;
+  if (q * 4u >= f.band_lo && q * 4u < f.band_hi) return make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+  return make_uint4(hash_mix(f.base + HASH_K0 * p) & keep, hash_mix(f.base + HASH_K0 * (p + 1u)) & keep,
+                    hash_mix(f.base + HASH_K0 * (p + 2u)) & keep, hash_mix(f.base + HASH_K0 * (p + 3u)) & keep);
+}
+// the whole block writes the 84 x 84 x 4 frame
 template <int THREADS>
 __device__ __forceinline__ void env_write_frame(const EnvFrame f, uint8_t* frame, int pattern_actions) {
-  const uint32_t keep = pattern_actions > 0 ? 0x3F3F3F3Fu : 0xFFFFFFFFu;
   uint4* out = reinterpret_cast<uint4*>(frame);
-  for (int q = threadIdx.x; q < FRAME_WORDS / 4; q += THREADS) {
-    const uint32_t p = (uint32_t)q * 4u + 1u;
-    uint4 v;
-    v.x = hash_mix(f.base + HASH_K0 * p);
-    v.y = hash_mix(f.base + HASH_K0 * (p + 1u));
-    v.z = hash_mix(f.base + HASH_K0 * (p + 2u));
-    v.w = hash_mix(f.base + HASH_K0 * (p + 3u));
-    v.x &= keep; v.y &= keep; v.z &= keep; v.w &= keep;
-    if ((uint32_t)q * 4u >= f.band_lo && (uint32_t)q * 4u < f.band_hi) v = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-    out[q] = v;
-  }
+  for (int q = threadIdx.x; q < FRAME_WORDS / 4; q += THREADS) out[q] = env_frame_quad(f, (uint32_t)q, pattern_actions);
 }
 
 }  // namespace paac

@@ -147,6 +147,23 @@ void heads_backward(LaunchCtx& lc, int prec, const NetDims& nd, const float* the
                     const bf16* theta16, const void* h, int n, const float* dz, const float* dV, void* gact_fc,
                     float* grad, float* scratch, GradSegments* segs);
 
+// ---- all forward passes of a rollout in one launch, small batches of the smaller network (rollout_small.cu) ----------
+bool rollout_small_supported(const LaunchCtx& lc, int arch, int n);
+size_t rollout_small_part_floats(int n);        // scratch
+size_t rollout_small_barrier_words(int n);      // uint32, zero before the first launch and after a device error
+struct SmallRollout {
+  int n, steps, sample_steps; uint32_t t0;      // passes over slots t0 .. t0 + steps - 1; the first sample_steps sample an action
+  bool step_env;                                // ... and step the synthetic environments with it (env)
+  const uint8_t* frames; size_t frame_step;     // states of slot t0, bytes from one slot to the next
+  void* const* act;                             // stored activations of slot t0, by layer
+  float* part; uint32_t* barriers;
+  float *logits, *values, *uniforms; int32_t *actions, *sampled; const int32_t* forced;      // of slot t0
+  uint64_t seed; uint64_t* step_base; uint32_t advance;      // > 0: added to the step index at the end
+  HeadMode mode; EnvStepArgs env;               // env.next_frames: the state after the last step; rewards, terminals of slot t0
+  uint32_t* error_word;
+};
+void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const SmallRollout& r);
+
 // ---- optimiser (optim.cu) -------------------------------------------------------------------
 constexpr int NORM_BLOCKS = 1184;
 void launch_clip_rmsprop(LaunchCtx& lc, size_t P, float* theta, float* rms, const float* grad,

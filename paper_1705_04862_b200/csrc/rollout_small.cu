@@ -1,0 +1,387 @@
+// The forward passes of a whole rollout of the smaller network in one launch, for batches of a few environments.
+//
+// With 1 to 64 states a step of the layer-by-layer path is four launches of 5 us whose work is a fraction of that.  Here one
+// block per SM stays for the rollout and walks its steps.  Environment e belongs to a group of C blocks (C = 16, 8, 4 or
+// 2, as many as fit): each computes its share of the first layer's positions, and after a barrier of the group its share of
+// the second layer's.  The fully connected layer is where the states meet: 21 runs of 128 inputs x 4 tiles of 64 units are
+// dealt to 84 blocks, whose weight tile stays in shared memory for the whole rollout, so that each step reads only
+// activations; this takes one device-wide barrier before and one after.  Every block of a group then finishes its
+// environment's state by itself (sum over the runs, heads, draw, transition: the same numbers in each), and writes its
+// share of the next frame, of which it keeps the rows its next share of the first layer reads.
+//
+// Arithmetic is that of the layer-by-layer path to the bit: one chain of fused multiply-adds per output in ascending k,
+// 128-long runs of the fully connected layer added in double.
+//
+// What bounds a step: latency; two barriers over 148 blocks (about 1.4 us each), one over the group, and five passes of one
+// to three microseconds: 15 us a step for 4 states and 22 us for 32, against 22 and 36 us for the launches it replaces
+// (4 environments, five steps and the bootstrap: 131 -> 94 us; 32: 215 -> 137 us).
+//
+// Every wait is bounded: a block that gives up raises the error word and leaves, and so, one after the other, do all.
+#include <type_traits>
+
+#include "env_device.cuh"
+#include "kernels.h"
+#include "tc_common.cuh"
+
+namespace paac {
+
+constexpr int RS_THREADS = 256, RS_F = 256, RS_IN = 2592, RS_RUN = 128, RS_RUNS = (RS_IN + RS_RUN - 1) / RS_RUN, RS_COLS = 64;
+constexpr int RS_TILES = RS_RUNS * (RS_F / RS_COLS), RS_FC_LD = RS_RUN + 4, RS_ROWS = 32;
+typedef NipsConv1 RC1;
+typedef NipsConv2 RC2;
+constexpr int RS_POS1 = RC1::OH * RC1::OW, RS_POS2 = RC2::OH * RC2::OW;        // 400 and 81
+constexpr uint32_t RS_POLLS = 2000000u;
+
+struct RsArgs {
+  int n, C, A, steps, blocks;             // forward passes: slots t0 .. t0 + steps - 1
+  uint32_t t0;
+  const uint8_t* frames; size_t frame_step;       // states of slot t0, and from one slot to the next
+  uint8_t* next_frames;                           // states of the slot after the last one that steps (rollout)
+  int sample_steps;                               // of the passes, so many sample an action (and, with `env`, step it)
+  bool env;
+  float* part;                                    // [RS_RUNS][n][RS_F]
+  const float *b1, *b2, *bfc, *bpi, *bv;
+  float *logits, *values, *uniforms;
+  int32_t *actions, *sampled, *counters;
+  const int32_t* forced;
+  int8_t* rewards; uint8_t* terminals;
+  uint64_t seed; uint64_t* step_base; uint32_t advance;
+  uint32_t term_denom; int pattern_actions;
+  HeadMode mode;
+  unsigned long long* grid_bar; unsigned long long* group_bar;      // arrivals so far: [1], [n]
+  uint32_t* error_word;
+};
+
+// A barrier over `count` blocks is a counter of arrivals that only grows, by `count` at every use, so the target of the next
+// use follows from any value read before this block arrives; arriving costs no round trip.  What the blocks wrote before is
+// visible to all after.  false after a bounded wait.
+struct RsBarrier {
+  unsigned long long* arrivals; uint32_t count; unsigned long long target;
+  __device__ __forceinline__ void init(unsigned long long* a, uint32_t c) {
+    arrivals = a; count = c; target = 0;
+    if (threadIdx.x == 0) {
+      const unsigned long long now = *reinterpret_cast<volatile unsigned long long*>(a);
+      target = now - now % c;
+    }
+  }
+  __device__ __forceinline__ bool sync(uint32_t* error_word, int* s_ok) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      target += count;
+      asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(arrivals) : "memory");
+      unsigned long long now;
+      uint32_t polls = 0;
+      do {
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(arrivals) : "memory");
+      } while (now < target && ++polls < RS_POLLS);
+      *s_ok = now >= target;
+      if (now < target) atomicOr(error_word, tc::ERR_WAIT_FULL);
+    }
+    __syncthreads();
+    return *s_ok != 0;
+  }
+};
+
+__device__ __forceinline__ float4 rs_bytes(uint32_t v) {
+  constexpr float BIAS = 8388608.f;       // a byte in the low mantissa bits of 2^23 is 2^23 + byte
+  return make_float4(__uint_as_float(__byte_perm(v, 0x4B000000u, 0x7440)) - BIAS, __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7441)) - BIAS,
+                     __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7442)) - BIAS, __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7443)) - BIAS);
+}
+__device__ __forceinline__ void rs_fma4(float (&acc)[4], float a, const float4 w) {
+  acc[0] = fmaf(a, w.x, acc[0]); acc[1] = fmaf(a, w.y, acc[1]); acc[2] = fmaf(a, w.z, acc[2]); acc[3] = fmaf(a, w.w, acc[3]);
+}
+__device__ __forceinline__ float4 rs_relu(const float (&acc)[4], float scale, const float* b) {
+  return make_float4(fmaxf(fmaf(acc[0], scale, b[0]), 0.f), fmaxf(fmaf(acc[1], scale, b[1]), 0.f), fmaxf(fmaf(acc[2], scale, b[2]), 0.f),
+                     fmaxf(fmaf(acc[3], scale, b[3]), 0.f));
+}
+__device__ __forceinline__ void rs_store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void rs_store4(bf16* p, float4 v) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
+// written by other blocks during this launch: past the first-level cache
+__device__ __forceinline__ float4 rs_load4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 rs_load4(const bf16* p) {
+  const uint2 v = __ldcg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+}
+
+// shared memory, in floats
+constexpr int RS_W1 = 0, RS_W2 = RS_W1 + RC1::KK * RC1::CO, RS_FCW = RS_W2 + RC2::KK * RC2::CO, RS_FCA = RS_FCW + RS_COLS * RS_FC_LD,
+              RS_ACT1 = RS_FCA + RS_ROWS * RS_FC_LD, RS_FRAME = RS_ACT1 + RS_POS1 * RC1::CO, RS_HEADW = RS_FRAME + FRAME_BYTES / 4;
+
+// First layer: `share` positions from pos0, 4 channels and PP positions (`apart` apart) per thread.  The passes of both
+// convolutions are bound by weights going from shared memory to registers (16 floats a thread for four k, whatever PP is),
+// so PP is as large as leaves every scheduler one warp.
+template <class T, int PP>
+__device__ __forceinline__ void rs_conv1(const float* sm, const float* b1, T* act, int pos0, int share) {
+  const int q = threadIdx.x & 3, p = threadIdx.x >> 2, apart = (share + PP - 1) / PP;
+  const uint32_t* frame = reinterpret_cast<const uint32_t*>(sm + RS_FRAME);
+  const float4* w = reinterpret_cast<const float4*>(sm + RS_W1) + q;                   // [k][16]
+  float acc[PP][4];
+  int base[PP];
+#pragma unroll
+  for (int i = 0; i < PP; ++i) {
+    const int pos = pos0 + min(p + apart * i, share - 1);
+    base[i] = (pos / RC1::OW * RC1::S) * RC1::W + pos % RC1::OW * RC1::S;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+  }
+  if (p < apart)
+    for (int r = 0; r < RC1::K; ++r) {
+#pragma unroll
+      for (int s = 0; s < RC1::K; ++s) {
+        float4 a[PP];
+#pragma unroll
+        for (int i = 0; i < PP; ++i) a[i] = rs_bytes(frame[base[i] + r * RC1::W + s]);
+        const int k = (r * RC1::K + s) * 4;
+        const float4 w0 = w[k * 4], w1 = w[(k + 1) * 4], w2 = w[(k + 2) * 4], w3 = w[(k + 3) * 4];
+#pragma unroll
+        for (int i = 0; i < PP; ++i) { rs_fma4(acc[i], a[i].x, w0); rs_fma4(acc[i], a[i].y, w1); rs_fma4(acc[i], a[i].z, w2); rs_fma4(acc[i], a[i].w, w3); }
+      }
+    }
+#pragma unroll
+  for (int i = 0; i < PP; ++i)
+    if (p < apart && p + apart * i < share) rs_store4(act + (size_t)(pos0 + p + apart * i) * RC1::CO + 4 * q, rs_relu(acc[i], 1.0f / 255.0f, b1 + 4 * q));
+}
+// Second layer: the same with 8 groups of 4 channels, the input rows in shared memory.
+template <class T, int PP>
+__device__ __forceinline__ void rs_conv2(const float* sm, const float* b2, T* act, int pos0, int share) {
+  const int q = threadIdx.x & 7, p = threadIdx.x >> 3, apart = (share + PP - 1) / PP;
+  const float4* in = reinterpret_cast<const float4*>(sm + RS_ACT1);                    // [20][20][16]
+  const float4* w = reinterpret_cast<const float4*>(sm + RS_W2) + q;                   // [k][32]
+  float acc[PP][4];
+  int base[PP];
+#pragma unroll
+  for (int i = 0; i < PP; ++i) {
+    const int pos = pos0 + min(p + apart * i, share - 1);
+    base[i] = ((pos / RC2::OW * RC2::S) * RC2::W + pos % RC2::OW * RC2::S) * (RC2::C / 4);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+  }
+  if (p < apart)
+    for (int r = 0; r < RC2::K; ++r) {
+#pragma unroll 4
+      for (int sc = 0; sc < RC2::K * RC2::C / 4; ++sc) {                               // (s, four input channels)
+        float4 a[PP];
+#pragma unroll
+        for (int i = 0; i < PP; ++i) a[i] = in[base[i] + r * (RC2::W * RC2::C / 4) + sc];
+        const int k = r * RC2::K * RC2::C + sc * 4;
+        const float4 w0 = w[k * 8], w1 = w[(k + 1) * 8], w2 = w[(k + 2) * 8], w3 = w[(k + 3) * 8];
+#pragma unroll
+        for (int i = 0; i < PP; ++i) { rs_fma4(acc[i], a[i].x, w0); rs_fma4(acc[i], a[i].y, w1); rs_fma4(acc[i], a[i].z, w2); rs_fma4(acc[i], a[i].w, w3); }
+      }
+    }
+#pragma unroll
+  for (int i = 0; i < PP; ++i)
+    if (p < apart && p + apart * i < share) rs_store4(act + (size_t)(pos0 + p + apart * i) * RC2::CO + 4 * q, rs_relu(acc[i], 1.f, b2 + 4 * q));
+}
+
+template <class T, class TW, int C>
+__global__ void __launch_bounds__(RS_THREADS, 1)
+rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const TW* wpi, const TW* wv, T* act1, T* act2, T* h) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float xs[RS_F], zs[33];
+  __shared__ EnvFrame s_frame;
+  __shared__ int32_t s_action;
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = q.n, A = q.A;
+  const bool conv = (int)blockIdx.x < n * C;
+  const int e = blockIdx.x / C, rank = blockIdx.x % C;
+  const int tile = q.blocks - 1 - (int)blockIdx.x;                 // of the fully connected layer; the last blocks have one each
+  const bool fc = tile < RS_TILES;
+  const int run = tile / (RS_F / RS_COLS), col0 = tile % (RS_F / RS_COLS) * RS_COLS, k0 = run * RS_RUN;
+  const int len = min(RS_RUN, RS_IN - k0);
+  constexpr int SHARE1 = RS_POS1 / C, PP1 = C == 16 ? 1 : (C == 8 ? 2 : (C == 4 ? 2 : 7)), PP2 = C == 16 ? 1 : (C == 8 ? 2 : (C == 4 ? 3 : 6));
+  static_assert(RS_POS1 % C == 0, "equal shares of the first layer");
+  const int pos1 = rank * SHARE1, pos2 = RS_POS2 * rank / C, share2 = RS_POS2 * (rank + 1) / C - pos2;
+  const int row_lo = pos1 / RC1::OW * RC1::S, row_hi = (pos1 + SHARE1 - 1) / RC1::OW * RC1::S + RC1::K;      // frame rows read
+  constexpr int IN_ROW = RC1::OW * RC1::CO / 4;                    // 16-byte words of a row of the first layer's map
+  const int in_lo = pos2 / RC2::OW * RC2::S * IN_ROW, in_hi = ((pos2 + share2 - 1) / RC2::OW * RC2::S + RC2::K) * IN_ROW;
+  RsBarrier grid, group;
+  grid.init(q.grid_bar, q.blocks);
+  if (conv) group.init(q.group_bar + e, C);
+  uint4* frame = reinterpret_cast<uint4*>(sm + RS_FRAME);
+  constexpr int QUADS = FRAME_W / 4;                               // 16-byte words of a frame row
+
+  // what stays for the rollout: both convolutions' weights as [k][channel], the head weights, the weight tile
+  if (conv) {
+    for (int i = tid; i < RC1::KK * RC1::CO; i += RS_THREADS) sm[RS_W1 + i % RC1::KK * RC1::CO + i / RC1::KK] = to_f(w1[i]);
+    for (int i = tid; i < RC2::KK * RC2::CO; i += RS_THREADS) sm[RS_W2 + i % RC2::KK * RC2::CO + i / RC2::KK] = to_f(w2[i]);
+    for (int i = tid; i < (A + 1) * RS_F; i += RS_THREADS) sm[RS_HEADW + i] = i < A * RS_F ? to_f(wpi[i]) : to_f(wv[i - A * RS_F]);
+    const uint4* src = reinterpret_cast<const uint4*>(q.frames + (size_t)e * FRAME_BYTES);
+    for (int i = row_lo * QUADS + tid; i < row_hi * QUADS; i += RS_THREADS) frame[i] = __ldcg(src + i);
+  }
+  if (fc)
+    for (int i = tid; i < RS_COLS * RS_RUN; i += RS_THREADS) {
+      const int c = i / RS_RUN, k = i % RS_RUN;
+      sm[RS_FCW + c * RS_FC_LD + k] = k < len ? to_f(wfc[(size_t)(col0 + c) * RS_IN + k0 + k]) : 0.f;
+    }
+  const uint64_t step0 = *q.step_base + q.t0;
+  __syncthreads();
+
+  for (int t = 0; t < q.steps; ++t) {
+    const size_t slot = (size_t)t * n;
+    if (conv) {
+      T* a1 = act1 + (slot + e) * RC1::OUT_SIZE;
+      T* a2 = act2 + (slot + e) * RC2::OUT_SIZE;
+      rs_conv1<T, PP1>(sm, q.b1, a1, pos1, SHARE1);
+      if (!group.sync(q.error_word, &s_ok)) return;
+      for (int i = in_lo + tid; i < in_hi; i += RS_THREADS) reinterpret_cast<float4*>(sm + RS_ACT1)[i] = rs_load4(a1 + 4 * i);
+      __syncthreads();
+      rs_conv2<T, PP2>(sm, q.b2, a2, pos2, share2);
+    }
+    if (!grid.sync(q.error_word, &s_ok)) return;
+    if (fc) {
+      for (int r0 = 0; r0 < n; r0 += RS_ROWS) {
+        const int rows = min(RS_ROWS, n - r0);
+        if (r0 > 0) __syncthreads();
+        for (int i = tid; i < rows * (RS_RUN / 4); i += RS_THREADS) {
+          const int r = i / (RS_RUN / 4), k = i % (RS_RUN / 4) * 4;
+          if (k < len) *reinterpret_cast<float4*>(sm + RS_FCA + r * RS_FC_LD + k) = rs_load4(act2 + (slot + r0 + r) * RS_IN + k0 + k);
+        }
+        __syncthreads();
+        const int cx = tid & 15, ry = tid >> 4;
+        const float* pa = sm + RS_FCA + ry * RS_FC_LD;
+        const float* pb = sm + RS_FCW + cx * RS_FC_LD;
+        float acc[2][4] = {};
+        auto columns = [&](auto two_rows) {
+          constexpr int R = decltype(two_rows)::value;
+#pragma unroll 4
+          for (int k = 0; k < len; k += 4) {
+            float4 a[R], b[4];
+#pragma unroll
+            for (int i = 0; i < R; ++i) a[i] = *reinterpret_cast<const float4*>(pa + i * 16 * RS_FC_LD + k);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(pb + j * 16 * RS_FC_LD + k);
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]); acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]); acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+              }
+          }
+        };
+        if (ry < rows) { if (rows > 16) columns(std::integral_constant<int, 2>{}); else columns(std::integral_constant<int, 1>{}); }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (ry + 16 * i < rows)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q.part[((size_t)run * n + r0 + ry + 16 * i) * RS_F + col0 + cx + 16 * j] = acc[i][j];
+      }
+    }
+    if (!grid.sync(q.error_word, &s_ok)) return;
+    if (!conv) continue;
+    // ---- the end of the state's pass, in every block of the group ----
+    const bool sample = t < q.sample_steps, stepping = sample && q.env;
+    {
+      float v[RS_RUNS];
+#pragma unroll
+      for (int p = 0; p < RS_RUNS; ++p) v[p] = __ldcg(q.part + ((size_t)p * n + e) * RS_F + tid);
+      double s = 0.0;
+#pragma unroll
+      for (int p = 0; p < RS_RUNS; ++p) s += (double)v[p];
+      const T x = from_f<T>(fmaxf((float)(s + (double)q.bfc[tid]), 0.f));
+      if (rank == 0) h[(slot + e) * RS_F + tid] = x;
+      xs[tid] = to_f(x);
+    }
+    EnvPrep prep{};
+    if (stepping && tid == 32) prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, q.counters);
+    __syncthreads();
+    for (int k = warp; k <= A; k += RS_THREADS / 32) {
+      float acc = 0.f;
+#pragma unroll
+      for (int i = 0; i < RS_F / 32; ++i) {
+        const int at = sizeof(T) == 2 ? lane * (RS_F / 32) + i : lane + 32 * i;
+        acc = fmaf(sm[RS_HEADW + k * RS_F + at], xs[at], acc);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) zs[k] = acc + (k < A ? q.bpi[k] : q.bv[0]);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const int32_t a = warp_finish_heads(q.mode, lane < A ? zs[lane] : -INFINITY, zs[A], lane, A, (size_t)e, q.logits + slot * A, q.values + slot,
+                                          sample, q.seed, step0 + t, q.forced ? q.forced + slot : nullptr, q.actions + slot, q.sampled + slot,
+                                          q.uniforms + slot);
+      if (lane == 0) s_action = a;
+    }
+    if (!stepping) { __syncthreads(); continue; }
+    __syncthreads();
+    EnvOutcome o{0, false, 0u};
+    if (tid == 32) {
+      o = env_outcome(prep, s_action, q.term_denom, q.pattern_actions);
+      s_frame = env_frame_of(prep.pre_next, o.tag, q.pattern_actions);
+    }
+    __syncthreads();
+    if (tid == 32 && rank == 0) env_record(prep, o, (uint32_t)e, n, q.rewards + slot, q.terminals + slot, q.counters);
+    const EnvFrame f = s_frame;
+    // this block's share of the frame for everyone, and the rows it will read itself
+    uint4* out = reinterpret_cast<uint4*>((t + 1 < q.sample_steps ? const_cast<uint8_t*>(q.frames) + (size_t)(t + 1) * q.frame_step : q.next_frames) + (size_t)e * FRAME_BYTES);
+    const int own_lo = FRAME_WORDS / 4 * rank / C, own_hi = FRAME_WORDS / 4 * (rank + 1) / C;
+    const int lo = min(own_lo, row_lo * QUADS), hi = max(own_hi, row_hi * QUADS);
+    for (int i = lo + tid; i < hi; i += RS_THREADS) {
+      const bool own = i >= own_lo && i < own_hi, keep = i >= row_lo * QUADS && i < row_hi * QUADS;
+      if (!own && !keep) continue;
+      const uint4 v = env_frame_quad(f, (uint32_t)i, q.pattern_actions);
+      if (own) out[i] = v;
+      if (keep) frame[i] = v;
+    }
+    __syncthreads();
+  }
+  if (q.advance && blockIdx.x == 0 && tid == 0) *q.step_base += q.advance;        // every block has read it
+}
+
+// Blocks per environment: as many of 16, 8, 4, 2 as leave each a multiprocessor of its own; 0: use the layer-by-layer path.
+static int rs_blocks_per_env(int n) { return n <= 9 ? 16 : (n <= 18 ? 8 : (n <= 37 ? 4 : (n <= 74 ? 2 : 0))); }
+bool rollout_small_supported(const LaunchCtx& lc, int arch, int n) {
+  if (arch != PAAC_ARCH_NIPS || lc.fp32_tensor_cores || rs_blocks_per_env(n) == 0) return false;
+  static const int fits = [] {
+    int dev = 0, sms = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return coop && sms >= 148 ? 1 : 0;
+  }();
+  return fits != 0;
+}
+size_t rollout_small_part_floats(int n) { return (size_t)RS_RUNS * n * RS_F; }
+size_t rollout_small_barrier_words(int n) { return 2 * ((size_t)n + 1); }      // 64-bit counters
+
+template <class T, class TW>
+static void rs_launch(LaunchCtx& lc, const RsArgs& q, const TW* w, const NetDims& nd, void* const act[]) {
+  const LayerDims* d = nd.layer;
+  const size_t smem = (size_t)(RS_HEADW + (q.A + 1) * RS_F) * sizeof(float);
+  auto go = [&](auto kern) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { lc.host_failure = true; return; }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(q.blocks); cfg.blockDim = dim3(RS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = lc.st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    lc.serialize_next = false;
+    KernelScope scope(lc, KID_SMALL_ROLLOUT);
+    if (cudaLaunchKernelEx(&cfg, kern, q, w + d[0].w_off, w + d[1].w_off, w + d[2].w_off, w + nd.pi_w, w + nd.v_w, (T*)act[0], (T*)act[1], (T*)act[2]) != cudaSuccess)
+      lc.host_failure = true;
+  };
+  if (q.C == 16) go(rollout_small_kernel<T, TW, 16>);
+  else if (q.C == 8) go(rollout_small_kernel<T, TW, 8>);
+  else if (q.C == 4) go(rollout_small_kernel<T, TW, 4>);
+  else go(rollout_small_kernel<T, TW, 2>);
+}
+
+void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const SmallRollout& r) {
+  const LayerDims* d = nd.layer;
+  RsArgs q{};
+  q.n = r.n; q.C = rs_blocks_per_env(r.n); q.A = nd.A; q.steps = r.steps; q.blocks = 148; q.t0 = r.t0;
+  q.frames = r.frames; q.frame_step = r.frame_step; q.next_frames = r.env.next_frames; q.sample_steps = r.sample_steps; q.env = r.step_env;
+  q.part = r.part; q.b1 = theta + d[0].b_off; q.b2 = theta + d[1].b_off; q.bfc = theta + d[2].b_off; q.bpi = theta + nd.pi_b; q.bv = theta + nd.v_b;
+  q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
+  q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
+  q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode;
+  q.grid_bar = reinterpret_cast<unsigned long long*>(r.barriers); q.group_bar = q.grid_bar + 1; q.error_word = r.error_word;
+  if (prec == PAAC_BF16) rs_launch<bf16, bf16>(lc, q, theta16, nd, r.act);
+  else rs_launch<float, float>(lc, q, theta, nd, r.act);
+}
+
+}  // namespace paac

@@ -641,3 +641,19 @@ def test_float_contraction_shapes(orc, arch, n_e, t_max, A):
     check_update(orc, o, g, TOL["fp32"], inject=True)
     assert g.error_word() == 0
     g.close()
+
+
+@pytest.mark.parametrize("n_e,prec,A", [(1, "fp32", 2), (9, "bf16", 18), (10, "fp32", 32), (18, "bf16", 4), (19, "fp32", 6), (37, "bf16", 3),
+                                        (38, "fp32", 5), (74, "fp32", 9), (75, "bf16", 6)])
+def test_small_batches_one_launch_rollout(orc, n_e, prec, A):
+    """The smaller network's rollout in one launch: the smallest and largest batch of every group size, the first one beyond,
+    both storage types; two iterations (the barriers' counters go on), the second through recorded sequences' first use."""
+    cfg = dict(arch="nips", precision=prec, n_e=n_e, t_max=2, n_actions=A, lr=0.0028, term_denom=3)
+    o, g = make_pair(orc, cfg)
+    for it in range(2):
+        if it and prec == "bf16":
+            resync(o, g)
+        check_rollout(orc, o, g, TOL[prec])
+        check_update(orc, o, g, TOL[prec], inject=True)
+    assert g.error_word() == 0
+    g.close()
