@@ -213,17 +213,17 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
   int32_t* sampled = sample ? c->sampled + row : nullptr;
   float* uniforms = sample ? c->uniforms + row : nullptr;
   if (use_tc(c) && heads_fused_supported(c->nd)) {
-    int splits = 0;
+    int splits = 0, parts = 2;
     tc_forward(c->lc, c->arch, c->nd, c->theta, c->theta16, c->w_images, frames, c->n_e, act, c->scratch,
-               &c->stats->error_word, &splits);
+               &c->stats->error_word, &splits, &parts);
     if (tail != nullptr && splits == 0 && sample) {
-      *tail = HeadsTail{c->scratch, c->theta + c->nd.pi_b, c->theta + c->nd.v_b, c->A, c->logits + row * c->A,
+      *tail = HeadsTail{c->scratch, parts, c->theta + c->nd.pi_b, c->theta + c->nd.v_b, c->A, c->logits + row * c->A,
                         c->values + row, forced, actions, sampled, uniforms, head_mode(c)};
       return true;
     }
     launch_heads_fused(c->lc, c->nd, c->theta, c->theta16, c->scratch, splits, (bf16*)act[c->nd.n_conv], c->n_e,
                        c->logits + row * c->A, c->values + row, c->seed, c->step_dev, (uint32_t)slot, forced, actions,
-                       sampled, uniforms, head_mode(c), (advanced && splits == 0 && !sample) ? c->step_dev : nullptr, (uint32_t)c->t_max);
+                       sampled, uniforms, head_mode(c), (advanced && splits == 0 && !sample) ? c->step_dev : nullptr, (uint32_t)c->t_max, parts);
     if (advanced) *advanced = splits == 0 && !sample;      // the sampling kernel has moved the step index on
     return false;
   }
@@ -514,7 +514,7 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
       if (l == 2 && all_finished) {
         // what has piled up so far (the heads, the fully connected layer, the third convolution) is most of the gradient:
         // finished beside the rest of the chain
-        auto finish = [&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2, nullptr); };
+        auto finish = [&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2); };
         if (side.on) side.append(finish);
       }
       if (chunked && l == 1) {
@@ -539,16 +539,11 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
       }
     }
     side.join();
-    ready += finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials + ready : nullptr, NORM_BLOCKS - ready, c->stats);
-    if (all_finished && tc_supported(c->arch, c->prec)) {
-      tc_close_update(c->lc, c->nd, c->theta, c->rms, c->grad, c->theta16, c->w_images, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
-                      c->norm_partials, ready, c->stats);
-    } else {
-      launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad,
-                          c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
-                          c->norm_partials, c->stats, all_finished ? ready : 0);
-      if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
-    }
+    ready += finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials + ready : nullptr, NORM_BLOCKS - ready);
+    launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad,
+                        c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
+                        c->norm_partials, c->stats, all_finished ? ready : 0);
+    if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
     if (stats) launch_publish_stats(c->lc, c->stats, &c->box->stats, &c->box->done);
   });
   c->N += (uint64_t)c->B;

@@ -53,6 +53,21 @@ __host__ __device__ __forceinline__ float philox_uniform(uint32_t c0, uint32_t c
 struct HeadMode { int algo; float eps; };
 
 #ifdef __CUDACC__
+// Head output `lane` of state e (of n) from its shares hp[PARTS][n][32], PARTS / 2 for each half of the hidden units: what is
+// left of the tree the fully connected kernel adds a half's sums up in, then the two halves.
+template <int PARTS>
+__device__ __forceinline__ float sum_head_parts(const float* hp, int n, size_t e, int lane) {
+  const float* p = hp + e * 32 + lane;
+  float v[PARTS];
+#pragma unroll
+  for (int i = 0; i < PARTS; ++i) v[i] = p[(size_t)i * n * 32];
+#pragma unroll
+  for (int o = PARTS / 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < o; ++i) { v[i] += v[i + o]; v[PARTS / 2 + i] += v[PARTS / 2 + i + o]; }
+  return v[0] + v[PARTS / 2];
+}
+
 // Everything that follows the heads' dot products, done by one full warp for state e.  Lane k < A holds head output
 // z_k (the other lanes -inf); v is the value head's output, the same in all lanes.  Writes the A outputs and the
 // stored value; with `sample` it also draws the action from the Philox uniform of (e, step) -- inverse CDF of the
@@ -303,7 +318,6 @@ struct DeviceStats {
   float policy_loss, value_loss, entropy, grad_norm, clip_scale;
   int32_t status;
   uint32_t error_word;   // bit set by a kernel whose bounded wait or bounds check gave up
-  uint32_t error_taken;  // error_word as the finishing kernel found it: what the kernel that closes the update goes by
   uint32_t arrivals;     // blocks of the head-gradient kernel that have finished (back to zero when it ends)
 };
 

@@ -57,11 +57,11 @@ void launch_cast_bf16(LaunchCtx& lc, const float* src, bf16* dst, size_t n) {
 // little endian, are the four channels), as 16-byte stores.
 constexpr int ENV_THREADS = 256;
 
-// With SAMPLE the block's first warp also takes the action first: it finishes the heads of its environment from the
-// two partial dot products hp[half][e][k] the fully connected kernel left (k < A policy rows, k = A value row;
+// With PARTS > 0 (SAMPLE) the block's first warp also takes the action first: it finishes the heads of its environment from the
+// partial dot products hp[part][e][k] the fully connected kernel left (k < A policy rows, k = A value row;
 // rows 32 floats apart), softmax, inverse-CDF draw from the Philox uniform of (env, step) exactly as the stand-alone
 // sampling kernel does, and writes logits, value, uniform and action; the transition then uses that action.
-template <bool SAMPLE>
+template <int PARTS>
 __global__ void __launch_bounds__(ENV_THREADS)
 env_step_kernel(uint64_t seed, int n_e, const uint64_t* __restrict__ step_base, uint32_t t,
                 const int32_t* actions, uint32_t term_denom,
@@ -71,27 +71,30 @@ env_step_kernel(uint64_t seed, int n_e, const uint64_t* __restrict__ step_base, 
   // the second warp prepares everything of the transition that does not depend on it -- the hash chains of this step
   // and the next up to the point where the action enters, and the environment's counters, whose loads would otherwise
   // be waited for after the draw.  One hash step, the reward / terminal bits and the frame's base remain.
+  constexpr bool SAMPLE = PARTS > 0;
   __shared__ EnvFrame s_frame;
   __shared__ int32_t s_action;
   const uint32_t e = blockIdx.x;
   const bool stepping = SAMPLE || actions != nullptr;          // else: the start frames (step 0, tag 0)
   EnvPrep prep{};
+  // what precedes the wait was written at least five kernels ago (the counters, the step index, the biases)
+  if (SAMPLE && threadIdx.x == 32) prep = env_prepare(seed, e, n_e, (uint32_t)(*step_base) + t, counters);     // step index of this transition
   if (SAMPLE && threadIdx.x < 32) {
     const int lane = threadIdx.x, A = ht.A;
     const float bias = lane < A ? __ldg(ht.bpi + lane) : (lane == A ? __ldg(ht.bv) : 0.f);   // older than the previous kernel
     pdl_entry();
     float sum = -INFINITY;
-    if (lane <= A) sum = (ht.hp[(size_t)e * 32 + lane] + ht.hp[((size_t)n_e + e) * 32 + lane]) + bias;
+    if (lane <= A) sum = sum_head_parts<SAMPLE ? PARTS : 2>(ht.hp, n_e, e, lane) + bias;
     const float z = lane < A ? sum : -INFINITY;
     const int32_t a = warp_finish_heads(ht.mode, z, __shfl_sync(0xffffffffu, sum, A), lane, A, (size_t)e, ht.logits, ht.values, true,
                                         seed, *step_base + t, ht.forced, ht.actions, ht.sampled, ht.uniforms);
     if (lane == 0) s_action = a;
   } else {
     pdl_entry();
-    if (threadIdx.x == 32) {
+    if (!SAMPLE && threadIdx.x == 32) {
       if (stepping) {
-        prep = env_prepare(seed, e, n_e, (uint32_t)(*step_base) + t, counters);     // global step index of this transition
-        if (!SAMPLE) s_action = actions[e];
+        prep = env_prepare(seed, e, n_e, (uint32_t)(*step_base) + t, counters);
+        s_action = actions[e];
       } else {
         prep.pre_next = env_hash_prefix(seed, e, 0u);
       }
@@ -112,7 +115,7 @@ void launch_env_step(LaunchCtx& lc, uint64_t seed, int n_e, const uint64_t* step
                      const int32_t* actions, uint32_t term_denom, uint8_t* next_frames, int8_t* rewards,
                      uint8_t* terminals, int32_t* counters, int pattern_actions) {
   KernelScope scope(lc, KID_ENV_STEP);
-  launch_kernel(lc, env_step_kernel<false>, n_e, ENV_THREADS, 0, seed, n_e, step_base, t, actions, term_denom, next_frames, rewards,
+  launch_kernel(lc, env_step_kernel<0>, n_e, ENV_THREADS, 0, seed, n_e, step_base, t, actions, term_denom, next_frames, rewards,
                                                   terminals, counters, HeadsTail{}, pattern_actions);
 }
 
@@ -120,8 +123,13 @@ void launch_env_step_sampling(LaunchCtx& lc, uint64_t seed, int n_e, const uint6
                               uint8_t* next_frames, int8_t* rewards, uint8_t* terminals, int32_t* counters,
                               const HeadsTail& ht, int pattern_actions) {
   KernelScope scope(lc, KID_ENV_STEP);
-  launch_kernel(lc, env_step_kernel<true>, n_e, ENV_THREADS, 0, seed, n_e, step_base, t, (const int32_t*)nullptr, term_denom,
-                next_frames, rewards, terminals, counters, ht, pattern_actions);
+  // up to two blocks per SM may set up while the previous kernel drains; more of them would pile up on the first free SMs
+  auto launch = [&](auto how) {
+    how(lc, ht.parts == 2 ? env_step_kernel<2> : (ht.parts == 4 ? env_step_kernel<4> : env_step_kernel<8>), dim3(n_e), dim3(ENV_THREADS), (size_t)0, seed, n_e, step_base, t, (const int32_t*)nullptr, term_denom,
+        next_frames, rewards, terminals, counters, ht, pattern_actions);
+  };
+  if (n_e <= 296) launch([](auto&&... a) { launch_kernel_overlapped(a...); });
+  else launch([](auto&&... a) { launch_kernel(a...); });
 }
 
 // the environments' global step index lives on the device, so that a recorded sequence of launches can be

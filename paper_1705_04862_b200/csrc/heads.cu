@@ -248,9 +248,10 @@ heads_fused_kernel(const float* __restrict__ part, int splits, const float* __re
 }
 
 // The tail of the heads for the cluster path of the fully connected layer, which has already taken the head dot
-// products over each half of the hidden units: hp[half][e][k], k < A the policy rows, k = A the value row, rows
-// HS_LD floats apart.  One warp per state, lane k holds logit k; softmax and sampling as above.
-constexpr int HS_LD = 32, HS_WARPS = 4;
+// products over each part of the hidden units: hp[part][e][k], k < A the policy rows, k = A the value row, rows
+// 32 floats apart.  One warp per state, lane k holds logit k; softmax and sampling as above.
+constexpr int HS_WARPS = 4;
+template <int PARTS>
 __global__ void __launch_bounds__(HS_WARPS * 32)
 heads_sample_kernel(const float* __restrict__ hp, const float* __restrict__ bpi, const float* __restrict__ bv, int n, int A,
                     float* __restrict__ logits, float* __restrict__ values, uint64_t seed,
@@ -265,7 +266,7 @@ heads_sample_kernel(const float* __restrict__ hp, const float* __restrict__ bpi,
   if (advance_step != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *advance_step += advance_by;
   if (e >= n) return;
   float s = -INFINITY;
-  if (lane <= A) s = (hp[(size_t)e * HS_LD + lane] + hp[((size_t)n + e) * HS_LD + lane]) + b;
+  if (lane <= A) s = sum_head_parts<PARTS>(hp, n, (size_t)e, lane) + b;
   const float z = lane < A ? s : -INFINITY;
   warp_finish_heads(mode, z, __shfl_sync(0xffffffffu, s, A), lane, A, (size_t)e, logits, values, actions != nullptr, seed,
                     actions != nullptr ? *step_base + t : 0ull, forced, actions, sampled, uniforms);
@@ -276,10 +277,10 @@ bool heads_fused_supported(const NetDims& nd) { return nd.F == 512 && nd.pi_w % 
 void launch_heads_fused(LaunchCtx& lc, const NetDims& nd, const float* theta, const bf16* theta16, const float* part,
                         int splits, bf16* h_out, int n, float* logits, float* values, uint64_t seed,
                         const uint64_t* step_base, uint32_t t, const int32_t* forced, int32_t* actions, int32_t* sampled,
-                        float* uniforms, HeadMode mode, uint64_t* advance_step, uint32_t advance_by) {
+                        float* uniforms, HeadMode mode, uint64_t* advance_step, uint32_t advance_by, int parts) {
   KernelScope scope(lc, KID_HEADS_FWD);
-  if (splits == 0) {          // `part` holds the head dot products of the two halves of the hidden units
-    launch_kernel_overlapped(lc, heads_sample_kernel, (n + HS_WARPS - 1) / HS_WARPS, HS_WARPS * 32, 0, part, theta + nd.pi_b,
+  if (splits == 0) {          // `part` holds the head dot products of the parts of the hidden units
+    launch_kernel_overlapped(lc, parts == 2 ? heads_sample_kernel<2> : (parts == 4 ? heads_sample_kernel<4> : heads_sample_kernel<8>), (n + HS_WARPS - 1) / HS_WARPS, HS_WARPS * 32, 0, part, theta + nd.pi_b,
                              theta + nd.v_b, n, nd.A, logits, values, seed, advance_step ? nullptr : step_base, t, forced,
                              actions, sampled, uniforms, advance_step, advance_by, mode);
     return;

@@ -14,10 +14,10 @@ void launch_env_step(LaunchCtx& lc, uint64_t seed, int n_e, const uint64_t* step
                      uint8_t* terminals, int32_t* counters /* [3][n_e] */, int pattern_actions = 0 /* > 0: the learnable
                      environment with that many actions */);
 
-// What is left of the heads after the cluster kernel of the fully connected layer: the two halves' dot products
-// hp[2][n_e][32], the head biases, and where logits, values, uniforms and actions go (see launch_heads_fused).
+// What is left of the heads after the cluster kernel of the fully connected layer: the shares of the dot products,
+// hp[parts][n_e][32], the head biases, and where logits, values, uniforms and actions go (see launch_heads_fused).
 struct HeadsTail {
-  const float* hp; const float* bpi; const float* bv; int A;
+  const float* hp; int parts; const float* bpi; const float* bv; int A;
   float* logits; float* values; const int32_t* forced; int32_t* actions; int32_t* sampled; float* uniforms;
   HeadMode mode;
 };
@@ -51,9 +51,8 @@ struct GradSegments { GradSegment seg[12]; int n; int total_groups; };
 // false: list full
 bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale, bool in_order = false);
 // sumsq_partials != nullptr: every block also leaves the sum of squares of the gradient values it wrote in
-// sumsq_partials[block]; returns the number of blocks launched (at most max_blocks).  stats != nullptr: the error word is
-// taken down for the kernel that closes the update.
-int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, int max_blocks, DeviceStats* stats);
+// sumsq_partials[block]; returns the number of blocks launched (at most max_blocks)
+int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, int max_blocks);
 
 // ---- network on the CUDA cores (net_simt.cu) --------------------------------------------
 // act[l]: stored activation of layer l for the n states, storage float (PAAC_FP32) or bf16.  Returns the number of split-k
@@ -70,21 +69,16 @@ bool tc_supported(int arch, int prec);
 size_t tc_fc_scratch_floats(int n);
 // with fc_splits != nullptr the end of the fully connected layer is shared with launch_heads_fused: either the layer
 // is left as *fc_splits > 0 split-k partial sums in fc_scratch (part[split][n][512]) for that kernel to finish, or
-// (*fc_splits == 0) the layer is complete and fc_scratch holds the head dot products of the two halves of the
-// hidden units, hp[2][n][32], which that call only has to add up
+// (*fc_splits == 0) the layer is complete and fc_scratch holds the head dot products in *head_parts shares,
+// hp[parts][n][32], which that call only has to add up (see sum_head_parts)
 void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, const bf16* theta16, const bf16* images,
                 const uint8_t* frames, int n, void* const act[], float* fc_scratch, uint32_t* error_word,
-                int* fc_splits = nullptr);
+                int* fc_splits = nullptr, int* head_parts = nullptr);
 // transposed / regrouped bf16 weight images the backward contractions read (refreshed after every
 // parameter change), and the data-gradient kernels that use them
 size_t tc_weight_image_elems();
 // (a first-layer weight whose fp16 image would overflow raises DEV_ERR_RANGE in *error_word)
-// (afterwards tc_close_update() keeps them up to date)
 void tc_relayout_weights(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, bf16* images, uint32_t* error_word);
-// The end of a tensor-core update: clipping and RMSProp as launch_clip_rmsprop, and in the same pass the bf16 copy and the
-// weight images.  norm_partials[0 .. n_partials) hold the squared norm, stats->error_taken the error word (finish_gradients).
-void tc_close_update(LaunchCtx& lc, const NetDims& nd, float* theta, float* rms, const float* grad, bf16* theta16, bf16* images,
-                     float lr, float rho, float eps, float clip, const float* norm_partials, int n_partials, DeviceStats* stats);
 // one block waits at most max_polls polls on a barrier nobody signals, then records the time-out in *error_word
 void launch_wait_probe(LaunchCtx& lc, uint32_t max_polls, uint32_t* error_word);
 void tc_backward_dgrad_fc(LaunchCtx& lc, const bf16* images, int n, void* const act[], void* const gact[], uint32_t* err);
@@ -133,7 +127,7 @@ bool heads_fused_supported(const NetDims& nd);
 void launch_heads_fused(LaunchCtx& lc, const NetDims& nd, const float* theta, const bf16* theta16, const float* part,
                         int splits, bf16* h_out, int n, float* logits, float* values, uint64_t seed,
                         const uint64_t* step_base, uint32_t t, const int32_t* forced, int32_t* actions, int32_t* sampled,
-                        float* uniforms, HeadMode mode, uint64_t* advance_step = nullptr, uint32_t advance_by = 0);
+                        float* uniforms, HeadMode mode, uint64_t* advance_step = nullptr, uint32_t advance_by = 0, int parts = 2);
 // advance_step (only honoured with splits == 0, only valid without sampling): the kernel also adds advance_by to the
 // environments' step index, which saves the rollout its last launch
 // n-step returns and advantages, the loss gradient at the heads and the loss statistics, in one launch

@@ -17,7 +17,6 @@
 #include <cuda.h>          // CUtensorMap and its enums only; the encoder is looked up at run time, nothing links to libcuda
 
 #include "kernels.h"
-#include "optim_device.cuh"
 #include "tc_common.cuh"
 
 namespace paac {
@@ -33,13 +32,24 @@ constexpr size_t TC_IMG_W2 = 0, TC_IMG_W3 = 4 * 32 * 256, TC_IMG_WFC = TC_IMG_W3
 // map of matrix x[rows][cols] (row pitch `ld` elements) for boxes of box_rows x 64 elements with the 128-byte swizzle.
 // Maps are cached by their defining values: the matrices live at fixed places of the workspace, so after the first
 // iteration every call is a look-up.  Returns nullptr if the driver's encoder is unavailable or refuses.
+// the driver's encoder, looked up at run time (nothing links to libcuda); nullptr if it cannot be had
+typedef CUresult (*TmapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                 const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+static TmapEncodeFn tc_tmap_encoder() {
+  static const TmapEncodeFn encode = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
+        qres != cudaDriverEntryPointSuccess) fn = nullptr;
+    return (TmapEncodeFn)fn;
+  }();
+  return encode;
+}
+
 struct TmapKey { const void* p; uint64_t rows, cols, ld; uint32_t box_rows; };
 static const CUtensorMap* tc_tensor_map(const bf16* x, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows) {
-  typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn encode = nullptr;
-  static bool looked_up = false;
+  const TmapEncodeFn encode = tc_tmap_encoder();
   constexpr int MAX_MAPS = 64;
   static TmapKey keys[MAX_MAPS];
   static CUtensorMap maps[MAX_MAPS];
@@ -47,14 +57,6 @@ static const CUtensorMap* tc_tensor_map(const bf16* x, uint64_t rows, uint64_t c
   for (int i = 0; i < n_maps; ++i)
     if (keys[i].p == x && keys[i].rows == rows && keys[i].cols == cols && keys[i].ld == ld && keys[i].box_rows == box_rows)
       return &maps[i];
-  if (!looked_up) {
-    looked_up = true;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      encode = (EncodeFn)fn;
-  }
   if (encode == nullptr) return nullptr;
   static int next = 0;                                   // a full cache is overwritten in turn: launches copy the map
   const int slot = n_maps < MAX_MAPS ? n_maps : next++ % MAX_MAPS;
@@ -87,19 +89,7 @@ static const CUtensorMap* tc_tensor_map3(const bf16* x, uint64_t d1, uint64_t d2
   const int slot = n_maps < MAX_MAPS ? n_maps : next++ % MAX_MAPS;
   CUtensorMap* out = &maps[slot];
   keys[slot].p = nullptr;
-  typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn encode = nullptr;
-  static bool looked_up = false;
-  if (!looked_up) {
-    looked_up = true;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      encode = (EncodeFn)fn;
-  }
+  const TmapEncodeFn encode = tc_tmap_encoder();
   if (encode == nullptr) return nullptr;
   const cuuint64_t gdim[3] = {64, d1, d2}, gstride[2] = {stride1, stride2};
   const cuuint32_t box[3] = {64u, box1, box2}, estride[3] = {1u, 1u, 1u};
@@ -110,6 +100,33 @@ static const CUtensorMap* tc_tensor_map3(const bf16* x, uint64_t d1, uint64_t d2
   keys[slot] = Key{x, d1, d2, stride1, stride2, box1, box2};
   if (n_maps < MAX_MAPS) ++n_maps;
   return out;
+}
+
+// Map of the fully connected weights w[512][cols] for the narrow column tiles of the forward kernel: rows seen as
+// [8 groups of 64][64 / group runs][group], boxes of four neighbouring rows of every run of four groups (64 / group * 16
+// rows in all), 128-byte swizzle; cached like the others.
+static const CUtensorMap* tc_tensor_map_runs(const bf16* w, uint64_t cols, uint32_t group) {
+  struct Key { const void* p; uint64_t cols; uint32_t group; };
+  constexpr int MAX_MAPS = 16;
+  static Key keys[MAX_MAPS];
+  static CUtensorMap maps[MAX_MAPS];
+  static int n_maps = 0, next = 0;
+  for (int i = 0; i < n_maps; ++i)
+    if (keys[i].p == w && keys[i].cols == cols && keys[i].group == group) return &maps[i];
+  const TmapEncodeFn encode = tc_tmap_encoder();
+  if (encode == nullptr) return nullptr;
+  const int slot = n_maps < MAX_MAPS ? n_maps : next++ % MAX_MAPS;
+  keys[slot].p = nullptr;
+  const uint64_t row = cols * sizeof(bf16);
+  const cuuint64_t gdim[4] = {cols, group, 64 / group, 8}, gstride[3] = {row, group * row, 64 * row};
+  const cuuint32_t box[4] = {64u, 4u, 64 / group, 4u}, estride[4] = {1u, 1u, 1u, 1u};
+  if (encode(&maps[slot], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(w), gdim, gstride, box, estride,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return nullptr;
+  keys[slot] = Key{w, cols, group};
+  if (n_maps < MAX_MAPS) ++n_maps;
+  return &maps[slot];
 }
 
 struct TcShared {
@@ -1488,24 +1505,30 @@ __global__ void __launch_bounds__(256) fc_finish_kernel(const float* __restrict_
 
 // ---- fully connected layer, forward, as one cluster per output tile --------------------------------------------
 // h[m][n] = bf16(relu(sum_k A[m][k] W[n][k] + bias[n])) and the head dot products that follow it, in one launch.
-// An output tile is 128 rows x 256 columns; the CTAs of a cluster (its size = the number of K slices, chosen on
+// An output tile is 128 rows x BN columns; the CTAs of a cluster (its size = the number of K slices, chosen on
 // the host so that all clusters are resident at once) each multiply a slice of K into a tensor-memory accumulator,
 // park it as floats in their own shared memory (on top of the operand stages, which are no longer needed), write
-// it from there with whole-row accesses to their slice of part[split][m][n] and meet at a cluster barrier.  The
+// it from there with whole-row accesses to their slice of part[split][m][tile column] and meet at a cluster barrier.  The
 // slices are read back microseconds later, from L2.  (Reading the parked tiles of the other CTAs directly through
 // distributed shared memory was measured two to three times slower than this round trip, in every access order
 // tried.)  CTA r of the cluster then owns an equal share of the tile's rows: it adds the slices in split order (so
 // the sum does not depend on timing), applies bias, ReLU and the bf16 rounding, stores h for the backward pass
-// and, from the rounded values, its share of the A + 1 head dot products (256 of the 512 hidden units) as
-// hp[column tile][m][k]; heads_sample_kernel adds the two shares.
-// Warps 0-3 move the accumulator, one thread of warp 4 streams the operands (tiled bulk copies), lane 0 of warp 8
-// issues the MMAs; all twelve warps share the finishing phase (warps 9-11 are there only for it: with two rows per
-// warp a CTA's 21 or 22 rows then take one pass, and a pass costs a round trip to L2 however few rows it has).
-constexpr int FCC_BN = 256, FCC_STAGES = 4, FCC_MAX_SPLITS = 8, FCC_THREADS = 384, FCC_HP_LD = 32;
-constexpr int FCC_FIN_ROWS = 2 * (FCC_THREADS / 32);      // rows of the finishing phase per pass: 24 >= ceil(128 / 6)
-constexpr uint32_t FCC_STAGE_BYTES = TC_BM * 128 + FCC_BN * 128, FCC_ACC_BYTES = TC_BM * FCC_BN * 4;
-constexpr uint32_t FCC_HEADW_BYTES = 33 * FCC_BN * 2;
-static_assert(FCC_ACC_BYTES <= FCC_STAGES * FCC_STAGE_BYTES, "the parked accumulator reuses the operand stages");
+// and, from the rounded values, its share of the A + 1 head dot products (BN of the 512 hidden units) as
+// hp[column tile][m][k]; whoever draws the action adds the shares.
+// BN is 256 where the rows alone fill the device, and 128 or 64 as long as all clusters stay resident: up to 128 rows a CTA
+// then brings 50 KB of weights from L2 instead of 200, and every phase after the K loop handles a quarter of the numbers
+// (rollout step at 32 states 24 -> 21 us, at 256 states 33 -> 31 us).  No sum depends on BN: the K slices are the same, and
+// a head's dot product over 256 units is always made of sixteen running sums, sum cg over columns 4 (cg + 16 j) .. + 3,
+// j < 4, added as a tree (cg with cg ^ 8, then ^ 4, ^ 2, ^ 1).  A narrow tile takes the cg that agree in their low bits, so
+// that it holds whole subtrees, and whoever draws the action adds the tiles' shares: columns 64 j + GROUP q + 4 tile + i,
+// GROUP = 1024 / BN, which one four-dimensional copy per K block gathers.
+constexpr int FCC_MAX_BN = 256, FCC_MAX_PARTS = 8, FCC_STAGES = 4, FCC_MAX_SPLITS = 8, FCC_THREADS = 384, FCC_HP_LD = 32;
+template <int BN> struct FccSize {
+  static constexpr uint32_t STAGE_BYTES = TC_BM * 128 + BN * 128, ACC_BYTES = TC_BM * BN * 4, HEADW_BYTES = 33 * BN * 2;
+  static constexpr int SMEM = FCC_STAGES * STAGE_BYTES + HEADW_BYTES + 1024;
+  static_assert(ACC_BYTES <= FCC_STAGES * STAGE_BYTES, "the parked accumulator reuses the operand stages");
+  static_assert(SMEM <= 227 * 1024, "shared memory budget");
+};
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -1523,12 +1546,16 @@ struct FccShared {
   volatile uint32_t abort;
 };
 
+template <int FCC_BN>
 __global__ void __launch_bounds__(FCC_THREADS, 1)
 tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
                      const float* __restrict__ bias,
                      const bf16* __restrict__ wpi, const bf16* __restrict__ wv, int A, bf16* __restrict__ h_out,
                      float* part, float* __restrict__ hp, int M, int N, int K, int tiles_n, int splits,
                      uint32_t* error_word) {
+  constexpr uint32_t FCC_STAGE_BYTES = FccSize<FCC_BN>::STAGE_BYTES;
+  constexpr bool WIDE = FCC_BN == FCC_MAX_BN;
+  constexpr int CH = FCC_BN / 4, CGN = FCC_BN / 16, RUN = FCC_BN / 4, GROUP = 1024 / FCC_BN;      // 16-byte chunks of a parked row; running sums of a tile
   extern __shared__ uint8_t dyn_smem[];
   __shared__ FccShared sh;
   const uint32_t base = (smem_u32(dyn_smem) + 1023u) & ~1023u;
@@ -1536,6 +1563,8 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank(), tile = blockIdx.x / splits;
   const int nt = tile % tiles_n, mt = tile / tiles_n;
+  // local column RUN j + 4 q + i of this tile is column col0 + 64 j + GROUP q + i of the layer
+  const int half = nt / (FCC_MAX_BN / FCC_BN), share = nt % (FCC_MAX_BN / FCC_BN), col0 = half * FCC_MAX_BN + 4 * share;
   const int kb_total = K / TC_BK, kb_base = kb_total / splits, kb_rem = kb_total % splits;
   const int kb0 = rank * kb_base + min(rank, kb_rem), kb1 = kb0 + kb_base + (rank < kb_rem ? 1 : 0);
 
@@ -1565,7 +1594,8 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
         const uint32_t stage = base + s * FCC_STAGE_BYTES;
         mbar_arrive_expect_tx(&sh.full[s], FCC_STAGE_BYTES);
         tma_load_2d(stage, &tm_a, kb * TC_BK, mt * TC_BM, &sh.full[s]);
-        tma_load_2d(stage + TC_BM * 128, &tm_w, kb * TC_BK, nt * FCC_BN, &sh.full[s]);
+        if constexpr (WIDE) tma_load_2d(stage + TC_BM * 128, &tm_w, kb * TC_BK, col0, &sh.full[s]);
+        else tma_load_4d(stage + TC_BM * 128, &tm_w, kb * TC_BK, 4 * share, 0, 4 * half, &sh.full[s]);
       }
     }
   } else if (warp == 8) {
@@ -1593,14 +1623,13 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     // weights of this column tile (row k = policy row k, k < A, 16-byte aligned, or the value row, k = A, which follows
     // the policy biases in the parameter vector and is only 2-byte aligned; 256 bf16 each).  The weights are several
     // kernels old; the block-wide barrier after the accumulator is parked makes them visible to the finishing phase.
-    for (int i = threadIdx.x; i < A * (FCC_BN / 8); i += 128) {
-      const int k = i / (FCC_BN / 8), c = i % (FCC_BN / 8);
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(wpi + (size_t)k * N + nt * FCC_BN) + c);
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(headw + (uint32_t)(k * FCC_BN + 8 * c) * 2u),
-                   "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+    for (int i = threadIdx.x; i < A * CH; i += 128) {
+      const int k = i / CH, c = i % CH;
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(wpi + (size_t)k * N + col0 + 64 * (c / CGN) + GROUP * (c % CGN)));
+      asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(headw + (uint32_t)(k * FCC_BN + 4 * c) * 2u), "r"(v.x), "r"(v.y) : "memory");
     }
     for (int c = threadIdx.x; c < FCC_BN / 2; c += 128) {
-      const bf16* src = wv + nt * FCC_BN + 2 * c;
+      const bf16* src = wv + col0 + 64 * (2 * c / RUN) + GROUP * (2 * c % RUN / 4) + 2 * c % 4;
       const uint32_t v = (uint32_t)__bfloat16_as_ushort(src[0]) | ((uint32_t)__bfloat16_as_ushort(src[1]) << 16);
       asm volatile("st.shared.b32 [%0], %1;" ::"r"(headw + (uint32_t)(A * FCC_BN + 2 * c) * 2u), "r"(v) : "memory");
     }
@@ -1627,13 +1656,13 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   if (threadIdx.x < 256) {
 #pragma unroll 4
     for (int i = 0; i < TC_BM * FCC_BN / 4 / 256; ++i) {
-      const uint32_t q = (uint32_t)threadIdx.x + 256u * i, row = q >> 6, c = q & 63u;
+      const uint32_t q = (uint32_t)threadIdx.x + 256u * i, row = q / CH, c = q % CH;
       const int m = mt * TC_BM + (int)row;
       uint32_t r0, r1, r2, r3;
       asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                    : "r"(base + row * (FCC_BN * 4u) + ((c ^ (row & 7u)) << 4)) : "memory");
       if (m < M)
-        __stcg(reinterpret_cast<float4*>(part + ((size_t)rank * M + m) * N + nt * FCC_BN) + c,
+        __stcg(reinterpret_cast<float4*>(part + ((size_t)rank * M + m) * N + nt * FCC_BN + 4 * c),
                make_float4(__uint_as_float(r0), __uint_as_float(r1), __uint_as_float(r2), __uint_as_float(r3)));
     }
     __threadfence();
@@ -1643,20 +1672,25 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   __syncwarp();
   cluster_sync_all();
   // ---------------- this CTA's share of the tile's rows: sum over the cluster, bias, ReLU, heads ----------------
-  // rows [128 rank / splits, 128 (rank + 1) / splits), two per warp; thread (rl, cg) owns the 16-byte chunks
-  // cg, cg + 16, cg + 32, cg + 48 of row rl, i.e. columns 4 (cg + 16 j) .. + 3: the sixteen threads of a row read
-  // 256 contiguous bytes at a time
-  const int row_lo = TC_BM * rank / splits, row_hi = TC_BM * (rank + 1) / splits;
-  for (int row0 = row_lo + 2 * warp; row0 < row_hi; row0 += FCC_FIN_ROWS) {
-    const int cg = lane & 15;
-    const uint32_t row = (uint32_t)(row0 + (lane >> 4));
+  // rows [128 rank / splits, 128 (rank + 1) / splits), 32 / CGN per warp; thread (rl, cg) owns columns
+  // col0 + 64 j + GROUP cg .. + 3, j < 4, of row rl
+  // With narrow tiles the rows are few: the tile's valid rows are dealt out, and the warps a CTA's rows leave idle repeat their
+  // sums (a few KB from L2) and take every groups-th head.
+  const int rows_here = WIDE ? TC_BM : min(TC_BM, M - mt * TC_BM);
+  const int row_lo = rows_here * rank / splits, row_hi = rows_here * (rank + 1) / splits;
+  constexpr int WROWS = 32 / CGN;
+  const int group_warps = WIDE ? FCC_THREADS / 32 : max(1, (row_hi - row_lo + WROWS - 1) / WROWS), groups = FCC_THREADS / 32 / group_warps;
+  const int group = warp / group_warps;
+  for (int row0 = row_lo + WROWS * (warp % group_warps); row0 < row_hi && group < groups; row0 += WROWS * (FCC_THREADS / 32)) {
+    const int cg = lane % CGN;
+    const uint32_t row = (uint32_t)(row0 + lane / CGN);
     const bool live = (int)row < row_hi;
     const int m = live ? mt * TC_BM + (int)row : M;
     float v[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = 0.f;
     if (m < M) {
-      const float4* src = reinterpret_cast<const float4*>(part + (size_t)m * N + nt * FCC_BN) + cg;
+      const float4* src = reinterpret_cast<const float4*>(part + (size_t)m * N + nt * FCC_BN + 4 * cg);
       // the first six slices are asked for in one go (24 loads in flight per thread: the phase is a chain of L2
       // latencies otherwise), a seventh and eighth, if any, after them; the additions keep the slice order
       {
@@ -1665,7 +1699,7 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
         for (int s = 0; s < 6; ++s)
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            t[s][j] = s < splits ? __ldcg(src + (size_t)s * M * (N / 4) + 16 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
+            t[s][j] = s < splits ? __ldcg(src + (size_t)s * M * (N / 4) + CGN * j) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int s = 0; s < 6; ++s)
 #pragma unroll
@@ -1679,7 +1713,7 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
         for (int s = 0; s < 2; ++s)
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            t[s][j] = 6 + s < splits ? __ldcg(src + (size_t)(6 + s) * M * (N / 4) + 16 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
+            t[s][j] = 6 + s < splits ? __ldcg(src + (size_t)(6 + s) * M * (N / 4) + CGN * j) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -1691,13 +1725,13 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     float x[16];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = nt * FCC_BN + 4 * (cg + 16 * j);
+      const int n = col0 + 64 * j + GROUP * cg;
       const float4 b = __ldg(reinterpret_cast<const float4*>(bias + n));
       const bf16 h0 = __float2bfloat16_rn(fmaxf(v[4 * j] + b.x, 0.f)), h1 = __float2bfloat16_rn(fmaxf(v[4 * j + 1] + b.y, 0.f));
       const bf16 h2 = __float2bfloat16_rn(fmaxf(v[4 * j + 2] + b.z, 0.f)), h3 = __float2bfloat16_rn(fmaxf(v[4 * j + 3] + b.w, 0.f));
       x[4 * j] = __bfloat162float(h0); x[4 * j + 1] = __bfloat162float(h1);
       x[4 * j + 2] = __bfloat162float(h2); x[4 * j + 3] = __bfloat162float(h3);
-      if (m < M)
+      if (m < M && group == 0)
         *reinterpret_cast<uint2*>(h_out + (size_t)m * N + n) =
             make_uint2((uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16),
                        (uint32_t)__bfloat16_as_ushort(h2) | ((uint32_t)__bfloat16_as_ushort(h3) << 16));
@@ -1705,36 +1739,44 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     // head dot products over this thread's 16 hidden units: independent sums first, then a butterfly over the 16
     // threads of the row that halves the number of live values at each step and leaves thread cg with heads
     // 2 cg and 2 cg + 1 (the additions pair up in a fixed pattern)
-    float pr[FCC_HP_LD];
+    auto dot = [&](int k) {
+      float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll
-    for (int k = 0; k < FCC_HP_LD; ++k) {
-      pr[k] = 0.f;
-      if (k <= A) {
-        float acc0 = 0.f, acc1 = 0.f;
+      for (int j = 0; j < 4; ++j) {
+        uint32_t w0, w1;
+        asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(w0), "=r"(w1)
+                     : "r"(headw + (uint32_t)(k * FCC_BN + 4 * (cg + CGN * j)) * 2u) : "memory");
+        acc0 = fmaf(__uint_as_float(w0 << 16), x[4 * j], acc0);
+        acc1 = fmaf(__uint_as_float(w0 & 0xFFFF0000u), x[4 * j + 1], acc1);
+        acc0 = fmaf(__uint_as_float(w1 << 16), x[4 * j + 2], acc0);
+        acc1 = fmaf(__uint_as_float(w1 & 0xFFFF0000u), x[4 * j + 3], acc1);
+      }
+      return acc0 + acc1;
+    };
+    if constexpr (!WIDE) {
+      // the subtree over this tile's running sums; hp[2 halves x tiles][M][32]
+      for (int k = group; k <= A; k += groups) {
+        float v = dot(k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t w0, w1;
-          asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(w0), "=r"(w1)
-                       : "r"(headw + (uint32_t)(k * FCC_BN + 4 * (cg + 16 * j)) * 2u) : "memory");
-          acc0 = fmaf(__uint_as_float(w0 << 16), x[4 * j], acc0);
-          acc1 = fmaf(__uint_as_float(w0 & 0xFFFF0000u), x[4 * j + 1], acc1);
-          acc0 = fmaf(__uint_as_float(w1 << 16), x[4 * j + 2], acc0);
-          acc1 = fmaf(__uint_as_float(w1 & 0xFFFF0000u), x[4 * j + 3], acc1);
+        for (int o = CGN / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (m < M && cg == 0) hp[((size_t)nt * M + m) * FCC_HP_LD + k] = v;
+      }
+    } else {
+      float pr[FCC_HP_LD];
+#pragma unroll
+      for (int k = 0; k < FCC_HP_LD; ++k) pr[k] = k <= A ? dot(k) : 0.f;
+  #pragma unroll
+      for (int o = 8, len = FCC_HP_LD / 2; o > 0; o >>= 1, len >>= 1) {
+        const bool up = (cg & o) != 0;
+  #pragma unroll
+        for (int i = 0; i < len; ++i) {
+          const float send = up ? pr[i] : pr[i + len];
+          const float keep = up ? pr[i + len] : pr[i];
+          pr[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-        pr[k] = acc0 + acc1;
       }
+      if (m < M) *reinterpret_cast<float2*>(hp + ((size_t)nt * M + m) * FCC_HP_LD + 2 * cg) = make_float2(pr[0], pr[1]);
     }
-#pragma unroll
-    for (int o = 8, len = FCC_HP_LD / 2; o > 0; o >>= 1, len >>= 1) {
-      const bool up = (cg & o) != 0;
-#pragma unroll
-      for (int i = 0; i < len; ++i) {
-        const float send = up ? pr[i] : pr[i + len];
-        const float keep = up ? pr[i + len] : pr[i];
-        pr[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    }
-    if (m < M) *reinterpret_cast<float2*>(hp + ((size_t)nt * M + m) * FCC_HP_LD + 2 * cg) = make_float2(pr[0], pr[1]);
   }
   tcgen05_fence_before();
   __syncthreads();
@@ -1746,50 +1788,47 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
 }
 
 static bool tc_fc_cluster_supported(int N, int K, int A) {
-  return N % FCC_BN == 0 && K % TC_BK == 0 && K / TC_BK >= FCC_MAX_SPLITS && A + 1 <= FCC_HP_LD;
+  return N == 2 * FCC_MAX_BN && K % TC_BK == 0 && K / TC_BK >= FCC_MAX_SPLITS && A + 1 <= FCC_HP_LD;
 }
 
-constexpr int FCC_SMEM = FCC_STAGES * FCC_STAGE_BYTES + FCC_HEADW_BYTES + 1024;
-static_assert(FCC_SMEM <= 227 * 1024, "shared memory budget");
-
-// The largest cluster size (= number of K slices) with which all `tiles` clusters are resident at once, so that
-// the launch is one wave; how many clusters of a size fit depends on how the SMs are grouped on the part.
-static int tc_fc_cluster_splits(int tiles) {
+// How many clusters of `splits` CTAs are resident at once (depends on how the SMs are grouped on the part).
+static int tc_fc_max_clusters(int splits) {
   static int max_active[FCC_MAX_SPLITS + 1] = {};          // 0 = not asked yet, -1 = the query failed
-  for (int sp = FCC_MAX_SPLITS; sp >= 4; --sp) {
-    if (max_active[sp] == 0) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(sp * 16); cfg.blockDim = dim3(FCC_THREADS); cfg.dynamicSmemBytes = FCC_SMEM;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = sp; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr; cfg.numAttrs = 1;
-      int n = 0;
-      max_active[sp] = cudaOccupancyMaxActiveClusters(&n, tc_fc_cluster_kernel, &cfg) == cudaSuccess && n > 0 ? n : -1;
-    }
-    if (max_active[sp] >= tiles) return sp;
+  if (max_active[splits] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cudaFuncSetAttribute(tc_fc_cluster_kernel<FCC_MAX_BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, FccSize<FCC_MAX_BN>::SMEM);
+    cfg.gridDim = dim3(splits * 16); cfg.blockDim = dim3(FCC_THREADS); cfg.dynamicSmemBytes = FccSize<FCC_MAX_BN>::SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = splits; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int n = 0;
+    max_active[splits] = cudaOccupancyMaxActiveClusters(&n, tc_fc_cluster_kernel<FCC_MAX_BN>, &cfg) == cudaSuccess && n > 0 ? n : -1;
   }
+  return max_active[splits];
+}
+// The largest cluster size (= number of K slices) with which all `tiles` clusters are resident at once, so that
+// the launch is one wave.
+static int tc_fc_cluster_splits(int tiles) {
+  for (int sp = FCC_MAX_SPLITS; sp >= 4; --sp)
+    if (tc_fc_max_clusters(sp) >= tiles) return sp;
   return 4;
 }
 
-// false (nothing launched) if the tensor maps cannot be made; the caller then takes the split-k kernel
-static bool tc_fc_forward_cluster(LaunchCtx& lc, const bf16* a, const bf16* w, const float* bias, const bf16* wpi,
-                                  const bf16* wv, int A, bf16* h_out, float* part, float* hp, int M, int N, int K,
-                                  uint32_t* err) {
-  constexpr int smem = FCC_SMEM;
-  const CUtensorMap* tm_a = tc_tensor_map(a, (uint64_t)M, (uint64_t)K, (uint64_t)K, TC_BM);
-  const CUtensorMap* tm_w = tc_tensor_map(w, (uint64_t)N, (uint64_t)K, (uint64_t)K, FCC_BN);
-  if (tm_a == nullptr || tm_w == nullptr) return false;
+template <int BN>
+static bool tc_fc_cluster_launch(LaunchCtx& lc, const CUtensorMap* tm_a, const bf16* w, const float* bias, const bf16* wpi, const bf16* wv,
+                                 int A, bf16* h_out, float* part, float* hp, int M, int N, int K, int splits, uint32_t* err) {
+  const CUtensorMap* tm_w = BN == FCC_MAX_BN ? tc_tensor_map(w, (uint64_t)N, (uint64_t)K, (uint64_t)K, BN) : tc_tensor_map_runs(w, (uint64_t)K, 1024 / BN);
+  if (tm_w == nullptr) return false;
   static bool configured = false;
   if (!configured) {
-    cudaFuncSetAttribute(tc_fc_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(tc_fc_cluster_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, FccSize<BN>::SMEM);
     configured = true;
   }
-  const int tiles_m = (M + TC_BM - 1) / TC_BM, tiles_n = N / FCC_BN;
-  const int splits = tc_fc_cluster_splits(tiles_m * tiles_n);
+  const int tiles_m = (M + TC_BM - 1) / TC_BM, tiles_n = N / BN;
   KernelScope scope(lc, KID_FC_FWD);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tiles_m * tiles_n * splits); cfg.blockDim = dim3(FCC_THREADS); cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(tiles_m * tiles_n * splits); cfg.blockDim = dim3(FCC_THREADS); cfg.dynamicSmemBytes = FccSize<BN>::SMEM;
   cfg.stream = lc.st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1798,8 +1837,23 @@ static bool tc_fc_forward_cluster(LaunchCtx& lc, const bf16* a, const bf16* w, c
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = (pdl_enabled() && !lc.serialize_next) ? 2 : 1;
   lc.serialize_next = false;
-  cudaLaunchKernelEx(&cfg, tc_fc_cluster_kernel, *tm_a, *tm_w, bias, wpi, wv, A, h_out, part, hp, M, N, K, tiles_n, splits, err);
+  cudaLaunchKernelEx(&cfg, tc_fc_cluster_kernel<BN>, *tm_a, *tm_w, bias, wpi, wv, A, h_out, part, hp, M, N, K, tiles_n, splits, err);
   return true;
+}
+
+// The number of shares of the head dot products in hp (2, 4 or 8: one per column tile), 0 (nothing launched) if the tensor maps cannot be
+// made; the caller then takes the split-k kernel.
+static int tc_fc_forward_cluster(LaunchCtx& lc, const bf16* a, const bf16* w, const float* bias, const bf16* wpi,
+                                 const bf16* wv, int A, bf16* h_out, float* part, float* hp, int M, int N, int K,
+                                 uint32_t* err) {
+  const CUtensorMap* tm_a = tc_tensor_map(a, (uint64_t)M, (uint64_t)K, (uint64_t)K, TC_BM);
+  if (tm_a == nullptr) return 0;
+  const int tiles_m = (M + TC_BM - 1) / TC_BM, splits = tc_fc_cluster_splits(tiles_m * (N / FCC_MAX_BN)), room = tc_fc_max_clusters(splits);
+  bool ok;
+  if (tiles_m * (N / 64) <= room) ok = tc_fc_cluster_launch<64>(lc, tm_a, w, bias, wpi, wv, A, h_out, part, hp, M, N, K, splits, err);
+  else if (tiles_m * (N / 128) <= room) ok = tc_fc_cluster_launch<128>(lc, tm_a, w, bias, wpi, wv, A, h_out, part, hp, M, N, K, splits, err);
+  else ok = tc_fc_cluster_launch<256>(lc, tm_a, w, bias, wpi, wv, A, h_out, part, hp, M, N, K, splits, err);
+  return !ok ? 0 : (tiles_m * (N / 64) <= room ? N / 64 : (tiles_m * (N / 128) <= room ? N / 128 : N / 256));
 }
 
 // ---- first layer, forward: uint8 frames -> bf16 operand on the fly --------------------------------------
@@ -2220,7 +2274,7 @@ static void tc_gemm(LaunchCtx& lc, int kid, ASrc a, BSrc b, Epi e, int M, int N,
 }
 
 constexpr int FC_SPLITS = 7;
-size_t tc_fc_scratch_floats(int n) { return (size_t)FCC_MAX_SPLITS * n * 512 + (size_t)2 * n * FCC_HP_LD; }
+size_t tc_fc_scratch_floats(int n) { return (size_t)FCC_MAX_SPLITS * n * 512 + (size_t)FCC_MAX_PARTS * n * FCC_HP_LD; }
 
 static void tc_fc_forward(LaunchCtx& lc, const bf16* a, const bf16* w, const float* bias, bf16* out, int M, int N, int K,
                           float* part, uint32_t* err, int* splits_out) {
@@ -2248,7 +2302,7 @@ static void tc_fc_forward(LaunchCtx& lc, const bf16* a, const bf16* w, const flo
 bool tc_supported(int arch, int prec) { return arch == PAAC_ARCH_NATURE && prec == PAAC_BF16; }
 
 void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, const bf16* w, const bf16* images,
-                const uint8_t* frames, int n, void* const act[], float* fc_scratch, uint32_t* err, int* fc_splits) {
+                const uint8_t* frames, int n, void* const act[], float* fc_scratch, uint32_t* err, int* fc_splits, int* head_parts) {
   const LayerDims* d = nd.layer;
   if (arch != PAAC_ARCH_NATURE) return;   // the caller routes the smaller network to the CUDA-core path
   {
@@ -2269,10 +2323,13 @@ void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, 
           ShiftBiasReluEpi<Map, 7, 7>{Map{n}, (bf16*)act[2], theta + d[2].b_off, nullptr}, n * 81, err);
     }
     (void)M2; (void)M3;
-    if (fc_splits != nullptr && tc_fc_cluster_supported(512, 3136, nd.A) &&
-        tc_fc_forward_cluster(lc, (const bf16*)act[2], w + d[3].w_off, theta + d[3].b_off, w + nd.pi_w, w + nd.v_w, nd.A,
-                              (bf16*)act[3], fc_scratch + (size_t)2 * n * FCC_HP_LD, fc_scratch, n, 512, 3136, err)) {
-      // cluster path: h is complete and fc_scratch holds the head dot products as hp[2][n][32] (*fc_splits = 0)
+    // cluster path: h is complete and fc_scratch holds the head dot products as hp[parts][n][32] (*fc_splits = 0)
+    if (fc_splits != nullptr && tc_fc_cluster_supported(512, 3136, nd.A))
+      *head_parts = tc_fc_forward_cluster(lc, (const bf16*)act[2], w + d[3].w_off, theta + d[3].b_off, w + nd.pi_w, w + nd.v_w, nd.A,
+                                          (bf16*)act[3], fc_scratch + (size_t)FCC_MAX_PARTS * n * FCC_HP_LD, fc_scratch, n, 512, 3136, err);
+    else if (head_parts != nullptr)
+      *head_parts = 0;
+    if (head_parts != nullptr && *head_parts > 0) {
       *fc_splits = 0;
     } else {
       tc_fc_forward(lc, (const bf16*)act[2], w + d[3].w_off, theta + d[3].b_off, (bf16*)act[3], n, 512, 3136, fc_scratch, err,
@@ -2520,9 +2577,8 @@ __global__ void tc_bias_final_kernel(const float* __restrict__ part, int blocks,
 constexpr int FG_J = 2;          // rows of j per group of a many-split segment
 constexpr int FG_CHUNK = 128;    // splits at a time of a segment added in order
 enum { FG_FEW = 0, FG_MANY = 1, FG_IN_ORDER = 2 };
-__global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments segs, float* __restrict__ sumsq_partials, DeviceStats* stats) {
+__global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments segs, float* __restrict__ sumsq_partials) {
   pdl_entry();
-  if (stats != nullptr && blockIdx.x == 0 && threadIdx.x == 0) stats->error_taken = *reinterpret_cast<const volatile uint32_t*>(&stats->error_word);
   __shared__ float sh[FG_CHUNK * FG_J * 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float ss = 0.f;                       // sum of squares of the gradient values this thread writes
@@ -3253,12 +3309,12 @@ size_t tc_scratch_floats(int n) { return tc_layer_scratch_offset(n, 4) + tc_head
 
 // Enqueues the weight-gradient kernel of `layer` (0 = conv1 .. 3 = fc) and notes in *segs where its partial
 // sums are; finish_gradients() then turns all noted partial sums into the gradient vector in one launch.
-int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, int max_blocks, DeviceStats* stats) {
+int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, int max_blocks) {
   int blocks = 0;
   if (segs->n > 0) {
     KernelScope scope(lc, KID_WGRAD_REDUCE);
     blocks = segs->total_groups < max_blocks ? segs->total_groups : max_blocks;
-    launch_kernel(lc, tc_finalize_grads_kernel, blocks, 256, 0, *segs, sumsq_partials, stats);
+    launch_kernel(lc, tc_finalize_grads_kernel, blocks, 256, 0, *segs, sumsq_partials);
   }
   segs->n = 0; segs->total_groups = 0;
   return blocks;
@@ -3457,110 +3513,9 @@ size_t tc_weight_image_elems() { return TC_IMG_END; }
 void tc_relayout_weights(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, bf16* images, uint32_t* error_word) {
   const LayerDims* d = nd.layer;
   KernelScope scope(lc, KID_CAST);
-  launch_kernel(lc, relayout_weights_kernel, RL_FC_TILES + RL_SMALL_BLOCKS, 256, 0, theta16 + d[0].w_off, theta16 + d[1].w_off, theta16 + d[2].w_off,
+  launch_kernel_overlapped(lc, relayout_weights_kernel, RL_FC_TILES + RL_SMALL_BLOCKS, 256, 0, theta16 + d[0].w_off, theta16 + d[1].w_off, theta16 + d[2].w_off,
                                                   theta16 + d[3].w_off, images + TC_IMG_W2, images + TC_IMG_W3,
                                                   images + TC_IMG_WFC, images + TC_IMG_W1, error_word);
-}
-
-// The end of an update in one launch: clipping, RMSProp, the bf16 copy and the weight images.  Blocks 0 .. RL_FC_TILES - 1
-// take a 64 x 64 tile of the fully connected matrix each and write its transposed bf16 tile through shared memory; the
-// others take 4096 of the remaining parameters each and scatter the bf16 values of the convolution weights into their
-// images.  Parameters and RMSProp state are fetched before the wait on the finishing kernel, gradients after it.  A launch
-// of its own for the images (5.6 us, and its wait for the optimiser kernel) is what this saves; what bounds the rest is
-// latency: 37 MB, most of it in L2, over 414 blocks.
-constexpr int CU_THREADS = 256, CU_PER = 4;                       // float4 per thread
-constexpr size_t CU_CHUNK = (size_t)CU_THREADS * CU_PER * 4;
-__global__ void __launch_bounds__(CU_THREADS, 3)
-tc_close_update_kernel(size_t P, size_t w1_off, size_t w2_off, size_t w3_off, size_t wfc_off, float* theta, float* rms, const float* grad,
-                       bf16* theta16, bf16* w2_d, bf16* w3_d, bf16* wfc_t, bf16* w1_b, float lr, float rho, float eps, float clip,
-                       const float* partials, int n_partials, DeviceStats* stats) {
-  typedef NatConv1 C1; typedef NatConv2 C2; typedef NatConv3 C3;
-  constexpr size_t NF = 3136 * 512;
-  __shared__ uint16_t tile[64][66];                              // row pitch of 33 words: column reads spread over the banks
-  const bool fc = blockIdx.x < RL_FC_TILES;
-  const int o0 = (blockIdx.x % 8) * 64, in0 = (blockIdx.x / 8) * 64, r = threadIdx.x >> 2, c = threadIdx.x & 3;
-  const size_t rest = P - NF;                                    // everything else, the fully connected matrix cut out
-  size_t at[CU_PER];                                             // first parameter of each group of four (P: none)
-#pragma unroll
-  for (int j = 0; j < CU_PER; ++j) {
-    if (fc) {
-      at[j] = wfc_off + (size_t)(o0 + r) * 3136 + in0 + 4 * c + 16 * j;
-    } else {
-      const size_t q = (blockIdx.x - RL_FC_TILES) * CU_CHUNK + ((size_t)j * CU_THREADS + threadIdx.x) * 4;
-      at[j] = q >= rest ? P : (q < wfc_off ? q : q + NF);
-    }
-  }
-  float4 t4[CU_PER], m4[CU_PER], g4[CU_PER];
-  auto load = [&](const float* p, size_t i) {
-    if (i + 4 <= P) return *reinterpret_cast<const float4*>(p + i);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i < P) v.x = p[i];
-    if (i + 1 < P) v.y = p[i + 1];
-    if (i + 2 < P) v.z = p[i + 2];
-    return v;
-  };
-#pragma unroll
-  for (int j = 0; j < CU_PER; ++j) { t4[j] = load(theta, at[j]); m4[j] = load(rms, at[j]); }
-  pdl_entry();
-#pragma unroll
-  for (int j = 0; j < CU_PER; ++j) g4[j] = load(grad, at[j]);
-  const RmsStep step{lr, rho, eps, clip_scale_of<CU_THREADS>(partials, n_partials, clip, stats->error_taken, stats)};
-  if (step.scale < 0.f) return;
-#pragma unroll
-  for (int j = 0; j < CU_PER; ++j) {
-    const size_t i = at[j];
-    if (i >= P) continue;
-    float* t = &t4[j].x; float* m = &m4[j].x; const float* g = &g4[j].x;
-    uint16_t h[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { step(t[e], m[e], g[e]); h[e] = __bfloat16_as_ushort(__float2bfloat16_rn(t[e])); }
-    const uint2 packed = make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
-    if (i + 4 <= P) {
-      *reinterpret_cast<float4*>(theta + i) = t4[j]; *reinterpret_cast<float4*>(rms + i) = m4[j];
-      *reinterpret_cast<uint2*>(theta16 + i) = packed;
-    } else {
-      for (int e = 0; e < 4 && i + e < P; ++e) { theta[i + e] = t[e]; rms[i + e] = m[e]; reinterpret_cast<uint16_t*>(theta16)[i + e] = h[e]; }
-    }
-    if (fc) {
-      *reinterpret_cast<uint32_t*>(&tile[r][4 * c + 16 * j]) = packed.x;
-      *reinterpret_cast<uint32_t*>(&tile[r][4 * c + 16 * j + 2]) = packed.y;
-    } else if (i >= w3_off && i < w3_off + C3::CO * C3::KK) {     // four neighbours share all but the input channel
-      const int k = (int)(i - w3_off), ci = k % 64, tap = (k / 64) % 9, co = k / 576;
-      for (int e = 0; e < 4; ++e) reinterpret_cast<uint16_t*>(w3_d)[((ci + e) * 9 + tap) * 64 + co] = h[e];
-    } else if (i >= w2_off && i < w2_off + C2::CO * C2::KK) {
-      const int k = (int)(i - w2_off), ci = k % 32, s = (k / 32) % 4, rr = (k / 128) % 4, co = k / 512;
-      const int z = 2 * (rr & 1) + (s & 1), tap = 2 * (rr >> 1) + (s >> 1);
-      for (int e = 0; e < 4; ++e) reinterpret_cast<uint16_t*>(w2_d)[((z * 32 + ci + e) * 4 + tap) * 64 + co] = h[e];
-    } else if (i >= w1_off && i < w1_off + C1::CO * C1::KK) {
-      const int k = (int)(i - w1_off), s = (k / 4) % 8, rr = (k / 32) % 8, co = k / 256;
-      const int to = ((co * 4 + 2 * (rr >> 2) + (s >> 2)) * 4 + (rr & 3)) * 16 + (s & 3) * 4;
-      for (int e = 0; e < 4; ++e) {
-        // the forward kernel's copy of the first layer is fp16, scaled by 2^8 (see u8x4_to_f16x4)
-        const float scaled = __bfloat162float(__ushort_as_bfloat16(h[e])) * C1_F16_WEIGHT_SCALE;
-        if (!(fabsf(scaled) <= 65504.f)) atomicOr(&stats->error_word, DEV_ERR_RANGE);      // beyond fp16 (or not a number)
-        reinterpret_cast<__half*>(w1_b)[to + e] = __float2half_rn(scaled);
-      }
-    }
-  }
-  if (!fc) return;
-  __syncthreads();
-  uint32_t v[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e)
-    v[e] = (uint32_t)tile[16 * c + 2 * e][r] | ((uint32_t)tile[16 * c + 2 * e + 1][r] << 16);
-  uint4* dst = reinterpret_cast<uint4*>(wfc_t + (size_t)(in0 + r) * 512 + o0 + 16 * c);
-  dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
-  dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
-}
-
-void tc_close_update(LaunchCtx& lc, const NetDims& nd, float* theta, float* rms, const float* grad, bf16* theta16, bf16* images,
-                     float lr, float rho, float eps, float clip, const float* norm_partials, int n_partials, DeviceStats* stats) {
-  const LayerDims* d = nd.layer;
-  const size_t rest = nd.P - (size_t)3136 * 512;
-  KernelScope scope(lc, KID_CLIP_RMSPROP);
-  launch_kernel_overlapped(lc, tc_close_update_kernel, RL_FC_TILES + (int)((rest + CU_CHUNK - 1) / CU_CHUNK), CU_THREADS, 0, nd.P, d[0].w_off,
-                           d[1].w_off, d[2].w_off, d[3].w_off, theta, rms, grad, theta16, images + TC_IMG_W2, images + TC_IMG_W3,
-                           images + TC_IMG_WFC, images + TC_IMG_W1, lr, rho, eps, clip, norm_partials, n_partials, stats);
 }
 
 // ---- failure-path probe: a bounded wait that is made to run out ------------------------------------------------

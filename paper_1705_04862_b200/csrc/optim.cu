@@ -1,6 +1,5 @@
 // Global-norm clipping fused with RMSProp.
 #include "kernels.h"
-#include "optim_device.cuh"
 
 namespace paac {
 
@@ -33,7 +32,51 @@ sumsq_kernel(const float* __restrict__ g, size_t P, float* __restrict__ partials
   if (threadIdx.x == 0) partials[blockIdx.x] = sh[0];
 }
 
-// pass 2: norm, clipping factor, RMSProp and the refreshed bf16 copy (see optim_device.cuh).
+struct RmsStep {
+  float lr, rho, eps, scale;
+  // m <- rho m + (1 - rho) (scale g)^2,  theta <- theta - lr (scale g) / sqrt(m + eps)
+  __device__ __forceinline__ void operator()(float& t, float& m, float g) const {
+    const float gs = scale * g;
+    m = fmaf(rho, m, (1.f - rho) * gs * gs);
+    t = t - lr * gs / sqrtf(m + eps);
+  }
+};
+
+// Every block re-adds the partials in the same order (so all agree bit for bit) and forms scale = min(1, clip / norm); -1
+// means that parameters and state stay as they are: a non-finite norm, or a device error left by any earlier kernel (a
+// bounded wait that gave up means some tile or partial sum of this update is garbage), which the status then names.
+template <int THREADS>
+__device__ __forceinline__ float clip_scale_of(const float* partials, int n_partials, float clip, uint32_t dev_err, DeviceStats* stats) {
+  __shared__ float sh[THREADS / 32];
+  __shared__ float s_scale;
+  float acc = 0.f;
+  for (int i = threadIdx.x; i < n_partials; i += THREADS) acc += partials[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float total = 0.f;
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) total += sh[w];
+    const float norm = sqrtf(total);
+    float scale = 1.f;
+    const bool ok = isfinite(norm) && dev_err == 0u;
+    if (ok && clip > 0.f && norm > clip) scale = clip / norm;
+    s_scale = ok ? scale : -1.f;
+    if (blockIdx.x == 0) {
+      stats->grad_norm = norm;
+      stats->clip_scale = ok ? scale : 0.f;
+      stats->status = ok ? PAAC_OK
+                         : ((dev_err & DEV_ERR_WAIT_MASK) ? PAAC_ERR_TIMEOUT
+                                                           : ((dev_err & DEV_ERR_RANGE) ? PAAC_ERR_RANGE : PAAC_ERR_NONFINITE));
+    }
+  }
+  __syncthreads();
+  return s_scale;
+}
+
+// pass 2: norm, clipping factor, RMSProp and the refreshed bf16 copy.
 // One wave of two blocks per SM, launched so that it may start while the finishing kernel drains: a thread's first
 // UPD_AHEAD groups of parameters and state (all of them, up to 1.8 M parameters) are fetched before the wait, the
 // gradients right after it, together with the partial sums of the norm.

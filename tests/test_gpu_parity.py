@@ -657,3 +657,50 @@ def test_small_batches_one_launch_rollout(orc, n_e, prec, A):
         check_update(orc, o, g, TOL[prec], inject=True)
     assert g.error_word() == 0
     g.close()
+
+
+@pytest.mark.parametrize("n_e,A", [(1, 2), (127, 19), (128, 30), (129, 18), (384, 31)])
+def test_fully_connected_column_tiles(orc, n_e, A):
+    """The fully connected forward kernel with each of its column tiles (64, 128 and 256), full and ragged row tiles, few and
+    many head outputs: one rollout against the oracle."""
+    cfg = dict(arch="nature", precision="bf16", n_e=n_e, t_max=1, n_actions=A, lr=0.01, term_denom=3)
+    o, g = make_pair(orc, cfg)
+    check_rollout(orc, o, g, TOL["bf16"])
+    assert g.error_word() == 0
+    g.close()
+
+
+@pytest.mark.parametrize("n_e", [3, 1027])
+def test_pulled_planes_match_whole_states(n_e):
+    """External-environment steps whose planes the stacking kernel reads from pinned memory, with restarts: values,
+    actions and parameters equal those of a learner that is sent whole states, over recorded and plain sequences."""
+    import torch
+    gen = torch.Generator().manual_seed(n_e)
+    hp = dict(lr=0.01, term_denom=50)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        a, b = (pb.Paac("nature", n_e, 2, 6, 3, precision=pb.BF16, **hp) for _ in range(2))
+    state = torch.randint(0, 256, (n_e, 84, 84, 4), dtype=torch.uint8, generator=gen).pin_memory()
+    planes = torch.empty(n_e, 84, 84, dtype=torch.uint8).pin_memory()
+    out = [torch.zeros(2, n_e, dtype=torch.int32).pin_memory() for _ in range(2)]
+    val = [torch.zeros(n_e).pin_memory() for _ in range(2)]
+    for it in range(5):
+        for t in range(3):
+            if t > 0:
+                planes.copy_(torch.randint(0, 256, planes.shape, dtype=torch.uint8, generator=gen))
+                restart = (torch.rand(n_e, generator=gen) < 0.1).to(torch.uint8)
+                nxt = torch.cat([state[..., 1:], planes[..., None]], dim=-1)
+                fresh = planes[..., None].expand(-1, -1, -1, 4)
+                state.copy_(torch.where(restart[:, None, None, None] != 0, fresh, nxt))
+            for i, g in enumerate((a, b)):
+                acts = out[i][t] if t < 2 else None
+                if t == 0 or i == 1:
+                    g.act_host(t, state, acts, val[i])
+                else:
+                    g.act_host_newest(t, planes, restart, acts, val[i])
+                if t < 2:
+                    g.observe_host(t, torch.zeros(n_e, dtype=torch.int8), torch.zeros(n_e, dtype=torch.uint8))
+            assert torch.equal(val[0], val[1]), (it, t)
+        assert torch.equal(out[0], out[1])
+        assert a.update()["status"] == 0 and b.update()["status"] == 0
+        assert np.array_equal(a.params(), b.params())
+    a.close(), b.close()
