@@ -33,7 +33,8 @@ static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_
 // backward on the larger network (TMAC/s, of 36 the multiply-add pipe could do; every shape ends near 20, at 75 % of the
 // issue slots): the wide shape (8 x 8 per lane for 64 columns, 8 x 4 below, where 8 x 8 leaves tiles of too many rows) wins
 // from two warps per scheduler on (1184 of them; 19.8 against 18.4), below that 4 x 4 (18.4 against 12.2 with one and a half),
-// and 2 x 4 where even that leaves a scheduler without a warp (592).
+// and 2 x 4 where even that leaves a scheduler without a warp (592).  4 x 4 with 64 columns comes in blocks of two warps: the
+// second layer's 10368 rows then fill the device in more even rounds (34 -> 30 us, the third layer's 6272 the same).
 constexpr int FF_SMS = 148;
 static size_t ff_heads_scratch_floats(const NetDims& nd, int n);
 static int ff_shape(int N, long long outputs) {              // outputs of all classes and splits
@@ -53,7 +54,7 @@ static void ff_launch(LaunchCtx& lc, int kid, int M, int n_cols, int K, int kps,
     else gemm_ffma<4, 2, 4, 4, 1, 64>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
   } else {
     if constexpr (SHAPE == 2) gemm_ffma<4, 8, 8, 4, 1, 16>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
-    else if constexpr (SHAPE == 1) gemm_ffma<4, 4, 4, 2, 2, 32>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
+    else if constexpr (SHAPE == 1) gemm_ffma<4, 4, 4, 1, 2, 32>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
     else gemm_ffma<4, 2, 4, 2, 2, 64>(lc, kid, M, n_cols, K, kps, classes, la, lb, ep);
   }
 }
