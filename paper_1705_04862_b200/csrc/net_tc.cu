@@ -2201,19 +2201,19 @@ static void tc_shift(LaunchCtx& lc, int kid, Cfg cfg, const bf16* w, Epi e, int 
   }
   const int tiles = (positions + TC_BM - 1) / TC_BM;
   // bulk-copied stages: the layer input as a matrix of 128-byte rows, fetched in boxes of one stage
-  static CUtensorMap no_map;
-  const CUtensorMap* tm_a = &no_map;
-  const CUtensorMap* tm_b = &no_map;
+  CUtensorMap map_a = {}, map_b = {};            // copies: the second look-up may give the cache slot of the first away
+  bool have = true;
+  auto take = [&](CUtensorMap& to, const CUtensorMap* from) { if (from == nullptr) have = false; else to = *from; };
   if constexpr (Cfg::BULK == 1) {
-    tm_a = tc_tensor_map(cfg.base_host(), (uint64_t)cfg.row_count(), 64, 64, Cfg::STAGE_ROWS);
+    take(map_a, tc_tensor_map(cfg.base_host(), (uint64_t)cfg.row_count(), 64, 64, Cfg::STAGE_ROWS));
   } else if constexpr (Cfg::BULK == 2) {
     // plane p: [states * 10][10 pairs][64], 2560 bytes from one oh to the next, starting 10 p pair rows in
-    tm_a = tc_tensor_map3(cfg.base_host(), 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10);
-    tm_b = tc_tensor_map3(cfg.base_host() + 10 * 64, 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10);
+    take(map_a, tc_tensor_map3(cfg.base_host(), 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10));
+    take(map_b, tc_tensor_map3(cfg.base_host() + 10 * 64, 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10));
   }
-  if (tm_a == nullptr || tm_b == nullptr) { lc.host_failure = true; return; }      // no tensor-map encoder
+  if (!have) { lc.host_failure = true; return; }      // no tensor-map encoder
   KernelScope scope(lc, kid);
-  launch_kernel_overlapped(lc, kern, tiles < sm_count() ? tiles : sm_count(), SH_THREADS, smem, *tm_a, *tm_b, cfg, w, e, tiles, err);
+  launch_kernel_overlapped(lc, kern, tiles < sm_count() ? tiles : sm_count(), SH_THREADS, smem, map_a, map_b, cfg, w, e, tiles, err);
 }
 
 template <class Cfg, class Epi, int STAGES>
@@ -2228,18 +2228,18 @@ static void tc_shift_t(LaunchCtx& lc, int kid, Cfg cfg, const bf16* w, Epi e, in
     configured = true;
   }
   const int tiles = (positions + ST_TILE - 1) / ST_TILE;
-  static CUtensorMap no_map;
-  const CUtensorMap* tm_a = &no_map;
-  const CUtensorMap* tm_b = &no_map;
+  CUtensorMap map_a = {}, map_b = {};            // copies: the second look-up may give the cache slot of the first away
+  bool have = true;
+  auto take = [&](CUtensorMap& to, const CUtensorMap* from) { if (from == nullptr) have = false; else to = *from; };
   if constexpr (Cfg::BULK == 1) {
-    tm_a = tc_tensor_map(cfg.base_host(), (uint64_t)cfg.row_count(), 64, 64, Cfg::STAGE_ROWS);
+    take(map_a, tc_tensor_map(cfg.base_host(), (uint64_t)cfg.row_count(), 64, 64, Cfg::STAGE_ROWS));
   } else if constexpr (Cfg::BULK == 2) {
-    tm_a = tc_tensor_map3(cfg.base_host(), 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10);
-    tm_b = tc_tensor_map3(cfg.base_host() + 10 * 64, 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10);
+    take(map_a, tc_tensor_map3(cfg.base_host(), 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10));
+    take(map_b, tc_tensor_map3(cfg.base_host() + 10 * 64, 10, (uint64_t)cfg.states * 10, 128, 2560, 10, Cfg::STAGE_ROWS / 10));
   }
-  if (tm_a == nullptr || tm_b == nullptr) { lc.host_failure = true; return; }      // no tensor-map encoder
+  if (!have) { lc.host_failure = true; return; }      // no tensor-map encoder
   KernelScope scope(lc, kid);
-  launch_kernel_overlapped(lc, kern, tiles < sm_count() ? tiles : sm_count(), ST_THREADS, smem, *tm_a, *tm_b, cfg, w, e, tiles, err);
+  launch_kernel_overlapped(lc, kern, tiles < sm_count() ? tiles : sm_count(), ST_THREADS, smem, map_a, map_b, cfg, w, e, tiles, err);
 }
 
 template <class G, class Epi>
