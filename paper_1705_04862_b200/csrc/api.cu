@@ -1,5 +1,6 @@
 // C boundary of the PAAC library: context, workspace carving, and the order in which the
 // kernels of one pass of Algorithm 1 are enqueued.
+#include <mutex>
 #include <new>
 #include <string.h>
 
@@ -18,6 +19,65 @@ struct HostBox {
   uint8_t* outcomes;                            // rewards and terminal flags, laid out as on the device (outcome_bytes())
 };
 
+// What a learner needs beside its own stream: a stream the weight gradients run on, next to the chain of data gradients
+// (see SideBranch), events to fork and join with, and a stream to record on when the learner's is the legacy default one
+// (nothing runs there).
+struct SideSet {
+  cudaStream_t st, record;
+  cudaEvent_t ev[MAX_LAYERS + 1];
+  bool complete() const { return st != nullptr; }
+  bool make() {
+    bool ok = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&record, cudaStreamNonBlocking) == cudaSuccess;
+    for (int i = 0; ok && i <= MAX_LAYERS; ++i) ok = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); destroy(); }
+    return ok;
+  }
+  void destroy() {
+    if (st) cudaStreamDestroy(st);
+    if (record) cudaStreamDestroy(record);
+    for (cudaEvent_t e : ev) if (e) cudaEventDestroy(e);
+    *this = SideSet{};
+  }
+};
+// Both kinds of helper cost some 100 us to make, more than a first iteration of a small learner; a destroyed learner's are
+// kept for the next one, at most POOL_MAX of each (idle by then: paac_destroy has waited for the learner's stream, which
+// every side branch joins).  Everything belongs to the one device of the process.
+struct HelperPool {
+  static constexpr int POOL_MAX = 4;
+  struct Box { HostBox* p; size_t bytes; };
+  std::mutex lock;
+  SideSet sides[POOL_MAX]; int n_sides = 0;
+  Box boxes[POOL_MAX]; int n_boxes = 0;
+  bool take(SideSet& out) {
+    std::lock_guard<std::mutex> g(lock);
+    if (n_sides == 0) return false;
+    out = sides[--n_sides];
+    return true;
+  }
+  void give(SideSet& s) {
+    {
+      std::lock_guard<std::mutex> g(lock);
+      if (n_sides < POOL_MAX) { sides[n_sides++] = s; s = SideSet{}; return; }
+    }
+    s.destroy();
+  }
+  bool take(size_t need, Box& out) {
+    std::lock_guard<std::mutex> g(lock);
+    for (int i = 0; i < n_boxes; ++i)
+      if (boxes[i].bytes >= need && boxes[i].bytes <= 4 * need) { out = boxes[i]; boxes[i] = boxes[--n_boxes]; return true; }
+    return false;
+  }
+  void give(Box b) {
+    {
+      std::lock_guard<std::mutex> g(lock);
+      if (n_boxes < POOL_MAX) { boxes[n_boxes++] = b; return; }
+    }
+    cudaFreeHost(b.p);
+  }
+};
+static HelperPool& helper_pool() { static HelperPool* p = new HelperPool; return *p; }      // never torn down: the driver may go first
+
 struct paac_ctx {
   int arch, n_e, t_max, A, prec, B;
   paac_hparams hp;
@@ -33,6 +93,7 @@ struct paac_ctx {
   uint64_t env_step;       // global step index of the environments (same for all)
   bool rollout_fresh;      // a rollout has completed since the last update
   uint8_t* newest;         // staging for paac_act_host_newest with pageable planes: [n_e][84][84]
+  size_t box_bytes;
   HostBox* box;            // pinned, device-visible: what host and device hand each other (made on first use)
   bool observed;           // outcomes of this rollout wait in the box for their copy to the device
   int host_t;              // external-environment mode: next expected step
@@ -46,9 +107,7 @@ struct paac_ctx {
   // second iteration (the two frame buffers alternate), so after two plain iterations each parity is captured
   // once into a CUDA graph and replayed from then on.  Anything that changes the sequence drops the graphs.
   bool graphs_on;          // option: allow recording
-  cudaStream_t side_st;    // weight gradients run here, next to the chain of data gradients (see SideBranch)
-  cudaEvent_t side_ev[MAX_LAYERS + 1];
-  cudaStream_t record_st;  // where sequences are recorded when st is the legacy default stream (made on first use)
+  SideSet side;            // made, or taken from the pool, on first use
   // recorded launch sequences: kind 0 = rollout, 1 = update, 2 = update that reports, 3 + 2 t + v = step t of the external-environment mode
   // (v = 1: with the frame stack built on the device), each for both parities of the frame buffers
   static constexpr int GRAPH_KINDS = 3 + 2 * 65;
@@ -245,10 +304,13 @@ size_t outcome_bytes(const paac_ctx* c) { return (size_t)((const char*)c->termin
 bool host_box(paac_ctx* c) {
   if (c->box) return true;
   const size_t n = c->n_e, head = (sizeof(HostBox) + 255) / 256 * 256;
-  void* p = nullptr;
-  if (cudaHostAlloc(&p, head + n * 9 + outcome_bytes(c), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+  HelperPool::Box found{nullptr, (head + n * 9 + outcome_bytes(c) + 4095) / 4096 * 4096};
+  if (!helper_pool().take(found.bytes, found) &&
+      cudaHostAlloc((void**)&found.p, found.bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
     cudaGetLastError(); return false;
   }
+  void* p = found.p;
+  c->box_bytes = found.bytes;
   c->box = new (p) HostBox{};
   char* q = (char*)p + head;
   c->box->actions = (int32_t*)q; c->box->values = (float*)(q + 4 * n);
@@ -276,6 +338,8 @@ int send_outcomes(paac_ctx* c) {
   return PAAC_ERR_CUDA;
 }
 
+bool side_set(paac_ctx* c) { return c->side.complete() || helper_pool().take(c->side) || c->side.make(); }
+
 void drop_graphs(paac_ctx* c) {
   for (int k = 0; k < paac_ctx::GRAPH_KINDS; ++k)
     for (int par = 0; par < 2; ++par) {
@@ -298,9 +362,7 @@ template <class F> void run_recorded(paac_ctx* c, int kind, int parity, F enqueu
     // The legacy default stream cannot be captured, but a graph can be launched into it: the sequence is recorded on a
     // stream of the context's own (nothing runs there).  Default-stream contexts replay like all others from then on.
     const bool legacy = c->st == nullptr || c->st == cudaStreamLegacy;
-    if (legacy && c->record_st == nullptr && cudaStreamCreateWithFlags(&c->record_st, cudaStreamNonBlocking) != cudaSuccess)
-      c->record_st = nullptr;
-    const cudaStream_t rec = legacy && c->record_st != nullptr ? c->record_st : c->st;
+    const cudaStream_t rec = legacy && side_set(c) ? c->side.record : c->st;
     if (cudaStreamBeginCapture(rec, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       const uint64_t before = c->lc.count;
       c->lc.serialize_next = true;
@@ -336,20 +398,16 @@ template <class F> void run_recorded(paac_ctx* c, int kind, int parity, F enqueu
 struct SideBranch {
   paac_ctx* c; cudaStream_t main; bool on, forked; int used;
   explicit SideBranch(paac_ctx* ctx) : c(ctx), main(ctx->lc.st), on(!ctx->lc.profiling), forked(false), used(0) {
-    if (on && !c->side_st) {
-      on = cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking) == cudaSuccess;
-      for (int i = 0; on && i <= MAX_LAYERS; ++i) on = cudaEventCreateWithFlags(&c->side_ev[i], cudaEventDisableTiming) == cudaSuccess;
-      if (!on) cudaGetLastError();
-    }
+    if (on) on = side_set(c);
   }
   // `enqueue` runs on the side stream, after everything the main one holds so far and after the side's own launches
   template <class F> void run(F enqueue) {
     if (!on || used >= MAX_LAYERS) { enqueue(); return; }
-    cudaEventRecord(c->side_ev[used], main);
-    cudaStreamWaitEvent(c->side_st, c->side_ev[used], 0);
+    cudaEventRecord(c->side.ev[used], main);
+    cudaStreamWaitEvent(c->side.st, c->side.ev[used], 0);
     ++used; forked = true;
     const bool keep = c->lc.serialize_next;
-    c->lc.st = c->side_st; c->lc.serialize_next = true;
+    c->lc.st = c->side.st; c->lc.serialize_next = true;
     enqueue();
     c->lc.st = main; c->lc.serialize_next = keep;
   }
@@ -357,14 +415,14 @@ struct SideBranch {
   template <class F> void append(F enqueue) {
     if (!forked) { enqueue(); return; }
     const bool keep = c->lc.serialize_next;
-    c->lc.st = c->side_st; c->lc.serialize_next = true;
+    c->lc.st = c->side.st; c->lc.serialize_next = true;
     enqueue();
     c->lc.st = main; c->lc.serialize_next = keep;
   }
   void join() {
     if (!forked) return;
-    cudaEventRecord(c->side_ev[MAX_LAYERS], c->side_st);
-    cudaStreamWaitEvent(main, c->side_ev[MAX_LAYERS], 0);
+    cudaEventRecord(c->side.ev[MAX_LAYERS], c->side.st);
+    cudaStreamWaitEvent(main, c->side.ev[MAX_LAYERS], 0);
     c->lc.serialize_next = true;
   }
 };
@@ -618,10 +676,8 @@ int paac_destroy(paac_ctx* c) {
   cudaStreamSynchronize(c->st);
   drop_graphs(c);
   c->lc.release();
-  if (c->box) cudaFreeHost(c->box);
-  if (c->side_st) cudaStreamDestroy(c->side_st);
-  for (cudaEvent_t e : c->side_ev) if (e) cudaEventDestroy(e);
-  if (c->record_st) cudaStreamDestroy(c->record_st);
+  if (c->box) helper_pool().give(HelperPool::Box{c->box, c->box_bytes});
+  if (c->side.complete()) helper_pool().give(c->side);
   if (c->owns_workspace) cudaFree(c->ws);
   cudaGetLastError();
   delete c;
