@@ -224,8 +224,10 @@ static void backward_layer_t(LaunchCtx& lc, int arch, const NetDims& nd, const T
   }
 }
 
-// Where layer l's partial sums start in the update's scratch (a region of its own for every layer, since they are kept
-// until finish_gradients() has run); l = number of layers: the heads' region; one more: the end.
+// Where layer l's partial sums start in the update's scratch; l = number of layers: the heads' region; one more: the end.
+// Every layer has a region of its own in both contractions: the CUDA-core one keeps its partial sums until
+// finish_gradients() has run, and the three-pass one, which adds each layer's up at once, may do so for one layer on the
+// side stream while the main stream works on another.  Both split alike, splits * (J + 1) * CO floats each.
 static size_t ff_scratch_offset(const NetDims& nd, int n, int l) {
   size_t off = 0;
   for (int q = 0; q < l && q <= nd.n_conv; ++q) {
@@ -239,7 +241,7 @@ static size_t ff_scratch_offset(const NetDims& nd, int n, int l) {
 void simt_backward_layer(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const float* theta, const bf16* theta16,
                          const uint8_t* frames, int n, void* const act[], void* const gact[], float* grad,
                          float* scratch, GradSegments* segs, int layer, bool wgrad, bool dgrad) {
-  float* sc = use_tc3(lc) ? scratch : scratch + ff_scratch_offset(nd, n, layer);
+  float* sc = scratch + ff_scratch_offset(nd, n, layer);
   if (prec == PAAC_BF16)
     backward_layer_t<bf16, bf16>(lc, arch, nd, theta16, frames, n, act, gact, grad, sc, segs, layer, wgrad, dgrad);
   else
@@ -254,18 +256,7 @@ int simt_forward(LaunchCtx& lc, int arch, int prec, const NetDims& nd, const flo
 
 size_t simt_scratch_floats(int arch, const NetDims& nd, int n, int n_fwd) {
   (void)arch;
-  // an update on the CUDA cores keeps all its partial sums; one through the three-pass kernel finishes layer by layer
-  size_t best = ff_scratch_offset(nd, n, nd.n_conv + 2);
-  for (int l = 0; l <= nd.n_conv; ++l) {
-    const LayerDims& d = nd.layer[l];
-    const int M = d.CO;
-    const int N = (l < nd.n_conv ? d.K * d.K * d.C : d.H * d.W * d.C) + 1;
-    const int K = n * d.OH * d.OW;
-    const size_t need = (size_t)pick_splits(M, N, K) * M * N;
-    if (need > best) best = need;
-  }
-  const size_t heads = (size_t)pick_splits(nd.A + 1, nd.F + 1, n) * (nd.A + 1) * (nd.F + 1);
-  if (heads > best) best = heads;
+  const size_t best = ff_scratch_offset(nd, n, nd.n_conv + 2);      // all of an update's partial sums
   // split-k partial sums of the fully connected layer's forward pass, which only ever sees n_fwd states at a time
   const LayerDims& f = nd.layer[nd.n_conv];
   const int IN = f.H * f.W * f.C;
@@ -376,10 +367,11 @@ static void heads_backward_t(LaunchCtx& lc, const NetDims& nd, const TW* w, cons
     gemm_tc3(lc, KID_HEADS_BWD, n, F, A + 1, 1, HeadGradOp{dz, dV, A}, HeadWeightOp<TW>{w + nd.pi_w, w + nd.v_w, F, A},
               ReluMaskEp<T>{gact_fc, h, F});
     const int splits = pick_splits(A + 1, F + 1, n);
+    float* part = scratch + ff_scratch_offset(nd, n, nd.n_conv + 1);
     gemm_tc3(lc, KID_HEADS_BWD, A + 1, F + 1, n, splits, HeadGradTOp{dz, dV, A}, ColMajorOnesOp<T>{h, F, F},
-              PartialEp{scratch, A + 1, F + 1});
-    reduce_wgrad(lc, scratch, splits, A + 1, 0, A, F, 1.f, grad + nd.pi_w, grad + nd.pi_b);
-    reduce_wgrad(lc, scratch, splits, A + 1, A, 1, F, 1.f, grad + nd.v_w, grad + nd.v_b);
+              PartialEp{part, A + 1, F + 1});
+    reduce_wgrad(lc, part, splits, A + 1, 0, A, F, 1.f, grad + nd.pi_w, grad + nd.pi_b);
+    reduce_wgrad(lc, part, splits, A + 1, A, 1, F, 1.f, grad + nd.v_w, grad + nd.v_b);
     return;
   }
   const int splits = pick_splits(A + 1, F + 1, n), rows_per = gemm_k_per_split(n, splits);

@@ -65,6 +65,29 @@ def test_float_configurations_on_the_tensor_cores(orc, index, updates):
     g.close()
 
 
+@pytest.mark.parametrize("arch,prec,n_e,options", [("nips", "fp32", 32, {}), ("nature", "fp32", 9, {}),
+                                                   ("nature", "bf16", 37, {pb.OPT_CUDA_CORES_ONLY: 1}),
+                                                   ("nature", "bf16", 37, {pb.OPT_TC_WGRAD_LAYERS: 0b1100})])
+def test_three_pass_update_is_the_same_beside_the_chain_and_in_line(arch, prec, n_e, options):
+    """With the three-pass contraction each layer's partial sums are added up as soon as they are there, some layers on the
+    side stream: the gradient has the same bits in every run, and those of a run that is timed kernel by kernel, which
+    keeps everything on one stream.  (Layers that shared their scratch would overwrite one another's sums.)"""
+    outs = []
+    for timed in (True, False, False, False):
+        g = pb.Paac(arch, n_e, 3, 6, seed=5, precision=pb.BF16 if prec == "bf16" else pb.FP32, lr=0.0224, term_denom=50)
+        g.set_option(pb.OPT_FP32_TENSOR_CORES, 1)
+        for option, value in options.items():
+            g.set_option(option, value)
+        g.profile(timed)
+        for _ in range(3):
+            g.rollout()
+            assert g.update()["status"] == 0
+        outs.append((g.debug_read(pb.DBG_GRAD).copy(), g.params()))
+        g.close()
+    for grad, theta in outs[1:]:
+        assert np.array_equal(grad, outs[0][0]) and np.array_equal(theta, outs[0][1])
+
+
 def test_float_tensor_core_option_on_the_nature_network(orc):
     """The three-pass kernel with bf16 storage and the larger network (CUDA-core-only mode routed through it): ragged
     batch, several tiles in every dimension; compared with the CUDA-core contractions on the same rollout."""
