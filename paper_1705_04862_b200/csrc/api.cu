@@ -1,9 +1,12 @@
 // C boundary of the PAAC library: context, workspace carving, and the order in which the
 // kernels of one pass of Algorithm 1 are enqueued.
+#include <cuda.h>
+
 #include <mutex>
 #include <new>
 #include <string.h>
 
+#include "host_view.h"
 #include "kernels.h"
 
 using namespace paac;
@@ -785,11 +788,26 @@ int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, f
   return act_host_finish(c, t, nullptr, dst, actions, values);
 }
 
-// the device's view of pinned host memory, nullptr for anything else
-static const uint8_t* pinned_view(const uint8_t* p) {
-  cudaPointerAttributes a{};
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-  return a.type == cudaMemoryTypeHost ? (const uint8_t*)a.devicePointer : nullptr;
+// what the driver knows of a host address (its entry point is looked up at run time: nothing links to libcuda)
+static bool query_host_range(const uint8_t* p, HostRange& r) {
+  typedef CUresult (*Attributes)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Attributes attributes = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError(); fn = nullptr;
+    }
+    return (Attributes)fn;
+  }();
+  unsigned type = 0, managed = 0;
+  CUdeviceptr device = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute which[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* where[] = {&type, &managed, &device, &start, &size};
+  if (attributes == nullptr || attributes(5, which, where, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return false;
+  r = HostRange{type == CU_MEMORYTYPE_HOST && !managed, (uintptr_t)device, (uintptr_t)start, size};
+  return true;
 }
 
 int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_t* restart, int32_t* actions, float* values) {
@@ -800,9 +818,9 @@ int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES, plane = (size_t)c->n_e * FRAME_H * FRAME_W;
   const uint8_t* prev = c->frames[c->cur] + (size_t)(t - 1) * fstep;
   uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
-  // Pinned planes (16-byte aligned) are read over the link by the kernel that builds the states, which saves the copy's
+  // Pinned planes (16-byte aligned, all of them in one allocation) are read over the link by the kernel that builds the states, which saves the copy's
   // set-up, its hand-over to the first kernel and a round trip through device memory; others are copied first.
-  const uint8_t* view = ((uintptr_t)newest & 15u) == 0 ? pinned_view(newest) : nullptr;
+  const uint8_t* view = ((uintptr_t)newest & 15u) == 0 ? host_view(newest, plane, query_host_range) : nullptr;
   c->box->planes.newest = view ? view : c->newest;
   c->box->planes.restart = restart ? c->box->restart : nullptr;
   if (restart) memcpy(c->box->restart, restart, c->n_e);

@@ -3,6 +3,9 @@ declares, sizes workspaces, validates arguments, and refuses to run without a de
 import ctypes as C
 import os
 import re
+import subprocess
+
+import pytest
 
 from paper_1705_04862_b200 import binding as pb
 from paper_1705_04862_b200 import build as pbuild
@@ -71,3 +74,41 @@ def test_init_fails_loudly_without_a_gpu():
     hp = pb.default_hparams()
     assert L.paac_init(C.byref(h), pb.ARCH_NIPS, 4, 5, 4, C.byref(hp), 1) == pb.ERR_CUDA
     assert not h.value
+
+
+HOST_VIEW = """
+#include "host_view.h"
+// ranges: start, size, device address of the start, pinned -- four numbers each
+extern "C" uintptr_t view(uintptr_t p, size_t bytes, const uint64_t* ranges, int n) {
+  return (uintptr_t)paac::host_view((const uint8_t*)p, bytes, [&](const uint8_t* at, paac::HostRange& r) {
+    for (int i = 0; i < n; ++i, ranges += 4)
+      if ((uintptr_t)at - ranges[0] < ranges[1]) {
+        r = paac::HostRange{ranges[3] != 0, (uintptr_t)at - ranges[0] + ranges[2], ranges[2], (size_t)ranges[1]};
+        return true;
+      }
+    return false;
+  });
+}
+"""
+
+
+@pytest.mark.parametrize("p,size,ranges,readable", [
+    (0x1000, 0x1000, [(0x1000, 0x1000, 0x1000, 1)], True),                               # the whole allocation
+    (0x1010, 0xFF0, [(0x1000, 0x1000, 0x1000, 1)], True),                                # up to its last byte
+    (0x1010, 0xFF1, [(0x1000, 0x1000, 0x1000, 1)], False),                               # one byte further
+    (0x1000, 0x3000, [(0x1000, 0x1000, 0x1000, 1)], False),                              # a registered piece of a larger array
+    (0x1000, 0x3000, [(0x1000, 0x1000, 0x1000, 1), (0x3000, 0x1000, 0x3000, 1)], False),   # both ends, not the middle
+    (0x1000, 0x2000, [(0x1000, 0x1000, 0x1000, 1), (0x2000, 0x1000, 0x2000, 1)], False),   # two allocations side by side
+    (0x1000, 16, [], False),                                                            # nothing known
+    (0x1000, 16, [(0x1000, 0x1000, 0x1000, 0)], False),                                  # known, not pinned
+    (0x1000, 16, [(0x1000, 0x1000, 0x9000, 1)], False),                                  # seen elsewhere by the device
+    (0x1000, 2 ** 64 - 1, [(0x1000, 0x1000, 0x1000, 1)], False),                         # a length that wraps around
+])
+def test_host_buffers_are_read_in_place_only_where_all_of_them_is_pinned(tmp_path, p, size, ranges, readable):
+    src, so = tmp_path / "view.cpp", tmp_path / "view.so"
+    src.write_text(HOST_VIEW)
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_1705_04862_b200", "csrc"), str(src), "-o", str(so)], check=True)
+    view = C.CDLL(str(so)).view
+    view.argtypes, view.restype = [C.c_uint64, C.c_size_t, C.POINTER(C.c_uint64), C.c_int], C.c_uint64
+    flat = [x for r in ranges for x in r] or [0]
+    assert view(p, size, (C.c_uint64 * len(flat))(*flat), len(ranges)) == (p if readable else 0)

@@ -727,3 +727,36 @@ def test_pulled_planes_match_whole_states(n_e):
         assert a.update()["status"] == 0 and b.update()["status"] == 0
         assert np.array_equal(a.params(), b.params())
     a.close(), b.close()
+
+
+@pytest.mark.parametrize("kind,offset", [("pinned", 0), ("pinned", 4096), ("pinned", 4), ("pageable", 0), ("registered", 0), ("registered", 8192)])
+def test_planes_from_any_host_memory(kind, offset):
+    """Planes at the start, in the middle and at the very end of a pinned allocation or a registered piece of an array, at an
+    address the kernel cannot read in place, and in ordinary memory: the state built from them is the same."""
+    import torch
+    n_e, rng = 7, np.random.RandomState(3)
+    size = n_e * 84 * 84
+    room = torch.zeros(offset + size + 8192, dtype=torch.uint8)
+    base = (-room.data_ptr()) % 4096                                  # registration works on whole pages
+    pages = (offset + size + 4095) // 4096 * 4096
+    if kind == "pinned":
+        room = room[:offset + size].pin_memory()                      # the planes end where the buffer does
+        base = 0
+    elif kind == "registered":
+        room = torch.zeros(base + pages + 8192, dtype=torch.uint8)
+        base = (-room.data_ptr()) % 4096
+        assert int(torch.cuda.cudart().cudaHostRegister(room.data_ptr() + base, pages, 0)) == 0
+    planes = room[base + offset:base + offset + size].view(n_e, 84, 84)
+    want = rng.randint(0, 256, (n_e, 84, 84), dtype=np.uint8)
+    planes.copy_(torch.from_numpy(want))
+    state = rng.randint(0, 256, (n_e, 84, 84, 4), dtype=np.uint8)
+    g = pb.Paac("nips", n_e, 1, 4, seed=2)
+    a = np.zeros(n_e, np.int32)
+    g.act_host(0, state, a)
+    g.observe_host(0, np.zeros(n_e, np.int8), np.zeros(n_e, np.uint8))
+    g.act_host_newest(1, planes)
+    got = g.debug_read(pb.DBG_NEXT_FRAMES).reshape(n_e, 84, 84, 4)
+    assert np.array_equal(got[..., :3], state[..., 1:]) and np.array_equal(got[..., 3], want)
+    g.close()
+    if kind == "registered":
+        assert int(torch.cuda.cudart().cudaHostUnregister(room.data_ptr() + base)) == 0
