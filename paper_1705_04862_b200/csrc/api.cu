@@ -19,7 +19,8 @@ struct HostBox {
   HostPlanes planes;                            // the newest frames and the restart flags of the step in flight
   DeviceStats stats;
   int32_t* actions; float* values; uint8_t* restart;      // [n_e] each, behind this struct
-  uint8_t* outcomes;                            // rewards and terminal flags, laid out as on the device (outcome_bytes())
+  uint8_t* outcomes;                            // rewards and terminal flags, laid out as on the device (outcome_bytes());
+                                                // only the steps in paac_ctx::observed hold anything
 };
 
 // What a learner needs beside its own stream: a stream the weight gradients run on, next to the chain of data gradients
@@ -98,7 +99,7 @@ struct paac_ctx {
   uint8_t* newest;         // staging for paac_act_host_newest with pageable planes: [n_e][84][84]
   size_t box_bytes;
   HostBox* box;            // pinned, device-visible: what host and device hand each other (made on first use)
-  bool observed;           // outcomes of this rollout wait in the box for their copy to the device
+  uint64_t observed;       // bit t: step t's outcomes wait in the box for their copy to the device (t_max is at most 64)
   int host_t;              // external-environment mode: next expected step
   int update_chunks;       // > 1: conv2 data gradient and conv1 weight gradient alternate over this many groups of states
   bool host_next_valid;    // the bootstrap state of the last host-mode rollout sits where step 0 of the next one goes
@@ -332,13 +333,29 @@ bool await_box(paac_ctx* c) {
   __atomic_thread_fence(__ATOMIC_ACQUIRE);
   return true;
 }
-// the rollout's outcomes, gathered by paac_observe_host, to the device in one copy
+// The outcomes gathered by paac_observe_host, to the device: in one copy where the whole rollout was observed, else run by
+// run of observed steps, so that a step nobody observed keeps what the device holds for it.
 int send_outcomes(paac_ctx* c) {
-  if (!c->observed) return PAAC_OK;
-  c->observed = false;
-  if (cudaMemcpyAsync(c->rewards, c->box->outcomes, outcome_bytes(c), cudaMemcpyHostToDevice, c->st) == cudaSuccess) return PAAC_OK;
-  cudaGetLastError();
-  return PAAC_ERR_CUDA;
+  const uint64_t steps = c->observed, all = ~0ull >> (64 - c->t_max);
+  c->observed = 0;
+  const size_t to_terminals = outcome_bytes(c) - c->B;
+  auto send = [&](void* dst, size_t at, size_t bytes) {
+    return cudaMemcpyAsync(dst, c->box->outcomes + at, bytes, cudaMemcpyHostToDevice, c->st) == cudaSuccess;
+  };
+  bool ok = true;
+  if (steps == all) {
+    ok = send(c->rewards, 0, outcome_bytes(c));
+  } else {
+    for (int t = 0; t < c->t_max && ok; ++t) {
+      if (!(steps >> t & 1)) continue;
+      const size_t row = (size_t)t * c->n_e;
+      while (t + 1 < c->t_max && steps >> (t + 1) & 1) ++t;
+      const size_t bytes = (size_t)(t + 1) * c->n_e - row;
+      ok = send(c->rewards + row, row, bytes) && send(c->terminals + row, to_terminals + row, bytes);
+    }
+  }
+  if (!ok) cudaGetLastError();
+  return ok ? PAAC_OK : PAAC_ERR_CUDA;
 }
 
 bool side_set(paac_ctx* c) { return c->side.complete() || helper_pool().take(c->side) || c->side.make(); }
@@ -839,7 +856,7 @@ int paac_observe_host(paac_ctx* c, int t, const int8_t* rewards, const uint8_t* 
   const size_t row = (size_t)t * c->n_e;
   memcpy(c->box->outcomes + row, rewards, c->n_e);
   memcpy(c->box->outcomes + (outcome_bytes(c) - c->B) + row, terminals, c->n_e);
-  c->observed = true;
+  c->observed |= 1ull << t;
   return PAAC_OK;
 }
 

@@ -760,3 +760,39 @@ def test_planes_from_any_host_memory(kind, offset):
     g.close()
     if kind == "registered":
         assert int(torch.cuda.cudart().cudaHostUnregister(room.data_ptr() + base)) == 0
+
+
+@pytest.mark.parametrize("t_max", [3, 64])
+def test_steps_that_were_not_observed_keep_what_the_learner_has(t_max):
+    """Nothing obliges the host to report a step's outcome.  Such a step has the rewards and terminals the learner's own
+    buffers hold -- zeros in a new learner, whatever one before it in the process was told -- and what is written into them
+    in the middle of a rollout stays for the steps not observed afterwards."""
+    n_e, frames = 3, np.zeros((3, 84, 84, 4), np.uint8)
+    a, ones = np.zeros(n_e, np.int32), np.ones(n_e, np.uint8)
+
+    def rollout(g, observe, at=None, write=None):
+        for t in range(t_max + 1):
+            g.act_host(t, frames, a)
+            if t in observe:
+                g.observe_host(t, observe[t].astype(np.int8), ones)
+            if t == at:
+                g.debug_write(pb.DBG_REWARDS, write)
+        return g.debug_read(pb.DBG_REWARDS).reshape(t_max, n_e), g.debug_read(pb.DBG_TERMINALS).reshape(t_max, n_e)
+
+    g = pb.Paac("nips", n_e, t_max, 4, seed=2)
+    rewards, terminals = rollout(g, {t: ones for t in range(t_max)})
+    assert rewards.all() and terminals.all()
+    g.close()
+    g = pb.Paac("nips", n_e, t_max, 4, seed=2)
+    want = np.zeros((t_max, n_e), np.int8)
+    rewards, terminals = rollout(g, {1: -ones})
+    want[1] = -1
+    assert np.array_equal(rewards, want) and np.array_equal(terminals, want != 0)
+    rewards, terminals = rollout(g, {0: ones, t_max - 1: ones}, at=1, write=np.full((t_max, n_e), -1, np.int8))
+    want[:] = -1                                    # step 0 was observed before the write
+    want[t_max - 1] = 1
+    assert np.array_equal(rewards, want)
+    assert np.array_equal(np.nonzero(terminals.all(1))[0], sorted({0, 1, t_max - 1})) and terminals.sum() == n_e * len({0, 1, t_max - 1})
+    rewards, _ = rollout(g, {t: ones for t in range(t_max)})
+    assert (rewards == 1).all()
+    g.close()
