@@ -2,7 +2,6 @@
 // kernels of one pass of Algorithm 1 are enqueued.
 #include <cuda.h>
 
-#include <mutex>
 #include <new>
 #include <string.h>
 
@@ -23,19 +22,18 @@ struct HostBox {
                                                 // only the steps in paac_ctx::observed hold anything
 };
 
-// What a learner needs beside its own stream: a stream the weight gradients run on, next to the chain of data gradients
-// (see SideBranch), events to fork and join with, and a stream to record on when the learner's is the legacy default one
-// (nothing runs there).
+// What a learner needs beside its own stream, made with it: a stream the weight gradients run on, next to the chain of data
+// gradients (see SideBranch), events to fork and join with, and, where the learner's stream is the legacy default one, a
+// stream to record on (nothing runs there).
 struct SideSet {
   cudaStream_t st, record;
   cudaEvent_t ev[MAX_LAYERS + 1];
   bool complete() const { return st != nullptr; }
-  bool make() {
+  void make(bool recorder) {
     bool ok = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&record, cudaStreamNonBlocking) == cudaSuccess;
+              (!recorder || cudaStreamCreateWithFlags(&record, cudaStreamNonBlocking) == cudaSuccess);
     for (int i = 0; ok && i <= MAX_LAYERS; ++i) ok = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) { cudaGetLastError(); destroy(); }
-    return ok;
   }
   void destroy() {
     if (st) cudaStreamDestroy(st);
@@ -44,43 +42,6 @@ struct SideSet {
     *this = SideSet{};
   }
 };
-// Both kinds of helper cost some 100 us to make, more than a first iteration of a small learner; a destroyed learner's are
-// kept for the next one, at most POOL_MAX of each (idle by then: paac_destroy has waited for the learner's stream, which
-// every side branch joins).  Everything belongs to the one device of the process.
-struct HelperPool {
-  static constexpr int POOL_MAX = 4;
-  struct Box { HostBox* p; size_t bytes; };
-  std::mutex lock;
-  SideSet sides[POOL_MAX]; int n_sides = 0;
-  Box boxes[POOL_MAX]; int n_boxes = 0;
-  bool take(SideSet& out) {
-    std::lock_guard<std::mutex> g(lock);
-    if (n_sides == 0) return false;
-    out = sides[--n_sides];
-    return true;
-  }
-  void give(SideSet& s) {
-    {
-      std::lock_guard<std::mutex> g(lock);
-      if (n_sides < POOL_MAX) { sides[n_sides++] = s; s = SideSet{}; return; }
-    }
-    s.destroy();
-  }
-  bool take(size_t need, Box& out) {
-    std::lock_guard<std::mutex> g(lock);
-    for (int i = 0; i < n_boxes; ++i)
-      if (boxes[i].bytes >= need && boxes[i].bytes <= 4 * need) { out = boxes[i]; boxes[i] = boxes[--n_boxes]; return true; }
-    return false;
-  }
-  void give(Box b) {
-    {
-      std::lock_guard<std::mutex> g(lock);
-      if (n_boxes < POOL_MAX) { boxes[n_boxes++] = b; return; }
-    }
-    cudaFreeHost(b.p);
-  }
-};
-static HelperPool& helper_pool() { static HelperPool* p = new HelperPool; return *p; }      // never torn down: the driver may go first
 
 struct paac_ctx {
   int arch, n_e, t_max, A, prec, B;
@@ -97,8 +58,7 @@ struct paac_ctx {
   uint64_t env_step;       // global step index of the environments (same for all)
   bool rollout_fresh;      // a rollout has completed since the last update
   uint8_t* newest;         // staging for paac_act_host_newest with pageable planes: [n_e][84][84]
-  size_t box_bytes;
-  HostBox* box;            // pinned, device-visible: what host and device hand each other (made on first use)
+  HostBox* box;            // pinned, device-visible: what host and device hand each other (nullptr: it could not be had)
   uint64_t observed;       // bit t: step t's outcomes wait in the box for their copy to the device (t_max is at most 64)
   int host_t;              // external-environment mode: next expected step
   int update_chunks;       // > 1: conv2 data gradient and conv1 weight gradient alternate over this many groups of states
@@ -111,7 +71,7 @@ struct paac_ctx {
   // second iteration (the two frame buffers alternate), so after two plain iterations each parity is captured
   // once into a CUDA graph and replayed from then on.  Anything that changes the sequence drops the graphs.
   bool graphs_on;          // option: allow recording
-  SideSet side;            // made, or taken from the pool, on first use
+  SideSet side;            // incomplete if it could not be had: everything then stays on the learner's stream
   // recorded launch sequences: kind 0 = rollout, 1 = update, 2 = update that reports, 3 + 2 t + v = step t of the external-environment mode
   // (v = 1: with the frame stack built on the device), each for both parities of the frame buffers
   static constexpr int GRAPH_KINDS = 3 + 2 * 65;
@@ -305,21 +265,14 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
 }
 
 size_t outcome_bytes(const paac_ctx* c) { return (size_t)((const char*)c->terminals - (const char*)c->rewards) + c->B; }
-bool host_box(paac_ctx* c) {
-  if (c->box) return true;
+void make_box(paac_ctx* c) {
   const size_t n = c->n_e, head = (sizeof(HostBox) + 255) / 256 * 256;
-  HelperPool::Box found{nullptr, (head + n * 9 + outcome_bytes(c) + 4095) / 4096 * 4096};
-  if (!helper_pool().take(found.bytes, found) &&
-      cudaHostAlloc((void**)&found.p, found.bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-    cudaGetLastError(); return false;
-  }
-  void* p = found.p;
-  c->box_bytes = found.bytes;
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, head + n * 9 + outcome_bytes(c), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return; }
   c->box = new (p) HostBox{};
   char* q = (char*)p + head;
   c->box->actions = (int32_t*)q; c->box->values = (float*)(q + 4 * n);
   c->box->restart = (uint8_t*)(q + 8 * n); c->box->outcomes = (uint8_t*)(q + 9 * n);
-  return true;
 }
 // Waits for the flag that the last kernel of a launch sequence sets; a failed launch or kernel shows in the stream's
 // status instead.
@@ -358,8 +311,6 @@ int send_outcomes(paac_ctx* c) {
   return ok ? PAAC_OK : PAAC_ERR_CUDA;
 }
 
-bool side_set(paac_ctx* c) { return c->side.complete() || helper_pool().take(c->side) || c->side.make(); }
-
 void drop_graphs(paac_ctx* c) {
   for (int k = 0; k < paac_ctx::GRAPH_KINDS; ++k)
     for (int par = 0; par < 2; ++par) {
@@ -367,6 +318,8 @@ void drop_graphs(paac_ctx* c) {
       c->plain_calls[k][par] = 0;
     }
 }
+
+bool legacy_stream(const paac_ctx* c) { return c->st == nullptr || c->st == cudaStreamLegacy; }
 
 // Runs `enqueue` (which only launches kernels on c->st) either directly, or -- once this kind/parity has run
 // directly before -- records it into a graph and replays the graph.
@@ -381,8 +334,7 @@ template <class F> void run_recorded(paac_ctx* c, int kind, int parity, F enqueu
     cudaGraph_t g = nullptr;
     // The legacy default stream cannot be captured, but a graph can be launched into it: the sequence is recorded on a
     // stream of the context's own (nothing runs there).  Default-stream contexts replay like all others from then on.
-    const bool legacy = c->st == nullptr || c->st == cudaStreamLegacy;
-    const cudaStream_t rec = legacy && side_set(c) ? c->side.record : c->st;
+    const cudaStream_t rec = legacy_stream(c) && c->side.complete() ? c->side.record : c->st;
     if (cudaStreamBeginCapture(rec, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       const uint64_t before = c->lc.count;
       c->lc.serialize_next = true;
@@ -414,12 +366,10 @@ template <class F> void run_recorded(paac_ctx* c, int kind, int parity, F enqueu
 }
 
 // A second stream beside the context's, for launches that nothing on the main one waits for until the join.  Off (all
-// launches stay on the main stream) while kernels are being timed one by one, or if the stream cannot be had.
+// launches stay on the main stream) while kernels are being timed one by one, or if the stream could not be had.
 struct SideBranch {
   paac_ctx* c; cudaStream_t main; bool on, forked; int used;
-  explicit SideBranch(paac_ctx* ctx) : c(ctx), main(ctx->lc.st), on(!ctx->lc.profiling), forked(false), used(0) {
-    if (on) on = side_set(c);
-  }
+  explicit SideBranch(paac_ctx* ctx) : c(ctx), main(ctx->lc.st), on(!ctx->lc.profiling && ctx->side.complete()), forked(false), used(0) {}
   // `enqueue` runs on the side stream, after everything the main one holds so far and after the side's own launches
   template <class F> void run(F enqueue) {
     if (!on || used >= MAX_LAYERS) { enqueue(); return; }
@@ -446,6 +396,15 @@ struct SideBranch {
     c->lc.serialize_next = true;
   }
 };
+
+// what paac_init made
+void release(paac_ctx* c) {
+  if (c->box) cudaFreeHost(c->box);
+  c->side.destroy();
+  if (c->owns_workspace) cudaFree(c->ws);
+  cudaGetLastError();
+  delete c;
+}
 
 }  // namespace
 
@@ -501,9 +460,12 @@ int paac_init(paac_ctx** out, int arch, int n_e, int t_max, int n_actions, const
   c->cur = 1;   // the first rollout flips to buffer 0; its start states are written there now
   launch_env_step(c->lc, seed, n_e, c->step_dev, 0u, nullptr, hp->term_denom, c->frames[0], nullptr, nullptr, nullptr,
                   pattern_actions(c));
-  if (cudaStreamSynchronize(c->st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
-    if (c->owns_workspace) cudaFree(c->ws);
-    delete c;
+  const bool launched = cudaGetLastError() == cudaSuccess;
+  // host work of some 100 us (50 to 60 per stream) while the device clears the workspace and writes the start states
+  make_box(c);
+  c->side.make(legacy_stream(c));
+  if (cudaStreamSynchronize(c->st) != cudaSuccess || cudaGetLastError() != cudaSuccess || !launched) {
+    release(c);
     return PAAC_ERR_CUDA;
   }
   *out = c;
@@ -555,7 +517,7 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
 int paac_update(paac_ctx* c, paac_update_stats* stats) {
   if (!c) return PAAC_ERR_ARG;
   if (!c->rollout_fresh) return PAAC_ERR_STATE;
-  if (stats && !host_box(c)) return PAAC_ERR_CUDA;
+  if (stats && !c->box) return PAAC_ERR_CUDA;
   if (stats) c->box->done = 0u;
   const paac_hparams& hp = c->hp;
   run_recorded(c, stats ? 2 : 1, c->cur, [&]() {
@@ -696,11 +658,7 @@ int paac_destroy(paac_ctx* c) {
   cudaStreamSynchronize(c->st);
   drop_graphs(c);
   c->lc.release();
-  if (c->box) helper_pool().give(HelperPool::Box{c->box, c->box_bytes});
-  if (c->side.complete()) helper_pool().give(c->side);
-  if (c->owns_workspace) cudaFree(c->ws);
-  cudaGetLastError();
-  delete c;
+  release(c);
   return PAAC_OK;
 }
 
@@ -794,7 +752,7 @@ int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, f
   if (t != c->host_t) return PAAC_ERR_STATE;
   // s_0 of a rollout is s_{t_max} of the one before (Algorithm 1): those frames are on the device already
   if (!frames && !(t == 0 && c->host_next_valid)) return PAAC_ERR_ARG;
-  if (!host_box(c)) return PAAC_ERR_CUDA;
+  if (!c->box) return PAAC_ERR_CUDA;
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
   if (t == 0) c->cur ^= 1;
   uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
@@ -831,7 +789,7 @@ int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_
   if (c) c->lc.serialize_next = true;
   if (!c || !newest || t < 1 || t > c->t_max || (t < c->t_max && !actions)) return PAAC_ERR_ARG;
   if (t != c->host_t) return PAAC_ERR_STATE;
-  if (!host_box(c)) return PAAC_ERR_CUDA;
+  if (!c->box) return PAAC_ERR_CUDA;
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES, plane = (size_t)c->n_e * FRAME_H * FRAME_W;
   const uint8_t* prev = c->frames[c->cur] + (size_t)(t - 1) * fstep;
   uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
@@ -852,7 +810,7 @@ int paac_observe_host(paac_ctx* c, int t, const int8_t* rewards, const uint8_t* 
   if (c) c->lc.serialize_next = true;
   if (!c || !rewards || !terminals || t < 0 || t >= c->t_max) return PAAC_ERR_ARG;
   if (t + 1 != c->host_t) return PAAC_ERR_STATE;
-  if (!host_box(c)) return PAAC_ERR_CUDA;
+  if (!c->box) return PAAC_ERR_CUDA;
   const size_t row = (size_t)t * c->n_e;
   memcpy(c->box->outcomes + row, rewards, c->n_e);
   memcpy(c->box->outcomes + (outcome_bytes(c) - c->B) + row, terminals, c->n_e);

@@ -796,3 +796,26 @@ def test_steps_that_were_not_observed_keep_what_the_learner_has(t_max):
     rewards, _ = rollout(g, {t: ones for t in range(t_max)})
     assert (rewards == 1).all()
     g.close()
+
+
+def test_destroyed_learners_leave_nothing_behind():
+    """Learners that own their workspace, created, used in both modes and destroyed again and again: device memory and the
+    process's memory (pinned memory among it) end where they were after the first few."""
+    import ctypes as C
+    import torch
+
+    def resident():
+        return int(open("/proc/self/statm").read().split()[1]) * 4096
+
+    n_e, L, hp = 2048, pb.lib(), pb.default_hparams()
+    frames, a = np.zeros((n_e, 84, 84, 4), np.uint8), np.zeros(n_e, np.int32)
+    seen = []
+    for _ in range(24):
+        h = C.c_void_p()
+        assert L.paac_init(C.byref(h), pb.ARCH_NIPS, n_e, 1, 4, C.byref(hp), 1) == pb.OK
+        assert L.paac_rollout(h, None) == pb.OK and L.paac_update(h, C.byref(pb.UpdateStats())) == pb.OK
+        assert L.paac_act_host(h, 0, frames.ctypes.data, a.ctypes.data, None) == pb.OK
+        assert L.paac_destroy(h) == pb.OK
+        seen.append((torch.cuda.mem_get_info()[0], resident()))
+    assert seen[-1][0] >= seen[7][0] - (4 << 20)
+    assert seen[-1][1] <= seen[7][1] + (4 << 20)
