@@ -7,9 +7,8 @@
 // file therefore carries that scratch itself, as a file-scope __device__ array that is part of the loaded
 // module: every GPU that loads the library holds these 16 KB until the process exits, and no call here
 // allocates or frees anything, on the device or through a library.
-#include <mutex>
-
 #include "common.cuh"
+#include "per_device.h"
 
 namespace {
 
@@ -17,7 +16,6 @@ constexpr int NA_SLICE = 4096;                        // parameters per partial 
 constexpr int NA_MAX_SLICES = 4096;                   // capacity of the static scratch
 constexpr size_t NA_MAX_PARAMS = (size_t)NA_SLICE * NA_MAX_SLICES;   // 16,777,216
 constexpr int NA_THREADS = 256;
-constexpr int NA_MAX_DEVICES = 64;
 
 // One partial sum per block of the first launch.  Shared by every call on the device and never cleared: each call overwrites
 // the entries it will read before reading them, so stale contents are harmless, but two calls that overlap
@@ -26,19 +24,20 @@ static __device__ __align__(256) float g_noalloc_partials[NA_MAX_SLICES];
 
 // In host code the array's name is only a handle for the runtime; the device address has to be asked for,
 // once per device, with that device current.
-std::mutex g_setup_mutex;
-float* g_partials_addr[NA_MAX_DEVICES] = {};
+paac::PerDevice<float*> g_partials_addr;
 
 int partials_for_current_device(float** out) {
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NA_MAX_DEVICES) { cudaGetLastError(); return PAAC_ERR_CUDA; }
-  std::lock_guard<std::mutex> lock(g_setup_mutex);
-  if (g_partials_addr[dev] == nullptr) {
-    void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_noalloc_partials) != cudaSuccess || p == nullptr) { cudaGetLastError(); return PAAC_ERR_CUDA; }
-    g_partials_addr[dev] = static_cast<float*>(p);
-  }
-  *out = g_partials_addr[dev];
+  float* const* p = nullptr;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    p = g_partials_addr.get(dev, [](float*& at) {
+      void* found = nullptr;
+      if (cudaGetSymbolAddress(&found, g_noalloc_partials) != cudaSuccess) return false;
+      at = static_cast<float*>(found);
+      return at != nullptr;
+    });
+  if (p == nullptr) { cudaGetLastError(); return PAAC_ERR_CUDA; }
+  *out = *p;
   return PAAC_OK;
 }
 

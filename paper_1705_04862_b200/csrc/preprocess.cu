@@ -2,6 +2,7 @@
 // 210 x 160 -> 84 x 84, newest channel of the four-frame state.  Integer arithmetic throughout.
 #include "common.cuh"
 #include "kernels.h"
+#include "per_device.h"
 
 namespace paac {
 
@@ -253,8 +254,13 @@ extern "C" int paac_preprocess(const uint8_t* raw_prev, const uint8_t* raw_last,
   if (!raw_prev || !raw_last || !state_out || n < 1 || n > 65535) return PAAC_ERR_ARG;
   if (((uintptr_t)raw_prev | (uintptr_t)raw_last) & 15u) return PAAC_ERR_ARG;
   if (((uintptr_t)state_out | (uintptr_t)state_in) & 3u) return PAAC_ERR_ARG;
-  static const cudaError_t attr = cudaFuncSetAttribute(preprocess_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PpShared));
-  if (attr != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
+  // a function's attributes belong to the current device, and this entry point works on any
+  static PerDevice<bool> ready;
+  int device = -1;
+  const bool ok = cudaGetDevice(&device) == cudaSuccess && ready.get(device, [](bool&) {
+    return cudaFuncSetAttribute(preprocess_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PpShared)) == cudaSuccess;
+  }) != nullptr;
+  if (!ok) { cudaGetLastError(); return PAAC_ERR_CUDA; }
   const int tasks = PP_BANDS * n, blocks = tasks < 2 * 148 ? tasks : 2 * 148;      // two blocks per SM are resident
   preprocess_kernel<<<blocks, PP_THREADS, sizeof(PpShared), (cudaStream_t)stream>>>(raw_prev, raw_last, state_in, state_out, tasks);
   return cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;

@@ -76,6 +76,15 @@ def test_init_fails_loudly_without_a_gpu():
     assert not h.value
 
 
+def _compiled(tmp_path, source):
+    """A library of plain C++ that includes one of the headers the host code shares with nothing on a device."""
+    src, so = tmp_path / "host.cpp", tmp_path / "host.so"
+    src.write_text(source)
+    csrc = os.path.join(ROOT, "paper_1705_04862_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", csrc, str(src), "-o", str(so)], check=True)
+    return C.CDLL(str(so))
+
+
 HOST_VIEW = """
 #include "host_view.h"
 // ranges: start, size, device address of the start, pinned -- four numbers each
@@ -105,10 +114,27 @@ extern "C" uintptr_t view(uintptr_t p, size_t bytes, const uint64_t* ranges, int
     (0x1000, 2 ** 64 - 1, [(0x1000, 0x1000, 0x1000, 1)], False),                         # a length that wraps around
 ])
 def test_host_buffers_are_read_in_place_only_where_all_of_them_is_pinned(tmp_path, p, size, ranges, readable):
-    src, so = tmp_path / "view.cpp", tmp_path / "view.so"
-    src.write_text(HOST_VIEW)
-    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_1705_04862_b200", "csrc"), str(src), "-o", str(so)], check=True)
-    view = C.CDLL(str(so)).view
+    view = _compiled(tmp_path, HOST_VIEW).view
     view.argtypes, view.restype = [C.c_uint64, C.c_size_t, C.POINTER(C.c_uint64), C.c_int], C.c_uint64
     flat = [x for r in ranges for x in r] or [0]
     assert view(p, size, (C.c_uint64 * len(flat))(*flat), len(ranges)) == (p if readable else 0)
+
+
+PER_DEVICE = """
+#include "per_device.h"
+static paac::PerDevice<int> cache;
+static int calls = 0;
+extern "C" int get(int device, int works) {          // 100 * device + the call it was made in, or -1
+  const int* v = cache.get(device, [&](int& out) { out = 100 * device + ++calls; return works != 0; });
+  return v ? *v : -1;
+}
+"""
+
+
+def test_what_belongs_to_a_device_is_made_once_on_each(tmp_path):
+    """The pre-processing kernel's attribute and the built-in array's address: looked up on every device that is used,
+    once, and again after a failure."""
+    get = _compiled(tmp_path, PER_DEVICE).get
+    assert [get(0, 1), get(0, 1), get(1, 1), get(0, 1), get(1, 0)] == [1, 1, 102, 1, 102]
+    assert [get(63, 0), get(63, 1), get(63, 0)] == [-1, 6304, 6304]
+    assert [get(-1, 1), get(64, 1)] == [-1, -1]
