@@ -226,7 +226,7 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
   for (int l = 0; l <= c->nd.n_conv; ++l)
     act[l] = (char*)c->act[l] + (size_t)slot * c->n_e * c->nd.layer[l].out_size * c->elt;
   const size_t row = (size_t)slot * c->n_e;
-  if (rollout_small_supported(c->lc, c->arch, c->n_e)) {
+  if (rollout_small_supported(c->lc, c->arch, c->prec, c->n_e)) {
     small_rollout(c, frames, slot, 1, sample ? 1 : 0, nullptr, advanced && !sample);
     if (advanced) *advanced = !sample;
     return false;
@@ -481,7 +481,7 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
   uint8_t* nxt = c->frames[c->cur ^ 1];
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
   run_recorded(c, 0, c->cur, [&]() {
-    if (rollout_small_supported(c->lc, c->arch, c->n_e)) {
+    if (rollout_small_supported(c->lc, c->arch, c->prec, c->n_e)) {
       const EnvStepArgs env{c->hp.term_denom, nxt, c->rewards, c->terminals, c->counters, pattern_actions(c)};
       small_rollout(c, fr, 0, c->t_max + 1, c->t_max, &env, true);
       return;

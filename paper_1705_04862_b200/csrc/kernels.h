@@ -142,7 +142,7 @@ void heads_backward(LaunchCtx& lc, int prec, const NetDims& nd, const float* the
                     float* grad, float* scratch, GradSegments* segs);
 
 // ---- all forward passes of a rollout in one launch, small batches of the smaller network (rollout_small.cu) ----------
-bool rollout_small_supported(const LaunchCtx& lc, int arch, int n);
+bool rollout_small_supported(const LaunchCtx& lc, int arch, int prec, int n);      // sizes, and that all its blocks are resident
 size_t rollout_small_part_floats(int n);        // scratch
 size_t rollout_small_barrier_words(int n);      // uint32, zero before the first launch and after a device error
 struct SmallRollout {

@@ -335,53 +335,72 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
 
 // Blocks per environment: as many of 16, 8, 4, 2 as leave each a multiprocessor of its own; 0: use the layer-by-layer path.
 static int rs_blocks_per_env(int n) { return n <= 9 ? 16 : (n <= 18 ? 8 : (n <= 37 ? 4 : (n <= 74 ? 2 : 0))); }
-bool rollout_small_supported(const LaunchCtx& lc, int arch, int n) {
-  if (arch != PAAC_ARCH_NIPS || lc.fp32_tensor_cores || rs_blocks_per_env(n) == 0) return false;
-  static const int fits = [] {
-    int dev = 0, sms = 0, coop = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) { cudaGetLastError(); return 0; }
-    return coop && sms >= 148 ? 1 : 0;
-  }();
-  return fits != 0;
+// One block per SM of a whole device; shared memory up to the largest head.
+constexpr int RS_BLOCKS = 148;
+static size_t rs_smem(int A) { return (size_t)(RS_HEADW + (A + 1) * RS_F) * sizeof(float); }
+
+template <class T_, int C> struct RsKernel {
+  typedef T_ T;                                        // storage of weights and activations
+  static auto kernel() { return rollout_small_kernel<T, T, C>; }
+  // Blocks that wait for one another all have to be resident: what a cooperative launch checks, asked for beforehand so that
+  // a device with fewer multiprocessors, or a build that takes more registers, goes layer by layer instead of failing.
+  static bool fits() {
+    static const bool resident = [] {
+      int dev = 0, sms = 0, coop = 0, per_sm = 0;
+      const int smem = (int)rs_smem(32);
+      const bool known = cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+                         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess &&
+                         cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel(), RS_THREADS, smem) == cudaSuccess;
+      if (!known) cudaGetLastError();
+      return known && coop != 0 && per_sm * sms >= RS_BLOCKS;
+    }();
+    return resident;
+  }
+};
+template <class F> static auto rs_pick(int prec, int C, F f) {
+  auto of = [&](auto t) {
+    typedef decltype(t) T;
+    if (C == 16) return f(RsKernel<T, 16>{});
+    if (C == 8) return f(RsKernel<T, 8>{});
+    if (C == 4) return f(RsKernel<T, 4>{});
+    return f(RsKernel<T, 2>{});
+  };
+  return prec == PAAC_BF16 ? of(bf16{}) : of(float{});
+}
+
+bool rollout_small_supported(const LaunchCtx& lc, int arch, int prec, int n) {
+  const int C = rs_blocks_per_env(n);
+  return arch == PAAC_ARCH_NIPS && !lc.fp32_tensor_cores && C != 0 && rs_pick(prec, C, [](auto k) { return k.fits(); });
 }
 size_t rollout_small_part_floats(int n) { return (size_t)RS_RUNS * n * RS_F; }
 size_t rollout_small_barrier_words(int n) { return 2 * ((size_t)n + 1); }      // 64-bit counters
 
-template <class T, class TW>
-static void rs_launch(LaunchCtx& lc, const RsArgs& q, const TW* w, const NetDims& nd, void* const act[]) {
-  const LayerDims* d = nd.layer;
-  const size_t smem = (size_t)(RS_HEADW + (q.A + 1) * RS_F) * sizeof(float);
-  auto go = [&](auto kern) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { lc.host_failure = true; return; }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(q.blocks); cfg.blockDim = dim3(RS_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = lc.st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    lc.serialize_next = false;
-    KernelScope scope(lc, KID_SMALL_ROLLOUT);
-    if (cudaLaunchKernelEx(&cfg, kern, q, w + d[0].w_off, w + d[1].w_off, w + d[2].w_off, w + nd.pi_w, w + nd.v_w, (T*)act[0], (T*)act[1], (T*)act[2]) != cudaSuccess)
-      lc.host_failure = true;
-  };
-  if (q.C == 16) go(rollout_small_kernel<T, TW, 16>);
-  else if (q.C == 8) go(rollout_small_kernel<T, TW, 8>);
-  else if (q.C == 4) go(rollout_small_kernel<T, TW, 4>);
-  else go(rollout_small_kernel<T, TW, 2>);
-}
-
 void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const SmallRollout& r) {
   const LayerDims* d = nd.layer;
   RsArgs q{};
-  q.n = r.n; q.C = rs_blocks_per_env(r.n); q.A = nd.A; q.steps = r.steps; q.blocks = 148; q.t0 = r.t0;
+  q.n = r.n; q.C = rs_blocks_per_env(r.n); q.A = nd.A; q.steps = r.steps; q.blocks = RS_BLOCKS; q.t0 = r.t0;
   q.frames = r.frames; q.frame_step = r.frame_step; q.next_frames = r.env.next_frames; q.sample_steps = r.sample_steps; q.env = r.step_env;
   q.part = r.part; q.b1 = theta + d[0].b_off; q.b2 = theta + d[1].b_off; q.bfc = theta + d[2].b_off; q.bpi = theta + nd.pi_b; q.bv = theta + nd.v_b;
   q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
   q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
   q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode;
   q.grid_bar = reinterpret_cast<unsigned long long*>(r.barriers); q.group_bar = q.grid_bar + 1; q.error_word = r.error_word;
-  if (prec == PAAC_BF16) rs_launch<bf16, bf16>(lc, q, theta16, nd, r.act);
-  else rs_launch<float, float>(lc, q, theta, nd, r.act);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(q.blocks); cfg.blockDim = dim3(RS_THREADS); cfg.dynamicSmemBytes = rs_smem(q.A); cfg.stream = lc.st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative; attr[0].val.cooperative = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  lc.serialize_next = false;
+  KernelScope scope(lc, KID_SMALL_ROLLOUT);
+  const bool launched = rs_pick(prec, q.C, [&](auto k) {
+    typedef typename decltype(k)::T T;
+    const T* w;
+    if constexpr (sizeof(T) == 2) w = theta16; else w = theta;
+    return k.fits() && cudaLaunchKernelEx(&cfg, k.kernel(), q, w + d[0].w_off, w + d[1].w_off, w + d[2].w_off, w + nd.pi_w, w + nd.v_w,
+                                          (T*)r.act[0], (T*)r.act[1], (T*)r.act[2]) == cudaSuccess;
+  });
+  if (!launched) lc.host_failure = true;
 }
 
 }  // namespace paac

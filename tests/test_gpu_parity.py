@@ -819,3 +819,18 @@ def test_destroyed_learners_leave_nothing_behind():
         seen.append((torch.cuda.mem_get_info()[0], resident()))
     assert seen[-1][0] >= seen[7][0] - (4 << 20)
     assert seen[-1][1] <= seen[7][1] + (4 << 20)
+
+
+@pytest.mark.parametrize("prec", [pb.FP32, pb.BF16])
+def test_small_batches_are_one_launch(prec):
+    """Up to 74 environments of the smaller network all blocks of the one-launch rollout are resident on this device, with the
+    largest head too; beyond, and with the three-pass option, the layers are launched one by one."""
+    for n_e, A, three_pass, one in ((1, 32, 0, True), (9, 2, 0, True), (10, 32, 0, True), (18, 6, 0, True), (19, 32, 0, True),
+                                    (37, 6, 0, True), (38, 32, 0, True), (74, 32, 0, True), (75, 6, 0, False), (9, 6, 1, False)):
+        g = pb.Paac("nips", n_e, 2, A, seed=1, precision=prec)
+        g.set_option(pb.OPT_FP32_TENSOR_CORES, three_pass)
+        before = g.launch_count()
+        g.rollout()
+        assert (g.launch_count() - before == 1) == one, (n_e, A, three_pass)
+        assert g.error_word() == 0
+        g.close()
