@@ -21,6 +21,22 @@ __device__ __forceinline__ float to_f(uint8_t x) { return (float)x; }
 template <class T> __device__ __forceinline__ T from_f(float x);
 template <> __device__ __forceinline__ float from_f<float>(float x) { return x; }
 template <> __device__ __forceinline__ bf16 from_f<bf16>(float x) { return __float2bfloat16_rn(x); }
+// four neighbouring values: a byte in the low mantissa bits of 2^23 is 2^23 + byte (two full-rate instructions instead of
+// a conversion), a bf16 is the upper half of a float
+__device__ __forceinline__ float4 widen4(uint32_t bytes) {
+  constexpr float BIAS = 8388608.f;
+  return make_float4(__uint_as_float(__byte_perm(bytes, 0x4B000000u, 0x7440)) - BIAS, __uint_as_float(__byte_perm(bytes, 0x4B000000u, 0x7441)) - BIAS,
+                     __uint_as_float(__byte_perm(bytes, 0x4B000000u, 0x7442)) - BIAS, __uint_as_float(__byte_perm(bytes, 0x4B000000u, 0x7443)) - BIAS);
+}
+__device__ __forceinline__ float4 widen4(uint2 halves) {
+  return make_float4(__uint_as_float(halves.x << 16), __uint_as_float(halves.x & 0xFFFF0000u), __uint_as_float(halves.y << 16),
+                     __uint_as_float(halves.y & 0xFFFF0000u));
+}
+__device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void store4(bf16* p, float4 v) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
 
 // ---- Philox4x32-10 (Salmon et al., SC'11) -------------------------------------
 __host__ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
@@ -205,7 +221,7 @@ inline NetDims make_net(int arch, int A) {
 enum KernelId {
   KID_INIT = 0, KID_ENV_STEP, KID_CONV1_FWD, KID_CONV2_FWD, KID_CONV3_FWD, KID_FC_FWD, KID_HEADS_FWD,
   KID_RETURNS, KID_HEAD_GRAD, KID_HEADS_BWD, KID_FC_WGRAD, KID_FC_DGRAD, KID_CONV3_WGRAD, KID_CONV3_DGRAD,
-  KID_CONV2_WGRAD, KID_CONV2_DGRAD, KID_CONV1_WGRAD, KID_WGRAD_REDUCE, KID_SUMSQ, KID_CLIP_RMSPROP, KID_CAST, KID_BIAS_GRAD,
+  KID_CONV2_WGRAD, KID_CONV2_DGRAD, KID_CONV1_WGRAD, KID_WGRAD_REDUCE, KID_SUMSQ, KID_CLIP_RMSPROP, KID_CAST,
   KID_SMALL_ROLLOUT,
   KID_COUNT
 };
@@ -213,7 +229,7 @@ inline const char* kernel_name(int id) {
   static const char* names[KID_COUNT] = {
       "init_params", "env_step", "conv1_fwd", "conv2_fwd", "conv3_fwd", "fc_fwd", "heads_fwd_sample", "returns",
       "head_grad", "heads_bwd", "fc_wgrad", "fc_dgrad", "conv3_wgrad", "conv3_dgrad", "conv2_wgrad", "conv2_dgrad",
-      "conv1_wgrad", "wgrad_reduce", "grad_sumsq", "clip_rmsprop", "cast_bf16", "bias_grad", "small_rollout"};
+      "conv1_wgrad", "wgrad_reduce", "grad_sumsq", "clip_rmsprop", "cast_bf16", "small_rollout"};
   return id >= 0 && id < KID_COUNT ? names[id] : "?";
 }
 

@@ -124,9 +124,10 @@ void launch_env_step_sampling(LaunchCtx& lc, uint64_t seed, int n_e, const uint6
                               const HeadsTail& ht, int pattern_actions) {
   KernelScope scope(lc, KID_ENV_STEP);
   // up to two blocks per SM may set up while the previous kernel drains; more of them would pile up on the first free SMs
+  auto kern = ht.parts == 2 ? env_step_kernel<2> : (ht.parts == 4 ? env_step_kernel<4> : env_step_kernel<8>);
   auto launch = [&](auto how) {
-    how(lc, ht.parts == 2 ? env_step_kernel<2> : (ht.parts == 4 ? env_step_kernel<4> : env_step_kernel<8>), dim3(n_e), dim3(ENV_THREADS), (size_t)0, seed, n_e, step_base, t, (const int32_t*)nullptr, term_denom,
-        next_frames, rewards, terminals, counters, ht, pattern_actions);
+    how(lc, kern, dim3(n_e), dim3(ENV_THREADS), (size_t)0, seed, n_e, step_base, t, (const int32_t*)nullptr, term_denom, next_frames, rewards,
+        terminals, counters, ht, pattern_actions);
   };
   if (n_e <= 296) launch([](auto&&... a) { launch_kernel_overlapped(a...); });
   else launch([](auto&&... a) { launch_kernel(a...); });

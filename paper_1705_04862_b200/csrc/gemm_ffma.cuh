@@ -24,28 +24,13 @@ __device__ __forceinline__ void widen(const uint4 v, const float*, float4 (&f)[1
   f[0] = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
 }
 __device__ __forceinline__ void widen(const uint4 v, const bf16*, float4 (&f)[2]) {
-  f[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
-  f[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xFFFF0000u));
+  f[0] = widen4(make_uint2(v.x, v.y)); f[1] = widen4(make_uint2(v.z, v.w));
 }
-// a byte in the low mantissa bits of 2^23 is 2^23 + byte: two full-rate instructions instead of a conversion
 __device__ __forceinline__ void widen(const uint4 v, const uint8_t*, float4 (&f)[4]) {
-  constexpr float BIAS = 8388608.f;
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    f[i] = make_float4(__uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7440)) - BIAS, __uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7441)) - BIAS,
-                       __uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7442)) - BIAS, __uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7443)) - BIAS);
+  f[0] = widen4(v.x); f[1] = widen4(v.y); f[2] = widen4(v.z); f[3] = widen4(v.w);
 }
 __device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 load4(const bf16* p) {
-  const uint2 v = *reinterpret_cast<const uint2*>(p);
-  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
-}
-__device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ void store4(bf16* p, float4 v) {
-  const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-}
+__device__ __forceinline__ float4 load4(const bf16* p) { return widen4(*reinterpret_cast<const uint2*>(p)); }
 
 // A k block of R rows in shared memory: [R][BK + 4] or [BK][R + 4] (the padding keeps the reads below free of conflicts).
 template <class OP, int R, int BK> struct FfTile {
@@ -134,7 +119,7 @@ template <bool K_CONTIG, int T, int LANES> __device__ __forceinline__ int ff_ind
   return K_CONTIG ? lane + i * LANES : ((i / RUN) * LANES + lane) * RUN + i % RUN;
 }
 
-// Four warps, WM x WN; a warp's lanes are LM x (32 / LM), TM x TN outputs each.  Grid (m tiles, n tiles, splits x classes).
+// WM x WN warps; a warp's lanes are LM x (32 / LM), TM x TN outputs each.  Grid (m tiles, n tiles, splits x classes).
 // With EP::COLSUM the epilogue also gets the sum over k of every row of B (bias gradients), once per split.
 constexpr int FF_STAGES = 3;
 template <int LM, int TM, int TN, int WM, int WN, int BK, class LA, class LB> struct FfCfg {

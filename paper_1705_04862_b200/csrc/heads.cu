@@ -280,9 +280,10 @@ void launch_heads_fused(LaunchCtx& lc, const NetDims& nd, const float* theta, co
                         float* uniforms, HeadMode mode, uint64_t* advance_step, uint32_t advance_by, int parts) {
   KernelScope scope(lc, KID_HEADS_FWD);
   if (splits == 0) {          // `part` holds the head dot products of the parts of the hidden units
-    launch_kernel_overlapped(lc, parts == 2 ? heads_sample_kernel<2> : (parts == 4 ? heads_sample_kernel<4> : heads_sample_kernel<8>), (n + HS_WARPS - 1) / HS_WARPS, HS_WARPS * 32, 0, part, theta + nd.pi_b,
-                             theta + nd.v_b, n, nd.A, logits, values, seed, advance_step ? nullptr : step_base, t, forced,
-                             actions, sampled, uniforms, advance_step, advance_by, mode);
+    auto kern = parts == 2 ? heads_sample_kernel<2> : (parts == 4 ? heads_sample_kernel<4> : heads_sample_kernel<8>);
+    launch_kernel_overlapped(lc, kern, (n + HS_WARPS - 1) / HS_WARPS, HS_WARPS * 32, 0, part, theta + nd.pi_b, theta + nd.v_b, n, nd.A, logits,
+                             values, seed, advance_step ? nullptr : step_base, t, forced, actions, sampled, uniforms, advance_step, advance_by,
+                             mode);
     return;
   }
   launch_kernel(lc, heads_fused_kernel, (n + HF_WARPS - 1) / HF_WARPS, HF_WARPS * 32, 0, part, splits, theta + nd.layer[nd.n_conv].b_off, h_out,

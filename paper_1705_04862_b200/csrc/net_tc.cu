@@ -28,10 +28,7 @@ constexpr size_t TC_IMG_W2 = 0, TC_IMG_W3 = 4 * 32 * 256, TC_IMG_WFC = TC_IMG_W3
                  TC_IMG_W1 = TC_IMG_WFC + (size_t)3136 * 512, TC_IMG_END = TC_IMG_W1 + 32 * 256;
 
 
-// ---- tensor maps for the plain row-major bf16 matrices (fully connected layer) ---------------------------------
-// map of matrix x[rows][cols] (row pitch `ld` elements) for boxes of box_rows x 64 elements with the 128-byte swizzle.
-// Maps are cached by their defining values: the matrices live at fixed places of the workspace, so after the first
-// iteration every call is a look-up.  Returns nullptr if the driver's encoder is unavailable or refuses.
+// ---- tensor maps ------------------------------------------------------------------------------------------------
 // the driver's encoder, looked up at run time (nothing links to libcuda); nullptr if it cannot be had
 typedef CUresult (*TmapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -47,6 +44,10 @@ static TmapEncodeFn tc_tmap_encoder() {
   return encode;
 }
 
+// Map of a plain row-major bf16 matrix x[rows][cols] (row pitch `ld` elements; the fully connected layer's operands) for boxes
+// of box_rows x 64 elements with the 128-byte swizzle.  Maps are cached by their defining values: the matrices live at fixed
+// places of the workspace, so after the first iteration every call is a look-up.  Returns nullptr if the driver's encoder is
+// unavailable or refuses.
 struct TmapKey { const void* p; uint64_t rows, cols, ld; uint32_t box_rows; };
 static const CUtensorMap* tc_tensor_map(const bf16* x, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows) {
   const TmapEncodeFn encode = tc_tmap_encoder();
@@ -516,16 +517,14 @@ tc_gemm_kernel(ASrc a_src, BSrc b_src, Epi epi, int num_kb, uint32_t* error_word
   }
 }
 
-// ---- persistent variant: weights resident in shared memory, A streamed with cp.async -------------------
+// ---- persistent variant: weights resident in shared memory, A streamed by tiled bulk copies -------------
 // One CTA per SM walks over output tiles t = blockIdx.x, blockIdx.x + gridDim.x, ...; tile t is row tile
 // t % tiles_m of class t / tiles_m (classes: the parity classes of a stride-2 data gradient, else one).
 // The whole K extent of the CTA's weight slice (BN rows, KB blocks, all classes) is loaded once.
 //   warps 0-3  epilogue: tile i is read out of its TMEM buffer while tile i+1 is being multiplied
-//   warps 4-7  producers: one tile row per thread, eight 16-byte cp.async per K block straight into the
-//              swizzled image; a stage is published LAG blocks later, after the thread's copies of it
-//              have landed (cp.async.wait_group) and were fenced towards the async proxy
+//   warp 4     lane 0 asks the copy engine for the 128 x 64 boxes of A, straight into the swizzled image
 //   warp 8     lane 0 issues the MMAs and commits stages / accumulators
-constexpr int PK_THREADS = 288, PK_LAG = 5;
+constexpr int PK_THREADS = 288;
 struct PkShared {
   uint64_t full[8], empty[8], acc_full[2], acc_empty[2], mask_full[2], mask_empty[2];
   uint32_t tmem_base;
@@ -1765,10 +1764,10 @@ tc_fc_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
       float pr[FCC_HP_LD];
 #pragma unroll
       for (int k = 0; k < FCC_HP_LD; ++k) pr[k] = k <= A ? dot(k) : 0.f;
-  #pragma unroll
+#pragma unroll
       for (int o = 8, len = FCC_HP_LD / 2; o > 0; o >>= 1, len >>= 1) {
         const bool up = (cg & o) != 0;
-  #pragma unroll
+#pragma unroll
         for (int i = 0; i < len; ++i) {
           const float send = up ? pr[i] : pr[i + len];
           const float keep = up ? pr[i + len] : pr[i];
@@ -2345,8 +2344,8 @@ void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, 
 // of m): atom column a -> 8 groups of 8 rows -> 128-byte swizzled rows; leading (atom-column) stride 8 KB,
 // stride between 8-row groups 1 KB; a K=16 MMA step covers two groups.
 // A CTA owns JT row tiles of 128 j each and a contiguous range of 64-row blocks of m (split-k); it writes
-// its float partial tile to scratch, and a second kernel adds the partials in a fixed order.
-constexpr int WG_ROWS = 64, WG_LAG = 3;
+// its float partial tile to scratch; tc_finalize_grads_kernel adds the partials in a fixed order.
+constexpr int WG_ROWS = 64;
 
 // G rows: BN (64 or 128) bf16 starting at column n0; rows past M read as zero so that the tail of the last
 // block adds nothing.  VALID < 64 pads a narrower matrix (conv1: 32 channels) with zero columns.
@@ -2533,38 +2532,6 @@ tc_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
   }
 }
 
-// dW[co][j] = scale * sum over splits of partial[split][j][co].  A block owns 32 consecutive outputs;
-// its 8 thread rows each add every 8th split, then the 8 sums are added in a fixed order.
-__global__ void __launch_bounds__(256) tc_wgrad_reduce_kernel(const float* __restrict__ partial, int splits, int J, int CO,
-                                                              float scale, float* __restrict__ gw) {
-  pdl_entry();
-  __shared__ float sh[8][33];
-  const int total = J * CO, lane = threadIdx.x & 31, part = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + lane;
-  float s = 0.f;
-  if (i < total)
-    for (int p = part; p < splits; p += 8) s += partial[(size_t)p * total + i];
-  sh[part][lane] = s;
-  __syncthreads();
-  if (part == 0 && i < total) {
-    float t = 0.f;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) t += sh[q][lane];
-    const int j = i / CO, co = i % CO;
-    gw[(size_t)co * J + j] = t * scale;
-  }
-}
-
-// bias gradient: the per-split column sums written by the weight-gradient kernel, added in split order
-__global__ void tc_bias_final_kernel(const float* __restrict__ part, int blocks, int CO, float* __restrict__ gb) {
-  pdl_entry();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= CO) return;
-  float s = 0.f;
-  for (int b = 0; b < blocks; ++b) s += part[(size_t)b * CO + c];
-  gb[c] = s;
-}
-
 // One launch finishes every tensor-core weight gradient of an update: for each segment (a layer's weights, or
 // its bias with J = 1) dst[co * J + j] = scale * sum over splits of part[split][j][co], the splits added in a
 // fixed order.  The partial sums have co innermost and the gradient has j innermost, so every group of outputs
@@ -2730,7 +2697,6 @@ template <class XSrc, class GSrc, int JT, int BN, int STAGES, int CO>
 static void tc_wgrad(LaunchCtx& lc, int kid, XSrc xs, GSrc gs, int rows, int n_atoms, float scale,
                      float* gw, float* gb, float* scratch, GradSegments* segs, uint32_t* err) {
   constexpr int smem = STAGES * ((2 * JT + BN / 64) * WG_ROWS * 128) + 2 * WG_ROWS * 128 + 1024;
-  static_assert(STAGES >= WG_LAG || !XSrc::ASYNC, "pipeline depth");
   auto kern = tc_wgrad_kernel<XSrc, GSrc, (CO < 64 ? CO : 64), JT, BN, STAGES>;
   static bool configured = false;
   if (!configured) {
@@ -3464,7 +3430,7 @@ __global__ void __launch_bounds__(256) relayout_weights_kernel(const bf16* __res
                                         bf16* __restrict__ w1_b, uint32_t* __restrict__ error_word) {
   pdl_entry();
   typedef NatConv2 C2; typedef NatConv3 C3;
-  constexpr int N2 = 4 * C2::C * 4 * C2::CO, N3 = C3::C * 9 * C3::CO, NF = 3136 * 512, N1 = 32 * 256;
+  constexpr int N2 = 4 * C2::C * 4 * C2::CO, N3 = C3::C * 9 * C3::CO, N1 = 32 * 256;
   // Blocks 0 .. RL_FC_TILES - 1 transpose the fully connected matrix, the bulk of the work, one 64 x 64 tile each
   // through shared memory, so that both sides are whole 128-byte rows; the other blocks gather the small images.
   if (blockIdx.x < RL_FC_TILES) {

@@ -82,11 +82,6 @@ struct RsBarrier {
   }
 };
 
-__device__ __forceinline__ float4 rs_bytes(uint32_t v) {
-  constexpr float BIAS = 8388608.f;       // a byte in the low mantissa bits of 2^23 is 2^23 + byte
-  return make_float4(__uint_as_float(__byte_perm(v, 0x4B000000u, 0x7440)) - BIAS, __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7441)) - BIAS,
-                     __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7442)) - BIAS, __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7443)) - BIAS);
-}
 __device__ __forceinline__ void rs_fma4(float (&acc)[4], float a, const float4 w) {
   acc[0] = fmaf(a, w.x, acc[0]); acc[1] = fmaf(a, w.y, acc[1]); acc[2] = fmaf(a, w.z, acc[2]); acc[3] = fmaf(a, w.w, acc[3]);
 }
@@ -94,17 +89,9 @@ __device__ __forceinline__ float4 rs_relu(const float (&acc)[4], float scale, co
   return make_float4(fmaxf(fmaf(acc[0], scale, b[0]), 0.f), fmaxf(fmaf(acc[1], scale, b[1]), 0.f), fmaxf(fmaf(acc[2], scale, b[2]), 0.f),
                      fmaxf(fmaf(acc[3], scale, b[3]), 0.f));
 }
-__device__ __forceinline__ void rs_store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ void rs_store4(bf16* p, float4 v) {
-  const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-}
 // written by other blocks during this launch: past the first-level cache
 __device__ __forceinline__ float4 rs_load4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float4 rs_load4(const bf16* p) {
-  const uint2 v = __ldcg(reinterpret_cast<const uint2*>(p));
-  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
-}
+__device__ __forceinline__ float4 rs_load4(const bf16* p) { return widen4(__ldcg(reinterpret_cast<const uint2*>(p))); }
 
 // shared memory, in floats
 constexpr int RS_W1 = 0, RS_W2 = RS_W1 + RC1::KK * RC1::CO, RS_FCW = RS_W2 + RC2::KK * RC2::CO, RS_FCA = RS_FCW + RS_COLS * RS_FC_LD,
@@ -133,7 +120,7 @@ __device__ __forceinline__ void rs_conv1(const float* sm, const float* b1, T* ac
       for (int s = 0; s < RC1::K; ++s) {
         float4 a[PP];
 #pragma unroll
-        for (int i = 0; i < PP; ++i) a[i] = rs_bytes(frame[base[i] + r * RC1::W + s]);
+        for (int i = 0; i < PP; ++i) a[i] = widen4(frame[base[i] + r * RC1::W + s]);
         const int k = (r * RC1::K + s) * 4;
         const float4 w0 = w[k * 4], w1 = w[(k + 1) * 4], w2 = w[(k + 2) * 4], w3 = w[(k + 3) * 4];
 #pragma unroll
@@ -142,7 +129,7 @@ __device__ __forceinline__ void rs_conv1(const float* sm, const float* b1, T* ac
     }
 #pragma unroll
   for (int i = 0; i < PP; ++i)
-    if (p < apart && p + apart * i < share) rs_store4(act + (size_t)(pos0 + p + apart * i) * RC1::CO + 4 * q, rs_relu(acc[i], 1.0f / 255.0f, b1 + 4 * q));
+    if (p < apart && p + apart * i < share) store4(act + (size_t)(pos0 + p + apart * i) * RC1::CO + 4 * q, rs_relu(acc[i], 1.0f / 255.0f, b1 + 4 * q));
 }
 // Second layer: the same with 8 groups of 4 channels, the input rows in shared memory.
 template <class T, int PP>
@@ -174,7 +161,7 @@ __device__ __forceinline__ void rs_conv2(const float* sm, const float* b2, T* ac
     }
 #pragma unroll
   for (int i = 0; i < PP; ++i)
-    if (p < apart && p + apart * i < share) rs_store4(act + (size_t)(pos0 + p + apart * i) * RC2::CO + 4 * q, rs_relu(acc[i], 1.f, b2 + 4 * q));
+    if (p < apart && p + apart * i < share) store4(act + (size_t)(pos0 + p + apart * i) * RC2::CO + 4 * q, rs_relu(acc[i], 1.f, b2 + 4 * q));
 }
 
 template <class T, class TW, int C>
@@ -318,7 +305,8 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
     if (tid == 32 && rank == 0) env_record(prep, o, (uint32_t)e, n, q.rewards + slot, q.terminals + slot, q.counters);
     const EnvFrame f = s_frame;
     // this block's share of the frame for everyone, and the rows it will read itself
-    uint4* out = reinterpret_cast<uint4*>((t + 1 < q.sample_steps ? const_cast<uint8_t*>(q.frames) + (size_t)(t + 1) * q.frame_step : q.next_frames) + (size_t)e * FRAME_BYTES);
+    uint8_t* states = t + 1 < q.sample_steps ? const_cast<uint8_t*>(q.frames) + (size_t)(t + 1) * q.frame_step : q.next_frames;
+    uint4* out = reinterpret_cast<uint4*>(states + (size_t)e * FRAME_BYTES);
     const int own_lo = FRAME_WORDS / 4 * rank / C, own_hi = FRAME_WORDS / 4 * (rank + 1) / C;
     const int lo = min(own_lo, row_lo * QUADS), hi = max(own_hi, row_hi * QUADS);
     for (int i = lo + tid; i < hi; i += RS_THREADS) {
