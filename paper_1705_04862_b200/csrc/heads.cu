@@ -106,18 +106,24 @@ simt_tail_kernel(TailArgs q, T* h, const TW* wpi, const float* bpi, const TW* wv
   }
 }
 
+template <class T, class TW, int F, bool STEP>
+static void tail_launch(LaunchCtx& lc, const TailArgs& q, T* h, const TW* wpi, const float* bpi, const TW* wv, const float* bv,
+                        const EnvStepArgs& env) {
+  constexpr size_t ROW = F * sizeof(float);
+  auto kern = simt_tail_kernel<T, TW, F, STEP>;
+  // for the largest head: beside the static arrays even one of 20 actions passes the default limit
+  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(33 * ROW));
+  if (attr != cudaSuccess) lc.host_failure = true;
+  const size_t smem = (q.A + 1) * ROW;
+  // few blocks: they may set up while the previous kernel drains; many small blocks would pile up on the first free SMs
+  if (q.n <= 148) launch_kernel_overlapped(lc, kern, dim3(q.n), dim3(2 * F), smem, q, h, wpi, bpi, wv, bv, env);
+  else launch_kernel(lc, kern, dim3(q.n), dim3(2 * F), smem, q, h, wpi, bpi, wv, bv, env);
+}
 template <class T, class TW, int F>
 static void tail_launch(LaunchCtx& lc, const TailArgs& q, T* h, const TW* wpi, const float* bpi, const TW* wv, const float* bv,
                         const EnvStepArgs* env) {
-  const size_t smem = (size_t)(q.A + 1) * F * sizeof(float);
-  auto go = [&](auto kern) {
-    if (smem + 4096 > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      lc.host_failure = true;
-    // few blocks: they may set up while the previous kernel drains; many small blocks would pile up on the first free SMs
-    if (q.n <= 148) launch_kernel_overlapped(lc, kern, dim3(q.n), dim3(2 * F), smem, q, h, wpi, bpi, wv, bv, env ? *env : EnvStepArgs{});
-    else launch_kernel(lc, kern, dim3(q.n), dim3(2 * F), smem, q, h, wpi, bpi, wv, bv, env ? *env : EnvStepArgs{});
-  };
-  if (env) go(simt_tail_kernel<T, TW, F, true>); else go(simt_tail_kernel<T, TW, F, false>);
+  if (env) tail_launch<T, TW, F, true>(lc, q, h, wpi, bpi, wv, bv, *env);
+  else tail_launch<T, TW, F, false>(lc, q, h, wpi, bpi, wv, bv, EnvStepArgs{});
 }
 
 void launch_simt_tail(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const float* part, int splits,

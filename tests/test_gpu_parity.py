@@ -834,3 +834,25 @@ def test_small_batches_are_one_launch(prec):
         assert (g.launch_count() - before == 1) == one, (n_e, A, three_pass)
         assert g.error_word() == 0
         g.close()
+
+
+@pytest.mark.parametrize("arch,prec,three_pass", [("nature", "FP32", 0), ("nips", "FP32", 0), ("nips", "BF16", 1), ("nature", "BF16", 0)])
+def test_every_head_size_as_the_first_of_its_process(arch, prec, three_pass):
+    """What a kernel is allowed for its largest head stays allowed for the rest of the process, so a limit that one head size
+    passes unnoticed shows only where that size is used first: every number of actions in a process of its own would
+    take minutes, the sizes in ascending order in one process do as well."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import paper_1705_04862_b200.binding as pb
+for A in range(2, 33):
+    g = pb.Paac("%s", 80, 1, A, seed=1, precision=pb.%s)
+    g.set_option(pb.OPT_FP32_TENSOR_CORES, %d)
+    g.rollout()
+    assert g.update()["status"] == 0 and g.error_word() == 0, A
+    g.close()
+""" % (arch, prec, three_pass)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    done = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr[-2000:]
