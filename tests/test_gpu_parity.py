@@ -115,9 +115,9 @@ def test_float_tensor_core_option_on_the_nature_network(orc):
 
 @pytest.mark.parametrize("own_stream", [False, True])
 def test_config2_free_running_actions_agree(orc, own_stream):
-    """Without forcing: both sides sample for themselves; with float parameters the draws agree.  On a stream
-    of its own the library replays recorded CUDA graphs from the third iteration on (the legacy default stream
-    cannot be captured, so there every iteration is plain launches): both must walk with the oracle."""
+    """Without forcing: both sides sample for themselves; with float parameters the draws agree.  From the third
+    iteration on the library replays recorded CUDA graphs (learners on the legacy default stream, which cannot be
+    captured, record on a stream of the library's own): both must walk with the oracle."""
     import torch
     cfg = CONFIGS[1]
     stream = torch.cuda.Stream() if own_stream else torch.cuda.current_stream()
@@ -280,7 +280,8 @@ def test_resync_after_many_updates(orc):
 
 
 def test_determinism_bitwise(orc):
-    """Same seed, same bits -- with plain launches and with replayed graphs (own stream), tensor-core path."""
+    """Same seed, same bits -- with plain launches, and with replayed graphs on the default and on an own stream,
+    tensor-core path."""
     import torch
     cfg = CONFIGS[2]
     outs = []
@@ -288,6 +289,7 @@ def test_determinism_bitwise(orc):
         stream = torch.cuda.Stream() if rep == 2 else torch.cuda.current_stream()
         with torch.cuda.stream(stream):
             _, g = make_pair(orc, cfg)
+            g.set_option(pb.OPT_CUDA_GRAPHS, int(rep > 0))
             for it in range(5):
                 g.rollout()
                 g.update()
@@ -654,7 +656,7 @@ def test_pattern_environment_matches_the_oracle_and_can_be_learned(orc):
 
 
 @pytest.mark.parametrize("arch,n_e,t_max,A", [("nips", 1, 1, 2), ("nips", 49, 1, 32), ("nips", 97, 1, 7), ("nature", 3, 2, 20),
-                                              ("nature", 66, 1, 6)])
+                                              ("nature", 66, 1, 6), ("nips", 475, 1, 4), ("nature", 475, 1, 3)])
 def test_float_contraction_shapes(orc, arch, n_e, t_max, A):
     """The CUDA-core contraction in each of its tile shapes, with remainders in every dimension, and the kernel that ends a
     forward step with few and many head outputs: one update each, both passes from identical tensors."""
@@ -670,7 +672,8 @@ def test_float_contraction_shapes(orc, arch, n_e, t_max, A):
                                         (38, "fp32", 5), (74, "fp32", 9), (75, "bf16", 6)])
 def test_small_batches_one_launch_rollout(orc, n_e, prec, A):
     """The smaller network's rollout in one launch: the smallest and largest batch of every group size, the first one beyond,
-    both storage types; two iterations (the barriers' counters go on), the second through recorded sequences' first use."""
+    both storage types; two iterations (the barriers' counters go on).  (Forced actions keep these on plain launches: the
+    recorded ones are compared with them in test_recorded_sequences_are_the_plain_launches.)"""
     cfg = dict(arch="nips", precision=prec, n_e=n_e, t_max=2, n_actions=A, lr=0.0028, term_denom=3)
     o, g = make_pair(orc, cfg)
     for it in range(2):
@@ -682,7 +685,7 @@ def test_small_batches_one_launch_rollout(orc, n_e, prec, A):
     g.close()
 
 
-@pytest.mark.parametrize("n_e,A", [(1, 2), (127, 19), (128, 30), (129, 18), (384, 31)])
+@pytest.mark.parametrize("n_e,A", [(1, 2), (127, 19), (128, 30), (129, 18), (384, 31), (513, 5)])
 def test_fully_connected_column_tiles(orc, n_e, A):
     """The fully connected forward kernel with each of its column tiles (64, 128 and 256), full and ragged row tiles, few and
     many head outputs: one rollout against the oracle."""
@@ -693,7 +696,7 @@ def test_fully_connected_column_tiles(orc, n_e, A):
     g.close()
 
 
-@pytest.mark.parametrize("n_e", [3, 1027])
+@pytest.mark.parametrize("n_e", [3, 1027, 1100])
 def test_pulled_planes_match_whole_states(n_e):
     """External-environment steps whose planes the stacking kernel reads from pinned memory, with restarts: values,
     actions and parameters equal those of a learner that is sent whole states, over recorded and plain sequences."""
@@ -856,3 +859,39 @@ for A in range(2, 33):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     done = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert done.returncode == 0, done.stderr[-2000:]
+
+
+@pytest.mark.parametrize("arch,prec,n_e,algorithm,own_stream", [
+    ("nips", "fp32", 4, pb.ALGO_A2C, True), ("nips", "fp32", 74, pb.ALGO_NSTEP_Q, False), ("nips", "bf16", 80, pb.ALGO_A2C, True),
+    ("nature", "fp32", 5, pb.ALGO_A2C, False), ("nature", "bf16", 33, pb.ALGO_NSTEP_Q, True), ("nature", "bf16", 130, pb.ALGO_A2C, False)])
+def test_recorded_sequences_are_the_plain_launches(arch, prec, n_e, algorithm, own_stream):
+    """Both halves of an iteration and the steps of the external-environment mode, recorded and replayed (several times for
+    either frame buffer) and launched one by one: the same bits at every iteration, the same number of kernels."""
+    import torch
+    stream = torch.cuda.Stream() if own_stream else torch.cuda.current_stream()
+    with torch.cuda.stream(stream):
+        a, b = (pb.Paac(arch, n_e, 2, 5, seed=4, precision=pb.BF16 if prec == "bf16" else pb.FP32, lr=0.01, term_denom=5,
+                        algorithm=algorithm) for _ in range(2))
+    b.set_option(pb.OPT_CUDA_GRAPHS, 0)
+    rng = np.random.RandomState(n_e)
+    for it in range(12):
+        if it < 6:
+            assert a.rollout().frames and b.rollout().frames
+        else:
+            acts, vals = np.zeros((2, 2, n_e), np.int32), np.zeros((2, 3, n_e), np.float32)
+            first = rng.randint(0, 256, (n_e, 84, 84, 4), dtype=np.uint8)
+            planes = rng.randint(0, 256, (2, n_e, 84, 84), dtype=np.uint8)
+            rewards, ends = rng.randint(-1, 2, (2, n_e)).astype(np.int8), (rng.randint(0, 5, (2, n_e)) == 0).astype(np.uint8)
+            for i, g in enumerate((a, b)):
+                g.act_host(0, first, acts[i][0], vals[i][0])
+                for t in (1, 2):
+                    g.observe_host(t - 1, rewards[t - 1], ends[t - 1])
+                    g.act_host_newest(t, planes[t - 1], ends[t - 1], acts[i][t] if t < 2 else None, vals[i][t])
+            assert np.array_equal(acts[0], acts[1]) and np.array_equal(vals[0], vals[1])
+        sync = it % 2 == 0 or it > 8
+        assert a.update(sync=sync) == b.update(sync=sync)
+        for which in (pb.DBG_ACTIONS, pb.DBG_REWARDS, pb.DBG_TERMINALS, pb.DBG_VALUES, pb.DBG_GRAD, pb.DBG_RMS):
+            assert np.array_equal(a.debug_read(which), b.debug_read(which)), (it, which)
+        assert np.array_equal(a.params(), b.params()) and a.launch_count() == b.launch_count()
+    assert a.error_word() == 0
+    a.close(), b.close()
