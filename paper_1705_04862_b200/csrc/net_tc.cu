@@ -136,101 +136,10 @@ struct TcShared {
   volatile uint32_t abort;
 };
 
-// ---- A-operand sources: 64 bf16 (128 bytes) of row m for K block kb ---------------------------
-// plain row-major matrix x[m][k]
-// Asynchronous sources split the address of (row m, K block kb) into a per-row part, computed once per tile
-// row, and a cheap per-block part: row(m) -> RowRef, at(ref, kb, valid) -> address of the 128 bytes, with
-// valid = false meaning "reads as zeros".
-struct RowRef { uint32_t base; int32_t yx; };
-struct PlainSrc {
-  static constexpr bool ASYNC = true;
-  const bf16* x; int ld; int M;
-  __device__ __forceinline__ RowRef row(int m) const { return RowRef{(uint32_t)min(m, M - 1) * (uint32_t)ld, 0}; }
-  __device__ __forceinline__ const bf16* at(const RowRef& r, int kb, bool& valid) const {
-    valid = true;
-    return x + r.base + kb * TC_BK;
-  }
-  __device__ __forceinline__ const bf16* ptr(int m, int kb, int, bool& valid) const { return at(row(m), kb, valid); }
-  __device__ __forceinline__ void load(int m, int kb, int, uint4 (&v)[8]) const {
-    m = min(m, M - 1);
-    const uint4* p = reinterpret_cast<const uint4*>(x + (size_t)m * ld + kb * TC_BK);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  }
-};
-// convolution window over a bf16 NHWC tensor; k = (r, s, ci); a K block holds 64 / C taps of one kernel row
-template <class G> struct ConvSrc {
-  static constexpr bool ASYNC = true;
-  const bf16* x; int M;
-  __device__ __forceinline__ RowRef row(int m) const {
-    m = min(m, M - 1);
-    const int b = m / (G::OH * G::OW), rem = m % (G::OH * G::OW), oh = rem / G::OW, ow = rem % G::OW;
-    return RowRef{(uint32_t)(((b * G::H + oh * G::S) * G::W + ow * G::S) * G::C), 0};
-  }
-  __device__ __forceinline__ const bf16* at(const RowRef& rr, int kb, bool& valid) const {
-    valid = true;
-    const int tap = kb * (64 / G::C), r = tap / G::K, s = tap % G::K;
-    return x + rr.base + (r * G::W + s) * G::C;
-  }
-  __device__ __forceinline__ const bf16* ptr(int m, int kb, int, bool& valid) const { return at(row(m), kb, valid); }
-  __device__ __forceinline__ void load(int m, int kb, int, uint4 (&v)[8]) const {
-    static_assert(64 % G::C == 0 && G::K % (64 / G::C) == 0, "a K block must stay inside one kernel row");
-    m = min(m, M - 1);
-    const int b = m / (G::OH * G::OW), rem = m % (G::OH * G::OW), oh = rem / G::OW, ow = rem % G::OW;
-    const int tap = kb * (64 / G::C), r = tap / G::K, s = tap % G::K;
-    const uint4* p = reinterpret_cast<const uint4*>(
-        x + ((size_t)(b * G::H + oh * G::S + r) * G::W + (ow * G::S + s)) * G::C);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  }
-};
-// first layer: uint8 frames [84][84][4]; a kernel row is 8 pixels x 4 channels = 32 bytes, a K block two
-// kernel rows.  Pixel values 0..255 are exact in bf16; the 1/255 normalisation is applied in the epilogue.
-__device__ __forceinline__ uint32_t u8x2_to_bf16x2(uint32_t lo, uint32_t hi) {
-  __nv_bfloat162 t = __floats2bfloat162_rn((float)lo, (float)hi);
-  return *reinterpret_cast<uint32_t*>(&t);
-}
-__device__ __forceinline__ void u8x16_to_bf16(const uint4& q, uint4& a, uint4& b) {
-  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-  uint32_t o[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    o[2 * i] = u8x2_to_bf16x2(w[i] & 255u, (w[i] >> 8) & 255u);
-    o[2 * i + 1] = u8x2_to_bf16x2((w[i] >> 16) & 255u, w[i] >> 24);
-  }
-  a = make_uint4(o[0], o[1], o[2], o[3]);
-  b = make_uint4(o[4], o[5], o[6], o[7]);
-}
-template <class G> struct FrameSrc {
-  static constexpr bool ASYNC = false;     // needs the uint8 -> bf16 conversion, so it goes through registers
-  const uint8_t* x; int M;
-  __device__ __forceinline__ void load(int m, int kb, int, uint4 (&v)[8]) const {
-    static_assert(G::K * G::C == 32, "one kernel row must be 32 bytes");
-    m = min(m, M - 1);
-    const int b = m / (G::OH * G::OW), rem = m % (G::OH * G::OW), oh = rem / G::OW, ow = rem % G::OW;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int r = kb * 2 + j;
-      const uint4* p = reinterpret_cast<const uint4*>(
-          x + ((size_t)(b * G::H + oh * G::S + r) * G::W + ow * G::S) * G::C);
-      const uint4 q0 = __ldg(p), q1 = __ldg(p + 1);
-      u8x16_to_bf16(q0, v[4 * j], v[4 * j + 1]);
-      u8x16_to_bf16(q1, v[4 * j + 2], v[4 * j + 3]);
-    }
-  }
-};
+// ---- operands: plain row-major matrices x[m][k] of M rows, fetched as boxes through tensor maps -------------------
+struct PlainSrc { const bf16* x; int ld; int M; };
 
-// ---- B-operand source: K-major weight matrix w[n][k] -------------------------------------------------
-struct WeightSrc {
-  const bf16* w; int ld;
-  __device__ __forceinline__ void load(int n, int kb, int, uint4 (&v)[8]) const {
-    const uint4* p = reinterpret_cast<const uint4*>(w + (size_t)n * ld + kb * TC_BK);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  }
-};
-
-// ---- epilogues: 32 accumulator columns n0..n0+31 of row m --------------------------------------------
+// ---- epilogues ---------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&t);
@@ -258,263 +167,15 @@ __device__ __forceinline__ void warp_store_rows_f32(uint32_t stg, int lane, cons
 }
 
 // out[m][n] = bf16(relu(acc * scale + bias[n]))
-struct BiasReluEpiTc {
-  bf16* out; const float* bias; int ld; float scale; int M;
-  __device__ __forceinline__ void operator()(int m, int n0, int, const uint32_t (&r)[32]) const {
-    if (m >= M) return;
-    uint32_t o[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float a = fmaxf(fmaf(__uint_as_float(r[2 * j]), scale, __ldg(bias + n0 + 2 * j)), 0.f);
-      const float b = fmaxf(fmaf(__uint_as_float(r[2 * j + 1]), scale, __ldg(bias + n0 + 2 * j + 1)), 0.f);
-      o[j] = pack_bf16x2(a, b);
-    }
-    uint4* dst = reinterpret_cast<uint4*>(out + (size_t)m * ld + n0);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) dst[j] = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
-  }
-};
-
-// ---- data-gradient sources: rows of the layer INPUT, k = (tap, co) -------------------------------------
-// stride-1 convolution with CO = 64: K block kb is tap (r, s); the row for input pixel (y, x) is the
-// 64 output-channel gradients of window (y - r, x - s), or zeros where that window does not exist.
-template <class G> struct DgradSrcS1 {
-  const bf16* g; int M;
-  __device__ __forceinline__ RowRef row(int m) const {
-    m = min(m, M - 1);
-    const int b = m / (G::H * G::W), rem = m % (G::H * G::W), y = rem / G::W, x = rem % G::W;
-    return RowRef{(uint32_t)(b * G::OH * G::OW * G::CO), (y << 8) | x};
-  }
-  __device__ __forceinline__ const bf16* at(const RowRef& rr, int kb, bool& valid) const {
-    const int oh = (rr.yx >> 8) - kb / G::K, ow = (rr.yx & 255) - kb % G::K;
-    valid = oh >= 0 && oh < G::OH && ow >= 0 && ow < G::OW;
-    return valid ? g + rr.base + (oh * G::OW + ow) * G::CO : g;
-  }
-  __device__ __forceinline__ const bf16* ptr(int m, int kb, int, bool& valid) const { return at(row(m), kb, valid); }
-  __device__ __forceinline__ void load(int m, int kb, int, uint4 (&v)[8]) const {
-    static_assert(G::S == 1 && G::CO == 64, "one tap per K block");
-    m = min(m, M - 1);
-    const int b = m / (G::H * G::W), rem = m % (G::H * G::W), y = rem / G::W, x = rem % G::W;
-    const int oh = y - kb / G::K, ow = x - kb % G::K;
-    if (oh < 0 || oh >= G::OH || ow < 0 || ow >= G::OW) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = make_uint4(0u, 0u, 0u, 0u);
-      return;
-    }
-    const uint4* p = reinterpret_cast<const uint4*>(g + ((size_t)(b * G::OH + oh) * G::OW + ow) * G::CO);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  }
-};
-// stride-2, 4x4 kernel, CO = 64.  Input pixels are split into four parity classes z = (y&1, x&1); a
-// pixel of class z is touched only by the four taps (r, s) = (py + 2i, px + 2j), so each class is its
-// own dense contraction with K = 4 taps x 64 and no structural zeros.  Row m = (state, y>>1, x>>1).
-template <class G> struct DgradSrcS2 {
-  const bf16* g; int M;
-  __device__ __forceinline__ RowRef row(int m) const {
-    constexpr int HH = G::H / 2, WW = G::W / 2;
-    m = min(m, M - 1);
-    const int b = m / (HH * WW), rem = m % (HH * WW), yy = rem / WW, xx = rem % WW;
-    return RowRef{(uint32_t)(b * G::OH * G::OW * G::CO), (yy << 8) | xx};
-  }
-  __device__ __forceinline__ const bf16* at(const RowRef& rr, int kb, bool& valid) const {
-    const int oh = (rr.yx >> 8) - (kb >> 1), ow = (rr.yx & 255) - (kb & 1);
-    valid = oh >= 0 && oh < G::OH && ow >= 0 && ow < G::OW;
-    return valid ? g + rr.base + (oh * G::OW + ow) * G::CO : g;
-  }
-  __device__ __forceinline__ const bf16* ptr(int m, int kb, int, bool& valid) const { return at(row(m), kb, valid); }
-  __device__ __forceinline__ void load(int m, int kb, int, uint4 (&v)[8]) const {
-    static_assert(G::S == 2 && G::K == 4 && G::CO == 64 && G::H % 2 == 0 && G::W % 2 == 0, "parity split");
-    constexpr int HH = G::H / 2, WW = G::W / 2;
-    m = min(m, M - 1);
-    const int b = m / (HH * WW), rem = m % (HH * WW), yy = rem / WW, xx = rem % WW;
-    const int oh = yy - (kb >> 1), ow = xx - (kb & 1);
-    if (oh < 0 || oh >= G::OH || ow < 0 || ow >= G::OW) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = make_uint4(0u, 0u, 0u, 0u);
-      return;
-    }
-    const uint4* p = reinterpret_cast<const uint4*>(g + ((size_t)(b * G::OH + oh) * G::OW + ow) * G::CO);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  }
-};
-// per-class K-major weights w[z][n][k]
-struct ClassWeightSrc {
-  const bf16* w; int ld; int class_stride;
-  __device__ __forceinline__ void load(int n, int kb, int z, uint4 (&v)[8]) const {
-    const uint4* p = reinterpret_cast<const uint4*>(w + (size_t)z * class_stride + (size_t)n * ld + kb * TC_BK);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(p + i);
-  }
-};
+struct BiasReluEpiTc { bf16* out; const float* bias; int ld; float scale; int M; };
 
 // out[m][n] = act[m][n] > 0 ? bf16(acc) : 0     (gradient through the ReLU of the layer below)
-__device__ __forceinline__ void relu_mask_store(bf16* out, const bf16* act, size_t idx, const uint32_t (&r)[32]) {
-  const uint4* a4 = reinterpret_cast<const uint4*>(act + idx);
-  uint4* dst = reinterpret_cast<uint4*>(out + idx);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint4 a = __ldg(a4 + j);
-    const uint32_t aw[4] = {a.x, a.y, a.z, a.w};
-    uint32_t o[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      // stored activations are >= 0, so "positive" is "non-zero bit pattern other than -0"
-      const float lo = (aw[q] & 0x7FFFu) ? __uint_as_float(r[8 * j + 2 * q]) : 0.f;
-      const float hi = (aw[q] & 0x7FFF0000u) ? __uint_as_float(r[8 * j + 2 * q + 1]) : 0.f;
-      o[q] = pack_bf16x2(lo, hi);
-    }
-    dst[j] = make_uint4(o[0], o[1], o[2], o[3]);
-  }
-}
+struct ReluMaskEpiTc { bf16* out; const bf16* act; int ld; int M; };
 // value words (two bf16 each) survive where the activation word's halves are non-zero
 __device__ __forceinline__ uint32_t mask_pair(uint32_t v, uint32_t a) {
   // stored activations are ReLU outputs, never negative: non-zero is the same as greater than zero
   const __nv_bfloat162 a2 = *reinterpret_cast<const __nv_bfloat162*>(&a);
   return v & __hgt2_mask(a2, __floats2bfloat162_rn(0.f, 0.f));
-}
-
-// the same with the 32 activations of the slice already in registers (four 16-byte words)
-__device__ __forceinline__ void relu_mask_store_pre(bf16* out, size_t idx, const uint32_t (&r)[32], const uint4* a4) {
-  uint4* dst = reinterpret_cast<uint4*>(out + idx);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t aw[4] = {a4[j].x, a4[j].y, a4[j].z, a4[j].w};
-    uint32_t o[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float lo = (aw[q] & 0x7FFFu) ? __uint_as_float(r[8 * j + 2 * q]) : 0.f;
-      const float hi = (aw[q] & 0x7FFF0000u) ? __uint_as_float(r[8 * j + 2 * q + 1]) : 0.f;
-      o[q] = pack_bf16x2(lo, hi);
-    }
-    dst[j] = make_uint4(o[0], o[1], o[2], o[3]);
-  }
-}
-template <int BN> struct MaskPre { uint4 m[BN / 8]; size_t idx; bool valid; };
-struct ReluMaskEpiTc {
-  bf16* out; const bf16* act; int ld; int M;
-  __device__ __forceinline__ void operator()(int m, int n0, int, const uint32_t (&r)[32]) const {
-    if (m >= M) return;
-    relu_mask_store(out, act, (size_t)m * ld + n0, r);
-  }
-  // two-step form: fetch the BN activations of row m starting at column n0 early, use them later
-  template <class P> __device__ __forceinline__ void prefetch(int m, int n0, P& p) const {
-    p.valid = m < M;
-    p.idx = (size_t)m * ld + n0;
-    if (!p.valid) return;
-    const uint4* a4 = reinterpret_cast<const uint4*>(act + p.idx);
-#pragma unroll
-    for (int j = 0; j < (int)(sizeof(p.m) / sizeof(uint4)); ++j)
-      if (n0 + 8 * j < ld) p.m[j] = __ldg(a4 + j);          // a ragged last tile stops at the end of the row
-  }
-  template <class P> __device__ __forceinline__ void store(int col, const uint32_t (&r)[32], const P& p) const {
-    if (p.valid) relu_mask_store_pre(out, p.idx + col, r, &p.m[col / 8]);
-  }
-};
-// same for the stride-2 layer, whose four parity classes share one A operand and are laid side by side
-// along N: column n belongs to class n / C, channel n % C, and goes back to input pixel
-// (2 yy + class / 2, 2 xx + class % 2)
-template <class G> struct ReluMaskEpiS2 {
-  bf16* out; const bf16* act; int M;
-  __device__ __forceinline__ void operator()(int m, int n0, int, const uint32_t (&r)[32]) const {
-    static_assert(G::C == 32, "one class per 32-column slice");
-    if (m >= M) return;
-    constexpr int HH = G::H / 2, WW = G::W / 2;
-    const int cls = n0 / G::C;
-    const int b = m / (HH * WW), rem = m % (HH * WW), yy = rem / WW, xx = rem % WW;
-    const int y = 2 * yy + (cls >> 1), x = 2 * xx + (cls & 1);
-    relu_mask_store(out, act, ((size_t)(b * G::H + y) * G::W + x) * G::C, r);
-  }
-};
-
-// ---- the kernel ----------------------------------------------------------------------------------------
-template <class ASrc, class BSrc, class Epi, int BN, int STAGES>
-__global__ void __launch_bounds__(TC_THREADS)
-tc_gemm_kernel(ASrc a_src, BSrc b_src, Epi epi, int num_kb, uint32_t* error_word) {
-  pdl_entry();
-  static_assert(BN == 32 || BN == 64 || BN == 128, "tile width");
-  constexpr uint32_t A_BYTES = TC_BM * 128, B_BYTES = BN * 128, STAGE_BYTES = A_BYTES + B_BYTES;
-  extern __shared__ uint8_t dyn_smem[];
-  __shared__ TcShared sh;
-  const uint32_t tiles = (smem_u32(dyn_smem) + 1023u) & ~1023u;      // swizzle groups need 1024-byte alignment
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.x * TC_BM, n0 = blockIdx.y * BN, z = blockIdx.z;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) { mbar_init(&sh.full[s], 4); mbar_init(&sh.empty[s], 1); }
-    mbar_init(&sh.acc, 1);
-    sh.abort = 0u;
-    fence_barrier_init();
-  }
-  if (warp == 4) tmem_alloc(&sh.tmem_base, BN);
-  tcgen05_fence_before();
-  __syncthreads();
-  tcgen05_fence_after();
-  const uint32_t tmem = sh.tmem_base;
-
-  if (warp < 4) {
-    // ---------------- producers ----------------
-    const int row = threadIdx.x;                 // tile row owned by this thread
-    for (int kb = 0; kb < num_kb; ++kb) {
-      const int s = kb % STAGES;
-      uint4 va[8], vb[8];
-      a_src.load(m0 + row, kb, z, va);
-      if (row < BN) b_src.load(n0 + row, kb, z, vb);
-      // all lanes wait on the same phase; leave the loop together or not at all
-      const bool ok = mbar_wait(&sh.empty[s], ((kb / STAGES) & 1) ^ 1, &sh.abort, error_word, ERR_WAIT_EMPTY);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      const uint32_t a_base = tiles + s * STAGE_BYTES, b_base = a_base + A_BYTES;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const uint32_t off = sw128_offset(row, c);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a_base + off), "r"(va[c].x), "r"(va[c].y),
-                     "r"(va[c].z), "r"(va[c].w) : "memory");
-        if (row < BN)
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_base + off), "r"(vb[c].x), "r"(vb[c].y),
-                       "r"(vb[c].z), "r"(vb[c].w) : "memory");
-      }
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.full[s]);
-    }
-    // ---------------- epilogue ----------------
-    if (mbar_wait(&sh.acc, 0, &sh.abort, error_word, ERR_WAIT_ACC)) {
-      tcgen05_fence_after();
-#pragma unroll 1
-      for (int c = 0; c < BN / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld_32x32(tmem + ((uint32_t)(warp * 32) << 16) + c * 32, r);
-        epi(m0 + row, n0 + c * 32, z, r);
-      }
-    }
-  } else if (lane == 0) {
-    // ---------------- MMA issuer ----------------
-    constexpr uint32_t idesc = make_idesc_bf16(TC_BM, BN, 0, 0);
-    bool ok = true;
-    for (int kb = 0; kb < num_kb && ok; ++kb) {
-      const int s = kb % STAGES;
-      ok = mbar_wait(&sh.full[s], (kb / STAGES) & 1, &sh.abort, error_word, ERR_WAIT_FULL);
-      if (!ok) break;
-      tcgen05_fence_after();
-      const uint32_t a_base = tiles + s * STAGE_BYTES, b_base = a_base + A_BYTES;
-#pragma unroll
-      for (int k = 0; k < TC_BK / 16; ++k) {
-        const uint64_t ad = make_smem_desc(a_base + k * 32, 0, 1024, SWIZZLE_128B);
-        const uint64_t bd = make_smem_desc(b_base + k * 32, 0, 1024, SWIZZLE_128B);
-        mma_bf16(tmem, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
-      }
-      mma_commit(&sh.empty[s]);
-    }
-    if (ok) mma_commit(&sh.acc);
-  }
-  tcgen05_fence_before();
-  __syncthreads();
-  if (warp == 4) {
-    __syncwarp();
-    tcgen05_fence_after();
-    tmem_dealloc(tmem, BN);
-  }
 }
 
 // ---- persistent variant: weights resident in shared memory, A streamed by tiled bulk copies -------------
@@ -531,7 +192,7 @@ struct PkShared {
   volatile uint32_t abort;
 };
 
-template <class ASrc, class Epi, int BN, int KB, int NCLS, int STAGES, int KPS>
+template <class Epi, int BN, int KB, int NCLS, int STAGES, int KPS>
 __global__ void __launch_bounds__(PK_THREADS, 1)
 tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_a, const bf16* __restrict__ w, int n_total, Epi epi, int tiles_m,
                      uint32_t* error_word) {
@@ -1855,15 +1516,12 @@ static int tc_fc_forward_cluster(LaunchCtx& lc, const bf16* a, const bf16* w, co
   return !ok ? 0 : (tiles_m * (N / 64) <= room ? N / 64 : (tiles_m * (N / 128) <= room ? N / 128 : N / 256));
 }
 
-// ---- first layer, forward: uint8 frames -> bf16 operand on the fly --------------------------------------
-// Same persistent skeleton, with eight producer warps: the frame rows a tile needs are copied once into
-// shared memory with cp.async (two tiles ahead); thread (row, half) then expands window rows
-// 4*half .. 4*half+3 of its output pixel to bf16 into the two K blocks it owns.  Integers 0..255 are exact in bf16: the bytes are
-// spliced into floats 2^23 + n, 2^23 is subtracted, and the upper halves of two results are packed.
-// The forward kernel of the first layer multiplies in fp16 instead: a byte n placed in the low half of a 16-bit word
-// IS the fp16 subnormal n * 2^-24, so the expansion is two byte permutations per four pixels and nothing else (the
-// logic pipe that runs them was the kernel's bound with the ten instructions of the bf16 route).  Its weights are the
-// bf16 weights times 2^8 as fp16 (exact down to 2^-25); the epilogue's scale carries the 2^16 / 255.
+// ---- first layer, forward: uint8 frames -> fp16 operand on the fly --------------------------------------
+// Same persistent skeleton; eight warps expand the frame rows a tile needs, copied once into shared memory, block by block
+// (see the space-to-depth view below).  A byte n placed in the low half of a 16-bit word IS the fp16 subnormal n * 2^-24, so
+// the expansion is two byte permutations per four pixels and nothing else (ten instructions per four pixels, for bf16
+// integers, made the logic pipe that runs them the kernel's bound).  Its weights are the bf16 weights times 2^8 as fp16 (exact
+// down to 2^-25); the epilogue's scale carries the 2^16 / 255.
 __device__ __forceinline__ void u8x4_to_f16x4(uint32_t w, uint32_t& lo, uint32_t& hi) {
   lo = __byte_perm(w, 0u, 0x4140);
   hi = __byte_perm(w, 0u, 0x4342);
@@ -1878,14 +1536,6 @@ constexpr float C1_F16_WEIGHT_SCALE = 256.f, C1_F16_OUTPUT_SCALE = 16777216.f / 
 constexpr float C1_GRAD_SCALE = 18446744073709551616.f;                       // 2^64
 constexpr float C1_WGRAD_OUTPUT_SCALE = 590295810358705651712.f / 255.f;      // 2^69 / 255
 constexpr float C1_BIAS_OUTPUT_SCALE = 1.f / C1_GRAD_SCALE;
-__device__ __forceinline__ void u8x4_to_bf16x4(uint32_t w, uint32_t& lo, uint32_t& hi) {
-  const float f0 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440)) - 8388608.f;
-  const float f1 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7441)) - 8388608.f;
-  const float f2 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7442)) - 8388608.f;
-  const float f3 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7443)) - 8388608.f;
-  lo = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-  hi = __byte_perm(__float_as_uint(f2), __float_as_uint(f3), 0x7632);
-}
 
 // Space-to-depth view: with stride 4 and an 8 x 8 kernel, the window of output (oh, ow) is the 2 x 2 group of
 // 4 x 4-pixel blocks (oh + i, ow + j), i, j in {0, 1}.  A block is 4 x 4 x 4 channels = 64 values = one 128-byte
@@ -2167,13 +1817,13 @@ static int sm_count() {
   return n;
 }
 
-template <class ASrc, class Epi, int BN, int KB, int NCLS, int STAGES, int KPS>
-static void tc_persistent(LaunchCtx& lc, int kid, ASrc a, const bf16* w, int n_total, Epi e, int M, uint32_t* err) {
+template <class Epi, int BN, int KB, int NCLS, int STAGES, int KPS>
+static void tc_persistent(LaunchCtx& lc, int kid, PlainSrc a, const bf16* w, int n_total, Epi e, int M, uint32_t* err) {
   const CUtensorMap* tm_a = tc_tensor_map(a.x, (uint64_t)a.M, (uint64_t)KB * TC_BK, (uint64_t)a.ld, TC_BM);
   if (tm_a == nullptr) { lc.host_failure = true; return; }      // no tensor-map encoder: the API call reports PAAC_ERR_CUDA
   constexpr int smem = NCLS * KB * BN * 128 + STAGES * KPS * TC_BM * 128 + 4 * 32 * BN * 2 + 1024;      // weights, stages, staging tiles
   static_assert(smem <= 227 * 1024, "shared memory budget");
-  auto kern = tc_persistent_kernel<ASrc, Epi, BN, KB, NCLS, STAGES, KPS>;
+  auto kern = tc_persistent_kernel<Epi, BN, KB, NCLS, STAGES, KPS>;
   static bool configured = false;
   if (!configured) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -2258,20 +1908,6 @@ static void tc_conv1(LaunchCtx& lc, const uint8_t* frames, const bf16* w_blocks,
   launch_kernel_overlapped(lc, kern, gx, C1_THREADS, smem, frames, w_blocks, e, n_states, tiles, err);
 }
 
-template <class ASrc, class BSrc, class Epi, int BN, int STAGES>
-static void tc_gemm(LaunchCtx& lc, int kid, ASrc a, BSrc b, Epi e, int M, int N, int num_kb, int Z, uint32_t* error_word) {
-  constexpr int smem = STAGES * (TC_BM * 128 + BN * 128) + 1024;
-  auto kern = tc_gemm_kernel<ASrc, BSrc, Epi, BN, STAGES>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    configured = true;
-  }
-  KernelScope scope(lc, kid);
-  dim3 grid((M + TC_BM - 1) / TC_BM, N / BN, Z);
-  launch_kernel_overlapped(lc, kern, grid, TC_THREADS, smem, a, b, e, num_kb, error_word);
-}
-
 constexpr int FC_SPLITS = 7;
 size_t tc_fc_scratch_floats(int n) { return (size_t)FCC_MAX_SPLITS * n * 512 + (size_t)FCC_MAX_PARTS * n * FCC_HP_LD; }
 
@@ -2347,38 +1983,17 @@ void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, 
 // its float partial tile to scratch; tc_finalize_grads_kernel adds the partials in a fixed order.
 constexpr int WG_ROWS = 64;
 
-// G rows: BN (64 or 128) bf16 starting at column n0; rows past M read as zero so that the tail of the last
-// block adds nothing.  VALID < 64 pads a narrower matrix (conv1: 32 channels) with zero columns.
-template <int VALID> struct GradSrc {
-  const bf16* g; int ld; int M;
-  __device__ __forceinline__ const bf16* ptr(int m, int n0, bool& valid) const {
-    valid = m < M;
-    return valid ? g + (size_t)m * ld + n0 : g;
-  }
-  __device__ __forceinline__ void load(int m, int n0, uint4 (&v)[8]) const {
-    if (m >= M) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = make_uint4(0u, 0u, 0u, 0u);
-      return;
-    }
-    const uint4* p = reinterpret_cast<const uint4*>(g + (size_t)m * ld + n0);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = i < VALID / 8 ? __ldg(p + i) : make_uint4(0u, 0u, 0u, 0u);
-  }
-};
-
-template <class XSrc, class GSrc, int VALID_N, int JT, int BN, int STAGES>
+// Operands are plain row-major matrices: one thread fetches a stage as 64 x 64 boxes (rows and columns outside read as zeros,
+// so the tail of the last block adds nothing).
+template <int JT, int BN, int STAGES>
 __global__ void __launch_bounds__(TC_THREADS)
-tc_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_g, XSrc x_src, GSrc g_src,
-                float* __restrict__ partial, float* __restrict__ bias_partial, int n_atoms, int J, int CO, int num_blocks,
-                int blocks_per_split, uint32_t* error_word) {
-  // plain row-major matrices: one thread fetches a stage as 64 x 64 boxes (rows and columns outside read as zeros)
-  constexpr bool TMA = XSrc::ASYNC && VALID_N == 64;
+tc_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_g, float* __restrict__ partial,
+                float* __restrict__ bias_partial, int J, int CO, int num_blocks, int blocks_per_split, uint32_t* error_word) {
   static_assert(BN == 64 || BN == 128, "tile width");
   static_assert(JT == 1 || JT == 2, "row tiles per CTA");
   constexpr uint32_t ATOM_COL = WG_ROWS * 128;                      // 8 KB: one atom column of a stage
   constexpr uint32_t A_BYTES = 2 * JT * ATOM_COL, B_BYTES = (BN / 64) * ATOM_COL, STAGE_BYTES = A_BYTES + B_BYTES;
-  constexpr int A_PER_HALF = JT, B_COLS = BN / 64;
+  constexpr int B_COLS = BN / 64;
   extern __shared__ uint8_t dyn_smem[];
   __shared__ TcShared sh;
   const uint32_t tiles = (smem_u32(dyn_smem) + 1023u) & ~1023u;
@@ -2392,9 +2007,10 @@ tc_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
   const uint32_t ones_base = tiles + STAGES * STAGE_BYTES;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) { mbar_init(&sh.full[s], TMA ? 1 : 4); mbar_init(&sh.empty[s], 1); }
+    for (int s = 0; s < STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
     mbar_init(&sh.acc, 1);
-    if (TMA) { tma_prefetch_desc(&tm_x); tma_prefetch_desc(&tm_g); }
+    tma_prefetch_desc(&tm_x);
+    tma_prefetch_desc(&tm_g);
     sh.abort = 0u;
     fence_barrier_init();
   }
@@ -2415,51 +2031,20 @@ tc_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
   pdl_entry();          // everything above touches only this CTA's own resources and weights that are several kernels old
 
   if (warp < 4) {
-    // ---------------- producers: thread = (row of the block, half) ----------------
-    const int row = threadIdx.x & 63, half = threadIdx.x >> 6;
-    const uint32_t row_off = (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * 128u;
+    // ---------------- producer ----------------
     for (int kb = kb0; kb < kb1; ++kb) {
       const int it = kb - kb0, s = it % STAGES;
       const bool ok = mbar_wait(&sh.empty[s], ((it / STAGES) & 1) ^ 1, &sh.abort, error_word, ERR_WAIT_EMPTY);
       if (!__all_sync(0xffffffffu, ok)) break;
       const uint32_t a_base = tiles + s * STAGE_BYTES, b_base = a_base + A_BYTES;
-      const int m = kb * WG_ROWS + row;
-      if constexpr (TMA) {
-        if (threadIdx.x == 0) {
-          mbar_arrive_expect_tx(&sh.full[s], STAGE_BYTES);
+      if (threadIdx.x == 0) {
+        mbar_arrive_expect_tx(&sh.full[s], STAGE_BYTES);
 #pragma unroll
-          for (int col = 0; col < 2 * JT; ++col)
-            tma_load_2d(a_base + col * ATOM_COL, &tm_x, (atom0 + col) * 64, kb * WG_ROWS, &sh.full[s]);
+        for (int col = 0; col < 2 * JT; ++col)
+          tma_load_2d(a_base + col * ATOM_COL, &tm_x, (atom0 + col) * 64, kb * WG_ROWS, &sh.full[s]);
 #pragma unroll
-          for (int gc = 0; gc < B_COLS; ++gc)
-            tma_load_2d(b_base + gc * ATOM_COL, &tm_g, n0 + gc * 64, kb * WG_ROWS, &sh.full[s]);
-        }
-      } else {
-        uint4 v[8];
-#pragma unroll
-        for (int q = 0; q < A_PER_HALF; ++q) {
-          const int col = half * A_PER_HALF + q;                      // atom column inside the stage
-          const int atom = atom0 + col;
-          if (atom < n_atoms) x_src.load(m, atom, 0, v);
-          else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = make_uint4(0u, 0u, 0u, 0u);
-          }
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a_base + col * ATOM_COL + row_off +
-                         ((uint32_t)(c ^ (row & 7)) << 4)), "r"(v[c].x), "r"(v[c].y), "r"(v[c].z), "r"(v[c].w) : "memory");
-        }
-        if (half < B_COLS) {
-          g_src.load(m, n0 + half * 64, v);
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_base + half * ATOM_COL + row_off +
-                         ((uint32_t)(c ^ (row & 7)) << 4)), "r"(v[c].x), "r"(v[c].y), "r"(v[c].z), "r"(v[c].w) : "memory");
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.full[s]);
+        for (int gc = 0; gc < B_COLS; ++gc)
+          tma_load_2d(b_base + gc * ATOM_COL, &tm_g, n0 + gc * 64, kb * WG_ROWS, &sh.full[s]);
       }
     }
     // ---------------- epilogue: float partial tile to scratch ----------------
@@ -2693,11 +2278,11 @@ static size_t wg_scratch_floats(int rows, int J, int CO, int tiles_yz) {
   return (size_t)splits * J * CO + (size_t)splits * CO;
 }
 
-template <class XSrc, class GSrc, int JT, int BN, int STAGES, int CO>
-static void tc_wgrad(LaunchCtx& lc, int kid, XSrc xs, GSrc gs, int rows, int n_atoms, float scale,
+template <int JT, int BN, int STAGES>
+static void tc_wgrad(LaunchCtx& lc, int kid, PlainSrc xs, PlainSrc gs, int rows, int n_atoms, int CO, float scale,
                      float* gw, float* gb, float* scratch, GradSegments* segs, uint32_t* err) {
   constexpr int smem = STAGES * ((2 * JT + BN / 64) * WG_ROWS * 128) + 2 * WG_ROWS * 128 + 1024;
-  auto kern = tc_wgrad_kernel<XSrc, GSrc, (CO < 64 ? CO : 64), JT, BN, STAGES>;
+  auto kern = tc_wgrad_kernel<JT, BN, STAGES>;
   static bool configured = false;
   if (!configured) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -2710,10 +2295,10 @@ static void tc_wgrad(LaunchCtx& lc, int kid, XSrc xs, GSrc gs, int rows, int n_a
   const int splits = (num_blocks + bps - 1) / bps;
   float* bias_part = scratch + (size_t)splits * J * CO;
   const CUtensorMap* tm_x = tc_tensor_map(xs.x, (uint64_t)xs.M, (uint64_t)J, (uint64_t)xs.ld, WG_ROWS);
-  const CUtensorMap* tm_g = tc_tensor_map(gs.g, (uint64_t)gs.M, (uint64_t)CO, (uint64_t)gs.ld, WG_ROWS);
+  const CUtensorMap* tm_g = tc_tensor_map(gs.x, (uint64_t)gs.M, (uint64_t)CO, (uint64_t)gs.ld, WG_ROWS);
   if (tm_x == nullptr || tm_g == nullptr) { lc.host_failure = true; return; }      // no tensor-map encoder
   KernelScope scope(lc, kid);
-  launch_kernel_overlapped(lc, kern, dim3(splits, gy, gz), TC_THREADS, smem, *tm_x, *tm_g, xs, gs, scratch, bias_part, n_atoms, J, CO,
+  launch_kernel_overlapped(lc, kern, dim3(splits, gy, gz), TC_THREADS, smem, *tm_x, *tm_g, scratch, bias_part, J, CO,
                            num_blocks, bps, err);
   if (!add_grad_segment(segs, scratch, gw, splits, J, CO, scale) || !add_grad_segment(segs, bias_part, gb, splits, 1, CO, 1.f))
     lc.host_failure = true;
@@ -3303,8 +2888,8 @@ void tc_backward_wgrad(LaunchCtx& lc, const NetDims& nd, const uint8_t* frames, 
     tc_shift_wgrad<C3FwdCfg, GradCells<81, 9, 7, 7>, 5>(lc, KID_CONV3_WGRAD, C3FwdCfg{(const bf16*)act[1], n * 81}, g, n, n * 81,
                                                         gw, gb, sc, &segs, err);
   } else {
-    tc_wgrad<PlainSrc, GradSrc<64>, 2, 128, 4, 512>(lc, KID_FC_WGRAD, PlainSrc{(const bf16*)act[2], 3136, n},
-                                                    GradSrc<64>{g, 512, n}, n, 49, 1.f, gw, gb, sc, &segs, err);
+    tc_wgrad<2, 128, 4>(lc, KID_FC_WGRAD, PlainSrc{(const bf16*)act[2], 3136, n}, PlainSrc{g, 512, n}, n, 49, 512, 1.f, gw, gb, sc, &segs,
+                        err);
   }
 }
 
@@ -3502,7 +3087,7 @@ void launch_wait_probe(LaunchCtx& lc, uint32_t max_polls, uint32_t* error_word) 
 // ---- backward: data gradients ---------------------------------------------------------------------------
 void tc_backward_dgrad_fc(LaunchCtx& lc, const bf16* images, int n, void* const act[], void* const gact[], uint32_t* err) {
   const bf16* wfc_t = images + 4 * 32 * 256 + 64 * 576;
-  tc_persistent<PlainSrc, ReluMaskEpiTc, 128, 8, 1, 2, 2>(
+  tc_persistent<ReluMaskEpiTc, 128, 8, 1, 2, 2>(
       lc, KID_FC_DGRAD, PlainSrc{(const bf16*)gact[3], 512, n}, wfc_t, 3136,
       ReluMaskEpiTc{(bf16*)gact[2], (const bf16*)act[2], 3136, n}, n, err);
 }

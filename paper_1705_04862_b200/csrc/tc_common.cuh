@@ -7,8 +7,7 @@ namespace paac {
 namespace tc {
 
 constexpr uint32_t ERR_WAIT_FULL = 1u, ERR_WAIT_EMPTY = 2u, ERR_WAIT_ACC = 4u;
-// the three bits above: a bounded wait gave up (PAAC_ERR_TIMEOUT)
-constexpr uint32_t ERR_WAIT_ANY = 7u;
+// (a bounded wait gave up: PAAC_ERR_TIMEOUT, see DEV_ERR_WAIT_MASK)
 // A healthy wait ends within microseconds.  try_wait itself suspends the thread for a
 // hardware time slice, so this cap is of the order of a second before the kernel gives up.
 constexpr uint32_t WAIT_POLLS = 4000000u;
