@@ -16,8 +16,9 @@
  *     attributes) that are neither locked nor keyed by device: one calling thread and one device per
  *     process (paac_init on a second device returns PAAC_ERR_STATE).  Calls must follow
  *     init -> (rollout -> update)*.
- *   - Work is enqueued on the stream given at init; calls that return data to the
- *     host synchronise that stream, the others do not.
+ *   - Work is enqueued on the stream given at init (paac_update forks some kernels to a stream of the
+ *     library's own and joins it again); calls that return data to the host wait for the work that
+ *     produces it, the others do not.
  *   - Indices: t in [0, t_max) is the step inside the current rollout, e in [0, n_e)
  *     the environment, i = t*n_e + e the experience inside the update batch of
  *     B = n_e*t_max.  Frames are uint8 [84][84][4] (row, column, channel).
@@ -184,13 +185,16 @@ int paac_act_host(paac_ctx* ctx, int t, const uint8_t* frames /* host */, int32_
  * newest), oldest first.  Where restart[e] != 0 (host, [n_e], nullable = no restarts) environment e has begun a new
  * episode and the new frame fills all four channels.  t = 1 .. t_max (step 0 of a rollout has no new frame: it is the
  * state of the call before, see paac_act_host); calls of the two kinds may be mixed within a rollout.  Copies a
- * quarter of the bytes paac_act_host copies.  Errors as paac_act_host. */
+ * quarter of the bytes paac_act_host copies.  Planes at a 16-byte aligned address, all of them inside one pinned
+ * allocation or registration, are read in place over the link; others are copied first.  Either way they may be
+ * overwritten once the call has returned.  Errors as paac_act_host. */
 int paac_act_host_newest(paac_ctx* ctx, int t, const uint8_t* newest /* host */, const uint8_t* restart /* host, nullable */,
                          int32_t* actions /* host, out */, float* values /* host, out, nullable */);
 
 /* Outcome of the actions of step t, observed on the host: rewards in {-1,0,1} and
  * terminal flags, [n_e] each.  After step t_max-1 and the bootstrap paac_act_host(t_max),
- * paac_update() may be called. */
+ * paac_update() may be called.  A step that is not reported keeps the rewards and terminal flags the learner's
+ * buffers hold for it (zeros at first).  The arrays are copied before the call returns. */
 int paac_observe_host(paac_ctx* ctx, int t, const int8_t* rewards /* host */, const uint8_t* terminals /* host */);
 
 /* Frame pre-processing of Section 5.1 for real emulators feeding the external-environment mode: of the raw
@@ -204,8 +208,8 @@ int paac_observe_host(paac_ctx* ctx, int t, const int8_t* rewards /* host */, co
  *   state_in            device uint8 [n][84][84][4], nullable: the states before this step; NULL (after a reset):
  *                       the new frame fills all four channels
  *   state_out           device uint8 [n][84][84][4]; may be the same buffer as state_in
- *   n in [1, 65535]; stream: cudaStream_t.  Asynchronous; allocates nothing.  Integer arithmetic: results are
- *   the same bits on any machine. */
+ *   n in [1, 65535]; stream: cudaStream_t of the current device, which may be any (no context is involved).
+ *   Asynchronous; allocates nothing.  Integer arithmetic: results are the same bits on any machine. */
 int paac_preprocess(const uint8_t* raw_prev /* device */, const uint8_t* raw_last /* device */,
                     const uint8_t* state_in /* device, nullable */, uint8_t* state_out /* device */, int n, void* stream);
 
@@ -333,7 +337,9 @@ int paac_profile_read(paac_ctx* ctx, int max_entries, const char** names /* out 
  *   theta_bf16   device, nullable: bfloat16 bits of the new theta, [n]
  *   norm_and_scale  device float[2], nullable: gradient norm before clipping, factor applied (0 when
  *                   the norm was not finite and nothing was changed)
- *   stream       cudaStream_t; the two kernels are enqueued on it, the call does not synchronise
+ *   stream       cudaStream_t; the work is enqueued on it (one kernel up to 8192 parameters, else two, the second of
+ *                which may start while the first runs, whatever PAAC_OPT_DEPENDENT_LAUNCH says), the call does not
+ *                synchronise
  *
  * n may not exceed paac_noalloc_max_params() (16,777,216): beyond that the call returns PAAC_ERR_LIMIT
  * and does nothing.  The first call on each device looks up the device address of the built-in array

@@ -29,11 +29,12 @@ static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_
   launch_kernel(lc, wgrad_reduce_kernel, blocks, 256, 0, part, splits, part_rows, row0, rows, cols, scale, gw, gb);
 }
 
-// Shapes of the CUDA-core contraction for N columns (16, 32, or 64 and more).  Measured at 128 states forward and 640
-// backward on the larger network (TMAC/s, of 36 the multiply-add pipe could do; every shape ends near 20, at 75 % of the
-// issue slots): the wide shape (8 x 8 per lane for 64 columns, 8 x 4 below, where 8 x 8 leaves tiles of too many rows) wins
-// from two warps per scheduler on (1184 of them; 19.8 against 18.4), below that 4 x 4 (18.4 against 12.2 with one and a half),
-// and 2 x 4 where even that leaves a scheduler without a warp (592).  4 x 4 with 64 columns comes in blocks of two warps: the
+// Shapes of the CUDA-core contraction for N columns (16, 32, or 64 and more).  At 128 states forward and 640 backward the
+// larger network's layers run at 9 to 14 and 13 to 20 TMAC/s of the 36 the multiply-add pipe could do, with 54 to 65 and 58 to
+// 82 % of the issue slots busy.  The wide shape (8 x 8 per lane for 64 columns, 8 x 4 below, where 8 x 8 leaves tiles of too
+// many rows) wins from two warps per scheduler on (1184 of them; 19.8 against 18.4 TMAC/s for the fully connected layer's
+// weight gradient), below that 4 x 4 (18.4 against 12.2 with one and a half), and 2 x 4 where even that leaves a scheduler
+// without a warp (592).  4 x 4 with 64 columns comes in blocks of two warps: the
 // second layer's 10368 rows then fill the device in more even rounds (34 -> 30 us, the third layer's 6272 the same).
 constexpr int FF_SMS = 148;
 static size_t ff_heads_scratch_floats(const NetDims& nd, int n);

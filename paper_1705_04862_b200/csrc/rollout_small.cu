@@ -12,8 +12,8 @@
 // Arithmetic is that of the layer-by-layer path to the bit: one chain of fused multiply-adds per output in ascending k,
 // 128-long runs of the fully connected layer added in double.
 //
-// What bounds a step: latency; two barriers over 148 blocks (about 1.4 us each), one over the group, and five passes of one
-// to three microseconds: 15 us a step for 4 states and 22 us for 32, against 22 and 36 us for the launches it replaces
+// What bounds a step: latency; two barriers over 148 blocks and one over the group (1.3 us each by themselves), and five
+// passes of one to three microseconds: 15 us a step for 4 states and 22 us for 32, against 22 and 36 us for the launches it replaces
 // (4 environments, five steps and the bootstrap: 131 -> 94 us; 32: 215 -> 137 us).
 //
 // Every wait is bounded: a block that gives up raises the error word and leaves, and so, one after the other, do all.
