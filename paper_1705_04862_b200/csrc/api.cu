@@ -97,6 +97,8 @@ struct paac_ctx {
   uint8_t* terminals;
   DeviceStats* stats;
   uint32_t* barriers;      // of the one-launch rollout
+  uint4* words;            // and what its blocks hand each other (larger network)
+  size_t n_words;
   size_t elt;              // bytes of one stored activation element
 };
 
@@ -173,6 +175,8 @@ size_t carve(paac_ctx* c, char* base) {
   c->stats = k.take<DeviceStats>(1);
   c->step_dev = k.take<uint64_t>(1);
   c->barriers = k.take<uint32_t>(rollout_small_barrier_words((int)n_e));
+  c->n_words = tc_supported(c->arch, c->prec) ? rollout_tc_words((int)n_e) : 0;
+  c->words = k.take<uint4>(c->n_words);
   return (k.off + 255) & ~(size_t)255;
 }
 
@@ -198,7 +202,11 @@ void refresh_weight_copies(paac_ctx* c, bool cast) {
   if (tc_supported(c->arch, c->prec)) tc_relayout_weights(c->lc, c->nd, c->theta16, c->w_images, &c->stats->error_word);
 }
 
-// `steps` forward passes from slot t0 on in one launch (rollout_small_supported()); a rollout with `env`, else one pass
+// whether a rollout's forward passes go in one launch
+bool one_launch(const paac_ctx* c) {
+  return use_tc(c) ? rollout_tc_supported(c->n_e, c->A) : rollout_small_supported(c->lc, c->arch, c->prec, c->n_e);
+}
+// `steps` forward passes from slot t0 on in one launch (one_launch()); a rollout with `env`, else one pass
 void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sample_steps, const EnvStepArgs* env, bool advance) {
   void* act[MAX_LAYERS];
   for (int l = 0; l <= c->nd.n_conv; ++l)
@@ -210,9 +218,10 @@ void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sa
   r.logits = c->logits + row * c->A; r.values = c->values + row; r.uniforms = c->uniforms + row; r.actions = c->actions + row;
   r.sampled = c->sampled + row; r.forced = c->forced_on ? c->forced + row : nullptr;
   r.seed = c->seed; r.step_base = c->step_dev; r.advance = advance ? (uint32_t)c->t_max : 0u;
-  r.mode = head_mode(c); r.error_word = &c->stats->error_word;
+  r.mode = head_mode(c); r.error_word = &c->stats->error_word; r.words = c->words;
   if (env) r.env = *env;
-  launch_rollout_small(c->lc, c->prec, c->nd, c->theta, c->theta16, r);
+  if (use_tc(c)) launch_rollout_tc(c->lc, c->nd, c->theta, c->theta16, c->w_images, r);
+  else launch_rollout_small(c->lc, c->prec, c->nd, c->theta, c->theta16, r);
 }
 
 // network + heads on the n_e states of `frames`, activations into slot `slot`.  With `tail` the caller is about
@@ -226,7 +235,7 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
   for (int l = 0; l <= c->nd.n_conv; ++l)
     act[l] = (char*)c->act[l] + (size_t)slot * c->n_e * c->nd.layer[l].out_size * c->elt;
   const size_t row = (size_t)slot * c->n_e;
-  if (rollout_small_supported(c->lc, c->arch, c->prec, c->n_e)) {
+  if (one_launch(c)) {
     small_rollout(c, frames, slot, 1, sample ? 1 : 0, nullptr, advanced && !sample);
     if (advanced) *advanced = !sample;
     return false;
@@ -481,7 +490,7 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
   uint8_t* nxt = c->frames[c->cur ^ 1];
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
   run_recorded(c, 0, c->cur, [&]() {
-    if (rollout_small_supported(c->lc, c->arch, c->prec, c->n_e)) {
+    if (one_launch(c)) {
       const EnvStepArgs env{c->hp.term_denom, nxt, c->rewards, c->terminals, c->counters, pattern_actions(c)};
       small_rollout(c, fr, 0, c->t_max + 1, c->t_max, &env, true);
       return;
@@ -893,9 +902,11 @@ int paac_debug_write(paac_ctx* c, int which, const void* src, size_t bytes) {
   if (send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (cudaMemcpyAsync(p, src, b, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
-  // a wait that gave up may have left the one-launch rollout's barriers half full: clearing the error word resets them
+  // a wait that gave up may have left the one-launch rollout's barriers half full: clearing the error word resets them, and
+  // with the count of steps the words that carry it
   if (which == PAAC_DBG_ERROR_WORD &&
-      cudaMemsetAsync(c->barriers, 0, rollout_small_barrier_words(c->n_e) * sizeof(uint32_t), c->st) != cudaSuccess) {
+      (cudaMemsetAsync(c->barriers, 0, rollout_small_barrier_words(c->n_e) * sizeof(uint32_t), c->st) != cudaSuccess ||
+       cudaMemsetAsync(c->words, 0, c->n_words * sizeof(uint4), c->st) != cudaSuccess)) {
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
   return PAAC_OK;

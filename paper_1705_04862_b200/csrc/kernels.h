@@ -151,12 +151,23 @@ struct SmallRollout {
   const uint8_t* frames; size_t frame_step;     // states of slot t0, bytes from one slot to the next
   void* const* act;                             // stored activations of slot t0, by layer
   float* part; uint32_t* barriers;
+  void* words;                                  // larger network: rollout_tc_words() of 16 bytes
   float *logits, *values, *uniforms; int32_t *actions, *sampled; const int32_t* forced;      // of slot t0
   uint64_t seed; uint64_t* step_base; uint32_t advance;      // > 0: added to the step index at the end
   HeadMode mode; EnvStepArgs env;               // env.next_frames: the state after the last step; rewards, terminals of slot t0
   uint32_t* error_word;
 };
 void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const SmallRollout& r);
+
+// ---- the same for the larger network in bf16 (rollout_tc.cu) ----------
+bool rollout_tc_supported(int n, int n_actions);
+size_t rollout_tc_words(int n);                 // of 16 bytes; zero before the first launch and where the barriers are set to zero
+void launch_rollout_tc(LaunchCtx& lc, const NetDims& nd, const float* theta, const bf16* theta16, const bf16* images, const SmallRollout& r);
+// what that file shares with the layer-by-layer path: the first layer's fp16 weights in `images`, the scale of their sums, and
+// the number of slices of K that path adds up for n states
+const void* tc_conv1_weights(const bf16* images);
+float tc_conv1_scale();
+int tc_fc_slices(int n);
 
 // ---- optimiser (optim.cu) -------------------------------------------------------------------
 constexpr int NORM_BLOCKS = 1184;

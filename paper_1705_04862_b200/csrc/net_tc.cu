@@ -1934,6 +1934,9 @@ static void tc_fc_forward(LaunchCtx& lc, const bf16* a, const bf16* w, const flo
 }
 
 // ---- forward ---------------------------------------------------------------------------------------------
+const void* tc_conv1_weights(const bf16* images) { return images + TC_IMG_W1; }
+float tc_conv1_scale() { return C1_F16_OUTPUT_SCALE; }
+int tc_fc_slices(int n) { return tc_fc_cluster_splits((n + TC_BM - 1) / TC_BM * (512 / FCC_MAX_BN)); }
 bool tc_supported(int arch, int prec) { return arch == PAAC_ARCH_NATURE && prec == PAAC_BF16; }
 
 void tc_forward(LaunchCtx& lc, int arch, const NetDims& nd, const float* theta, const bf16* w, const bf16* images,
