@@ -11,13 +11,11 @@
 using namespace paac;
 
 // Pinned memory both sides see.  Results the host waits for are stored there by the kernel that ends a launch sequence
-// and picked up by polling a flag: no copy engine, no stream synchronisation.  The pointers let a recorded sequence
-// read buffers that differ from call to call.
+// and picked up by polling a flag: no copy engine, no stream synchronisation.
 struct HostBox {
   volatile uint32_t done;                       // set by the device when actions and values (or the statistics) are there
-  HostPlanes planes;                            // the newest frames and the restart flags of the step in flight
   DeviceStats stats;
-  int32_t* actions; float* values; uint8_t* restart;      // [n_e] each, behind this struct
+  int32_t* actions; float* values;              // [n_e] each, behind this struct
   uint8_t* outcomes;                            // rewards and terminal flags, laid out as on the device (outcome_bytes());
                                                 // only the steps in paac_ctx::observed hold anything
 };
@@ -72,9 +70,8 @@ struct paac_ctx {
   // once into a CUDA graph and replayed from then on.  Anything that changes the sequence drops the graphs.
   bool graphs_on;          // option: allow recording
   SideSet side;            // incomplete if it could not be had: everything then stays on the learner's stream
-  // recorded launch sequences: kind 0 = rollout, 1 = update, 2 = update that reports, 3 + 2 t + v = step t of the external-environment mode
-  // (v = 1: with the frame stack built on the device), each for both parities of the frame buffers
-  static constexpr int GRAPH_KINDS = 3 + 2 * 65;
+  // recorded launch sequences: kind 0 = rollout, 1 = update, 2 = update that reports, 3 + t = step t of the external-environment mode, each for both parities of the frame buffers
+  static constexpr int GRAPH_KINDS = 3 + 65;
   int plain_calls[GRAPH_KINDS][2];   // calls made with plain launches
   cudaGraphExec_t graph[GRAPH_KINDS][2];
   uint64_t graph_launches[GRAPH_KINDS][2];
@@ -207,7 +204,8 @@ bool one_launch(const paac_ctx* c) {
   return use_tc(c) ? rollout_tc_supported(c->n_e, c->A) : rollout_small_supported(c->lc, c->arch, c->prec, c->n_e);
 }
 // `steps` forward passes from slot t0 on in one launch (one_launch()); a rollout with `env`, else one pass
-void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sample_steps, const EnvStepArgs* env, bool advance) {
+void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sample_steps, const EnvStepArgs* env, bool advance,
+                   const HostStep* host = nullptr) {
   void* act[MAX_LAYERS];
   for (int l = 0; l <= c->nd.n_conv; ++l)
     act[l] = (char*)c->act[l] + (size_t)t0 * c->n_e * c->nd.layer[l].out_size * c->elt;
@@ -220,6 +218,7 @@ void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sa
   r.seed = c->seed; r.step_base = c->step_dev; r.advance = advance ? (uint32_t)c->t_max : 0u;
   r.mode = head_mode(c); r.error_word = &c->stats->error_word; r.words = c->words;
   if (env) r.env = *env;
+  if (host) r.host = *host;
   if (use_tc(c)) launch_rollout_tc(c->lc, c->nd, c->theta, c->theta16, c->w_images, r);
   else launch_rollout_small(c->lc, c->prec, c->nd, c->theta, c->theta16, r);
 }
@@ -277,11 +276,11 @@ size_t outcome_bytes(const paac_ctx* c) { return (size_t)((const char*)c->termin
 void make_box(paac_ctx* c) {
   const size_t n = c->n_e, head = (sizeof(HostBox) + 255) / 256 * 256;
   void* p = nullptr;
-  if (cudaHostAlloc(&p, head + n * 9 + outcome_bytes(c), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return; }
+  if (cudaHostAlloc(&p, head + n * 8 + outcome_bytes(c), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return; }
   c->box = new (p) HostBox{};
   char* q = (char*)p + head;
   c->box->actions = (int32_t*)q; c->box->values = (float*)(q + 4 * n);
-  c->box->restart = (uint8_t*)(q + 8 * n); c->box->outcomes = (uint8_t*)(q + 9 * n);
+  c->box->outcomes = (uint8_t*)(q + 8 * n);
 }
 // Waits for the flag that the last kernel of a launch sequence sets; a failed launch or kernel shows in the stream's
 // status instead.
@@ -733,20 +732,29 @@ int paac_profile_read(paac_ctx* c, int max_entries, const char** names, double* 
 }
 
 // ---- external-environment mode ------------------------------------------------------------------
-// The network on the state at `dst`, with `prev` after the frame stack has built that state, and the results into the
-// box: one launch sequence, recorded from the second time on.
-static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, uint8_t* dst, int32_t* actions, float* values) {
+// The network on the state at `dst`, with `prev` after the frame stack has built that state from `planes`, and the results into the
+// box.  The frame stack's arguments differ from step to step, so it is launched by itself; the rest is one launch sequence,
+// recorded from the second time on, or, for few environments, part of the same kernel.
+static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, uint8_t* dst, int32_t* actions,
+                           float* values) {
   const bool sample = t < c->t_max;
   const size_t row = (size_t)t * c->n_e;
   HostBox* box = c->box;
   box->done = 0u;
-  run_recorded(c, 3 + 2 * t + (prev ? 1 : 0), c->cur, [&]() {
-    if (prev) launch_stack_pull(c->lc, prev, &box->planes, dst, c->n_e);
-    bool advanced = false;
-    forward_slot(c, dst, t, sample, nullptr, sample ? nullptr : &advanced);
-    if (!sample && !advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
-    launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
-  });
+  if (use_tc(c) && one_launch(c)) {
+    HostStep host{prev, planes, {0u, 0u, 0u}, box->actions, box->values, &box->done};
+    if (restart)
+      for (int e = 0; e < c->n_e; ++e) host.fresh[e >> 5] |= (uint32_t)(restart[e] != 0) << (e & 31);
+    small_rollout(c, dst, t, 1, sample ? 1 : 0, nullptr, !sample, &host);
+  } else {
+    if (prev) launch_stack_pull(c->lc, prev, planes, restart, dst, c->n_e);
+    run_recorded(c, 3 + t, c->cur, [&]() {
+      bool advanced = false;
+      forward_slot(c, dst, t, sample, nullptr, sample ? nullptr : &advanced);
+      if (!sample && !advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
+      launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
+    });
+  }
   if (!await_box(c)) return PAAC_ERR_CUDA;
   if (sample) memcpy(actions, box->actions, c->n_e * sizeof(int32_t));
   if (values) memcpy(values, box->values, c->n_e * sizeof(float));
@@ -769,7 +777,7 @@ int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, f
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
   if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
-  return act_host_finish(c, t, nullptr, dst, actions, values);
+  return act_host_finish(c, t, nullptr, nullptr, nullptr, dst, actions, values);
 }
 
 // what the driver knows of a host address (its entry point is looked up at run time: nothing links to libcuda)
@@ -805,14 +813,11 @@ int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_
   // Pinned planes (16-byte aligned, all of them in one allocation) are read over the link by the kernel that builds the states, which saves the copy's
   // set-up, its hand-over to the first kernel and a round trip through device memory; others are copied first.
   const uint8_t* view = ((uintptr_t)newest & 15u) == 0 ? host_view(newest, plane, query_host_range) : nullptr;
-  c->box->planes.newest = view ? view : c->newest;
-  c->box->planes.restart = restart ? c->box->restart : nullptr;
-  if (restart) memcpy(c->box->restart, restart, c->n_e);
   if (!view && cudaMemcpyAsync(c->newest, newest, plane, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
   if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
-  return act_host_finish(c, t, prev, dst, actions, values);
+  return act_host_finish(c, t, prev, view ? view : c->newest, restart, dst, actions, values);
 }
 
 int paac_observe_host(paac_ctx* c, int t, const int8_t* rewards, const uint8_t* terminals) {

@@ -127,6 +127,7 @@ __device__ __forceinline__ int warp_finish_heads(const HeadMode hm, float z, flo
   int a = A - 1;
   bool found = false;
   // eight at a time, so that only the additions wait for one another; past the last action p = 0 and c stays what it is
+#pragma unroll 1
   for (int k0 = 0; k0 < A; k0 += 8) {
     float pk[8];
 #pragma unroll

@@ -66,4 +66,22 @@ __device__ __forceinline__ void env_write_frame(const EnvFrame f, uint8_t* frame
   for (int q = threadIdx.x; q < FRAME_WORDS / 4; q += THREADS) out[q] = env_frame_quad(f, (uint32_t)q, pattern_actions);
 }
 
+// Sixteen pixels of a frame stack: out = (three newest channels of prev, the plane's pixel), or four copies of the pixel for a fresh one.
+constexpr int STACK_ITEMS = FRAME_H * FRAME_W / 16;
+static_assert(STACK_ITEMS * 16 == FRAME_H * FRAME_W, "whole 16-byte words");
+__device__ __forceinline__ void stack_sixteen(const uint4 plane, bool fresh, const uint4* prev, uint4* out) {
+  const uint32_t w[4] = {plane.x, plane.y, plane.z, plane.w};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint4 o;
+    if (fresh) {
+      o = make_uint4((w[q] & 0xFFu) * 0x01010101u, ((w[q] >> 8) & 0xFFu) * 0x01010101u, ((w[q] >> 16) & 0xFFu) * 0x01010101u, (w[q] >> 24) * 0x01010101u);
+    } else {
+      const uint4 p = prev[q];
+      o = make_uint4((p.x >> 8) | (w[q] << 24), (p.y >> 8) | ((w[q] >> 8) << 24), (p.z >> 8) | ((w[q] >> 16) << 24), (p.w >> 8) | ((w[q] >> 24) << 24));
+    }
+    out[q] = o;
+  }
+}
+
 }  // namespace paac

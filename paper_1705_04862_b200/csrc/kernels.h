@@ -27,11 +27,14 @@ void launch_env_step_sampling(LaunchCtx& lc, uint64_t seed, int n_e, const uint6
                               const HeadsTail& ht, int pattern_actions = 0);
 
 // ---- external-environment mode (preprocess.cu) --------------------------------------------
-// The newest plane of every environment, [n][84][84] at a 16-byte aligned address, and restart flags [n] (nullable): both
-// may be pinned host memory.  The struct itself is read by the kernel too, so a recorded launch can be pointed elsewhere.
-struct HostPlanes { const uint8_t* newest; const uint8_t* restart; };
-// frame stack: out = (three newest channels of prev, newest plane), or four copies of the plane where restart[e] != 0
-void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const HostPlanes* planes, uint8_t* out, int n);
+// what a one-launch step of the external-environment mode does beside the network: the frame stack (newest != nullptr: the step's
+// states = prev's three newest channels and the planes, four copies of the plane where fresh has the environment's bit), and
+// actions (where sampled) and values to pinned memory, then *done = 1
+struct HostStep { const uint8_t* prev; const uint8_t* newest; uint32_t fresh[3]; int32_t* actions; float* values; volatile uint32_t* done; };
+// frame stack: out = (three newest channels of prev, newest plane), or four copies of the plane where restart[e] != 0.  planes: the
+// newest plane of every environment, [n][84][84] at a 16-byte aligned address, may be pinned host memory; restart: in host
+// memory (nullable), read before the call returns
+void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, uint8_t* out, int n);
 // actions (nullable) and values of n environments to pinned host memory, then *done = 1
 void launch_publish(LaunchCtx& lc, const int32_t* actions, const float* values, int n, int32_t* host_actions, float* host_values,
                     volatile uint32_t* done);
@@ -154,6 +157,7 @@ struct SmallRollout {
   void* words;                                  // larger network: rollout_tc_words() of 16 bytes
   float *logits, *values, *uniforms; int32_t *actions, *sampled; const int32_t* forced;      // of slot t0
   uint64_t seed; uint64_t* step_base; uint32_t advance;      // > 0: added to the step index at the end
+  HostStep host;
   HeadMode mode; EnvStepArgs env;               // env.next_frames: the state after the last step; rewards, terminals of slot t0
   uint32_t* error_word;
 };

@@ -1,6 +1,6 @@
 // Frame pre-processing (Section 5.1 of the paper): per-pixel maximum of the two latest raw frames, pixel intensity,
 // 210 x 160 -> 84 x 84, newest channel of the four-frame state.  Integer arithmetic throughout.
-#include "common.cuh"
+#include "env_device.cuh"
 #include "kernels.h"
 #include "per_device.h"
 
@@ -152,55 +152,41 @@ stack_push_kernel(const uint8_t* prev, const uint8_t* __restrict__ newest, const
 
 // The same for the external-environment mode, sixteen pixels per thread and all of a thread's plane words asked for before
 // any is used: they come over the host link, whose latency is a microsecond or two and whose bandwidth (about 50 GB/s) is
-// what bounds the kernel from a few dozen environments on.
-constexpr int PULL_ITEMS = FRAME_H * FRAME_W / 16, PULL_AHEAD = 3, PULL_BLOCKS = 592;
-static_assert(PULL_ITEMS * 16 == FRAME_H * FRAME_W, "whole 16-byte words");
+// what bounds the kernel from a few dozen environments on.  Which stacks start afresh comes as a launch argument, as does
+// where the planes are: read by every block from pinned memory, they cost 130 ns a block (reads of one address are served
+// one after the other) and as much for every warp's flags (1024 environments: 158 us, 147 without; 32: 10 us, 3 within rollout_tc_kernel).
+constexpr int PULL_AHEAD = 3, PULL_BLOCKS = 592, PULL_ENVS = 2048;
+struct PullFresh { uint32_t bits[PULL_ENVS / 32]; };
 __global__ void __launch_bounds__(SP_THREADS)
-stack_pull_kernel(const uint8_t* prev, const HostPlanes* planes, uint8_t* out, int n) {
-  __shared__ HostPlanes from;
+stack_pull_kernel(const uint8_t* prev, const uint8_t* planes, const __grid_constant__ PullFresh fresh, uint8_t* out, int n) {
   pdl_entry();
-  if (threadIdx.x == 0) from = *planes;
-  __syncthreads();
-  const uint32_t items = (uint32_t)n * PULL_ITEMS, stride = gridDim.x * SP_THREADS;
-  const uint4* newest = reinterpret_cast<const uint4*>(from.newest);
+  const uint32_t items = (uint32_t)n * STACK_ITEMS, stride = gridDim.x * SP_THREADS;
+  const uint4* newest = reinterpret_cast<const uint4*>(planes);
   for (uint32_t base = blockIdx.x * SP_THREADS + threadIdx.x; base < items; base += PULL_AHEAD * stride) {
     uint4 v[PULL_AHEAD];
-    bool fresh[PULL_AHEAD];
 #pragma unroll
-    for (int u = 0; u < PULL_AHEAD; ++u) {
-      const uint32_t i = base + u * stride;
-      if (i < items) {
-        v[u] = newest[i];
-        fresh[u] = from.restart != nullptr && from.restart[i / PULL_ITEMS] != 0;
-      }
-    }
+    for (int u = 0; u < PULL_AHEAD; ++u)
+      if (base + u * stride < items) v[u] = newest[base + u * stride];
 #pragma unroll
     for (int u = 0; u < PULL_AHEAD; ++u) {
       const uint32_t i = base + u * stride;
       if (i >= items) break;
-      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-      const uint4* src = reinterpret_cast<const uint4*>(prev) + (size_t)i * 4;
-      uint4* dst = reinterpret_cast<uint4*>(out) + (size_t)i * 4;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint4 o;
-        if (fresh[u]) {
-          o = make_uint4((w[q] & 0xFFu) * 0x01010101u, ((w[q] >> 8) & 0xFFu) * 0x01010101u, ((w[q] >> 16) & 0xFFu) * 0x01010101u,
-                         (w[q] >> 24) * 0x01010101u);
-        } else {
-          const uint4 p = src[q];
-          o = make_uint4((p.x >> 8) | (w[q] << 24), (p.y >> 8) | ((w[q] >> 8) << 24), (p.z >> 8) | ((w[q] >> 16) << 24),
-                         (p.w >> 8) | ((w[q] >> 24) << 24));
-        }
-        dst[q] = o;
-      }
+      const uint32_t e = i / STACK_ITEMS;
+      stack_sixteen(v[u], (fresh.bits[e >> 5] >> (e & 31u)) & 1u, reinterpret_cast<const uint4*>(prev) + (size_t)i * 4, reinterpret_cast<uint4*>(out) + (size_t)i * 4);
     }
   }
 }
-void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const HostPlanes* planes, uint8_t* out, int n) {
-  const size_t blocks = ((size_t)n * PULL_ITEMS + SP_THREADS - 1) / SP_THREADS;
-  KernelScope scope(lc, KID_ENV_STEP);
-  launch_kernel(lc, stack_pull_kernel, dim3(blocks < PULL_BLOCKS ? (unsigned)blocks : PULL_BLOCKS), dim3(SP_THREADS), 0, prev, planes, out, n);
+void launch_stack_pull(LaunchCtx& lc, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, uint8_t* out, int n) {
+  for (int e0 = 0; e0 < n; e0 += PULL_ENVS) {
+    const int count = n - e0 < PULL_ENVS ? n - e0 : PULL_ENVS;
+    PullFresh fresh{};
+    if (restart)
+      for (int e = 0; e < count; ++e) fresh.bits[e >> 5] |= (uint32_t)(restart[e0 + e] != 0) << (e & 31);
+    const size_t blocks = ((size_t)count * STACK_ITEMS + SP_THREADS - 1) / SP_THREADS, at = (size_t)e0 * FRAME_BYTES;
+    KernelScope scope(lc, KID_ENV_STEP);
+    launch_kernel(lc, stack_pull_kernel, dim3(blocks < PULL_BLOCKS ? (unsigned)blocks : PULL_BLOCKS), dim3(SP_THREADS), 0, prev + at,
+                  planes + at / FRAME_C, fresh, out + at, count);
+  }
 }
 
 // one block: a few kilobytes of posted writes over the host link, made visible before the flag

@@ -29,6 +29,12 @@
 // operands from shared memory at 128 bytes a clock), 0.8 and 0.5 handing the maps over, 2 in the fully connected layer, 0.9 waiting for
 // the other slices, 0.5 with the heads and 1.2 with the draw and the transition.
 //
+// With environments outside, a step is one such launch too: while the weights come in, each block of a cluster fetches its share of the
+// environment's newest plane over the host link and writes its share of the state, and the environment's action and value go straight
+// into pinned memory, the flag behind them set by the block that ends last.  Where the planes lie and which stacks start afresh are
+// launch arguments: read from pinned memory by every block, they took 16 us each (reads of one address are served one after
+// the other).
+//
 // Every wait for a word is bounded.  A block that gives up raises the error word and goes on without waiting (its cluster
 // waits for it at barriers), so that all blocks end.
 #include <cuda_fp16.h>
@@ -40,7 +46,7 @@
 namespace paac {
 
 typedef NatConv1 TC1; typedef NatConv2 TC2; typedef NatConv3 TC3;
-constexpr int RT_THREADS = 512, RT_WARPS = RT_THREADS / 32, RT_MAX_ENVS = 4;        // environments of a cluster
+constexpr int RT_THREADS = 512, RT_WARPS = RT_THREADS / 32, RT_MAX_ENVS = 1;        // environments of a cluster
 constexpr int RT_F = 512, RT_SLICES = 8, RT_TILE = 32, RT_FC_BLOCKS = RT_SLICES * (RT_F / RT_TILE), RT_ROWS = 64;
 constexpr int RT_POS3 = TC3::OH * TC3::OW, RT_FC_LD = 7 * 128;                      // 49 blocks of 64 k, six or seven to a slice
 constexpr uint32_t RT_POLLS = 2000000u;
@@ -67,6 +73,7 @@ struct RtArgs {
   uint64_t seed; uint64_t* step_base; uint32_t advance;
   uint32_t term_denom; int pattern_actions;
   HeadMode mode;
+  HostStep host;                                  // external environments (one pass)
   uint32_t* error_word;
 };
 
@@ -281,6 +288,13 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
   const int half = rank / STEP, low = rank % STEP;
   auto unit_of = [&](int col) { return half * 256 + 64 * (col / (4 * S::RUNS)) + 4 * ((col / 4 % S::RUNS) * STEP + low) + (col & 3); };
 
+  // the newest plane comes over the host link meanwhile: sixteen pixels to a thread
+  const int px_lo = STACK_ITEMS * rank / C, px_hi = STACK_ITEMS * (rank + 1) / C;
+  static_assert((STACK_ITEMS + C - 1) / C <= RT_THREADS && RT_MAX_ENVS == 1, "one piece to a thread");
+  uint4 plane{};
+  const bool pulls = q.host.newest != nullptr && envs > 0 && px_lo + tid < px_hi;
+  if (pulls) plane = reinterpret_cast<const uint4*>(q.host.newest)[(size_t)cluster * STACK_ITEMS + px_lo + tid];
+
   // ---- what stays for the rollout ----
   if (tid == 0) {
     s_dead = 0u; s_epoch = q.sync[0];
@@ -319,10 +333,15 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
     }
   tc::cp_async_commit();
   const uint64_t step0 = *q.step_base + q.t0;
+  if (pulls) {
+    const size_t at = (size_t)cluster * STACK_ITEMS + px_lo + tid;
+    stack_sixteen(plane, (q.host.fresh[cluster >> 5] >> (cluster & 31)) & 1u, reinterpret_cast<const uint4*>(q.host.prev) + 4 * at,
+                  reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames)) + 4 * at);
+  }
   tc::cp_async_wait<0>();
   __syncthreads();
   const uint32_t epoch = s_epoch;
-  rt_cluster_sync();                           // the other blocks have started: their shared memory may be written
+  rt_cluster_sync();                           // the other blocks have started: their shared memory may be written (and the state is there)
   uint32_t phase = 0u;                         // of the maps' barriers
   // this block's share of a map, complete here, to the others; then wait for theirs
   auto exchange = [&](uint64_t* bar, uint32_t at, uint32_t bytes) {
@@ -573,6 +592,11 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
       const int32_t a = warp_finish_heads(q.mode, lane < A ? s : -INFINITY, __shfl_sync(0xffffffffu, s, A), lane, A, (size_t)e, q.logits + slot * A,
                                           q.values + slot, sample, q.seed, step0 + t, q.forced ? q.forced + slot : nullptr, q.actions + slot,
                                           q.sampled + slot, q.uniforms + slot);
+      if (q.host.done != nullptr && rank == 0 && lane == 0) {
+        if (sample) q.host.actions[e] = a;
+        q.host.values[e] = q.values[slot + e];
+        __threadfence_system();
+      }
       if (stepping && lane == 0) {
         const EnvPrep prep = s_prep[ei];
         const EnvOutcome o = env_outcome(prep, a, q.term_denom, q.pattern_actions);
@@ -588,10 +612,12 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
   rt_cluster_sync();
   // Every block has read the counts when the last one ends.
   if (tid == 0) {
+    __threadfence();
     if (atomicAdd(q.sync + 1, 1u) == gridDim.x - 1) {
       q.sync[0] = epoch + (uint32_t)q.steps;
       q.sync[1] = 0u;
       if (q.advance) *q.step_base += q.advance;
+      if (q.host.done != nullptr) { __threadfence_system(); *q.host.done = 1u; }
     }
   }
 }
@@ -649,7 +675,7 @@ void launch_rollout_tc(LaunchCtx& lc, const NetDims& nd, const float* theta, con
   q.maps = (uint4*)r.words; q.sums = q.maps + rt_map_words(r.n); q.sync = r.barriers;
   q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
   q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
-  q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode; q.error_word = r.error_word;
+  q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode; q.host = r.host; q.error_word = r.error_word;
   lc.serialize_next = false;
   KernelScope scope(lc, KID_SMALL_ROLLOUT);
   const bool launched = rt_pick(r.n, [&](auto k) {

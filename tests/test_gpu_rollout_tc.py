@@ -42,3 +42,38 @@ def test_same_bits_as_layer_by_layer(A, hp):
                 x, y = x.reshape(slots, n, -1), y.reshape(slots, LAYERED, -1)[:, :n]
                 assert np.array_equal(x.view(np.uint8), np.ascontiguousarray(y).view(np.uint8)), (n, it, w, float(np.mean(x != y)))
 
+
+
+@pytest.mark.parametrize("n_e,ring", [(1, True), (33, True), (64, False), (74, True)])
+def test_outside_environments_same_bits_as_layer_by_layer(n_e, ring):
+    """Steps of the external-environment mode in one launch (planes read from pinned memory, or copied first) against the states they
+    should build and against the layer-by-layer kernels, restarts included; two iterations without sending step 0 again."""
+    import torch
+    T, A = 3, 6
+    gen = torch.Generator().manual_seed(n_e)
+    small, large = (pb.Paac("nature", n, T, A, seed=5, precision=pb.BF16, term_denom=3) for n in (n_e, LAYERED))
+    first = torch.randint(0, 256, (LAYERED, 84, 84, 4), dtype=torch.uint8, generator=gen)
+    state = first.clone()
+    acts = [np.zeros(n, np.int32) for n in (n_e, LAYERED)]
+    vals = [np.zeros(n, np.float32) for n in (n_e, LAYERED)]
+    for it in range(2):
+        for t in range(T + 1):
+            if t == 0:
+                for i, (g, n) in enumerate(((small, n_e), (large, LAYERED))):
+                    g.act_host(0, first[:n].contiguous().pin_memory() if it == 0 else None, acts[i], vals[i])
+            else:
+                planes = torch.randint(0, 256, (LAYERED, 84, 84), dtype=torch.uint8, generator=gen)
+                ends = (torch.rand(LAYERED, generator=gen) < 0.3).to(torch.uint8)
+                pushed = torch.cat([state[..., 1:], planes[..., None]], dim=-1)
+                state = torch.where(ends[:, None, None, None] != 0, planes[..., None].expand(-1, -1, -1, 4), pushed).contiguous()
+                for i, (g, n) in enumerate(((small, n_e), (large, LAYERED))):
+                    mine = planes[:n].contiguous()
+                    g.act_host_newest(t, mine.pin_memory() if ring else mine.numpy(), ends[:n].numpy().copy(), acts[i] if t < T else None, vals[i])
+            assert np.array_equal(vals[0].view(np.uint32), vals[1][:n_e].view(np.uint32)), (it, t)
+            if t < T:
+                assert np.array_equal(acts[0], acts[1][:n_e]), (it, t)
+                for g, n in ((small, n_e), (large, LAYERED)):
+                    g.observe_host(t, np.zeros(n, np.int8), np.zeros(n, np.uint8))
+        assert np.array_equal(small.debug_read(pb.DBG_NEXT_FRAMES), state[:n_e].numpy().reshape(-1))
+    assert small.error_word() == 0 and large.error_word() == 0
+    small.close(), large.close()
