@@ -113,6 +113,7 @@ __device__ __forceinline__ int warp_finish_heads(const HeadMode hm, float z, flo
     if (forced != nullptr && forced[e] >= 0) a = forced[e];
     const float qa = __shfl_sync(0xffffffffu, z, a);
     if (lane == 0) { sampled[e] = drawn; actions[e] = a; uniforms[e] = u; values[e] = qa; }
+    asm volatile("" : "+r"(a));
     return a;
   }
   if (lane == 0) values[e] = v;
@@ -141,6 +142,10 @@ __device__ __forceinline__ int warp_finish_heads(const HeadMode hm, float z, flo
   const int drawn = a;
   if (forced != nullptr && forced[e] >= 0) a = forced[e];
   if (lane == 0) { sampled[e] = drawn; actions[e] = a; uniforms[e] = u; }
+  // The action is a value of the whole warp.  Where the caller uses it in one lane only, the search for it was otherwise moved into
+  // that lane's branch, 1.6 us a step (a rollout of the smaller network 94 -> 84 us for 4 states, 131 -> 122 for 32; of the larger
+  // one in float for 32 states 331 -> 322).
+  asm volatile("" : "+r"(a));
   return a;
 }
 #endif
