@@ -93,8 +93,8 @@ struct paac_ctx {
   int8_t* rewards;
   uint8_t* terminals;
   DeviceStats* stats;
-  uint32_t* barriers;      // of the one-launch rollout
-  uint4* words;            // and what its blocks hand each other (larger network)
+  uint32_t* sync;          // of the one-launch rollouts: steps so far, blocks that have ended
+  uint4* words;            // and what their blocks hand each other
   size_t n_words;
   size_t elt;              // bytes of one stored activation element
 };
@@ -159,7 +159,6 @@ size_t carve(paac_ctx* c, char* base) {
       sc += c->simt_scratch_off;
       if (tc_fc_scratch_floats((int)n_e) > sc) sc = tc_fc_scratch_floats((int)n_e);
     }
-    if (c->arch == PAAC_ARCH_NIPS && rollout_small_part_floats((int)n_e) > sc) sc = rollout_small_part_floats((int)n_e);
     c->scratch = k.take<float>(sc);
   }
   c->norm_partials = k.take<float>(NORM_BLOCKS);
@@ -171,8 +170,8 @@ size_t carve(paac_ctx* c, char* base) {
   c->terminals = k.take<uint8_t>(B);
   c->stats = k.take<DeviceStats>(1);
   c->step_dev = k.take<uint64_t>(1);
-  c->barriers = k.take<uint32_t>(rollout_small_barrier_words((int)n_e));
-  c->n_words = tc_supported(c->arch, c->prec) ? rollout_tc_words((int)n_e) : 0;
+  c->sync = k.take<uint32_t>(2);
+  c->n_words = tc_supported(c->arch, c->prec) ? rollout_tc_words((int)n_e) : (c->arch == PAAC_ARCH_NIPS ? rollout_small_words((int)n_e) : 0);
   c->words = k.take<uint4>(c->n_words);
   return (k.off + 255) & ~(size_t)255;
 }
@@ -212,7 +211,7 @@ void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sa
   const size_t row = (size_t)t0 * c->n_e;
   SmallRollout r{};
   r.n = c->n_e; r.steps = steps; r.sample_steps = sample_steps; r.t0 = (uint32_t)t0; r.step_env = env != nullptr;
-  r.frames = frames; r.frame_step = (size_t)c->n_e * FRAME_BYTES; r.act = act; r.part = c->scratch; r.barriers = c->barriers;
+  r.frames = frames; r.frame_step = (size_t)c->n_e * FRAME_BYTES; r.act = act; r.sync = c->sync;
   r.logits = c->logits + row * c->A; r.values = c->values + row; r.uniforms = c->uniforms + row; r.actions = c->actions + row;
   r.sampled = c->sampled + row; r.forced = c->forced_on ? c->forced + row : nullptr;
   r.seed = c->seed; r.step_base = c->step_dev; r.advance = advance ? (uint32_t)c->t_max : 0u;
@@ -734,15 +733,15 @@ int paac_profile_read(paac_ctx* c, int max_entries, const char** names, double* 
 // ---- external-environment mode ------------------------------------------------------------------
 // The network on the state at `dst`, with `prev` after the frame stack has built that state from `planes`, and the results into the
 // box.  The frame stack's arguments differ from step to step, so it is launched by itself; the rest is one launch sequence,
-// recorded from the second time on, or, for few environments, part of the same kernel.
-static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, uint8_t* dst, int32_t* actions,
-                           float* values) {
+// recorded from the second time on, or, for few environments, part of the same kernel, which can also fetch whole `states`.
+static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, const uint8_t* states, uint8_t* dst,
+                           int32_t* actions, float* values) {
   const bool sample = t < c->t_max;
   const size_t row = (size_t)t * c->n_e;
   HostBox* box = c->box;
   box->done = 0u;
-  if (use_tc(c) && one_launch(c)) {
-    HostStep host{prev, planes, {0u, 0u, 0u}, box->actions, box->values, &box->done};
+  if (one_launch(c)) {
+    HostStep host{prev, planes, {0u, 0u, 0u}, states, box->actions, box->values, &box->done};
     if (restart)
       for (int e = 0; e < c->n_e; ++e) host.fresh[e >> 5] |= (uint32_t)(restart[e] != 0) << (e & 31);
     small_rollout(c, dst, t, 1, sample ? 1 : 0, nullptr, !sample, &host);
@@ -761,23 +760,6 @@ static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_
   if (t == c->t_max) { c->host_t = 0; c->env_step += c->t_max; c->rollout_fresh = true; c->host_next_valid = true; }
   else c->host_t = t + 1;
   return cuda_status(c);
-}
-
-int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, float* values) {
-  if (c) c->lc.serialize_next = true;
-  if (!c || t < 0 || t > c->t_max || (t < c->t_max && !actions)) return PAAC_ERR_ARG;
-  if (t != c->host_t) return PAAC_ERR_STATE;
-  // s_0 of a rollout is s_{t_max} of the one before (Algorithm 1): those frames are on the device already
-  if (!frames && !(t == 0 && c->host_next_valid)) return PAAC_ERR_ARG;
-  if (!c->box) return PAAC_ERR_CUDA;
-  const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
-  if (t == 0) c->cur ^= 1;
-  uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
-  if (frames && cudaMemcpyAsync(dst, frames, fstep, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
-    cudaGetLastError(); return PAAC_ERR_CUDA;
-  }
-  if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
-  return act_host_finish(c, t, nullptr, nullptr, nullptr, dst, actions, values);
 }
 
 // what the driver knows of a host address (its entry point is looked up at run time: nothing links to libcuda)
@@ -802,6 +784,24 @@ static bool query_host_range(const uint8_t* p, HostRange& r) {
   return true;
 }
 
+int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, float* values) {
+  if (c) c->lc.serialize_next = true;
+  if (!c || t < 0 || t > c->t_max || (t < c->t_max && !actions)) return PAAC_ERR_ARG;
+  if (t != c->host_t) return PAAC_ERR_STATE;
+  // s_0 of a rollout is s_{t_max} of the one before (Algorithm 1): those frames are on the device already
+  if (!frames && !(t == 0 && c->host_next_valid)) return PAAC_ERR_ARG;
+  if (!c->box) return PAAC_ERR_CUDA;
+  const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
+  if (t == 0) c->cur ^= 1;
+  uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
+  const uint8_t* view = frames && one_launch(c) && ((uintptr_t)frames & 15u) == 0 ? host_view(frames, fstep, query_host_range) : nullptr;
+  if (frames && !view && cudaMemcpyAsync(dst, frames, fstep, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
+    cudaGetLastError(); return PAAC_ERR_CUDA;
+  }
+  if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
+  return act_host_finish(c, t, nullptr, nullptr, nullptr, view, dst, actions, values);
+}
+
 int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_t* restart, int32_t* actions, float* values) {
   if (c) c->lc.serialize_next = true;
   if (!c || !newest || t < 1 || t > c->t_max || (t < c->t_max && !actions)) return PAAC_ERR_ARG;
@@ -817,7 +817,7 @@ int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
   if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
-  return act_host_finish(c, t, prev, view ? view : c->newest, restart, dst, actions, values);
+  return act_host_finish(c, t, prev, view ? view : c->newest, restart, nullptr, dst, actions, values);
 }
 
 int paac_observe_host(paac_ctx* c, int t, const int8_t* rewards, const uint8_t* terminals) {
@@ -907,10 +907,9 @@ int paac_debug_write(paac_ctx* c, int which, const void* src, size_t bytes) {
   if (send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
   if (cudaMemcpyAsync(p, src, b, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) { cudaGetLastError(); return PAAC_ERR_CUDA; }
-  // a wait that gave up may have left the one-launch rollout's barriers half full: clearing the error word resets them, and
-  // with the count of steps the words that carry it
+  // a wait that gave up may have left words of the one-launch rollout unwritten: clearing the error word starts them afresh
   if (which == PAAC_DBG_ERROR_WORD &&
-      (cudaMemsetAsync(c->barriers, 0, rollout_small_barrier_words(c->n_e) * sizeof(uint32_t), c->st) != cudaSuccess ||
+      (cudaMemsetAsync(c->sync, 0, 2 * sizeof(uint32_t), c->st) != cudaSuccess ||
        cudaMemsetAsync(c->words, 0, c->n_words * sizeof(uint4), c->st) != cudaSuccess)) {
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }

@@ -28,9 +28,9 @@ void launch_env_step_sampling(LaunchCtx& lc, uint64_t seed, int n_e, const uint6
 
 // ---- external-environment mode (preprocess.cu) --------------------------------------------
 // what a one-launch step of the external-environment mode does beside the network: the frame stack (newest != nullptr: the step's
-// states = prev's three newest channels and the planes, four copies of the plane where fresh has the environment's bit), and
-// actions (where sampled) and values to pinned memory, then *done = 1
-struct HostStep { const uint8_t* prev; const uint8_t* newest; uint32_t fresh[3]; int32_t* actions; float* values; volatile uint32_t* done; };
+// states = prev's three newest channels and the planes, four copies of the plane where fresh has the environment's bit) or
+// whole states from pinned memory (states != nullptr), and actions (where sampled) and values to pinned memory, then *done = 1
+struct HostStep { const uint8_t* prev; const uint8_t* newest; uint32_t fresh[3]; const uint8_t* states; int32_t* actions; float* values; volatile uint32_t* done; };
 // frame stack: out = (three newest channels of prev, newest plane), or four copies of the plane where restart[e] != 0.  planes: the
 // newest plane of every environment, [n][84][84] at a 16-byte aligned address, may be pinned host memory; restart: in host
 // memory (nullable), read before the call returns
@@ -146,15 +146,15 @@ void heads_backward(LaunchCtx& lc, int prec, const NetDims& nd, const float* the
 
 // ---- all forward passes of a rollout in one launch, small batches of the smaller network (rollout_small.cu) ----------
 bool rollout_small_supported(const LaunchCtx& lc, int arch, int prec, int n);      // sizes, and that all its blocks are resident
-size_t rollout_small_part_floats(int n);        // scratch
-size_t rollout_small_barrier_words(int n);      // uint32, zero before the first launch and after a device error
+// what the blocks hand each other, of 16 bytes; all zero, like the two counters of SmallRollout::sync, before the first launch and
+// after a device error
+size_t rollout_small_words(int n);
 struct SmallRollout {
   int n, steps, sample_steps; uint32_t t0;      // passes over slots t0 .. t0 + steps - 1; the first sample_steps sample an action
   bool step_env;                                // ... and step the synthetic environments with it (env)
   const uint8_t* frames; size_t frame_step;     // states of slot t0, bytes from one slot to the next
   void* const* act;                             // stored activations of slot t0, by layer
-  float* part; uint32_t* barriers;
-  void* words;                                  // larger network: rollout_tc_words() of 16 bytes
+  void* words; uint32_t* sync;                  // rollout_small_words() or rollout_tc_words()
   float *logits, *values, *uniforms; int32_t *actions, *sampled; const int32_t* forced;      // of slot t0
   uint64_t seed; uint64_t* step_base; uint32_t advance;      // > 0: added to the step index at the end
   HostStep host;
@@ -165,7 +165,7 @@ void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const floa
 
 // ---- the same for the larger network in bf16 (rollout_tc.cu) ----------
 bool rollout_tc_supported(int n, int n_actions);
-size_t rollout_tc_words(int n);                 // of 16 bytes; zero before the first launch and where the barriers are set to zero
+size_t rollout_tc_words(int n);
 void launch_rollout_tc(LaunchCtx& lc, const NetDims& nd, const float* theta, const bf16* theta16, const bf16* images, const SmallRollout& r);
 // what that file shares with the layer-by-layer path: the first layer's fp16 weights in `images`, the scale of their sums, and
 // the number of slices of K that path adds up for n states

@@ -2,26 +2,33 @@
 //
 // With 1 to 64 states a step of the layer-by-layer path is four launches of 5 us whose work is a fraction of that.  Here one
 // block per SM stays for the rollout and walks its steps.  Environment e belongs to a group of C blocks (C = 16, 8, 4 or
-// 2, as many as fit): each computes its share of the first layer's positions, and after a barrier of the group its share of
+// 2, as many as fit): each computes its share of the first layer's positions, and from the rows that it needs of everybody's its share of
 // the second layer's.  The fully connected layer is where the states meet: 21 runs of 128 inputs x 4 tiles of 64 units are
 // dealt to 84 blocks, whose weight tile stays in shared memory for the whole rollout, so that each step reads only
-// activations; this takes one device-wide barrier before and one after.  Every block of a group then finishes its
+// activations.  Every block of a group then finishes its
 // environment's state by itself (sum over the runs, heads, draw, transition: the same numbers in each), and writes its
 // share of the next frame, of which it keeps the rows its next share of the first layer reads.
 //
 // Arithmetic is that of the layer-by-layer path to the bit: one chain of fused multiply-adds per output in ascending k,
 // 128-long runs of the fully connected layer added in double.
 //
-// What bounds a step: latency; two barriers over 148 blocks and one over the group (1.3 us each by themselves), and five
-// passes of one to three microseconds: 15 us a step for 4 states and 22 us for 32, against 22 and 36 us for the launches it replaces
-// (4 environments, five steps and the bootstrap: 131 -> 94 us; 32: 215 -> 137 us).
+// The blocks hand each other both maps and the runs' sums as words that carry their step (step_words.cuh).  A word of a map is overwritten
+// for the next step only after all that read it have: a block starts a step with the sums of all runs of the one before, which
+// were made from all positions of the second map and they from all rows of the first.  A run's sums, however, need a few positions
+// only, whose blocks may be a step ahead of others of their group, so there are two sets of sums, used in turn: those of a step
+// are overwritten two steps later, when every block of the group has finished it.
 //
-// Every wait is bounded: a block that gives up raises the error word and leaves, and so, one after the other, do all.
+// What bounds a step: latency; three hand-overs of about a microsecond and five passes of one to four: @step
+//
+// With environments outside, a step is one such launch too: each block fetches the part of the state that it needs (or of the newest
+// plane) over the host link and writes its share out; actions and values go straight into pinned memory.
+//
+// Every wait is bounded: a block that gives up raises the error word and goes on without waiting.
 #include <type_traits>
 
 #include "env_device.cuh"
 #include "kernels.h"
-#include "tc_common.cuh"
+#include "step_words.cuh"
 
 namespace paac {
 
@@ -30,7 +37,6 @@ constexpr int RS_TILES = RS_RUNS * (RS_F / RS_COLS), RS_FC_LD = RS_RUN + 4, RS_R
 typedef NipsConv1 RC1;
 typedef NipsConv2 RC2;
 constexpr int RS_POS1 = RC1::OH * RC1::OW, RS_POS2 = RC2::OH * RC2::OW;        // 400 and 81
-constexpr uint32_t RS_POLLS = 2000000u;
 
 struct RsArgs {
   int n, C, A, steps, blocks;             // forward passes: slots t0 .. t0 + steps - 1
@@ -39,7 +45,10 @@ struct RsArgs {
   uint8_t* next_frames;                           // states of the slot after the last one that steps (rollout)
   int sample_steps;                               // of the passes, so many sample an action (and, with `env`, step it)
   bool env;
-  float* part;                                    // [RS_RUNS][n][RS_F]
+  uint4* map1;                                    // words: [n][400][8], two channels each
+  uint4* map2;                                    // [n][81][16]
+  uint2* sums;                                    // [2][RS_RUNS][n][RS_F], by the step's lowest bit
+  uint32_t* sync;
   const float *b1, *b2, *bfc, *bpi, *bv;
   float *logits, *values, *uniforms;
   int32_t *actions, *sampled, *counters;
@@ -48,38 +57,8 @@ struct RsArgs {
   uint64_t seed; uint64_t* step_base; uint32_t advance;
   uint32_t term_denom; int pattern_actions;
   HeadMode mode;
-  unsigned long long* grid_bar; unsigned long long* group_bar;      // arrivals so far: [1], [n]
+  HostStep host;
   uint32_t* error_word;
-};
-
-// A barrier over `count` blocks is a counter of arrivals that only grows, by `count` at every use, so the target of the next
-// use follows from any value read before this block arrives; arriving costs no round trip.  What the blocks wrote before is
-// visible to all after.  false after a bounded wait.
-struct RsBarrier {
-  unsigned long long* arrivals; uint32_t count; unsigned long long target;
-  __device__ __forceinline__ void init(unsigned long long* a, uint32_t c) {
-    arrivals = a; count = c; target = 0;
-    if (threadIdx.x == 0) {
-      const unsigned long long now = *reinterpret_cast<volatile unsigned long long*>(a);
-      target = now - now % c;
-    }
-  }
-  __device__ __forceinline__ bool sync(uint32_t* error_word, int* s_ok) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      target += count;
-      asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(arrivals) : "memory");
-      unsigned long long now;
-      uint32_t polls = 0;
-      do {
-        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(arrivals) : "memory");
-      } while (now < target && ++polls < RS_POLLS);
-      *s_ok = now >= target;
-      if (now < target) atomicOr(error_word, tc::ERR_WAIT_FULL);
-    }
-    __syncthreads();
-    return *s_ok != 0;
-  }
 };
 
 __device__ __forceinline__ void rs_fma4(float (&acc)[4], float a, const float4 w) {
@@ -89,9 +68,17 @@ __device__ __forceinline__ float4 rs_relu(const float (&acc)[4], float scale, co
   return make_float4(fmaxf(fmaf(acc[0], scale, b[0]), 0.f), fmaxf(fmaf(acc[1], scale, b[1]), 0.f), fmaxf(fmaf(acc[2], scale, b[2]), 0.f),
                      fmaxf(fmaf(acc[3], scale, b[3]), 0.f));
 }
-// written by other blocks during this launch: past the first-level cache
-__device__ __forceinline__ float4 rs_load4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float4 rs_load4(const bf16* p) { return widen4(__ldcg(reinterpret_cast<const uint2*>(p))); }
+// four neighbouring outputs: as they are stored, and as words with the value the next layer reads
+__device__ __forceinline__ float4 rs_stored(const float4 v, const float*) { return v; }
+__device__ __forceinline__ float4 rs_stored(const float4 v, const bf16*) {
+  return make_float4(to_f(from_f<bf16>(v.x)), to_f(from_f<bf16>(v.y)), to_f(from_f<bf16>(v.z)), to_f(from_f<bf16>(v.w)));
+}
+template <class T> __device__ __forceinline__ void rs_hand(T* at, uint4* words, const float4 v, uint32_t step) {
+  store4(at, v);
+  const float4 w = rs_stored(v, at);
+  word_store(words, __float_as_uint(w.x), __float_as_uint(w.y), step);
+  word_store(words + 1, __float_as_uint(w.z), __float_as_uint(w.w), step);
+}
 
 // shared memory, in floats
 constexpr int RS_W1 = 0, RS_W2 = RS_W1 + RC1::KK * RC1::CO, RS_FCW = RS_W2 + RC2::KK * RC2::CO, RS_FCA = RS_FCW + RS_COLS * RS_FC_LD,
@@ -101,7 +88,7 @@ constexpr int RS_W1 = 0, RS_W2 = RS_W1 + RC1::KK * RC1::CO, RS_FCW = RS_W2 + RC2
 // convolutions are bound by weights going from shared memory to registers (16 floats a thread for four k, whatever PP is),
 // so PP is as large as leaves every scheduler one warp.
 template <class T, int PP>
-__device__ __forceinline__ void rs_conv1(const float* sm, const float* b1, T* act, int pos0, int share) {
+__device__ __forceinline__ void rs_conv1(const float* sm, const float* b1, T* act, uint4* words, uint32_t step, int pos0, int share) {
   const int q = threadIdx.x & 3, p = threadIdx.x >> 2, apart = (share + PP - 1) / PP;
   const uint32_t* frame = reinterpret_cast<const uint32_t*>(sm + RS_FRAME);
   const float4* w = reinterpret_cast<const float4*>(sm + RS_W1) + q;                   // [k][16]
@@ -129,11 +116,14 @@ __device__ __forceinline__ void rs_conv1(const float* sm, const float* b1, T* ac
     }
 #pragma unroll
   for (int i = 0; i < PP; ++i)
-    if (p < apart && p + apart * i < share) store4(act + (size_t)(pos0 + p + apart * i) * RC1::CO + 4 * q, rs_relu(acc[i], 1.0f / 255.0f, b1 + 4 * q));
+    if (p < apart && p + apart * i < share) {
+      const int pos = pos0 + p + apart * i;
+      rs_hand(act + (size_t)pos * RC1::CO + 4 * q, words + pos * (RC1::CO / 2) + 2 * q, rs_relu(acc[i], 1.0f / 255.0f, b1 + 4 * q), step);
+    }
 }
 // Second layer: the same with 8 groups of 4 channels, the input rows in shared memory.
 template <class T, int PP>
-__device__ __forceinline__ void rs_conv2(const float* sm, const float* b2, T* act, int pos0, int share) {
+__device__ __forceinline__ void rs_conv2(const float* sm, const float* b2, T* act, uint4* words, uint32_t step, int pos0, int share) {
   const int q = threadIdx.x & 7, p = threadIdx.x >> 3, apart = (share + PP - 1) / PP;
   const float4* in = reinterpret_cast<const float4*>(sm + RS_ACT1);                    // [20][20][16]
   const float4* w = reinterpret_cast<const float4*>(sm + RS_W2) + q;                   // [k][32]
@@ -161,7 +151,10 @@ __device__ __forceinline__ void rs_conv2(const float* sm, const float* b2, T* ac
     }
 #pragma unroll
   for (int i = 0; i < PP; ++i)
-    if (p < apart && p + apart * i < share) store4(act + (size_t)(pos0 + p + apart * i) * RC2::CO + 4 * q, rs_relu(acc[i], 1.f, b2 + 4 * q));
+    if (p < apart && p + apart * i < share) {
+      const int pos = pos0 + p + apart * i;
+      rs_hand(act + (size_t)pos * RC2::CO + 4 * q, words + pos * (RC2::CO / 2) + 2 * q, rs_relu(acc[i], 1.f, b2 + 4 * q), step);
+    }
 }
 
 template <class T, class TW, int C>
@@ -171,7 +164,8 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
   __shared__ float xs[RS_F], zs[33];
   __shared__ EnvFrame s_frame;
   __shared__ int32_t s_action;
-  __shared__ int s_ok;
+  __shared__ volatile uint32_t s_dead;
+  __shared__ uint32_t s_epoch;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = q.n, A = q.A;
   const bool conv = (int)blockIdx.x < n * C;
   const int e = blockIdx.x / C, rank = blockIdx.x % C;
@@ -185,19 +179,59 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
   const int row_lo = pos1 / RC1::OW * RC1::S, row_hi = (pos1 + SHARE1 - 1) / RC1::OW * RC1::S + RC1::K;      // frame rows read
   constexpr int IN_ROW = RC1::OW * RC1::CO / 4;                    // 16-byte words of a row of the first layer's map
   const int in_lo = pos2 / RC2::OW * RC2::S * IN_ROW, in_hi = ((pos2 + share2 - 1) / RC2::OW * RC2::S + RC2::K) * IN_ROW;
-  RsBarrier grid, group;
-  grid.init(q.grid_bar, q.blocks);
-  if (conv) group.init(q.group_bar + e, C);
   uint4* frame = reinterpret_cast<uint4*>(sm + RS_FRAME);
   constexpr int QUADS = FRAME_W / 4;                               // 16-byte words of a frame row
 
+  // this block's share of a frame, and the rows of it that its share of the first layer reads
+  const int own_lo = FRAME_WORDS / 4 * rank / C, own_hi = FRAME_WORDS / 4 * (rank + 1) / C;
+  const int part_lo = min(own_lo, row_lo * QUADS), part_hi = max(own_hi, row_hi * QUADS);
+  auto place = [&](uint4* state, int i, const uint4 v) {
+    if (i >= own_lo && i < own_hi) state[i] = v;
+    if (i >= row_lo * QUADS && i < row_hi * QUADS) frame[i] = v;
+  };
+  if (conv && q.host.states != nullptr) {
+    // the whole state over the host link; a thread asks for all its words before it uses any
+    constexpr int MOST = (FRAME_WORDS / 4 + RS_THREADS - 1) / RS_THREADS;
+    const uint4* src = reinterpret_cast<const uint4*>(q.host.states) + (size_t)e * (FRAME_WORDS / 4);
+    uint4* state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
+    uint4 v[MOST];
+#pragma unroll
+    for (int u = 0; u < MOST; ++u)
+      if (part_lo + tid + u * RS_THREADS < part_hi) v[u] = src[part_lo + tid + u * RS_THREADS];
+#pragma unroll
+    for (int u = 0; u < MOST; ++u)
+      if (part_lo + tid + u * RS_THREADS < part_hi) place(state, part_lo + tid + u * RS_THREADS, v[u]);
+  }
+  if (conv && q.host.newest != nullptr) {
+    // or the newest plane, sixteen pixels to a word, onto the stack of the state before
+    constexpr int MOST = (STACK_ITEMS + RS_THREADS - 1) / RS_THREADS;
+    const uint4* src = reinterpret_cast<const uint4*>(q.host.newest) + (size_t)e * STACK_ITEMS;
+    const uint4* prev = reinterpret_cast<const uint4*>(q.host.prev) + (size_t)e * (FRAME_WORDS / 4);
+    uint4* state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
+    const bool fresh = (q.host.fresh[e >> 5] >> (e & 31)) & 1u;
+    uint4 v[MOST];
+#pragma unroll
+    for (int u = 0; u < MOST; ++u)
+      if (part_lo / 4 + tid + u * RS_THREADS < (part_hi + 3) / 4) v[u] = src[part_lo / 4 + tid + u * RS_THREADS];
+#pragma unroll
+    for (int u = 0; u < MOST; ++u) {
+      const int i = part_lo / 4 + tid + u * RS_THREADS;
+      if (i < (part_hi + 3) / 4) {
+        uint4 o[4];
+        stack_sixteen(v[u], fresh, prev + 4 * i, o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) place(state, 4 * i + k, o[k]);
+      }
+    }
+  }
   // what stays for the rollout: both convolutions' weights as [k][channel], the head weights, the weight tile
   if (conv) {
     for (int i = tid; i < RC1::KK * RC1::CO; i += RS_THREADS) sm[RS_W1 + i % RC1::KK * RC1::CO + i / RC1::KK] = to_f(w1[i]);
     for (int i = tid; i < RC2::KK * RC2::CO; i += RS_THREADS) sm[RS_W2 + i % RC2::KK * RC2::CO + i / RC2::KK] = to_f(w2[i]);
     for (int i = tid; i < (A + 1) * RS_F; i += RS_THREADS) sm[RS_HEADW + i] = i < A * RS_F ? to_f(wpi[i]) : to_f(wv[i - A * RS_F]);
-    const uint4* src = reinterpret_cast<const uint4*>(q.frames + (size_t)e * FRAME_BYTES);
-    for (int i = row_lo * QUADS + tid; i < row_hi * QUADS; i += RS_THREADS) frame[i] = __ldcg(src + i);
+    uint4* state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
+    if (q.host.newest == nullptr && q.host.states == nullptr)
+      for (int i = row_lo * QUADS + tid; i < row_hi * QUADS; i += RS_THREADS) frame[i] = __ldcg(state + i);
   }
   if (fc)
     for (int i = tid; i < RS_COLS * RS_RUN; i += RS_THREADS) {
@@ -205,27 +239,44 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
       sm[RS_FCW + c * RS_FC_LD + k] = k < len ? to_f(wfc[(size_t)(col0 + c) * RS_IN + k0 + k]) : 0.f;
     }
   const uint64_t step0 = *q.step_base + q.t0;
+  if (tid == 0) { s_dead = 0u; s_epoch = q.sync[0]; }
   __syncthreads();
+  const uint32_t epoch = s_epoch;
 
   for (int t = 0; t < q.steps; ++t) {
     const size_t slot = (size_t)t * n;
+    const uint32_t tag = epoch + 1u + (uint32_t)t;
+    uint2* sums = q.sums + (size_t)(tag & 1u) * RS_RUNS * n * RS_F;
     if (conv) {
       T* a1 = act1 + (slot + e) * RC1::OUT_SIZE;
       T* a2 = act2 + (slot + e) * RC2::OUT_SIZE;
-      rs_conv1<T, PP1>(sm, q.b1, a1, pos1, SHARE1);
-      if (!group.sync(q.error_word, &s_ok)) return;
-      for (int i = in_lo + tid; i < in_hi; i += RS_THREADS) reinterpret_cast<float4*>(sm + RS_ACT1)[i] = rs_load4(a1 + 4 * i);
+      rs_conv1<T, PP1>(sm, q.b1, a1, q.map1 + (size_t)e * (RS_POS1 * RC1::CO / 2), tag, pos1, SHARE1);
+      {
+        constexpr int MOST = 8;                    // 16-byte words, two values each: at most twelve rows (C = 2)
+        const uint4* src = q.map1 + (size_t)e * (RS_POS1 * RC1::CO / 2) + 2 * in_lo + tid;
+        const int count = (2 * (in_hi - in_lo) - tid + RS_THREADS - 1) / RS_THREADS;
+        uint4 v[MOST];
+        word_await(v, src, RS_THREADS, count, tag, &s_dead, q.error_word);
+#pragma unroll
+        for (int u = 0; u < MOST; ++u)
+          if (u < count) reinterpret_cast<float2*>(sm + RS_ACT1)[2 * in_lo + tid + u * RS_THREADS] = make_float2(__uint_as_float(v[u].x), __uint_as_float(v[u].z));
+      }
       __syncthreads();
-      rs_conv2<T, PP2>(sm, q.b2, a2, pos2, share2);
+      rs_conv2<T, PP2>(sm, q.b2, a2, q.map2 + (size_t)e * (RS_IN / 2), tag, pos2, share2);
     }
-    if (!grid.sync(q.error_word, &s_ok)) return;
     if (fc) {
       for (int r0 = 0; r0 < n; r0 += RS_ROWS) {
         const int rows = min(RS_ROWS, n - r0);
         if (r0 > 0) __syncthreads();
-        for (int i = tid; i < rows * (RS_RUN / 4); i += RS_THREADS) {
-          const int r = i / (RS_RUN / 4), k = i % (RS_RUN / 4) * 4;
-          if (k < len) *reinterpret_cast<float4*>(sm + RS_FCA + r * RS_FC_LD + k) = rs_load4(act2 + (slot + r0 + r) * RS_IN + k0 + k);
+        {
+          // 64 words (two inputs each) to a row of a whole run, 16 to one of the last
+          const int per = len / 2, r = tid / per, u = tid % per, apart = RS_THREADS / per, count = (rows - r + apart - 1) / apart;
+          const uint4* src = q.map2 + (size_t)(r0 + r) * (RS_IN / 2) + k0 / 2 + u;
+          uint4 v[RS_ROWS / 4];
+          word_await(v, src, (size_t)apart * (RS_IN / 2), count, tag, &s_dead, q.error_word);
+#pragma unroll
+          for (int i = 0; i < RS_ROWS / 4; ++i)
+            if (i < count) *reinterpret_cast<float2*>(sm + RS_FCA + (r + apart * i) * RS_FC_LD + 2 * u) = make_float2(__uint_as_float(v[i].x), __uint_as_float(v[i].z));
         }
         __syncthreads();
         const int cx = tid & 15, ry = tid >> 4;
@@ -255,26 +306,24 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
         for (int i = 0; i < 2; ++i)
           if (ry + 16 * i < rows)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) q.part[((size_t)run * n + r0 + ry + 16 * i) * RS_F + col0 + cx + 16 * j] = acc[i][j];
+            for (int j = 0; j < 4; ++j) word_store(sums + ((size_t)run * n + r0 + ry + 16 * i) * RS_F + col0 + cx + 16 * j, __float_as_uint(acc[i][j]), tag);
       }
     }
-    if (!grid.sync(q.error_word, &s_ok)) return;
     if (!conv) continue;
     // ---- the end of the state's pass, in every block of the group ----
     const bool sample = t < q.sample_steps, stepping = sample && q.env;
+    EnvPrep prep{};
+    if (stepping && tid == 32) prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, q.counters);
     {
-      float v[RS_RUNS];
-#pragma unroll
-      for (int p = 0; p < RS_RUNS; ++p) v[p] = __ldcg(q.part + ((size_t)p * n + e) * RS_F + tid);
+      uint2 v[RS_RUNS];
+      word_await(v, sums + (size_t)e * RS_F + tid, (size_t)n * RS_F, RS_RUNS, tag, &s_dead, q.error_word);
       double s = 0.0;
 #pragma unroll
-      for (int p = 0; p < RS_RUNS; ++p) s += (double)v[p];
+      for (int p = 0; p < RS_RUNS; ++p) s += (double)__uint_as_float(v[p].x);
       const T x = from_f<T>(fmaxf((float)(s + (double)q.bfc[tid]), 0.f));
       if (rank == 0) h[(slot + e) * RS_F + tid] = x;
       xs[tid] = to_f(x);
     }
-    EnvPrep prep{};
-    if (stepping && tid == 32) prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, q.counters);
     __syncthreads();
     for (int k = warp; k <= A; k += RS_THREADS / 32) {
       float acc = 0.f;
@@ -293,6 +342,11 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
                                           sample, q.seed, step0 + t, q.forced ? q.forced + slot : nullptr, q.actions + slot, q.sampled + slot,
                                           q.uniforms + slot);
       if (lane == 0) s_action = a;
+      if (q.host.done != nullptr && rank == 0 && lane == 0) {
+        if (sample) q.host.actions[e] = a;
+        q.host.values[e] = q.values[slot + e];
+        __threadfence_system();
+      }
     }
     if (!stepping) { __syncthreads(); continue; }
     __syncthreads();
@@ -307,18 +361,19 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
     // this block's share of the frame for everyone, and the rows it will read itself
     uint8_t* states = t + 1 < q.sample_steps ? const_cast<uint8_t*>(q.frames) + (size_t)(t + 1) * q.frame_step : q.next_frames;
     uint4* out = reinterpret_cast<uint4*>(states + (size_t)e * FRAME_BYTES);
-    const int own_lo = FRAME_WORDS / 4 * rank / C, own_hi = FRAME_WORDS / 4 * (rank + 1) / C;
-    const int lo = min(own_lo, row_lo * QUADS), hi = max(own_hi, row_hi * QUADS);
-    for (int i = lo + tid; i < hi; i += RS_THREADS) {
-      const bool own = i >= own_lo && i < own_hi, keep = i >= row_lo * QUADS && i < row_hi * QUADS;
-      if (!own && !keep) continue;
-      const uint4 v = env_frame_quad(f, (uint32_t)i, q.pattern_actions);
-      if (own) out[i] = v;
-      if (keep) frame[i] = v;
-    }
+    for (int i = part_lo + tid; i < part_hi; i += RS_THREADS) place(out, i, env_frame_quad(f, (uint32_t)i, q.pattern_actions));
     __syncthreads();
   }
-  if (q.advance && blockIdx.x == 0 && tid == 0) *q.step_base += q.advance;        // every block has read it
+  // Every block has read the counts when the last one ends.
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(q.sync + 1, 1u) == gridDim.x - 1) {
+      q.sync[0] = epoch + (uint32_t)q.steps;
+      q.sync[1] = 0u;
+      if (q.advance) *q.step_base += q.advance;
+      if (q.host.done != nullptr) { __threadfence_system(); *q.host.done = 1u; }
+    }
+  }
 }
 
 // Blocks per environment: as many of 16, 8, 4, 2 as leave each a multiprocessor of its own; 0: use the layer-by-layer path.
@@ -361,19 +416,22 @@ bool rollout_small_supported(const LaunchCtx& lc, int arch, int prec, int n) {
   const int C = rs_blocks_per_env(n);
   return arch == PAAC_ARCH_NIPS && !lc.fp32_tensor_cores && C != 0 && rs_pick(prec, C, [](auto k) { return k.fits(); });
 }
-size_t rollout_small_part_floats(int n) { return (size_t)RS_RUNS * n * RS_F; }
-size_t rollout_small_barrier_words(int n) { return 2 * ((size_t)n + 1); }      // 64-bit counters
+// of 16 bytes: both maps, and two sets of the runs' sums at two to a word
+static size_t rs_map1_words(int n) { return (size_t)n * RS_POS1 * RC1::CO / 2; }
+static size_t rs_map2_words(int n) { return (size_t)n * RS_IN / 2; }
+size_t rollout_small_words(int n) { return rs_blocks_per_env(n) == 0 ? 0 : rs_map1_words(n) + rs_map2_words(n) + (size_t)n * RS_RUNS * RS_F; }
 
 void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const SmallRollout& r) {
   const LayerDims* d = nd.layer;
   RsArgs q{};
   q.n = r.n; q.C = rs_blocks_per_env(r.n); q.A = nd.A; q.steps = r.steps; q.blocks = RS_BLOCKS; q.t0 = r.t0;
   q.frames = r.frames; q.frame_step = r.frame_step; q.next_frames = r.env.next_frames; q.sample_steps = r.sample_steps; q.env = r.step_env;
-  q.part = r.part; q.b1 = theta + d[0].b_off; q.b2 = theta + d[1].b_off; q.bfc = theta + d[2].b_off; q.bpi = theta + nd.pi_b; q.bv = theta + nd.v_b;
+  q.map1 = (uint4*)r.words; q.map2 = q.map1 + rs_map1_words(r.n); q.sums = (uint2*)(q.map2 + rs_map2_words(r.n)); q.sync = r.sync; q.host = r.host;
+  q.b1 = theta + d[0].b_off; q.b2 = theta + d[1].b_off; q.bfc = theta + d[2].b_off; q.bpi = theta + nd.pi_b; q.bv = theta + nd.v_b;
   q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
   q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
   q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode;
-  q.grid_bar = reinterpret_cast<unsigned long long*>(r.barriers); q.group_bar = q.grid_bar + 1; q.error_word = r.error_word;
+  q.error_word = r.error_word;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(q.blocks); cfg.blockDim = dim3(RS_THREADS); cfg.dynamicSmemBytes = rs_smem(q.A); cfg.stream = lc.st;
   cudaLaunchAttribute attr[1];

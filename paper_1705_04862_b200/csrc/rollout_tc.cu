@@ -19,15 +19,8 @@
 // sixteen k in the same order (the first layer's depend on the parity of the position, the second and third keep the two sums of
 // tc_shift_t_kernel, the fully connected layer its eight slices, the heads their tree).
 //
-// The words: a 16-byte access holds (value, step, value, step); each 8-byte half is written and read as one.  A word of a
-// step is overwritten by the next step only after everything that reads it has: an environment's blocks start a step with
-// the sums of the one before, which the fully connected blocks made from those words.  The step numbers go on from
-// launch to launch; the block that ends last moves the count on.
-//
-// What bounds a step: latency.  10.4 us for 32 states (20.2 layer by layer; a rollout 121.6 -> 72 us), of which a block spends 0.6
-// making the frame, 1.25, 1.15 and 0.95 in the three convolutions (chains of 16 and 24 dependent instructions of 44 clocks, and
-// operands from shared memory at 128 bytes a clock), 0.8 and 0.5 handing the maps over, 2 in the fully connected layer, 0.9 waiting for
-// the other slices, 0.5 with the heads and 1.2 with the draw and the transition.
+// A word (step_words.cuh) of a step is overwritten by the next step only after everything that reads it has: an environment's
+// blocks start a step with the sums of the one before, which the fully connected blocks made from those words.
 //
 // With environments outside, a step is one such launch too: while the weights come in, each block of a cluster fetches its share of the
 // environment's newest plane over the host link and writes its share of the state, and the environment's action and value go straight
@@ -35,13 +28,12 @@
 // launch arguments: read from pinned memory by every block, they took 16 us each (reads of one address are served one after
 // the other).
 //
-// Every wait for a word is bounded.  A block that gives up raises the error word and goes on without waiting (its cluster
-// waits for it at barriers), so that all blocks end.
+// Every wait is bounded; a block that gave up goes on without waiting, as its cluster waits for it at the end.
 #include <cuda_fp16.h>
 
 #include "env_device.cuh"
 #include "kernels.h"
-#include "tc_common.cuh"
+#include "step_words.cuh"
 
 namespace paac {
 
@@ -49,7 +41,6 @@ typedef NatConv1 TC1; typedef NatConv2 TC2; typedef NatConv3 TC3;
 constexpr int RT_THREADS = 512, RT_WARPS = RT_THREADS / 32, RT_MAX_ENVS = 1;        // environments of a cluster
 constexpr int RT_F = 512, RT_SLICES = 8, RT_TILE = 32, RT_FC_BLOCKS = RT_SLICES * (RT_F / RT_TILE), RT_ROWS = 64;
 constexpr int RT_POS3 = TC3::OH * TC3::OW, RT_FC_LD = 7 * 128;                      // 49 blocks of 64 k, six or seven to a slice
-constexpr uint32_t RT_POLLS = 2000000u;
 
 struct RtArgs {
   int n, A, steps, clusters;                      // forward passes: slots t0 .. t0 + steps - 1
@@ -116,29 +107,6 @@ __device__ __forceinline__ void rt_cluster_sync() {
 __device__ __forceinline__ void rt_pair_sync(int id) {                          // two warps
   __syncwarp();
   asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
-}
-
-// ---- words that carry their step ---------------------------------------------------------------------------------------
-__device__ __forceinline__ uint4 rt_peek(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-  return v;
-}
-// v[i] = the word at p + i * step, i < count (of N), once all are of step `tag`, or as they are after a bounded wait.  All are asked
-// for together, again and again: one after the other each would cost a round trip through L2.
-template <int N>
-__device__ __forceinline__ void rt_await(uint4 (&v)[N], const uint4* p, size_t step, int count, uint32_t tag, volatile uint32_t* dead, uint32_t* error_word) {
-  for (uint32_t polls = 0;; ++polls) {
-    bool ready = true;
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-      if (i < count) v[i] = rt_peek(p + i * step);
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-      if (i < count) ready = ready && v[i].y == tag && v[i].w == tag;
-    if (ready || *dead) return;
-    if (polls == RT_POLLS) { *dead = 1u; atomicOr(error_word, tc::ERR_WAIT_FULL); return; }
-  }
 }
 
 // Shared memory, in bytes.  Rows of weights are in groups of 128 bytes whose 16-byte pieces are permuted by the row's low bits, so
@@ -290,10 +258,17 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
 
   // the newest plane comes over the host link meanwhile: sixteen pixels to a thread
   const int px_lo = STACK_ITEMS * rank / C, px_hi = STACK_ITEMS * (rank + 1) / C;
-  static_assert((STACK_ITEMS + C - 1) / C <= RT_THREADS && RT_MAX_ENVS == 1, "one piece to a thread");
+  static_assert((STACK_ITEMS + C - 1) / C <= RT_THREADS && FRAME_WORDS / 4 / C <= 2 * RT_THREADS && RT_MAX_ENVS == 1, "one piece to a thread");
   uint4 plane{};
   const bool pulls = q.host.newest != nullptr && envs > 0 && px_lo + tid < px_hi;
   if (pulls) plane = reinterpret_cast<const uint4*>(q.host.newest)[(size_t)cluster * STACK_ITEMS + px_lo + tid];
+  // or the whole state: four such words
+  const int st_lo = FRAME_WORDS / 4 * rank / C, st_hi = FRAME_WORDS / 4 * (rank + 1) / C;
+  uint4 whole[2];
+  if (q.host.states != nullptr && envs > 0)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (st_lo + tid + i * RT_THREADS < st_hi) whole[i] = reinterpret_cast<const uint4*>(q.host.states)[(size_t)cluster * (FRAME_WORDS / 4) + st_lo + tid + i * RT_THREADS];
 
   // ---- what stays for the rollout ----
   if (tid == 0) {
@@ -338,6 +313,10 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
     stack_sixteen(plane, (q.host.fresh[cluster >> 5] >> (cluster & 31)) & 1u, reinterpret_cast<const uint4*>(q.host.prev) + 4 * at,
                   reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames)) + 4 * at);
   }
+  if (q.host.states != nullptr && envs > 0)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (st_lo + tid + i * RT_THREADS < st_hi) reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames))[(size_t)cluster * (FRAME_WORDS / 4) + st_lo + tid + i * RT_THREADS] = whole[i];
   tc::cp_async_wait<0>();
   __syncthreads();
   const uint32_t epoch = s_epoch;
@@ -465,7 +444,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
               for (int i = 0; i < 2; ++i) {
                 const int p = (2 * mg + m) * 16 + g + 8 * i;
                 if (p >= RT_POS3) continue;
-                asm volatile("st.volatile.global.v2.u32 [%0], {%1, %2};" ::"l"(reinterpret_cast<uint2*>(q.maps) + ((size_t)e * RT_POS3 + p) * 32 + ch / 2), "r"(v[i]), "r"(tag) : "memory");
+                word_store(reinterpret_cast<uint2*>(q.maps) + ((size_t)e * RT_POS3 + p) * 32 + ch / 2, v[i], tag);
                 *reinterpret_cast<uint32_t*>(q.act3 + (slot + e) * TC3::OUT_SIZE + p * 64 + ch) = v[i];
               }
             }
@@ -487,7 +466,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
         for (int r = tid >> 4; r < rows; r += RT_THREADS / 16) {
           const uint4* src = q.maps + ((size_t)(row0 + r) * RT_POS3 + kb0) * 16 + u;
           uint4 v[7];
-          rt_await(v, src, 16, kbs, tag, &s_dead, q.error_word);
+          word_await(v, src, 16, kbs, tag, &s_dead, q.error_word);
 #pragma unroll
           for (int p = 0; p < 7; ++p)
             if (p < kbs) {
@@ -525,8 +504,8 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
             for (int i = 0; i < 2; ++i) {
               const int r = row0 + mt * 16 + g + 8 * i;
               if (r < n)
-                asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %2};" ::"l"(q.sums + ((size_t)slice * n + r) * 256 + (unit0 + np * 16 + j * 8 + 2 * t4) / 2),
-                             "r"(__float_as_uint(acc[j][2 * i])), "r"(tag), "r"(__float_as_uint(acc[j][2 * i + 1])) : "memory");
+                word_store(q.sums + ((size_t)slice * n + r) * 256 + (unit0 + np * 16 + j * 8 + 2 * t4) / 2, __float_as_uint(acc[j][2 * i]),
+                           __float_as_uint(acc[j][2 * i + 1]), tag);
             }
         }
         __syncthreads();
@@ -543,7 +522,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
       const int e = cluster + ei * clusters, col = tid % (S::COLS / 2) * 2, u = unit_of(col);
       const uint4* src = q.sums + (size_t)e * 256 + u / 2;
       uint4 v[RT_SLICES];
-      rt_await(v, src, (size_t)n * 256, RT_SLICES, tag, &s_dead, q.error_word);
+      word_await(v, src, (size_t)n * 256, RT_SLICES, tag, &s_dead, q.error_word);
       float s0 = 0.f, s1 = 0.f;
 #pragma unroll
       for (int s = 0; s < RT_SLICES; ++s) {
@@ -672,7 +651,7 @@ void launch_rollout_tc(LaunchCtx& lc, const NetDims& nd, const float* theta, con
   q.wv = theta16 + nd.v_w; q.b1 = theta + d[0].b_off; q.b2 = theta + d[1].b_off; q.b3 = theta + d[2].b_off; q.bfc = theta + d[3].b_off;
   q.bpi = theta + nd.pi_b; q.bv = theta + nd.v_b; q.scale1 = tc_conv1_scale();
   q.act1 = (bf16*)r.act[0]; q.act2 = (bf16*)r.act[1]; q.act3 = (bf16*)r.act[2]; q.h = (bf16*)r.act[3];
-  q.maps = (uint4*)r.words; q.sums = q.maps + rt_map_words(r.n); q.sync = r.barriers;
+  q.maps = (uint4*)r.words; q.sums = q.maps + rt_map_words(r.n); q.sync = r.sync;
   q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
   q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
   q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode; q.host = r.host; q.error_word = r.error_word;
