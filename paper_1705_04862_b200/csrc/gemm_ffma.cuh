@@ -82,10 +82,21 @@ template <class OP, int R, int BK, int NT> struct FfLoader {
         const int i = threadIdx.x + it * NT;
         if (!FULL && i >= ITEMS) break;
         float4 f[V / 4];
-        widen(val[it], (const T*)nullptr, f);
         float4* dst = reinterpret_cast<float4*>(tile + (OP::K_CONTIG ? row_of(i) * Tile::LD + k_of(i) : k_of(i) * Tile::LD + row_of(i)));
+        if constexpr (sizeof(T) == 1 && !OP::K_CONTIG) {
+          // neighbouring threads' pieces are 64 bytes apart: each begins with another quarter of its own, so that eight threads'
+          // stores lie in different banks (a quarter of the first layer's weight gradient's shared-memory cycles were such conflicts)
+          const uint32_t turn = threadIdx.x >> 1;
+          const uint4 v = val[it];
+          const uint4 a = turn & 1u ? make_uint4(v.y, v.z, v.w, v.x) : v;
+          widen(turn & 2u ? make_uint4(a.z, a.w, a.x, a.y) : a, (const T*)nullptr, f);
 #pragma unroll
-        for (int q = 0; q < V / 4; ++q) dst[q] = f[q];
+          for (int q = 0; q < V / 4; ++q) dst[(q + turn) & 3u] = f[q];
+        } else {
+          widen(val[it], (const T*)nullptr, f);
+#pragma unroll
+          for (int q = 0; q < V / 4; ++q) dst[q] = f[q];
+        }
       }
     }
   }
