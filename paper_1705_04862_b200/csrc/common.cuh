@@ -118,26 +118,18 @@ __device__ __forceinline__ int warp_finish_heads(const HeadMode hm, float z, flo
   }
   if (lane == 0) values[e] = v;
   if (!sample) return -1;
-  const float u = philox_uniform((uint32_t)e, (uint32_t)step, (uint32_t)(step >> 32), RNG_STREAM_ACTION, seed);
   float ex = lane < A ? expf(z - m) : 0.f;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
   const float lse = m + logf(ex);
   const float p = lane < A ? expf(z - lse) : 0.f;
+  const float u = philox_uniform((uint32_t)e, (uint32_t)step, (uint32_t)(step >> 32), RNG_STREAM_ACTION, seed);
   float c = 0.f;
   int a = A - 1;
   bool found = false;
-  // eight at a time, so that only the additions wait for one another; past the last action p = 0 and c stays what it is
-#pragma unroll 1
-  for (int k0 = 0; k0 < A; k0 += 8) {
-    float pk[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) pk[k] = __shfl_sync(0xffffffffu, p, k0 + k);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      c += pk[k];
-      if (!found && u < c) { a = k0 + k; found = true; }
-    }
+  for (int k = 0; k < A; ++k) {
+    c += __shfl_sync(0xffffffffu, p, k);
+    if (!found && u < c) { a = k; found = true; }
   }
   const int drawn = a;
   if (forced != nullptr && forced[e] >= 0) a = forced[e];
