@@ -587,10 +587,14 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
     }
     side.join();
     ready += finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials + ready : nullptr, NORM_BLOCKS - ready);
-    launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad,
-                        c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps, hp.clip_norm,
-                        c->norm_partials, c->stats, all_finished ? ready : 0);
-    if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
+    if (tc_supported(c->arch, c->prec) && all_finished)
+      launch_clip_rmsprop_images(c->lc, c->nd.P, c->theta, c->rms, c->grad, c->theta16, tc_weight_images(c->nd, c->w_images, &c->stats->error_word), hp.lr,
+                                 hp.rms_decay, hp.rms_eps, hp.clip_norm, c->norm_partials, c->stats, ready);
+    else {
+      launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad, c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps,
+                          hp.clip_norm, c->norm_partials, c->stats, all_finished ? ready : 0);
+      if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
+    }
     if (stats) launch_publish_stats(c->lc, c->stats, &c->box->stats, &c->box->done);
   });
   c->N += (uint64_t)c->B;

@@ -179,5 +179,16 @@ void launch_clip_rmsprop(LaunchCtx& lc, size_t P, float* theta, float* rms, cons
                          bf16* theta16 /* nullable */, float lr, float rho, float eps, float clip,
                          float* norm_partials /* [NORM_BLOCKS] */, DeviceStats* stats,
                          int ready_partials = 0 /* > 0: norm_partials[0..ready_partials) already hold the squared norm */);
+// the same for the larger network in bf16, with the regrouped weight images (tc_weight_images()) written from the new parameters;
+// norm_partials[0..ready_partials) hold the squared norm
+struct WeightImages {
+  uint16_t *w1_b, *w2_d, *w3_d, *wfc_t;
+  size_t w1_end, w2_off, w3_off, fc_off;        // elements of the parameter vector
+  float w1_scale;
+  uint32_t* error_word;
+};
+WeightImages tc_weight_images(const NetDims& nd, bf16* images, uint32_t* error_word);
+void launch_clip_rmsprop_images(LaunchCtx& lc, size_t P, float* theta, float* rms, const float* grad, bf16* theta16, const WeightImages& img, float lr,
+                                float rho, float eps, float clip, const float* norm_partials, DeviceStats* stats, int ready_partials);
 
 }  // namespace paac

@@ -3063,6 +3063,11 @@ __global__ void __launch_bounds__(256) relayout_weights_kernel(const bf16* __res
   }
 }
 size_t tc_weight_image_elems() { return TC_IMG_END; }
+WeightImages tc_weight_images(const NetDims& nd, bf16* images, uint32_t* error_word) {
+  auto at = [&](size_t off) { return reinterpret_cast<uint16_t*>(images + off); };
+  return WeightImages{at(TC_IMG_W1), at(TC_IMG_W2), at(TC_IMG_W3), at(TC_IMG_WFC), nd.layer[0].b_off, nd.layer[1].w_off, nd.layer[2].w_off, nd.layer[3].w_off,
+                      C1_F16_WEIGHT_SCALE, error_word};
+}
 
 void tc_relayout_weights(LaunchCtx& lc, const NetDims& nd, const bf16* theta16, bf16* images, uint32_t* error_word) {
   const LayerDims* d = nd.layer;
