@@ -738,6 +738,10 @@ int paac_profile_read(paac_ctx* c, int max_entries, const char** names, double* 
 // The network on the state at `dst`, with `prev` after the frame stack has built that state from `planes`, and the results into the
 // box.  The frame stack's arguments differ from step to step, so it is launched by itself; the rest is one launch sequence,
 // recorded from the second time on, or, for few environments, part of the same kernel, which can also fetch whole `states`.
+// From HOST_PLAIN_FROM environments on the planes take longer over the link than the other launches take to be made, and launched
+// one by one the first layer sets itself up meanwhile (a recorded sequence starts when the frame stack has ended): an iteration of
+// 384, 512 and 1024 environments 820 -> 812, 990 -> 978 and 1620 -> 1609 us, but 668 -> 672 with 256.
+constexpr int HOST_PLAIN_FROM = 320;
 static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, const uint8_t* states, uint8_t* dst,
                            int32_t* actions, float* values) {
   const bool sample = t < c->t_max;
@@ -751,12 +755,14 @@ static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_
     small_rollout(c, dst, t, 1, sample ? 1 : 0, nullptr, !sample, &host);
   } else {
     if (prev) launch_stack_pull(c->lc, prev, planes, restart, dst, c->n_e);
-    run_recorded(c, 3 + t, c->cur, [&]() {
+    auto enqueue = [&]() {
       bool advanced = false;
       forward_slot(c, dst, t, sample, nullptr, sample ? nullptr : &advanced);
       if (!sample && !advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
       launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
-    });
+    };
+    if (prev && c->n_e >= HOST_PLAIN_FROM) enqueue();
+    else run_recorded(c, 3 + t, c->cur, enqueue);
   }
   if (!await_box(c)) return PAAC_ERR_CUDA;
   if (sample) memcpy(actions, box->actions, c->n_e * sizeof(int32_t));
