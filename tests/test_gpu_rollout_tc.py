@@ -77,3 +77,22 @@ def test_outside_environments_same_bits_as_layer_by_layer(n_e, ring):
         assert np.array_equal(small.debug_read(pb.DBG_NEXT_FRAMES), state[:n_e].numpy().reshape(-1))
     assert small.error_word() == 0 and large.error_word() == 0
     small.close(), large.close()
+
+
+def test_planes_of_more_environments_than_one_launch_takes():
+    """The frame stack's restart flags are launch arguments, 2048 environments to a launch: states of either side of that line."""
+    import torch
+    n = 2051
+    gen = torch.Generator().manual_seed(1)
+    g = pb.Paac("nips", n, 1, 4, seed=2, precision=pb.FP32)
+    first = torch.randint(0, 256, (n, 84, 84, 4), dtype=torch.uint8, generator=gen).pin_memory()
+    planes = torch.randint(0, 256, (n, 84, 84), dtype=torch.uint8, generator=gen).pin_memory()
+    ends = (torch.rand(n, generator=gen) < 0.5).to(torch.uint8)
+    acts, vals = np.zeros(n, np.int32), np.zeros(n, np.float32)
+    g.act_host(0, first, acts, vals)
+    g.observe_host(0, np.zeros(n, np.int8), ends.numpy())
+    g.act_host_newest(1, planes, ends.numpy(), None, vals)
+    pushed = torch.cat([first[..., 1:], planes[..., None]], dim=-1)
+    want = torch.where(ends[:, None, None, None] != 0, planes[..., None].expand(-1, -1, -1, 4), pushed)
+    assert np.array_equal(g.debug_read(pb.DBG_NEXT_FRAMES), want.contiguous().numpy().reshape(-1))
+    g.close()
