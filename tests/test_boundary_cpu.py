@@ -1,6 +1,7 @@
 """Host-side checks that need no GPU: the C-ABI library loads, exports every symbol the header
 declares, sizes workspaces, validates arguments, and refuses to run without a device."""
 import ctypes as C
+import itertools
 import os
 import re
 import subprocess
@@ -138,3 +139,36 @@ def test_what_belongs_to_a_device_is_made_once_on_each(tmp_path):
     assert [get(0, 1), get(0, 1), get(1, 1), get(0, 1), get(1, 0)] == [1, 1, 102, 1, 102]
     assert [get(63, 0), get(63, 1), get(63, 0)] == [-1, 6304, 6304]
     assert [get(-1, 1), get(64, 1)] == [-1, -1]
+
+
+def _word_accesses():
+    """(elements, bits of an element) of every load and store that step_words.cuh makes."""
+    text = open(os.path.join(ROOT, "paper_1705_04862_b200", "csrc", "step_words.cuh")).read()
+    found = re.findall(r'"(ld|st)\.[a-z.]*global\.(?:v(\d)\.)?[a-z](\d+) ', text)
+    return {kind: sorted({(int(n or 1), int(bits)) for k, n, bits in found if k == kind}) for kind in ("ld", "st")}
+
+
+def _torn_reads(store, load):
+    """Whether a reader may find the new step beside the old value.  Elements of a vector access are accesses of their own, in any
+    order; four-byte pieces, a value and then its step, eight bytes a word."""
+    pieces = store[0] * store[1] // 32
+    writes, reads = ([range(i * w // 32, (i + 1) * w // 32) for i in range(n)] for n, w in (store, load))
+    for order in itertools.permutations([("w", e) for e in writes] + [("r", e) for e in reads]):
+        memory, seen = [0] * pieces, [0] * pieces
+        for what, element in order:
+            for i in element:
+                if what == "w":
+                    memory[i] = 1
+                else:
+                    seen[i] = memory[i]
+        if any(seen[i + 1] > seen[i] for i in range(0, pieces, 2)):
+            return True
+    return False
+
+
+def test_a_word_that_carries_its_step_is_never_seen_in_part():
+    assert _torn_reads((4, 32), (4, 32)) and _torn_reads((2, 32), (1, 64)) and not _torn_reads((1, 64), (1, 64))
+    accesses = _word_accesses()
+    assert [n * bits for n, bits in accesses["ld"]] == [n * bits for n, bits in accesses["st"]] == [64, 128]
+    for load, store in zip(accesses["ld"], accesses["st"]):
+        assert not _torn_reads(store, load), (store, load)
