@@ -131,7 +131,12 @@ typedef struct {
 /* Algorithm 1, the inner loop and the bootstrap: for t = 0..t_max-1 evaluate the
  * network on s_t for all environments, sample a_t from the softmax policy by
  * inverse CDF with a Philox4x32-10 uniform, step every environment; then evaluate
- * V on the final states.  Asynchronous.  view may be NULL. */
+ * V on the final states.  Asynchronous.  view may be NULL.
+ * Up to 74 environments all of it can be one launch, whose blocks wait for one another and take nearly every
+ * multiprocessor.  It is made only while no learner of this process on another stream has work in flight (and not while
+ * the stream is being captured by the caller); else the layers are launched one by one, with the same results.  Kernels
+ * of the caller's own that hold multiprocessors beside it for more than about a second make its waits give up
+ * (PAAC_ERR_TIMEOUT, see PAAC_DBG_ERROR_WORD). */
 int paac_rollout(paac_ctx* ctx, paac_rollout_view* view /* host, out, nullable */);
 
 typedef struct {

@@ -2,6 +2,7 @@
 // kernels of one pass of Algorithm 1 are enqueued.
 #include <cuda.h>
 
+#include <mutex>
 #include <new>
 #include <string.h>
 
@@ -70,12 +71,14 @@ struct paac_ctx {
   // once into a CUDA graph and replayed from then on.  Anything that changes the sequence drops the graphs.
   bool graphs_on;          // option: allow recording
   SideSet side;            // incomplete if it could not be had: everything then stays on the learner's stream
-  // recorded launch sequences: kind 0 = rollout, 1 = update, 2 = update that reports, 3 + t = step t of the external-environment mode, each for both parities of the frame buffers
-  static constexpr int GRAPH_KINDS = 3 + 65;
+  // recorded launch sequences: kind 0 = rollout (in one launch where it can be), 1 = update, 2 = update that reports, 3 = rollout layer by layer of a
+  // learner that can do it in one launch, 4 + t = step t of the external-environment mode, each for both parities of the frame buffers
+  static constexpr int GRAPH_KINDS = 4 + 65;
   int plain_calls[GRAPH_KINDS][2];   // calls made with plain launches
   cudaGraphExec_t graph[GRAPH_KINDS][2];
   uint64_t graph_launches[GRAPH_KINDS][2];
   bool simt_only;          // keep the bf16 network on the CUDA cores (cross-check of the tensor-core path)
+  paac_ctx* next;          // the learners of this process (see Learners)
 
   // device buffers (all inside the workspace)
   float *theta, *grad, *rms;
@@ -198,10 +201,49 @@ void refresh_weight_copies(paac_ctx* c, bool cast) {
   if (tc_supported(c->arch, c->prec)) tc_relayout_weights(c->lc, c->nd, c->theta16, c->w_images, &c->stats->error_word);
 }
 
-// whether a rollout's forward passes go in one launch
-bool one_launch(const paac_ctx* c) {
+// whether a rollout's forward passes can go in one launch
+bool one_launch_supported(const paac_ctx* c) {
   return use_tc(c) ? rollout_tc_supported(c->n_e, c->A) : rollout_small_supported(c->lc, c->arch, c->prec, c->n_e);
 }
+
+// The learners of this process.  The blocks of a one-launch rollout wait for one another, and it takes nearly every multiprocessor:
+// two of them started side by side can each get a part of the device and wait for the rest until their waits give up (a
+// cooperative launch only checks that the device could hold the grid; seen with two learners of 64 environments).  So one is launched
+// only while no learner on another stream has work in flight, and a learner that is not alone goes layer by layer, with the same
+// numbers and in no more time: a round of four learners of 8 environments takes 306 us so, 412 with each rollout in one launch.
+struct Learners {
+  std::mutex lock;
+  paac_ctx* first = nullptr;
+  void add(paac_ctx* c) { std::lock_guard<std::mutex> hold(lock); c->next = first; first = c; }
+  void remove(paac_ctx* c) {
+    std::lock_guard<std::mutex> hold(lock);
+    for (paac_ctx** p = &first; *p; p = &(*p)->next) if (*p == c) { *p = c->next; return; }
+  }
+} learners;
+
+// whether a stream may have work in flight
+bool busy(cudaStream_t st) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;       // the question is allowed while some other stream is being captured
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  const bool idle = cudaStreamIsCapturing(st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone && cudaStreamQuery(st) == cudaSuccess;
+  if (!idle) cudaGetLastError();
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return !idle;
+}
+// Whether this pass goes in one launch.  If so `turn` is held, and is to be until the launch is in the stream.  A caller's
+// own graph gets the layers: nothing could order it against other learners when it is replayed.
+bool one_launch(const paac_ctx* c, std::unique_lock<std::mutex>& turn) {
+  if (!one_launch_supported(c)) return false;
+  turn = std::unique_lock<std::mutex>(learners.lock);
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  bool alone = cudaStreamIsCapturing(c->st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone;
+  if (!alone) cudaGetLastError();
+  for (const paac_ctx* o = learners.first; o != nullptr && alone; o = o->next) alone = o->st == c->st || !busy(o->st);
+  if (!alone) turn.unlock();
+  return alone;
+}
+
 // `steps` forward passes from slot t0 on in one launch (one_launch()); a rollout with `env`, else one pass
 void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sample_steps, const EnvStepArgs* env, bool advance,
                    const HostStep* host = nullptr) {
@@ -233,11 +275,6 @@ bool forward_slot(paac_ctx* c, const uint8_t* frames, int slot, bool sample, Hea
   for (int l = 0; l <= c->nd.n_conv; ++l)
     act[l] = (char*)c->act[l] + (size_t)slot * c->n_e * c->nd.layer[l].out_size * c->elt;
   const size_t row = (size_t)slot * c->n_e;
-  if (one_launch(c)) {
-    small_rollout(c, frames, slot, 1, sample ? 1 : 0, nullptr, advanced && !sample);
-    if (advanced) *advanced = !sample;
-    return false;
-  }
   const int32_t* forced = sample && c->forced_on ? c->forced + row : nullptr;
   int32_t* actions = sample ? c->actions + row : nullptr;
   int32_t* sampled = sample ? c->sampled + row : nullptr;
@@ -406,6 +443,7 @@ struct SideBranch {
 
 // what paac_init made
 void release(paac_ctx* c) {
+  learners.remove(c);
   if (c->box) cudaFreeHost(c->box);
   c->side.destroy();
   if (c->owns_workspace) cudaFree(c->ws);
@@ -459,6 +497,7 @@ int paac_init(paac_ctx** out, int arch, int n_e, int t_max, int n_actions, const
   }
   c->ws_bytes = need;
   carve(c, c->ws);
+  learners.add(c);
   c->lc.error_word = &c->stats->error_word;
   cudaMemsetAsync(c->ws, 0, need, c->st);
   cudaMemsetAsync(c->forced, 0xFF, (size_t)c->B * sizeof(int32_t), c->st);
@@ -487,8 +526,10 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
   uint8_t* fr = c->frames[c->cur];
   uint8_t* nxt = c->frames[c->cur ^ 1];
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
-  run_recorded(c, 0, c->cur, [&]() {
-    if (one_launch(c)) {
+  std::unique_lock<std::mutex> turn;
+  const bool one = one_launch(c, turn);
+  run_recorded(c, one || !one_launch_supported(c) ? 0 : 3, c->cur, [&]() {
+    if (one) {
       const EnvStepArgs env{c->hp.term_denom, nxt, c->rewards, c->terminals, c->counters, pattern_actions(c)};
       small_rollout(c, fr, 0, c->t_max + 1, c->t_max, &env, true);
       return;
@@ -512,6 +553,7 @@ int paac_rollout(paac_ctx* c, paac_rollout_view* view) {
     forward_slot(c, nxt, c->t_max, false, nullptr, &advanced);
     if (!advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
   });
+  if (turn) turn.unlock();
   c->env_step += c->t_max;
   c->rollout_fresh = true;
   if (view) {
@@ -742,17 +784,18 @@ int paac_profile_read(paac_ctx* c, int max_entries, const char** names, double* 
 // one by one the first layer sets itself up meanwhile (a recorded sequence starts when the frame stack has ended): an iteration of
 // 384, 512 and 1024 environments 820 -> 812, 990 -> 978 and 1620 -> 1609 us, but 668 -> 672 with 256.
 constexpr int HOST_PLAIN_FROM = 320;
-static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, const uint8_t* states, uint8_t* dst,
+static int act_host_finish(paac_ctx* c, int t, std::unique_lock<std::mutex> turn, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, const uint8_t* states, uint8_t* dst,
                            int32_t* actions, float* values) {
   const bool sample = t < c->t_max;
   const size_t row = (size_t)t * c->n_e;
   HostBox* box = c->box;
   box->done = 0u;
-  if (one_launch(c)) {
+  if (turn) {                // one_launch() said so
     HostStep host{prev, planes, {0u, 0u, 0u}, states, box->actions, box->values, &box->done};
     if (restart)
       for (int e = 0; e < c->n_e; ++e) host.fresh[e >> 5] |= (uint32_t)(restart[e] != 0) << (e & 31);
     small_rollout(c, dst, t, 1, sample ? 1 : 0, nullptr, !sample, &host);
+    turn.unlock();
   } else {
     if (prev) launch_stack_pull(c->lc, prev, planes, restart, dst, c->n_e);
     auto enqueue = [&]() {
@@ -762,7 +805,7 @@ static int act_host_finish(paac_ctx* c, int t, const uint8_t* prev, const uint8_
       launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
     };
     if (prev && c->n_e >= HOST_PLAIN_FROM) enqueue();
-    else run_recorded(c, 3 + t, c->cur, enqueue);
+    else run_recorded(c, 4 + t, c->cur, enqueue);
   }
   if (!await_box(c)) return PAAC_ERR_CUDA;
   if (sample) memcpy(actions, box->actions, c->n_e * sizeof(int32_t));
@@ -804,12 +847,13 @@ int paac_act_host(paac_ctx* c, int t, const uint8_t* frames, int32_t* actions, f
   const size_t fstep = (size_t)c->n_e * FRAME_BYTES;
   if (t == 0) c->cur ^= 1;
   uint8_t* dst = t < c->t_max ? c->frames[c->cur] + t * fstep : c->frames[c->cur ^ 1];
-  const uint8_t* view = frames && one_launch(c) && ((uintptr_t)frames & 15u) == 0 ? host_view(frames, fstep, query_host_range) : nullptr;
+  std::unique_lock<std::mutex> turn;
+  const uint8_t* view = one_launch(c, turn) && frames && ((uintptr_t)frames & 15u) == 0 ? host_view(frames, fstep, query_host_range) : nullptr;
   if (frames && !view && cudaMemcpyAsync(dst, frames, fstep, cudaMemcpyHostToDevice, c->st) != cudaSuccess) {
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
   if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
-  return act_host_finish(c, t, nullptr, nullptr, nullptr, view, dst, actions, values);
+  return act_host_finish(c, t, std::move(turn), nullptr, nullptr, nullptr, view, dst, actions, values);
 }
 
 int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_t* restart, int32_t* actions, float* values) {
@@ -827,7 +871,9 @@ int paac_act_host_newest(paac_ctx* c, int t, const uint8_t* newest, const uint8_
     cudaGetLastError(); return PAAC_ERR_CUDA;
   }
   if (t == c->t_max && send_outcomes(c) != PAAC_OK) return PAAC_ERR_CUDA;
-  return act_host_finish(c, t, prev, view ? view : c->newest, restart, nullptr, dst, actions, values);
+  std::unique_lock<std::mutex> turn;
+  one_launch(c, turn);
+  return act_host_finish(c, t, std::move(turn), prev, view ? view : c->newest, restart, nullptr, dst, actions, values);
 }
 
 int paac_observe_host(paac_ctx* c, int t, const int8_t* rewards, const uint8_t* terminals) {
