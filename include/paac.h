@@ -301,9 +301,11 @@ int paac_debug_write(paac_ctx* ctx, int which, const void* src /* host */, size_
  * PAAC_OPT_UPDATE_CHUNKS: 1 (default) .. 4.  With more than one, the tensor-core update runs the second layer's data
  * gradient and the first layer's weight gradient alternately over that many groups of states, so that a group's slice
  * of the gradient between them is read back from L2 instead of HBM.  The weight gradient's partial sums are then
- * added in a different grouping: results agree to float rounding, not bit for bit, with the default. */
+ * added in a different grouping: results agree to float rounding, not bit for bit, with the default.
+ * PAAC_OPT_WAIT_POLLS: 1 .. 2,000,000 (default): polls after which a wait between the blocks of a one-launch rollout gives
+ * up.  For tests of that path: with 1 the first waits run out, the kernel records it in the error word and returns. */
 enum { PAAC_OPT_CUDA_CORES_ONLY = 1, PAAC_OPT_TC_WGRAD_LAYERS = 2, PAAC_OPT_CUDA_GRAPHS = 3, PAAC_OPT_DEPENDENT_LAUNCH = 4,
-       PAAC_OPT_FP32_TENSOR_CORES = 5, PAAC_OPT_UPDATE_CHUNKS = 6 };
+       PAAC_OPT_FP32_TENSOR_CORES = 5, PAAC_OPT_UPDATE_CHUNKS = 6, PAAC_OPT_WAIT_POLLS = 7 };
 int paac_set_option(paac_ctx* ctx, int option, int value);
 
 /* Failure-path check that cannot hang: launches one small kernel whose only thread block waits, at most

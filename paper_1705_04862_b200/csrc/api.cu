@@ -98,6 +98,7 @@ struct paac_ctx {
   DeviceStats* stats;
   uint32_t* sync;          // of the one-launch rollouts: steps so far, blocks that have ended
   uint4* words;            // and what their blocks hand each other
+  uint32_t wait_polls;     // after which a wait there gives up
   size_t n_words;
   size_t elt;              // bytes of one stored activation element
 };
@@ -257,7 +258,7 @@ void small_rollout(paac_ctx* c, const uint8_t* frames, int t0, int steps, int sa
   r.logits = c->logits + row * c->A; r.values = c->values + row; r.uniforms = c->uniforms + row; r.actions = c->actions + row;
   r.sampled = c->sampled + row; r.forced = c->forced_on ? c->forced + row : nullptr;
   r.seed = c->seed; r.step_base = c->step_dev; r.advance = advance ? (uint32_t)c->t_max : 0u;
-  r.mode = head_mode(c); r.error_word = &c->stats->error_word; r.words = c->words;
+  r.mode = head_mode(c); r.error_word = &c->stats->error_word; r.polls = c->wait_polls; r.words = c->words;
   if (env) r.env = *env;
   if (host) r.host = *host;
   if (use_tc(c)) launch_rollout_tc(c->lc, c->nd, c->theta, c->theta16, c->w_images, r);
@@ -486,6 +487,7 @@ int paac_init(paac_ctx** out, int arch, int n_e, int t_max, int n_actions, const
   c->update_chunks = 1;
   c->gact0_scale = 1.f;
   c->graphs_on = true;
+  c->wait_polls = WORD_POLLS;
   c->seed = seed; c->device = dev; c->st = (cudaStream_t)hp->stream; c->lc.st = c->st;
   const size_t need = carve(c, nullptr);
   if (hp->workspace) {
@@ -749,6 +751,10 @@ int paac_set_option(paac_ctx* c, int option, int value) {
   if (option == PAAC_OPT_UPDATE_CHUNKS) {
     if (value < 1 || value > TC_MAX_UPDATE_CHUNKS) return PAAC_ERR_ARG;
     c->update_chunks = value; drop_graphs(c); return PAAC_OK;
+  }
+  if (option == PAAC_OPT_WAIT_POLLS) {
+    if (value < 1 || value > (int)WORD_POLLS) return PAAC_ERR_ARG;
+    c->wait_polls = (uint32_t)value; drop_graphs(c); return PAAC_OK;
   }
   if (option == PAAC_OPT_FP32_TENSOR_CORES) { c->lc.fp32_tensor_cores = value != 0; drop_graphs(c); return PAAC_OK; }
   return PAAC_ERR_ARG;

@@ -149,6 +149,7 @@ bool rollout_small_supported(const LaunchCtx& lc, int arch, int prec, int n);   
 // what the blocks hand each other, of 16 bytes; all zero, like the two counters of SmallRollout::sync, before the first launch and
 // after a device error
 size_t rollout_small_words(int n);
+constexpr uint32_t WORD_POLLS = 2000000u;       // a healthy wait of the one-launch rollouts ends within microseconds
 struct SmallRollout {
   int n, steps, sample_steps; uint32_t t0;      // passes over slots t0 .. t0 + steps - 1; the first sample_steps sample an action
   bool step_env;                                // ... and step the synthetic environments with it (env)
@@ -159,7 +160,7 @@ struct SmallRollout {
   uint64_t seed; uint64_t* step_base; uint32_t advance;      // > 0: added to the step index at the end
   HostStep host;
   HeadMode mode; EnvStepArgs env;               // env.next_frames: the state after the last step; rewards, terminals of slot t0
-  uint32_t* error_word;
+  uint32_t* error_word; uint32_t polls;         // after which a wait gives up
 };
 void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const float* theta, const bf16* theta16, const SmallRollout& r);
 

@@ -62,7 +62,7 @@ struct RsArgs {
   uint32_t term_denom; int pattern_actions;
   HeadMode mode;
   HostStep host;
-  uint32_t* error_word;
+  uint32_t* error_word; uint32_t polls;
 };
 
 __device__ __forceinline__ void rs_fma4(float (&acc)[4], float a, const float4 w) {
@@ -260,7 +260,7 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
         const uint4* src = q.map1 + (size_t)e * (RS_POS1 * RC1::CO / 2) + 2 * in_lo + tid;
         const int count = (2 * (in_hi - in_lo) - tid + RS_THREADS - 1) / RS_THREADS;
         uint4 v[MOST];
-        word_await(v, src, RS_THREADS, count, tag, &s_dead, q.error_word);
+        word_await(v, src, RS_THREADS, count, tag, &s_dead, q.error_word, q.polls);
 #pragma unroll
         for (int u = 0; u < MOST; ++u)
           if (u < count) reinterpret_cast<float2*>(sm + RS_ACT1)[2 * in_lo + tid + u * RS_THREADS] = make_float2(__uint_as_float(v[u].x), __uint_as_float(v[u].z));
@@ -277,7 +277,7 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
           const int per = len / 2, r = tid / per, u = tid % per, apart = RS_THREADS / per, count = (rows - r + apart - 1) / apart;
           const uint4* src = q.map2 + (size_t)(r0 + r) * (RS_IN / 2) + k0 / 2 + u;
           uint4 v[RS_ROWS / 4];
-          word_await(v, src, (size_t)apart * (RS_IN / 2), count, tag, &s_dead, q.error_word);
+          word_await(v, src, (size_t)apart * (RS_IN / 2), count, tag, &s_dead, q.error_word, q.polls);
 #pragma unroll
           for (int i = 0; i < RS_ROWS / 4; ++i)
             if (i < count) *reinterpret_cast<float2*>(sm + RS_FCA + (r + apart * i) * RS_FC_LD + 2 * u) = make_float2(__uint_as_float(v[i].x), __uint_as_float(v[i].z));
@@ -320,7 +320,7 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
     if (stepping && tid == 32) prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, q.counters);
     {
       uint2 v[RS_RUNS];
-      word_await(v, sums + (size_t)e * RS_F + tid, (size_t)n * RS_F, RS_RUNS, tag, &s_dead, q.error_word);
+      word_await(v, sums + (size_t)e * RS_F + tid, (size_t)n * RS_F, RS_RUNS, tag, &s_dead, q.error_word, q.polls);
       double s = 0.0;
 #pragma unroll
       for (int p = 0; p < RS_RUNS; ++p) s += (double)__uint_as_float(v[p].x);
@@ -435,7 +435,7 @@ void launch_rollout_small(LaunchCtx& lc, int prec, const NetDims& nd, const floa
   q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
   q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
   q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode;
-  q.error_word = r.error_word;
+  q.error_word = r.error_word; q.polls = r.polls;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(q.blocks); cfg.blockDim = dim3(RS_THREADS); cfg.dynamicSmemBytes = rs_smem(q.A); cfg.stream = lc.st;
   cudaLaunchAttribute attr[1];

@@ -28,7 +28,9 @@
 // launch arguments: read from pinned memory by every block, they took 16 us each (reads of one address are served one after
 // the other).
 //
-// Every wait is bounded; a block that gave up goes on without waiting, as its cluster waits for it at the end.
+// Every wait is bounded.  A block that gave up finishes its step without waiting (it arrives at each of its barriers once a step, so
+// none is told of more bytes than it can count) and leaves the loop.  The blocks of its cluster then linger together: nobody leaves
+// before what was sent to or from it can have arrived.
 #include <cuda_fp16.h>
 
 #include "env_device.cuh"
@@ -65,7 +67,7 @@ struct RtArgs {
   uint32_t term_denom; int pattern_actions;
   HeadMode mode;
   HostStep host;                                  // external environments (one pass)
-  uint32_t* error_word;
+  uint32_t* error_word; uint32_t polls;
 };
 
 // ---- instructions ------------------------------------------------------------------------------------------------------
@@ -92,6 +94,7 @@ __device__ __forceinline__ uint32_t rt_map(uint32_t addr, uint32_t rank) {      
   return r;
 }
 __device__ __forceinline__ void rt_sts(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void rt_store(uint32_t to, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(to), "r"(v) : "memory"); }
 // four bytes, or `bytes` of this block's shared memory, to another block's, counted at its barrier
 __device__ __forceinline__ void rt_send(uint32_t to, uint32_t v, uint32_t bar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(to), "r"(v), "r"(bar) : "memory");
@@ -239,7 +242,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
   extern __shared__ __align__(128) uint8_t rt_smem[];
   __shared__ EnvFrame s_frame[RT_MAX_ENVS];
   __shared__ EnvPrep s_prep[RT_MAX_ENVS];
-  __shared__ volatile uint32_t s_dead;
+  __shared__ volatile uint32_t s_dead, s_linger;                  // a wait here, or in a block of the cluster, gave up
   __shared__ uint32_t s_epoch;
   __shared__ __align__(8) uint64_t s_map1, s_map2, s_heads;       // the other blocks' shares have arrived
   const uint32_t sm = tc::smem_u32(rt_smem);
@@ -272,7 +275,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
 
   // ---- what stays for the rollout ----
   if (tid == 0) {
-    s_dead = 0u; s_epoch = q.sync[0];
+    s_dead = 0u; s_linger = 0u; s_epoch = q.sync[0];
     tc::mbar_init(&s_map1, 1); tc::mbar_init(&s_map2, 1); tc::mbar_init(&s_heads, 1);
     tc::fence_barrier_init();
   }
@@ -334,10 +337,11 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
         rt_send_bulk(rt_map(at, to), at, bytes, rt_map(tc::smem_u32(bar), to));
       }
     }
-    if (!s_dead) tc::mbar_wait(bar, phase, &s_dead, q.error_word, tc::ERR_WAIT_FULL);
+    if (!s_dead) tc::mbar_wait_limit(bar, phase, &s_dead, q.error_word, tc::ERR_WAIT_FULL, 2u * q.polls);
   };
 
   for (int t = 0; t < q.steps; ++t) {
+    if (t > 0 && __syncthreads_or(s_dead)) break;         // (the last step's frame, and all reads of its rows, are done)
     const uint32_t tag = epoch + 1u + (uint32_t)t;
     const size_t slot = (size_t)t * n;
     // ---- convolutions, environment by environment ----
@@ -466,7 +470,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
         for (int r = tid >> 4; r < rows; r += RT_THREADS / 16) {
           const uint4* src = q.maps + ((size_t)(row0 + r) * RT_POS3 + kb0) * 16 + u;
           uint4 v[7];
-          word_await(v, src, 16, kbs, tag, &s_dead, q.error_word);
+          word_await(v, src, 16, kbs, tag, &s_dead, q.error_word, q.polls);
 #pragma unroll
           for (int p = 0; p < 7; ++p)
             if (p < kbs) {
@@ -522,7 +526,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
       const int e = cluster + ei * clusters, col = tid % (S::COLS / 2) * 2, u = unit_of(col);
       const uint4* src = q.sums + (size_t)e * 256 + u / 2;
       uint4 v[RT_SLICES];
-      word_await(v, src, (size_t)n * 256, RT_SLICES, tag, &s_dead, q.error_word);
+      word_await(v, src, (size_t)n * 256, RT_SLICES, tag, &s_dead, q.error_word, q.polls);
       float s0 = 0.f, s1 = 0.f;
 #pragma unroll
       for (int s = 0; s < RT_SLICES; ++s) {
@@ -558,7 +562,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
       }
       if (tid == 0) tc::mbar_arrive_expect_tx(&s_heads, (uint32_t)(C * outputs * 4));
     }
-    if (warp < envs && !s_dead) tc::mbar_wait(&s_heads, t & 1, &s_dead, q.error_word, tc::ERR_WAIT_FULL);
+    if (warp < envs && !s_dead) tc::mbar_wait_limit(&s_heads, t & 1, &s_dead, q.error_word, tc::ERR_WAIT_FULL, 2u * q.polls);
     if (warp < envs) {
       const int ei = warp, e = cluster + ei * clusters;
       const float* z = reinterpret_cast<const float*>(rt_smem + S::ZS) + ei * C * 36;
@@ -583,12 +587,15 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
         if (rank == 0) env_record(prep, o, (uint32_t)e, n, q.rewards + slot, q.terminals + slot, q.counters);
       }
     }
-    __syncthreads();
   }
-  // Nobody leaves before all that others send it has arrived (which a block that gave up did not wait for).
-  if (s_dead)
-    for (int i = 0; i < 100; ++i) __nanosleep(1000u);
+  // Nobody leaves before all that others send it has arrived: it waited for that, unless it gave up.  Then, once every block of the cluster
+  // has sent its last, all of them stay for 100 us (a copy takes about one).
+  if (__syncthreads_or(s_dead) && tid < C) rt_store(rt_map(tc::smem_u32(const_cast<uint32_t*>(&s_linger)), tid), 1u);
   rt_cluster_sync();
+  if (s_linger) {
+    for (int i = 0; i < 100; ++i) __nanosleep(1000u);
+    rt_cluster_sync();
+  }
   // Every block has read the counts when the last one ends.
   if (tid == 0) {
     __threadfence();
@@ -655,6 +662,7 @@ void launch_rollout_tc(LaunchCtx& lc, const NetDims& nd, const float* theta, con
   q.logits = r.logits; q.values = r.values; q.uniforms = r.uniforms; q.actions = r.actions; q.sampled = r.sampled; q.counters = r.env.counters;
   q.forced = r.forced; q.rewards = r.env.rewards; q.terminals = r.env.terminals; q.seed = r.seed; q.step_base = r.step_base; q.advance = r.advance;
   q.term_denom = r.env.term_denom; q.pattern_actions = r.env.pattern_actions; q.mode = r.mode; q.host = r.host; q.error_word = r.error_word;
+  q.polls = r.polls;
   lc.serialize_next = false;
   KernelScope scope(lc, KID_SMALL_ROLLOUT);
   const bool launched = rt_pick(r.n, [&](auto k) {

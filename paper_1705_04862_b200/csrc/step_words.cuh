@@ -6,14 +6,13 @@
 // overwritten for the next step once all that read it have: the kernels say why that holds.  The step numbers go on from launch
 // to launch; the block that ends last moves the count on (sync[0] steps so far, sync[1] blocks that have ended).
 //
-// Every wait is bounded.  A thread that gives up raises the error word and *dead, with which its block goes on without waiting.
+// Every wait is bounded (`limit` polls; WORD_POLLS, of the order of a second, unless a test asks for less).  A thread that gives up
+// raises the error word and *dead, with which its block goes on without waiting.
 #pragma once
 #include "common.cuh"
 #include "tc_common.cuh"
 
 namespace paac {
-
-constexpr uint32_t WORD_POLLS = 2000000u;
 
 __device__ __forceinline__ uint64_t word_half(uint32_t value, uint32_t step) { return (uint64_t)step << 32 | value; }
 __device__ __forceinline__ void word_peek(const uint4* p, uint4& v) {
@@ -37,7 +36,8 @@ __device__ __forceinline__ void word_store(uint2* p, uint32_t a, uint32_t step) 
 // v[i] = the word at p + i * stride, i < count (of N), once all are of the step, or as they are after a bounded wait.  All are asked
 // for together, again and again: one after the other each would cost a round trip through L2.
 template <int N, class W>
-__device__ __forceinline__ void word_await(W (&v)[N], const W* p, size_t stride, int count, uint32_t step, volatile uint32_t* dead, uint32_t* error_word) {
+__device__ __forceinline__ void word_await(W (&v)[N], const W* p, size_t stride, int count, uint32_t step, volatile uint32_t* dead, uint32_t* error_word,
+                                           uint32_t limit) {
   for (uint32_t polls = 0;; ++polls) {
     bool ready = true;
 #pragma unroll
@@ -47,7 +47,7 @@ __device__ __forceinline__ void word_await(W (&v)[N], const W* p, size_t stride,
     for (int i = 0; i < N; ++i)
       if (i < count) ready = ready && word_of(v[i], step);
     if (ready || *dead) return;
-    if (polls == WORD_POLLS) { *dead = 1u; atomicOr(error_word, tc::ERR_WAIT_FULL); return; }
+    if (polls == limit) { *dead = 1u; atomicOr(error_word, tc::ERR_WAIT_FULL); return; }
   }
 }
 

@@ -96,3 +96,57 @@ def test_planes_of_more_environments_than_one_launch_takes():
     want = torch.where(ends[:, None, None, None] != 0, planes[..., None].expand(-1, -1, -1, 4), pushed)
     assert np.array_equal(g.debug_read(pb.DBG_NEXT_FRAMES), want.contiguous().numpy().reshape(-1))
     g.close()
+
+
+@pytest.mark.parametrize("arch,prec,n_e", [("nature", pb.BF16, 1), ("nature", pb.BF16, 33), ("nature", pb.BF16, 74), ("nips", pb.FP32, 3),
+                                           ("nips", pb.BF16, 18), ("nips", pb.FP32, 37), ("nips", pb.FP32, 74)])
+def test_waits_between_blocks_give_up(arch, prec, n_e):
+    """With one poll to a wait the first ones run out: the launch ends, the error word says so, the update is skipped.  Once the word is
+    cleared the learner goes on, with whole rollouts and with steps of environments outside, as one to which nothing happened."""
+    a, b = (pb.Paac(arch, n_e, 4, 6, seed=8, precision=prec, lr=0.01, term_denom=5) for _ in range(2))
+    for g in (a, b):
+        g.rollout()
+        assert g.update()["status"] == 0
+    theta, rms = a.params(), a.debug_read(pb.DBG_RMS).copy()
+    with pytest.raises(pb.PaacError):
+        a.set_option(pb.OPT_WAIT_POLLS, 0)
+    rng = np.random.RandomState(n_e)
+    first, planes = rng.randint(0, 256, (n_e, 84, 84, 4), dtype=np.uint8), rng.randint(0, 256, (4, n_e, 84, 84), dtype=np.uint8)
+    acts, vals = np.zeros((2, n_e), np.int32), np.zeros((2, n_e), np.float32)
+
+    def outside(i, g):
+        seen = []
+        for t in range(5):
+            if t == 0:
+                g.act_host(0, first, acts[i], vals[i])
+            else:
+                g.act_host_newest(t, planes[t - 1], None, acts[i] if t < 4 else None, vals[i])
+            seen += [acts[i].copy(), vals[i].copy()]
+            if t < 4:
+                g.observe_host(t, np.ones(n_e, np.int8), np.zeros(n_e, np.uint8))
+        return seen
+
+    for limited in (lambda: a.rollout(), lambda: outside(0, a)):
+        a.set_option(pb.OPT_WAIT_POLLS, 1)
+        limited()
+        assert a.error_word() == 1
+        st = a.update()
+        assert st["status"] == pb.ERR_TIMEOUT and st["clip_scale"] == 0.0
+        a.set_option(pb.OPT_WAIT_POLLS, 2000000)
+        a.clear_error_word()
+        assert np.array_equal(a.params(), theta) and np.array_equal(a.debug_read(pb.DBG_RMS), rms)
+        b.rollout()                                            # as many steps as the one that was cut short
+        for which in (pb.DBG_NEXT_FRAMES, pb.DBG_COUNTERS):
+            a.debug_write(which, b.debug_read(which))
+        for again in range(2):
+            for g in (a, b):
+                g.rollout()
+            for which in (pb.DBG_FRAMES, pb.DBG_NEXT_FRAMES, pb.DBG_ACTIONS, pb.DBG_REWARDS, pb.DBG_VALUES, pb.DBG_LOGITS, pb.DBG_UNIFORMS, pb.DBG_COUNTERS):
+                assert np.array_equal(a.debug_read(which).view(np.uint8), b.debug_read(which).view(np.uint8)), which
+        for x, y in zip(outside(0, a), outside(1, b)):
+            assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
+        for g in (a, b):
+            assert g.update()["status"] == 0
+        theta, rms = a.params(), a.debug_read(pb.DBG_RMS).copy()
+        assert np.array_equal(theta, b.params())
+    a.close(), b.close()
