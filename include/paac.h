@@ -288,10 +288,11 @@ int paac_debug_write(paac_ctx* ctx, int which, const void* src /* host */, size_
  * PAAC_OPT_CUDA_GRAPHS: != 0 (default) lets paac_rollout / paac_update record their kernel sequence into CUDA
  * graphs after two plain iterations and replay them; 0 keeps every call on plain launches.  (Graphs are also
  * bypassed while actions are forced or per-kernel profiling is on.)
- * PAAC_OPT_DEPENDENT_LAUNCH: != 0 (default) launches every kernel with programmatic stream serialization, so
+ * PAAC_OPT_DEPENDENT_LAUNCH: != 0 (default) launches kernels with programmatic stream serialization, so
  * that a kernel's CTAs are scheduled while the kernel before it drains (each kernel waits on the device for its
  * predecessor before it touches that kernel's data); 0 launches with plain stream order.  The setting is
- * process-wide.  Results are bit-identical either way.
+ * process-wide and holds for the entry points without a context too (paac_preprocess, paac_stack_push,
+ * paac_clip_rmsprop_noalloc).  Results are bit-identical either way.
  * PAAC_OPT_FP32_TENSOR_CORES: != 0 runs every contraction of the CUDA-core path (PAAC_FP32 on either network, and
  * PAAC_BF16 with PAAC_OPT_CUDA_CORES_ONLY) on the tensor cores at float accuracy: each float operand is split into two
  * TF32 pieces (22 significant bits together) and three tcgen05 passes (hi*hi + hi*lo + lo*hi) are accumulated in one
@@ -344,8 +345,7 @@ int paac_profile_read(paac_ctx* ctx, int max_entries, const char** names /* out 
  *   theta_bf16   device, nullable: bfloat16 bits of the new theta, [n]
  *   norm_and_scale  device float[2], nullable: gradient norm before clipping, factor applied (0 when
  *                   the norm was not finite and nothing was changed)
- *   stream       cudaStream_t; the work is enqueued on it (one kernel up to 8192 parameters, else two, the second of
- *                which may start while the first runs, whatever PAAC_OPT_DEPENDENT_LAUNCH says), the call does not
+ *   stream       cudaStream_t; the work is enqueued on it (one kernel up to 8192 parameters, else two), the call does not
  *                synchronise
  *
  * n may not exceed paac_noalloc_max_params() (16,777,216): beyond that the call returns PAAC_ERR_LIMIT

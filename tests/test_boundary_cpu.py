@@ -172,3 +172,32 @@ def test_a_word_that_carries_its_step_is_never_seen_in_part():
     assert [n * bits for n, bits in accesses["ld"]] == [n * bits for n, bits in accesses["st"]] == [64, 128]
     for load, store in zip(accesses["ld"], accesses["st"]):
         assert not _torn_reads(store, load), (store, load)
+
+
+# preprocess.cu as it is, but for launches that are recorded instead of made
+LAUNCHES = """
+#include <cuda_runtime.h>
+static int attributes = -1;
+template <class K, class... Args> static cudaError_t recorded(const cudaLaunchConfig_t* cfg, K, Args&&...) { attributes = (int)cfg->numAttrs; return cudaSuccess; }
+#define cudaLaunchKernelEx recorded
+#include "preprocess.cu"
+extern "C" int push_with(int dependent_launch) {
+  paac::pdl_enabled() = dependent_launch != 0;
+  attributes = -1;
+  const uint8_t* p = (const uint8_t*)4096;
+  paac_stack_push(p, p, nullptr, (uint8_t*)p, 1, nullptr);       // (its status is that of a machine without a device)
+  return attributes;
+}
+"""
+
+
+def _compiled_cuda(tmp_path, source):
+    src, so = tmp_path / "host.cu", tmp_path / "host.so"
+    src.write_text(source)
+    subprocess.run([pbuild.NVCC] + pbuild.FLAGS + ["-shared", "-I", pbuild.CSRC, str(src), "-o", str(so)], check=True)
+    return so
+
+
+def test_entry_points_without_a_context_follow_the_launch_option(tmp_path):
+    push = C.CDLL(str(_compiled_cuda(tmp_path, LAUNCHES))).push_with
+    assert [push(1), push(0), push(1)] == [1, 0, 1]
