@@ -341,6 +341,12 @@ inline cudaError_t launch_overlapped_on(cudaStream_t stream, void (*kern)(KArgs.
   return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
+// Their status.  A launch that failed has left its error behind: taken away here, or the caller's next check would find it.
+inline int launch_status(cudaError_t launched) {
+  const cudaError_t last = cudaGetLastError();
+  return launched == cudaSuccess && last == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
+}
+
 // bits of DeviceStats::error_word: 1, 2, 4 = a bounded wait gave up (which kind: see tc_common.cuh);
 // 8 = a first-layer weight does not fit the fp16 image the forward kernel multiplies with
 constexpr uint32_t DEV_ERR_WAIT_MASK = 7u, DEV_ERR_RANGE = 8u;

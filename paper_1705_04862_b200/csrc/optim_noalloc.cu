@@ -207,14 +207,15 @@ extern "C" int paac_clip_rmsprop_noalloc(float* theta, float* rms, const float* 
   if (st != PAAC_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool wide = (((uintptr_t)theta | (uintptr_t)rms | (uintptr_t)grad) & 15u) == 0 && ((uintptr_t)theta_bf16 & 7u) == 0;
+  cudaError_t launched;
   if (n <= (size_t)NA_ONE_BLOCK)
-    paac::launch_overlapped_on(s, noalloc_one_block_kernel, dim3(1), dim3(NA_ONE_THREADS), 0, theta, rms, grad, theta_bf16, (int)n, lr, rms_decay, rms_eps,
-                               clip_norm, norm_and_scale);
+    launched = paac::launch_overlapped_on(s, noalloc_one_block_kernel, dim3(1), dim3(NA_ONE_THREADS), 0, theta, rms, grad, theta_bf16, (int)n, lr, rms_decay,
+                                          rms_eps, clip_norm, norm_and_scale);
   else if (wide)
-    two_launches<4>(theta, rms, grad, theta_bf16, n, lr, rms_decay, rms_eps, clip_norm, partials, norm_and_scale, s);
+    launched = two_launches<4>(theta, rms, grad, theta_bf16, n, lr, rms_decay, rms_eps, clip_norm, partials, norm_and_scale, s);
   else
-    two_launches<1>(theta, rms, grad, theta_bf16, n, lr, rms_decay, rms_eps, clip_norm, partials, norm_and_scale, s);
-  return cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
+    launched = two_launches<1>(theta, rms, grad, theta_bf16, n, lr, rms_decay, rms_eps, clip_norm, partials, norm_and_scale, s);
+  return paac::launch_status(launched);
 }
 
 extern "C" size_t paac_noalloc_max_params(void) { return NA_MAX_PARAMS; }

@@ -233,7 +233,7 @@ extern "C" int paac_stack_push(const uint8_t* state_in, const uint8_t* newest, c
   if (((uintptr_t)state_in | (uintptr_t)state_out) & 15u) return PAAC_ERR_ARG;
   if ((uintptr_t)newest & 3u) return PAAC_ERR_ARG;
   const cudaError_t launched = launch_overlapped_on((cudaStream_t)stream, stack_push_kernel, dim3(2, n), dim3(SP_THREADS), 0, state_in, newest, restart, state_out);
-  return launched == cudaSuccess && cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
+  return launch_status(launched);
 }
 
 extern "C" int paac_preprocess(const uint8_t* raw_prev, const uint8_t* raw_last, const uint8_t* state_in,
@@ -252,5 +252,5 @@ extern "C" int paac_preprocess(const uint8_t* raw_prev, const uint8_t* raw_last,
   const int tasks = PP_BANDS * n, blocks = tasks < 2 * 148 ? tasks : 2 * 148;      // two blocks per SM are resident
   const cudaError_t launched = launch_overlapped_on((cudaStream_t)stream, preprocess_kernel, dim3(blocks), dim3(PP_THREADS), sizeof(PpShared), raw_prev, raw_last,
                                                     state_in, state_out, tasks);
-  return launched == cudaSuccess && cudaGetLastError() == cudaSuccess ? PAAC_OK : PAAC_ERR_CUDA;
+  return launch_status(launched);
 }

@@ -178,15 +178,31 @@ def test_a_word_that_carries_its_step_is_never_seen_in_part():
 LAUNCHES = """
 #include <cuda_runtime.h>
 static int attributes = -1;
-template <class K, class... Args> static cudaError_t recorded(const cudaLaunchConfig_t* cfg, K, Args&&...) { attributes = (int)cfg->numAttrs; return cudaSuccess; }
+static cudaError_t outcome = cudaSuccess, last = cudaSuccess;
+template <class K, class... Args> static cudaError_t recorded(const cudaLaunchConfig_t* cfg, K, Args&&...) {
+  attributes = (int)cfg->numAttrs;
+  if (outcome != cudaSuccess) last = outcome;
+  return outcome;
+}
+static cudaError_t take_last() { const cudaError_t e = last; last = cudaSuccess; return e; }
 #define cudaLaunchKernelEx recorded
+#define cudaGetLastError take_last
+#define cudaGetDevice(device) (*(device) = 0, cudaSuccess)
+#define cudaFuncSetAttribute(...) cudaSuccess
 #include "preprocess.cu"
 extern "C" int push_with(int dependent_launch) {
   paac::pdl_enabled() = dependent_launch != 0;
   attributes = -1;
   const uint8_t* p = (const uint8_t*)4096;
-  paac_stack_push(p, p, nullptr, (uint8_t*)p, 1, nullptr);       // (its status is that of a machine without a device)
-  return attributes;
+  return paac_stack_push(p, p, nullptr, (uint8_t*)p, 1, nullptr) == PAAC_OK ? attributes : -2;
+}
+extern "C" int status_and_error_left(int call, int outcome_of_launch, int error_before) {      // 100 * status + what the caller finds
+  const uint8_t* p = (const uint8_t*)4096;
+  outcome = (cudaError_t)outcome_of_launch;
+  last = (cudaError_t)error_before;
+  const int status = call == 0 ? paac_stack_push(p, p, nullptr, (uint8_t*)p, 1, nullptr) : paac_preprocess(p, p, nullptr, (uint8_t*)p, 1, nullptr);
+  outcome = cudaSuccess;
+  return 100 * status + (int)take_last();
 }
 """
 
@@ -201,3 +217,11 @@ def _compiled_cuda(tmp_path, source):
 def test_entry_points_without_a_context_follow_the_launch_option(tmp_path):
     push = C.CDLL(str(_compiled_cuda(tmp_path, LAUNCHES))).push_with
     assert [push(1), push(0), push(1)] == [1, 0, 1]
+
+
+@pytest.mark.parametrize("call", [0, 1])
+def test_a_failed_launch_leaves_no_error_behind(tmp_path, call):
+    of = C.CDLL(str(_compiled_cuda(tmp_path, LAUNCHES))).status_and_error_left
+    assert of(call, 0, 0) == 0
+    assert of(call, 9, 0) == 100 * pb.ERR_CUDA          # the launch fails
+    assert of(call, 0, 1) == 100 * pb.ERR_CUDA          # an error that the caller had not looked at
