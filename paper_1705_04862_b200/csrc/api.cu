@@ -786,9 +786,12 @@ int paac_profile_read(paac_ctx* c, int max_entries, const char** names, double* 
 // The network on the state at `dst`, with `prev` after the frame stack has built that state from `planes`, and the results into the
 // box.  The frame stack's arguments differ from step to step, so it is launched by itself; the rest is one launch sequence,
 // recorded from the second time on, or, for few environments, part of the same kernel, which can also fetch whole `states`.
-// From HOST_PLAIN_FROM environments on the planes take longer over the link than the other launches take to be made, and launched
-// one by one the first layer sets itself up meanwhile (a recorded sequence starts when the frame stack has ended): an iteration of
-// 384, 512 and 1024 environments 820 -> 812, 990 -> 978 and 1620 -> 1609 us, but 668 -> 672 with 256.
+// On the tensor-core path, from HOST_PLAIN_FROM environments on, the planes take longer over the link than the other launches take to
+// be made, and launched one by one the first layer sets itself up meanwhile (a recorded sequence starts when the frame stack has
+// ended): an iteration of 384, 512 and 1024 environments 820 -> 812, 990 -> 978 and 1620 -> 1609 us, but 668 -> 672 with 256 and 741 -> 744
+// with 320.  A slower host moves the line up.  The CUDA-core path's first layer has nothing to set up and its kernels are longer: float
+// storage with 320 and 512 environments takes 3199 us recorded and 3215 one by one, 4765 and 4782; the smaller network 1579 and 1578,
+// 2361 and 2352, 4224 and 4228 with 1024 (a run's iterations differ by 10 to 20).  It stays recorded.
 constexpr int HOST_PLAIN_FROM = 320;
 static int act_host_finish(paac_ctx* c, int t, std::unique_lock<std::mutex> turn, const uint8_t* prev, const uint8_t* planes, const uint8_t* restart, const uint8_t* states, uint8_t* dst,
                            int32_t* actions, float* values) {
@@ -810,7 +813,7 @@ static int act_host_finish(paac_ctx* c, int t, std::unique_lock<std::mutex> turn
       if (!sample && !advanced) launch_advance_step(c->lc, c->step_dev, (uint32_t)c->t_max);
       launch_publish(c->lc, sample ? c->actions + row : nullptr, c->values + row, c->n_e, box->actions, box->values, &box->done);
     };
-    if (prev && c->n_e >= HOST_PLAIN_FROM) enqueue();
+    if (prev && use_tc(c) && c->n_e >= HOST_PLAIN_FROM) enqueue();
     else run_recorded(c, 4 + t, c->cur, enqueue);
   }
   if (!await_box(c)) return PAAC_ERR_CUDA;
