@@ -69,3 +69,11 @@ def _compare(arch, prec, n_e, layered_too, iterations=3):
 def test_recorded_and_launched_one_by_one(arch, prec, n_e):
     """Either side of where a step's launches follow the frame stack one by one, and the path on which they stay recorded."""
     _compare(arch, prec, n_e, layered_too=False, iterations=5)
+
+
+@pytest.mark.parametrize("arch,prec,n_e", [("nature", pb.BF16, 1), ("nature", pb.BF16, 33), ("nature", pb.BF16, 34), ("nature", pb.BF16, 74),
+                                           ("nips", pb.FP32, 9), ("nips", pb.BF16, 10), ("nips", pb.FP32, 18), ("nips", pb.FP32, 19),
+                                           ("nips", pb.BF16, 37), ("nips", pb.FP32, 38), ("nips", pb.BF16, 74)])
+def test_steps_in_one_launch_fetch_what_was_sent(arch, prec, n_e):
+    """The smallest and the largest number of environments of every group of blocks, each block of which fetches a share of its own."""
+    _compare(arch, prec, n_e, layered_too=True)
