@@ -6,13 +6,15 @@ namespace paac {
 
 constexpr int FRAME_WORDS = FRAME_H * FRAME_W;   // 7056, a multiple of 4
 
-// what of a transition does not depend on the action: prepared by one thread while the action is being found
+// What of a transition does not depend on the action: prepared by one thread while the action is being found.  Without `counters` (a
+// block that will not record the transition, beside one that may be writing them) those are left out.
 struct EnvPrep { uint32_t pre_step, pre_next; int32_t len, ret, episodes; };
 __device__ __forceinline__ EnvPrep env_prepare(uint64_t seed, uint32_t e, int n_e, uint32_t step, const int32_t* counters) {
   EnvPrep p;
   p.pre_step = env_hash_prefix(seed, e, step);
   p.pre_next = env_hash_prefix(seed, e, step + 1u);
-  p.len = counters[e]; p.ret = counters[n_e + e]; p.episodes = counters[2 * n_e + e];
+  p.len = p.ret = p.episodes = 0;
+  if (counters != nullptr) { p.len = counters[e]; p.ret = counters[n_e + e]; p.episodes = counters[2 * n_e + e]; }
   return p;
 }
 // the frame of a state: its hash base, and the band of the learnable environment in pixel words (empty otherwise)

@@ -317,7 +317,7 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
     // ---- the end of the state's pass, in every block of the group ----
     const bool sample = t < q.sample_steps, stepping = sample && q.env;
     EnvPrep prep{};
-    if (stepping && tid == 32) prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, q.counters);
+    if (stepping && tid == 32) prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, rank == 0 ? q.counters : nullptr);
     {
       uint2 v[RS_RUNS];
       word_await(v, sums + (size_t)e * RS_F + tid, (size_t)n * RS_F, RS_RUNS, tag, &s_dead, q.error_word, q.polls);

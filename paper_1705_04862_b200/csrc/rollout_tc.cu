@@ -519,7 +519,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
     const bool sample = t < q.sample_steps, stepping = sample && q.env;
     if (stepping && lane == 0 && warp >= 8 && warp - 8 < envs) {
       const int ei = warp - 8;
-      s_prep[ei] = env_prepare(q.seed, (uint32_t)(cluster + ei * clusters), n, (uint32_t)step0 + t, q.counters);
+      s_prep[ei] = env_prepare(q.seed, (uint32_t)(cluster + ei * clusters), n, (uint32_t)step0 + t, rank == 0 ? q.counters : nullptr);
     }
     float* xs = reinterpret_cast<float*>(rt_smem + S::XS);
     for (int ei = tid / (S::COLS / 2); ei < envs; ei += RT_THREADS / (S::COLS / 2)) {
