@@ -40,12 +40,12 @@
 namespace paac {
 
 typedef NatConv1 TC1; typedef NatConv2 TC2; typedef NatConv3 TC3;
-constexpr int RT_THREADS = 512, RT_WARPS = RT_THREADS / 32, RT_MAX_ENVS = 1;        // environments of a cluster
+constexpr int RT_THREADS = 512, RT_WARPS = RT_THREADS / 32;
 constexpr int RT_F = 512, RT_SLICES = 8, RT_TILE = 32, RT_FC_BLOCKS = RT_SLICES * (RT_F / RT_TILE), RT_ROWS = 64;
 constexpr int RT_POS3 = TC3::OH * TC3::OW, RT_FC_LD = 7 * 128;                      // 49 blocks of 64 k, six or seven to a slice
 
 struct RtArgs {
-  int n, A, steps, clusters;                      // forward passes: slots t0 .. t0 + steps - 1
+  int n, A, steps;                                // forward passes: slots t0 .. t0 + steps - 1
   uint32_t t0;
   const uint8_t* frames; size_t frame_step;       // states of slot t0, and from one slot to the next
   uint8_t* next_frames;                           // states of the slot after the last one that steps (rollout)
@@ -125,7 +125,7 @@ template <int C> struct RtMem {
   static constexpr int W1 = 0, W2 = W1 + N1 * 4096, W3 = W2 + N2 * 8 * 1024, WFC = W3 + N2 * 8 * 1152, HEADW = WFC + RT_TILE * RT_FC_LD,
                        FRAME = HEADW + (33 * COLS * 2 + 127) / 128 * 128, ACT1 = FRAME + (FRAME_BYTES + 127) / 128 * 128, ACT2 = ACT1 + (4 * RT_PLANE1 + 127) / 128 * 128,
                        B1 = ACT2 + (8 * RT_PLANE2 + 127) / 128 * 128, B2 = B1 + N1 * 32, B3 = B2 + N2 * 32, BFC = B3 + N2 * 32, BHEAD = BFC + COLS * 4,
-                       XS = (BHEAD + 33 * 4 + 15) / 16 * 16, ZS = XS + RT_MAX_ENVS * COLS * 4, TOTAL = ZS + RT_MAX_ENVS * C * 36 * 4;
+                       XS = (BHEAD + 33 * 4 + 15) / 16 * 16, ZS = XS + COLS * 4, TOTAL = ZS + C * 36 * 4;
   static constexpr int ROWS = FRAME;              // the states' rows for the fully connected layer lie over the frame and the maps
   static_assert(ROWS + RT_ROWS * RT_FC_LD <= B1, "rows of the fully connected layer");
   static_assert(TOTAL <= 227 * 1024, "shared memory");
@@ -240,16 +240,16 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(RT_THREADS, 1)
 rollout_tc_kernel(const __grid_constant__ RtArgs q) {
   typedef RtMem<C> S;
   extern __shared__ __align__(128) uint8_t rt_smem[];
-  __shared__ EnvFrame s_frame[RT_MAX_ENVS];
-  __shared__ EnvPrep s_prep[RT_MAX_ENVS];
+  __shared__ EnvFrame s_frame;
+  __shared__ EnvPrep s_prep;
   __shared__ volatile uint32_t s_dead, s_linger;                  // a wait here, or in a block of the cluster, gave up
   __shared__ uint32_t s_epoch;
   __shared__ __align__(8) uint64_t s_map1, s_map2, s_heads;       // the other blocks' shares have arrived
   const uint32_t sm = tc::smem_u32(rt_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = q.n, A = q.A;
   const int g = lane >> 2, t4 = lane & 3;
-  const int rank = (int)rt_rank(), cluster = blockIdx.x / C, clusters = q.clusters;
-  const int envs = cluster < n ? (n - cluster + clusters - 1) / clusters : 0;          // this cluster's: cluster, cluster + clusters, ...
+  const int rank = (int)rt_rank(), e = blockIdx.x / C;             // this cluster's environment
+  const bool conv = e < n;
   const bool fc = blockIdx.x < RT_FC_BLOCKS;
   const int slice = blockIdx.x % RT_SLICES, unit0 = blockIdx.x / RT_SLICES * RT_TILE;
   const int kb0 = slice * 6 + (slice > 0 ? 1 : 0), kbs = slice == 0 ? 7 : 6;           // 49 blocks of 64 k: seven, then six each
@@ -261,17 +261,17 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
 
   // the newest plane comes over the host link meanwhile: sixteen pixels to a thread
   const int px_lo = STACK_ITEMS * rank / C, px_hi = STACK_ITEMS * (rank + 1) / C;
-  static_assert((STACK_ITEMS + C - 1) / C <= RT_THREADS && FRAME_WORDS / 4 / C <= 2 * RT_THREADS && RT_MAX_ENVS == 1, "one piece to a thread");
+  static_assert((STACK_ITEMS + C - 1) / C <= RT_THREADS && FRAME_WORDS / 4 / C <= 2 * RT_THREADS, "one piece to a thread");
   uint4 plane{};
-  const bool pulls = q.host.newest != nullptr && envs > 0 && px_lo + tid < px_hi;
-  if (pulls) plane = reinterpret_cast<const uint4*>(q.host.newest)[(size_t)cluster * STACK_ITEMS + px_lo + tid];
+  const bool pulls = q.host.newest != nullptr && conv && px_lo + tid < px_hi;
+  if (pulls) plane = reinterpret_cast<const uint4*>(q.host.newest)[(size_t)e * STACK_ITEMS + px_lo + tid];
   // or the whole state: four such words
   const int st_lo = FRAME_WORDS / 4 * rank / C, st_hi = FRAME_WORDS / 4 * (rank + 1) / C;
   uint4 whole[2];
-  if (q.host.states != nullptr && envs > 0)
+  if (q.host.states != nullptr && conv)
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-      if (st_lo + tid + i * RT_THREADS < st_hi) whole[i] = reinterpret_cast<const uint4*>(q.host.states)[(size_t)cluster * (FRAME_WORDS / 4) + st_lo + tid + i * RT_THREADS];
+      if (st_lo + tid + i * RT_THREADS < st_hi) whole[i] = reinterpret_cast<const uint4*>(q.host.states)[(size_t)e * (FRAME_WORDS / 4) + st_lo + tid + i * RT_THREADS];
 
   // ---- what stays for the rollout ----
   if (tid == 0) {
@@ -279,7 +279,7 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
     tc::mbar_init(&s_map1, 1); tc::mbar_init(&s_map2, 1); tc::mbar_init(&s_heads, 1);
     tc::fence_barrier_init();
   }
-  if (envs > 0) {
+  if (conv) {
     for (int i = tid; i < S::N1 * 16 * 32; i += RT_THREADS) {
       const int l = i & 31, step = i >> 5, j = step >> 4, co = (rank * S::N1 + j) * 8 + (l >> 2);
       *reinterpret_cast<uint2*>(rt_smem + S::W1 + i * 8) = __ldg(reinterpret_cast<const uint2*>(q.w1 + ((size_t)co * 16 + (step & 15)) * 16 + 4 * (l & 3)));
@@ -296,8 +296,6 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
       const int k = i / S::COLS, u = unit_of(i % S::COLS);
       reinterpret_cast<bf16*>(rt_smem + S::HEADW)[i] = k < A ? q.wpi[(size_t)k * RT_F + u] : q.wv[u];
     }
-  }
-  if (envs > 0) {
     float* b = reinterpret_cast<float*>(rt_smem);
     if (tid < S::N1 * 8) b[S::B1 / 4 + tid] = q.b1[rank * S::N1 * 8 + tid];
     if (tid < S::N2 * 8) { b[S::B2 / 4 + tid] = q.b2[rank * S::N2 * 8 + tid]; b[S::B3 / 4 + tid] = q.b3[rank * S::N2 * 8 + tid]; }
@@ -312,14 +310,14 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
   tc::cp_async_commit();
   const uint64_t step0 = *q.step_base + q.t0;
   if (pulls) {
-    const size_t at = (size_t)cluster * STACK_ITEMS + px_lo + tid;
-    stack_sixteen(plane, (q.host.fresh[cluster >> 5] >> (cluster & 31)) & 1u, reinterpret_cast<const uint4*>(q.host.prev) + 4 * at,
+    const size_t at = (size_t)e * STACK_ITEMS + px_lo + tid;
+    stack_sixteen(plane, (q.host.fresh[e >> 5] >> (e & 31)) & 1u, reinterpret_cast<const uint4*>(q.host.prev) + 4 * at,
                   reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames)) + 4 * at);
   }
-  if (q.host.states != nullptr && envs > 0)
+  if (q.host.states != nullptr && conv)
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-      if (st_lo + tid + i * RT_THREADS < st_hi) reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames))[(size_t)cluster * (FRAME_WORDS / 4) + st_lo + tid + i * RT_THREADS] = whole[i];
+      if (st_lo + tid + i * RT_THREADS < st_hi) reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames))[(size_t)e * (FRAME_WORDS / 4) + st_lo + tid + i * RT_THREADS] = whole[i];
   tc::cp_async_wait<0>();
   __syncthreads();
   const uint32_t epoch = s_epoch;
@@ -344,16 +342,15 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
     if (t > 0 && __syncthreads_or(s_dead)) break;         // (the last step's frame, and all reads of its rows, are done)
     const uint32_t tag = epoch + 1u + (uint32_t)t;
     const size_t slot = (size_t)t * n;
-    // ---- convolutions, environment by environment ----
-    for (int ei = 0; ei < envs; ++ei) {
-      const int e = cluster + ei * clusters;
+    // ---- convolutions ----
+    if (conv) {
       uint4* frame = reinterpret_cast<uint4*>(rt_smem + S::FRAME);
       if (t == 0) {
         const uint4* src = reinterpret_cast<const uint4*>(q.frames + (size_t)e * FRAME_BYTES);
         for (int i = tid; i < FRAME_WORDS / 4; i += RT_THREADS) frame[i] = __ldcg(src + i);
       } else {
         // the state the last step reached: for this block, and its share for everyone
-        const EnvFrame f = s_frame[ei];
+        const EnvFrame f = s_frame;
         uint8_t* states = t < q.sample_steps ? const_cast<uint8_t*>(q.frames) + (size_t)t * q.frame_step : q.next_frames;
         uint4* out = reinterpret_cast<uint4*>(states + (size_t)e * FRAME_BYTES);
         const int lo = FRAME_WORDS / 4 * rank / C, hi = FRAME_WORDS / 4 * (rank + 1) / C;
@@ -514,16 +511,13 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
         }
         __syncthreads();
       }
-    if (envs == 0) continue;
-    // ---- the end of the states' pass: this block's hidden units and their part of the heads ----
+    if (!conv) continue;
+    // ---- the end of the state's pass: this block's hidden units and their part of the heads ----
     const bool sample = t < q.sample_steps, stepping = sample && q.env;
-    if (stepping && lane == 0 && warp >= 8 && warp - 8 < envs) {
-      const int ei = warp - 8;
-      s_prep[ei] = env_prepare(q.seed, (uint32_t)(cluster + ei * clusters), n, (uint32_t)step0 + t, rank == 0 ? q.counters : nullptr);
-    }
+    if (stepping && lane == 0 && warp == 8) s_prep = env_prepare(q.seed, (uint32_t)e, n, (uint32_t)step0 + t, rank == 0 ? q.counters : nullptr);
     float* xs = reinterpret_cast<float*>(rt_smem + S::XS);
-    for (int ei = tid / (S::COLS / 2); ei < envs; ei += RT_THREADS / (S::COLS / 2)) {
-      const int e = cluster + ei * clusters, col = tid % (S::COLS / 2) * 2, u = unit_of(col);
+    if (tid < S::COLS / 2) {
+      const int col = tid * 2, u = unit_of(col);
       const uint4* src = q.sums + (size_t)e * 256 + u / 2;
       uint4 v[RT_SLICES];
       word_await(v, src, (size_t)n * 256, RT_SLICES, tag, &s_dead, q.error_word, q.polls);
@@ -535,19 +529,19 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
       const float2 b = *reinterpret_cast<const float2*>(rt_smem + S::BFC + col * 4);
       const __nv_bfloat162 x = __floats2bfloat162_rn(fmaxf(s0 + b.x, 0.f), fmaxf(s1 + b.y, 0.f));
       *reinterpret_cast<__nv_bfloat162*>(q.h + (slot + e) * RT_F + u) = x;
-      *reinterpret_cast<float2*>(xs + ei * S::COLS + col) = __bfloat1622float2(x);
+      *reinterpret_cast<float2*>(xs + col) = __bfloat1622float2(x);
     }
     __syncthreads();
     {
       // RUNS lanes to a head output: each its running sum over four groups of four units, then the tree over this block's sums
       constexpr int PER = 32 / S::RUNS;
-      const int run = lane % S::RUNS, outputs = envs * (A + 1);
+      const int run = lane % S::RUNS, outputs = A + 1;
       for (int o0 = warp * PER; o0 < outputs; o0 += RT_WARPS * PER) {
-        const int o = min(o0 + lane / S::RUNS, outputs - 1), ei = o / (A + 1), k = o - ei * (A + 1);
+        const int k = min(o0 + lane / S::RUNS, outputs - 1);
         float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float4 x = *reinterpret_cast<const float4*>(xs + ei * S::COLS + 4 * (run + S::RUNS * j));
+          const float4 x = *reinterpret_cast<const float4*>(xs + 4 * (run + S::RUNS * j));
           const uint2 w = *reinterpret_cast<const uint2*>(rt_smem + S::HEADW + (k * S::COLS + 4 * (run + S::RUNS * j)) * 2);
           acc0 = fmaf(__uint_as_float(w.x << 16), x.x, acc0);
           acc1 = fmaf(__uint_as_float(w.x & 0xFFFF0000u), x.y, acc1);
@@ -558,14 +552,13 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
 #pragma unroll
         for (int b = S::RUNS / 2; b > 0; b >>= 1) v += __shfl_xor_sync(0xffffffffu, v, b);
         if (run < C && o0 + lane / S::RUNS < outputs)
-          rt_send(rt_map(sm + S::ZS + (uint32_t)((ei * C + rank) * 36 + k) * 4u, run), __float_as_uint(v), rt_map(tc::smem_u32(&s_heads), run));
+          rt_send(rt_map(sm + S::ZS + (uint32_t)(rank * 36 + k) * 4u, run), __float_as_uint(v), rt_map(tc::smem_u32(&s_heads), run));
       }
       if (tid == 0) tc::mbar_arrive_expect_tx(&s_heads, (uint32_t)(C * outputs * 4));
     }
-    if (warp < envs && !s_dead) tc::mbar_wait_limit(&s_heads, t & 1, &s_dead, q.error_word, tc::ERR_WAIT_FULL, 2u * q.polls);
-    if (warp < envs) {
-      const int ei = warp, e = cluster + ei * clusters;
-      const float* z = reinterpret_cast<const float*>(rt_smem + S::ZS) + ei * C * 36;
+    if (warp == 0 && !s_dead) tc::mbar_wait_limit(&s_heads, t & 1, &s_dead, q.error_word, tc::ERR_WAIT_FULL, 2u * q.polls);
+    if (warp == 0) {
+      const float* z = reinterpret_cast<const float*>(rt_smem + S::ZS);
       float s = -INFINITY;
       if (lane <= A) {
         if constexpr (C == 2) s = z[lane] + z[36 + lane];
@@ -581,9 +574,9 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
         __threadfence_system();
       }
       if (stepping && lane == 0) {
-        const EnvPrep prep = s_prep[ei];
+        const EnvPrep prep = s_prep;
         const EnvOutcome o = env_outcome(prep, a, q.term_denom, q.pattern_actions);
-        s_frame[ei] = env_frame_of(prep.pre_next, o.tag, q.pattern_actions);
+        s_frame = env_frame_of(prep.pre_next, o.tag, q.pattern_actions);
         if (rank == 0) env_record(prep, o, (uint32_t)e, n, q.rewards + slot, q.terminals + slot, q.counters);
       }
     }
@@ -644,7 +637,7 @@ template <class F> static auto rt_pick(int n, F f) {
 // and this kernel 66 to 92.  With a second environment for some clusters it takes 135 us at 75 and 154 at 148, against 130 and 157.
 constexpr int RT_MOST = 74;
 bool rollout_tc_supported(int n, int n_actions) {
-  return n <= RT_MOST && n_actions < 32 && tc_fc_slices(n) == RT_SLICES && rt_pick(n, [&](auto k) { return n <= RT_MAX_ENVS * k.clusters(); });
+  return n <= RT_MOST && n_actions < 32 && tc_fc_slices(n) == RT_SLICES && rt_pick(n, [&](auto k) { return n <= k.clusters(); });
 }
 static size_t rt_map_words(int n) { return (size_t)n * RT_POS3 * 16; }
 size_t rollout_tc_words(int n) { return n > RT_MOST ? 0 : rt_map_words(n) + (size_t)n * RT_SLICES * 256; }
@@ -667,11 +660,11 @@ void launch_rollout_tc(LaunchCtx& lc, const NetDims& nd, const float* theta, con
   KernelScope scope(lc, KID_SMALL_ROLLOUT);
   const bool launched = rt_pick(r.n, [&](auto k) {
     typedef decltype(k) Kernel;
-    q.clusters = Kernel::clusters();
-    if (q.clusters == 0) return false;
+    const int clusters = Kernel::clusters();
+    if (clusters == 0) return false;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    Kernel::shape(cfg, attr, q.clusters);
+    Kernel::shape(cfg, attr, clusters);
     cfg.stream = lc.st;
     return cudaLaunchKernelEx(&cfg, Kernel::kernel(), q) == cudaSuccess;
   });
