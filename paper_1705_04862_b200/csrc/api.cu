@@ -240,7 +240,9 @@ bool one_launch(const paac_ctx* c, std::unique_lock<std::mutex>& turn) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
   bool alone = cudaStreamIsCapturing(c->st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone;
   if (!alone) cudaGetLastError();
-  for (const paac_ctx* o = learners.first; o != nullptr && alone; o = o->next) alone = o->st == c->st || !busy(o->st);
+  // (the per-thread default stream is another one in another thread, where it cannot be asked about)
+  for (const paac_ctx* o = learners.first; o != nullptr && alone; o = o->next)
+    alone = o == c || (o->st != cudaStreamPerThread && (o->st == c->st || !busy(o->st)));
   if (!alone) turn.unlock();
   return alone;
 }

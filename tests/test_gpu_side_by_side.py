@@ -117,3 +117,20 @@ def test_a_rollout_recorded_by_the_caller_goes_layer_by_layer(arch, prec):
     _same(a, b)
     del graph
     a.close(), b.close()
+
+
+def test_a_learner_on_the_per_thread_stream_counts_as_at_work():
+    """Its stream is another one in every thread, so another thread cannot ask about it."""
+    import torch
+    g = _learner(torch.cuda.Stream(), "nips", pb.FP32, 4)
+    assert _launches(g, g.rollout) == 1
+    per_thread = _learner(torch.cuda.ExternalStream(2), "nips", pb.FP32, 4)
+    assert per_thread.hp.stream == 2
+    torch.cuda.synchronize()
+    assert _launches(g, g.rollout) > 1
+    torch.cuda.synchronize()
+    assert _launches(per_thread, per_thread.rollout) == 1
+    per_thread.close()
+    torch.cuda.synchronize()
+    assert _launches(g, g.rollout) == 1
+    g.close()
