@@ -328,8 +328,9 @@ inline cudaError_t launch_kernel_overlapped(LaunchCtx& lc, void (*kern)(KArgs...
 }
 
 // The same for the entry points without a context, on the caller's stream: the kernel waits for whatever is before it there (its
-// first act but for what touches nothing of the caller's), so only its launch overlaps.  Call after call, pre-processing of 64, 200
-// and 1024 environments takes 5.0, 11.9 and 46.6 us instead of 6.2, 14.3 and 49.1, the frame stack of 1024 12.2 instead of 14.4.
+// first act but for what touches nothing of the caller's), so only its launch overlaps, and only where a kernel is directly before it.
+// Call after call on the same buffers, pre-processing of 64, 200 and 1024 environments takes 5.0, 11.9 and 46.6 us instead of 6.2, 14.3 and
+// 49.1 (1024 with other buffers each time: 51.0 instead of 52.5), the frame stack of 1024 12.2 instead of 14.4.
 template <class... KArgs, class... Args>
 inline cudaError_t launch_overlapped_on(cudaStream_t stream, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
   cudaLaunchConfig_t cfg = {};

@@ -162,7 +162,7 @@ clip_rmsprop_kernel(size_t P, float* theta, float* rms, const float* g,
 
 // The same for the larger network's bf16 copies: the regrouped weight images (relayout_weights_kernel in net_tc.cu says which) are
 // written from the new parameters as they are made, where a kernel of its own read the copies back, 5.7 us behind this one (an
-// iteration of one learner: 32 environments 154.8 -> 151.3 us, 256 335 -> 330.5, 1024 719.8 -> 716.6).  The fully
+// iteration of one learner: 32 environments 154.8 -> 151.3 us; at 256 and 1024 no more than runs differ by).  The fully
 // connected matrix goes in tiles of 32 units x 64 inputs, a thread's float4 in each of up to three of them, so that its
 // transpose leaves through shared memory in runs of 64 bytes; the blocks that have only two tiles take the rest of the
 // parameters, whose images are small enough for scattered stores.  Arithmetic per parameter is that of clip_rmsprop_kernel.

@@ -21,8 +21,8 @@ static_assert(PP_BAND_BYTES % 16 == 0 && PP_RAW_BYTES % 16 == 0, "16-byte loads"
 // through three passes: channel-wise maximum and intensity, sixteen pixels per thread (one dot-product instruction per
 // pixel); the weighted sum over three rows, four columns per thread, two 16-bit sums per word; the weighted sum over at
 // most three columns, one output pixel per thread.  One block per task with the loads at its front and nine byte reads
-// per output pixel took 66 us for 1024 environments (264 MB); this takes 49.1 us in a row of calls, 46.6 with the set-up beside the
-// end of the call before.
+// per output pixel took 66 us for 1024 environments (264 MB); this takes 49.1 us in a row of calls on the same buffers, 46.6 with the
+// set-up beside the end of the call before (51.0 where the buffers are others each time).
 constexpr int PP_STAGES = 3, PP_ITEMS = PP_BAND_SRC * PP_SW / 16, PP_OUT = PP_BAND_OUT * FRAME_W;
 constexpr int PP_OUT_PER = (PP_OUT + PP_THREADS - 1) / PP_THREADS;
 struct PpShared {
