@@ -98,7 +98,7 @@ typedef struct {
   void* workspace;      /* device; caller-owned scratch of >= paac_workspace_bytes(), 256-byte aligned;
                            NULL: the library allocates and owns it */
   size_t workspace_bytes;
-  void* stream;         /* cudaStream_t the work is enqueued on; NULL: the default stream */
+  void* stream;         /* cudaStream_t the work is enqueued on, which has to outlive the context; NULL: the default stream */
   int algorithm;        /* PAAC_ALGO_A2C (default) or PAAC_ALGO_NSTEP_Q */
   float epsilon;        /* PAAC_ALGO_NSTEP_Q: exploration probability in [0, 1] (default 0.1) */
   int environment;      /* PAAC_ENV_HASHED (default) or PAAC_ENV_PATTERN */
@@ -239,7 +239,7 @@ int paac_stack_push(const uint8_t* state_in, const uint8_t* newest, const uint8_
 int paac_set_params(paac_ctx* ctx, const float* src /* host */, size_t n);
 
 /* Actions to take instead of sampling in the following rollouts: host int32
- * [t_max][n_e], -1 = sample as usual.  NULL clears.  Lets a checker walk in lock
+ * [t_max][n_e], -1 = sample as usual.  NULL clears.  Lets an oracle walk in lock
  * step when a uniform falls within rounding of a CDF boundary. */
 int paac_force_actions(paac_ctx* ctx, const int32_t* actions /* host, nullable */);
 

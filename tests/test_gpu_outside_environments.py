@@ -42,7 +42,7 @@ def _compare(arch, prec, n_e, layered_too, iterations=3):
                 torch.cuda.synchronize()
                 if i == 1 and layered_too:
                     with torch.cuda.stream(other):
-                        torch.cuda._sleep(10_000_000)
+                        torch.cuda._sleep(40_000_000)
                 before = l.launch_count()
                 if whole:
                     l.act_host(t, state, acts[i] if t < T else None, vals[i])

@@ -45,7 +45,7 @@ def test_one_launch_only_while_nobody_else_is_at_work(arch, prec, n_e):
         torch.cuda.synchronize()
         with torch.cuda.stream(mine if it % 4 == 3 else other):
             if it % 2:
-                torch.cuda._sleep(40_000_000)                  # some 20 ms
+                torch.cuda._sleep(200_000_000)                 # some 100 ms
         layered = it % 4 == 1
         assert (_launches(g, g.rollout) > 1) == layered, it
         torch.cuda.synchronize()
@@ -58,7 +58,7 @@ def test_one_launch_only_while_nobody_else_is_at_work(arch, prec, n_e):
             torch.cuda.synchronize()
             if i == 0 and t != 2:
                 with torch.cuda.stream(other):
-                    torch.cuda._sleep(40_000_000)
+                    torch.cuda._sleep(200_000_000)
             def step():
                 if t == 0:
                     l.act_host(0, first, acts[i], vals[i])
