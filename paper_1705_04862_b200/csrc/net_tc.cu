@@ -638,17 +638,22 @@ struct C2FwdCfg {
   __host__ __device__ static constexpr int step_lo(int j) { return 2 * j; }
   __host__ __device__ static constexpr int step_hi(int j) { return 2 * j + 1; }
 };
-// conv3 data gradient: the 7 x 7 x 64 output gradient on a zero-padded 11 x 11 raster; input pixel (y, x) is
-// raster position 11 y + x and tap (r, s) reads (2 - r) * 11 + (2 - s) rows down
+// The data gradients read the output gradient on a raster that is zero-padded at the top and on the left only: a tap that
+// looks past the right edge finds the next row's left padding, one that looks past the bottom the next state's top rows, and
+// the rows past the last state are zeros.  So the raster is no wider than the layer's input and every position is an output.
+// (With padding on all sides, an 11 x 11 raster for either layer, 33 and 17 % of the positions were dropped: at 5120 states conv3's
+// kernel took 64.3 us, conv2's 76.1; now 44.2 and 59.7.  Both are bound by what a tile costs: instructions, staging.)
+// conv3 data gradient: the 7 x 7 x 64 output gradient at rows and columns 2 .. 8 of a 9 x 9 raster; input pixel (y, x) is
+// raster position 9 y + x and tap (r, s) reads (2 - r) * 9 + (2 - s) rows down
 struct C3DgradCfg {
-  static constexpr int PLANES = 1, NT = 9, STAGE_ROWS = 152, RASTER = 121;
+  static constexpr int PLANES = 1, NT = 9, STAGE_ROWS = 152, RASTER = 81;
   static constexpr int BULK = 0;
   const bf16* g3; int states;
   __device__ __forceinline__ const bf16* base() const { return g3; }
   // element offset of raster cell `rem` inside a state's 7 x 7 x 64 gradient, or -1 for a padding cell
   __device__ static __forceinline__ int cell(int rem) {
-    const int Y = rem / 11, X = rem % 11;
-    return (Y >= 2 && Y <= 8 && X >= 2 && X <= 8) ? ((Y - 2) * 7 + (X - 2)) * 64 : -1;
+    const int Y = rem / 9, X = rem % 9;
+    return (Y >= 2 && X >= 2) ? ((Y - 2) * 7 + (X - 2)) * 64 : -1;
   }
   __device__ __forceinline__ const bf16* src_cell(int g, bool& valid) const {
     const int b = g / RASTER, off = cell(g - b * RASTER);
@@ -656,18 +661,18 @@ struct C3DgradCfg {
     return valid ? g3 + (size_t)b * 49 * 64 + off : g3;
   }
   __host__ __device__ static constexpr int tap_plane(int) { return 0; }
-  __host__ __device__ static constexpr int tap_shift(int t) { return (2 - t / 3) * 11 + (2 - t % 3); }
+  __host__ __device__ static constexpr int tap_shift(int t) { return (2 - t / 3) * 9 + (2 - t % 3); }
 };
-// conv2 data gradient (all four parity classes along N): the 9 x 9 x 64 gradient on a zero-padded 11 x 11
-// raster; class pixel (yy, xx) is position 11 yy + xx and tap (i, j) reads (1 - i) * 11 + (1 - j) rows down
+// conv2 data gradient (all four parity classes along N): the 9 x 9 x 64 gradient at rows and columns 1 .. 9 of a 10 x 10
+// raster; class pixel (yy, xx) is position 10 yy + xx and tap (i, j) reads (1 - i) * 10 + (1 - j) rows down
 struct C2DgradCfg {
-  static constexpr int PLANES = 1, NT = 4, STAGE_ROWS = 144, RASTER = 121;
+  static constexpr int PLANES = 1, NT = 4, STAGE_ROWS = 144, RASTER = 100;
   static constexpr int BULK = 0;
   const bf16* g2; int states;
   __device__ __forceinline__ const bf16* base() const { return g2; }
   __device__ static __forceinline__ int cell(int rem) {
-    const int Y = rem / 11, X = rem % 11;
-    return (Y >= 1 && Y <= 9 && X >= 1 && X <= 9) ? ((Y - 1) * 9 + (X - 1)) * 64 : -1;
+    const int Y = rem / 10, X = rem % 10;
+    return (Y >= 1 && X >= 1) ? ((Y - 1) * 9 + (X - 1)) * 64 : -1;
   }
   __device__ __forceinline__ const bf16* src_cell(int g, bool& valid) const {
     const int b = g / RASTER, off = cell(g - b * RASTER);
@@ -675,7 +680,7 @@ struct C2DgradCfg {
     return valid ? g2 + (size_t)b * 81 * 64 + off : g2;
   }
   __host__ __device__ static constexpr int tap_plane(int) { return 0; }
-  __host__ __device__ static constexpr int tap_shift(int t) { return (1 - (t >> 1)) * 11 + (1 - (t & 1)); }
+  __host__ __device__ static constexpr int tap_shift(int t) { return (1 - (t >> 1)) * 10 + (1 - (t & 1)); }
 };
 
 // epilogues of the shifted kernels: raster position -> output row, or nothing for a margin position
@@ -3102,10 +3107,10 @@ void tc_backward_dgrad_fc(LaunchCtx& lc, const bf16* images, int n, void* const 
 void tc_backward_dgrad_conv3(LaunchCtx& lc, const bf16* images, int n, void* const act[], void* const gact[], uint32_t* err) {
   typedef NatConv3 C3;
   const int M = n * C3::H * C3::W;
-  typedef RasterMap<121, 11, 9, 9> Map;
+  typedef RasterMap<81, 9, 9, 9> Map;
   tc_shift<C3DgradCfg, ShiftReluMaskEpi<Map, 9, 9>, 64, 4, 1>(
       lc, KID_CONV3_DGRAD, C3DgradCfg{(const bf16*)gact[2], n}, images + 4 * 32 * 256,
-      ShiftReluMaskEpi<Map, 9, 9>{Map{n}, (bf16*)gact[1], (const bf16*)act[1]}, n * 121, err);
+      ShiftReluMaskEpi<Map, 9, 9>{Map{n}, (bf16*)gact[1], (const bf16*)act[1]}, n * C3DgradCfg::RASTER, err);
   (void)M;
 }
 float tc_conv1_grad_scale() { return C1_GRAD_SCALE; }
@@ -3118,7 +3123,7 @@ void tc_backward_conv2d_conv1w_chunked(LaunchCtx& lc, const NetDims& nd, const b
                                        GradSegments* segs, uint32_t* err) {
   typedef NatConv1 C1;
   typedef NatConv2 C2;
-  typedef RasterMap<121, 11, 10, 10> Map;
+  typedef RasterMap<100, 10, 10, 10> Map;
   if (chunks > TC_MAX_UPDATE_CHUNKS) chunks = TC_MAX_UPDATE_CHUNKS;
   if (chunks > n) chunks = n;
   const int per = (n + chunks - 1) / chunks;
@@ -3133,7 +3138,7 @@ void tc_backward_conv2d_conv1w_chunked(LaunchCtx& lc, const NetDims& nd, const b
     bf16* gact0 = (bf16*)gact[0] + (size_t)s0 * a0;
     tc_shift<C2DgradCfg, ShiftReluMaskEpiS2<Map>, 128, 3, 1>(
         lc, KID_CONV2_DGRAD, C2DgradCfg{(const bf16*)gact[1] + (size_t)s0 * g1, nc}, images,
-        ShiftReluMaskEpiS2<Map>{Map{nc}, gact0, (const bf16*)act[0] + (size_t)s0 * a0, C1_GRAD_SCALE}, nc * 121, err);
+        ShiftReluMaskEpiS2<Map>{Map{nc}, gact0, (const bf16*)act[0] + (size_t)s0 * a0, C1_GRAD_SCALE}, nc * C2DgradCfg::RASTER, err);
     done += tc_conv1_wgrad_launch<C1>(lc, frames + (size_t)s0 * FRAME_BYTES, gact0, nc, part + (size_t)done * 256 * 32,
                                       bias_part + (size_t)done * 2 * 32, err);
   }
@@ -3147,10 +3152,10 @@ void tc_backward_dgrad_conv2(LaunchCtx& lc, const bf16* images, int n, void* con
                              float out_scale) {
   typedef NatConv2 C2;
   const int M = n * (C2::H / 2) * (C2::W / 2);
-  typedef RasterMap<121, 11, 10, 10> Map;
+  typedef RasterMap<100, 10, 10, 10> Map;
   tc_shift<C2DgradCfg, ShiftReluMaskEpiS2<Map>, 128, 3, 1>(
       lc, KID_CONV2_DGRAD, C2DgradCfg{(const bf16*)gact[1], n}, images,
-      ShiftReluMaskEpiS2<Map>{Map{n}, (bf16*)gact[0], (const bf16*)act[0], out_scale}, n * 121, err);
+      ShiftReluMaskEpiS2<Map>{Map{n}, (bf16*)gact[0], (const bf16*)act[0], out_scale}, n * C2DgradCfg::RASTER, err);
   (void)M;
 }
 
