@@ -293,12 +293,12 @@ int paac_debug_write(paac_ctx* ctx, int which, const void* src /* host */, size_
  * predecessor before it touches that kernel's data); 0 launches with plain stream order.  The setting is
  * process-wide and holds for the entry points without a context too (paac_preprocess, paac_stack_push,
  * paac_clip_rmsprop_noalloc).  Results are bit-identical either way.
- * PAAC_OPT_FP32_TENSOR_CORES: != 0 runs every contraction of the CUDA-core path (PAAC_FP32 on either network, and
- * PAAC_BF16 with PAAC_OPT_CUDA_CORES_ONLY) on the tensor cores at float accuracy: each float operand is split into two
- * TF32 pieces (22 significant bits together) and three tcgen05 passes (hi*hi + hi*lo + lo*hi) are accumulated in one
- * float accumulator; what is dropped is below 2^-21 of a product, so results stay within the 1e-4 tolerance of the
- * float path, free-running over ten updates included.  Default 0:
- * with the 20 to 160 rows of the float configurations a 128-row tensor tile is mostly padding.
+ * PAAC_OPT_FP32_TENSOR_CORES: != 0 runs every contraction of the convolutions and the fully connected layer of the float path
+ * (PAAC_FP32 on either network, PAAC_BF16 on the smaller one and with PAAC_OPT_CUDA_CORES_ONLY) on the tensor cores at float accuracy:
+ * each float operand is split into two TF32 pieces (22 significant bits together) and three tcgen05 passes (hi*hi + hi*lo + lo*hi)
+ * are added up in float; what is dropped is below 2^-21 of a product, so results stay within the 1e-4 tolerance of the
+ * float path, free-running over ten updates included.  Default 0: the larger contractions do so, where it takes less time
+ * and the sums are at least as exact, the others run on the CUDA cores.
  * PAAC_OPT_UPDATE_CHUNKS: 1 (default) .. 4.  With more than one, the tensor-core update runs the second layer's data
  * gradient and the first layer's weight gradient alternately over that many groups of states, so that a group's slice
  * of the gradient between them is read back from L2 instead of HBM.  The weight gradient's partial sums are then

@@ -503,6 +503,7 @@ int paac_init(paac_ctx** out, int arch, int n_e, int t_max, int n_actions, const
   carve(c, c->ws);
   learners.add(c);
   c->lc.error_word = &c->stats->error_word;
+  c->lc.bf16_sums_on_tensor_cores = arch == PAAC_ARCH_NIPS;
   cudaMemsetAsync(c->ws, 0, need, c->st);
   cudaMemsetAsync(c->forced, 0xFF, (size_t)c->B * sizeof(int32_t), c->st);
   launch_init_params(c->lc, c->nd, seed, c->theta);
@@ -590,8 +591,6 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
     // The data gradients are a chain, and the first layer's weight gradient ends it; the other layers' weight gradients
     // only need their own layer's gradient and run beside the chain.
     SideBranch side(c);
-    // when every gradient goes through the finishing kernel, it also delivers the squared norm
-    const bool all_finished = !c->lc.fp32_tensor_cores || (use_tc(c) && c->tc_wgrad_mask == 0xF && tc_heads_backward_supported(c->nd));
     int ready = 0;
     for (int l = L; l >= 0; --l) {
       // tensor-core kernels where they exist, the CUDA-core contraction otherwise
@@ -604,7 +603,7 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
                               c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, true, false);
       };
       if (l > 0) side.run(wgrad); else wgrad();
-      if (l == 2 && all_finished) {
+      if (l == 2) {
         // what has piled up so far (the heads, the fully connected layer, the third convolution) is most of the gradient:
         // finished beside the rest of the chain
         auto finish = [&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2); };
@@ -632,15 +631,13 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
       }
     }
     side.join();
-    ready += finish_gradients(c->lc, &c->grad_segs, all_finished ? c->norm_partials + ready : nullptr, NORM_BLOCKS - ready);
-    if (tc_supported(c->arch, c->prec) && all_finished)
+    ready += finish_gradients(c->lc, &c->grad_segs, c->norm_partials + ready, NORM_BLOCKS - ready);
+    if (tc_supported(c->arch, c->prec))
       launch_clip_rmsprop_images(c->lc, c->nd.P, c->theta, c->rms, c->grad, c->theta16, tc_weight_images(c->nd, c->w_images, &c->stats->error_word), hp.lr,
                                  hp.rms_decay, hp.rms_eps, hp.clip_norm, c->norm_partials, c->stats, ready);
-    else {
+    else
       launch_clip_rmsprop(c->lc, c->nd.P, c->theta, c->rms, c->grad, c->prec == PAAC_BF16 ? c->theta16 : nullptr, hp.lr, hp.rms_decay, hp.rms_eps,
-                          hp.clip_norm, c->norm_partials, c->stats, all_finished ? ready : 0);
-      if (c->prec == PAAC_BF16) refresh_weight_copies(c, false);
-    }
+                          hp.clip_norm, c->norm_partials, c->stats, ready);
     if (stats) launch_publish_stats(c->lc, c->stats, &c->box->stats, &c->box->done);
   });
   c->N += (uint64_t)c->B;

@@ -21,6 +21,13 @@
 
 namespace paac {
 
+// k per split for a requested number of splits, and how many splits that gives
+inline int gemm_k_per_split(int K, int splits, int granule = 16) {
+  const int kps = (K + splits - 1) / splits;
+  return (kps + granule - 1) / granule * granule;
+}
+inline int gemm_k_splits(int K, int splits, int granule = 16) { const int kps = gemm_k_per_split(K, splits, granule); return (K + kps - 1) / kps; }
+
 // sixteen bytes of stored values as floats
 __device__ __forceinline__ void widen(const uint4 v, const float*, float4 (&f)[1]) {
   f[0] = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));

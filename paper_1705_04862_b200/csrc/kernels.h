@@ -178,10 +178,8 @@ int tc_fc_slices(int n);
 constexpr int NORM_BLOCKS = 1184;
 void launch_clip_rmsprop(LaunchCtx& lc, size_t P, float* theta, float* rms, const float* grad,
                          bf16* theta16 /* nullable */, float lr, float rho, float eps, float clip,
-                         float* norm_partials /* [NORM_BLOCKS] */, DeviceStats* stats,
-                         int ready_partials = 0 /* > 0: norm_partials[0..ready_partials) already hold the squared norm */);
-// the same for the larger network in bf16, with the regrouped weight images (tc_weight_images()) written from the new parameters;
-// norm_partials[0..ready_partials) hold the squared norm
+                         const float* norm_partials /* [0..ready_partials) hold the squared norm */, DeviceStats* stats, int ready_partials);
+// the same for the larger network in bf16, with the regrouped weight images (tc_weight_images()) written from the new parameters
 struct WeightImages {
   uint16_t *w1_b, *w2_d, *w3_d, *wfc_t;
   size_t w1_end, w2_off, w3_off, fc_off;        // elements of the parameter vector

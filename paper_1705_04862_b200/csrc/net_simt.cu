@@ -7,26 +7,14 @@
 
 namespace paac {
 
-// the three-pass tensor-core kernel instead of the CUDA cores (an option)
-static bool use_tc3(const LaunchCtx& lc) { return lc.fp32_tensor_cores && lc.error_word != nullptr; }
-
 static int pick_splits(int M, int N, int K) {
-  const int blocks = ((M + SG_BM - 1) / SG_BM) * ((N + SG_BN - 1) / SG_BN);
+  const int blocks = ((M + 63) / 64) * ((N + 63) / 64);
   int s = (592 + blocks - 1) / blocks;
   const int by_k = (K + 127) / 128;
   if (s > by_k) s = by_k;
   if (s > 512) s = 512;
   if (s < 1) s = 1;
   return gemm_k_splits(K, s);
-}
-
-static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_rows, int row0,
-                         int rows, int cols, float scale, float* gw, float* gb) {
-  const size_t total = (size_t)rows * (cols + 1);
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 2368) blocks = 2368;
-  KernelScope scope(lc, KID_WGRAD_REDUCE);
-  launch_kernel(lc, wgrad_reduce_kernel, blocks, 256, 0, part, splits, part_rows, row0, rows, cols, scale, gw, gb);
 }
 
 // Shapes of the CUDA-core contraction for N columns (16, 32, or 64 and more).  At 128 states forward and 640 backward the
@@ -37,6 +25,36 @@ static void reduce_wgrad(LaunchCtx& lc, const float* part, int splits, int part_
 // without a warp (592).  4 x 4 with 64 columns comes in blocks of two warps: the
 // second layer's 10368 rows then fill the device in more even rounds (34 -> 30 us, the third layer's 6272 the same).
 constexpr int FF_SMS = 148;
+
+// ---- which contractions go to the tensor cores ----
+// Splits of k for an M x N result there: two blocks per SM, four blocks of k and more to each.
+static int t3_splits(int M, int N, int K) {
+  const int bn = N < 64 ? N : 64, tiles = (M + T3_BM - 1) / T3_BM * ((N + bn - 1) / bn);
+  int s = 2 * FF_SMS / tiles;
+  const int by_k = K / (4 * T3_BK);
+  if (s > by_k) s = by_k;
+  return s < 1 ? 1 : gemm_k_splits(K, s, T3_BK);
+}
+// Data gradients, M rows.  A tile takes about a microsecond per block of 32 k, whatever the number of tiles up to two per SM, where the
+// CUDA cores take time with the multiply-adds: 11 M of them per block and 80 M in all is where the two meet.  (us, CUDA cores / tensor cores,
+// larger network: third layer, 18 blocks, 40 states 25 / 26, 64 states 29 / 25, 640 states 105 / 54; second layer, 8 blocks, 40 states 19 / 19, 80 states
+// 26 / 19, 640 states 126 / 67; fully connected layer, 16 blocks, 80 states 19 / 23, 120 states 25 / 23, 640 states 70 / 29.)  Errors against
+// sums in 64 bits, 2-norm: 1.2 to 1.5e-7 instead of 1.2 to 2.9e-7.
+// The forward pass stays on the CUDA cores, whose chains of multiply-adds are the same for every batch: sums as exact but in another order put
+// a unit or two per pass on the other side of the ReLU, and training then runs apart from there.
+template <class T> static bool t3_allowed(const LaunchCtx& lc) { return lc.error_word != nullptr && (sizeof(T) == 4 || lc.bf16_sums_on_tensor_cores); }
+template <class T> static bool t3_pays(const LaunchCtx& lc, long long M, int N, int K) {
+  if (lc.fp32_tensor_cores) return lc.error_word != nullptr;
+  const long long blocks = (K + T3_BK - 1) / T3_BK, macs = M * N * K;
+  return t3_allowed<T>(lc) && macs >= blocks * 11000000 && macs >= 80000000;
+}
+// Weight gradients, whose k is split until the device is full: from 64 M multiply-adds on (first layer of the smaller network, 40 states 14 / 11 us,
+// 160 states 31 / 20, 960 states 152 / 66; second layer 80 states 13 / 11, 640 states 43 / 20).  The fully connected layer's sums over fewer than
+// 256 rows are more exact on the CUDA cores (160 rows: 1.08e-7 against 1.41e-7).
+template <class T> static bool t3_wgrad_pays(const LaunchCtx& lc, int J, int CO, int K) {
+  if (lc.fp32_tensor_cores) return lc.error_word != nullptr;
+  return t3_allowed<T>(lc) && K >= 256 && (long long)J * CO * K >= 64000000;
+}
 static size_t ff_heads_scratch_floats(const NetDims& nd, int n);
 static int ff_shape(int N, long long outputs) {              // outputs of all classes and splits
   if (outputs >= 1184LL * 32 * 8 * (N >= 64 ? 8 : 4)) return 2;
@@ -69,12 +87,12 @@ static void ff_rows(LaunchCtx& lc, int kid, int M, int n_cols, int K, int kps, i
 
 // Weight gradients: C(j, co) = sum over output positions of window(j) * gradient(co), one run of positions per split;
 // the splits' sums (and the bias gradient's, the column sums of the second operand) are added, in split order, by
-// finish_gradients().  The runs are those of the three-pass path (pick_splits).
+// finish_gradients().
 struct FfWgradPlan { int splits, kps; size_t part, total; };      // floats: the weights' partial sums, and all of them
-static FfWgradPlan ff_wgrad_plan(int J, int CO, int K) {
+static FfWgradPlan ff_wgrad_plan(int J, int CO, int K, bool tensor) {
   FfWgradPlan p;
-  p.splits = pick_splits(CO, J + 1, K);
-  p.kps = gemm_k_per_split(K, p.splits);
+  p.splits = tensor ? t3_splits(J, CO, K) : pick_splits(CO, J + 1, K);
+  p.kps = gemm_k_per_split(K, p.splits, tensor ? T3_BK : 16);
   p.part = (size_t)p.splits * J * CO;
   p.total = (p.part + (size_t)p.splits * CO + 63) / 64 * 64;
   return p;
@@ -82,27 +100,33 @@ static FfWgradPlan ff_wgrad_plan(int J, int CO, int K) {
 template <int CO_TILE, class LA, class LB>
 static void ff_wgrad(LaunchCtx& lc, int kid, int J, int CO, int K, LA window, LB grad_rows, float scale, float* gw, float* gb,
                      float* scratch, GradSegments* segs) {
-  const FfWgradPlan p = ff_wgrad_plan(J, CO, K);
+  typedef typename LB::Elem T;
+  const bool tensor = t3_wgrad_pays<T>(lc, J, CO, K);
+  const FfWgradPlan p = ff_wgrad_plan(J, CO, K, tensor);
   FfPartialColsum ep;
   ep.part = scratch; ep.M = J; ep.N = CO; ep.colpart = scratch + p.part;
   // 64 x 64 tiles of 8 x 8 per lane where they give every SM three blocks, 128 x 32 of 8 x 4 where those give it one
-  if (CO_TILE == 64 && (J + 63) / 64 * ((CO + 63) / 64) * p.splits >= 3 * FF_SMS)
+  if (tensor)
+    gemm_tc3<CO_TILE>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
+  else if (CO_TILE == 64 && (J + 63) / 64 * ((CO + 63) / 64) * p.splits >= 3 * FF_SMS)
     gemm_ffma<4, 8, 8, 2, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
   else if (CO_TILE == 32 && (J + 127) / 128 * p.splits >= FF_SMS)
     gemm_ffma<4, 8, 4, 4, 1, 16>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
   else
     ff_rows<CO_TILE>(lc, kid, J, CO, K, p.kps, 1, window, grad_rows, ep);
-  if (!add_grad_segment(segs, scratch, gw, p.splits, J, CO, scale, true) || !add_grad_segment(segs, ep.colpart, gb, p.splits, 1, CO, 1.f, true))
+  if (!add_grad_segment(segs, scratch, gw, p.splits, J, CO, scale, !tensor) || !add_grad_segment(segs, ep.colpart, gb, p.splits, 1, CO, 1.f, !tensor))
     lc.host_failure = true;
 }
 
 template <class G, class TIn, class T, class TW>
 static void conv_fwd(LaunchCtx& lc, int kid, const TIn* x, const TW* w, const float* bias, T* out, int n,
                      float scale) {
-  if (use_tc3(lc))
-    gemm_tc3(lc, kid, n * G::OH * G::OW, G::CO, G::KK, 1, ConvWindowOp<G, TIn>{x}, RowMajorOp<TW>{w, G::KK}, BiasReluEp<T>{out, bias, G::CO, scale});
-  else
-    ff_rows<G::CO>(lc, kid, n * G::OH * G::OW, G::CO, G::KK, G::KK, 1, FfWindow<G, TIn>{x}, FfRows<TW>{w, G::KK}, FfBiasRelu<T>{out, bias, G::CO, scale});
+  const int M = n * G::OH * G::OW;
+  const FfWindow<G, TIn> window{x};
+  const FfRows<TW> weights{w, G::KK};
+  const FfBiasRelu<T> ep{out, bias, G::CO, scale};
+  if (lc.fp32_tensor_cores) gemm_tc3<G::CO>(lc, kid, M, G::CO, G::KK, G::KK, 1, window, weights, ep);
+  else ff_rows<G::CO>(lc, kid, M, G::CO, G::KK, G::KK, 1, window, weights, ep);
 }
 // With few states the fully connected layer is a handful of tiles over a reduction of thousands: the reduction is then
 // split over many blocks (partial sums in scratch, added by launch_simt_tail) so that the weight matrix is streamed by
@@ -110,15 +134,15 @@ static void conv_fwd(LaunchCtx& lc, int kid, const TIn* x, const TW* w, const fl
 template <class T, class TW>
 static int fc_fwd(LaunchCtx& lc, int kid, const T* x, const TW* w, const float* bias, T* out, int n,
                    int IN, int F, float* scratch) {
-  const int splits = pick_splits(n, F, IN);
-  if (use_tc3(lc)) {
-    if (splits <= 1) gemm_tc3(lc, kid, n, F, IN, 1, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, BiasReluEp<T>{out, bias, F, 1.f});
-    else gemm_tc3(lc, kid, n, F, IN, splits, RowMajorOp<T>{x, IN}, RowMajorOp<TW>{w, IN}, PartialEp{scratch, n, F});
-  } else if (splits <= 1) {
-    ff_rows<64>(lc, kid, n, F, IN, IN, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfBiasRelu<T>{out, bias, F, 1.f});
-  } else {
-    ff_rows<64>(lc, kid, n, F, IN, gemm_k_per_split(IN, splits), 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, FfPartial{scratch, n, F});
-  }
+  const bool tensor = lc.fp32_tensor_cores;
+  const int splits = tensor ? t3_splits(n, F, IN) : pick_splits(n, F, IN);
+  const int kps = splits <= 1 ? IN : gemm_k_per_split(IN, splits, tensor ? T3_BK : 16);
+  auto launch = [&](auto ep) {
+    if (tensor) gemm_tc3<64>(lc, kid, n, F, IN, kps, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, ep);
+    else ff_rows<64>(lc, kid, n, F, IN, kps, 1, FfRows<T>{x, IN}, FfRows<TW>{w, IN}, ep);
+  };
+  if (splits <= 1) launch(FfBiasRelu<T>{out, bias, F, 1.f});
+  else launch(FfPartial{scratch, n, F});
   return splits <= 1 ? 0 : splits;
 }
 template <class G, class T, class TW>
@@ -126,48 +150,38 @@ static void conv_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T*
   if constexpr (G::S == 2 && G::K == 4 && G::H % 2 == 0 && G::W % 2 == 0) {
     // four parity classes, each a dense contraction over its own four taps (a quarter of the multiply-adds)
     const int M = n * (G::H / 2) * (G::W / 2), K = 4 * G::CO;
-    if (use_tc3(lc))
-      for (int z = 0; z < 4; ++z)
-        gemm_tc3(lc, kid, M, G::C, K, 1, ConvDgradClassOp<G, T>{g, z >> 1, z & 1}, ConvWeightClassOp<G, TW>{w, z >> 1, z & 1},
-                 ReluMaskClassEp<G, T>{gin, act_in, z >> 1, z & 1});
+    const FfDgradClass<G, T> rows{g};
+    const FfWeightClass<G, TW> weights{w, 0};
+    const FfReluMaskClass<G, T> ep{gin, act_in, 0};
+    if (t3_pays<T>(lc, M, 4 * G::C, K))
+      gemm_tc3<64>(lc, kid, M, 4 * G::C, K, K, 1, rows, T3WeightClasses<G, TW>{w}, T3ReluMaskClasses<G, T>{gin, act_in});
     else
-      ff_rows<G::C>(lc, kid, M, G::C, K, K, 4, FfDgradClass<G, T>{g}, FfWeightClass<G, TW>{w, 0}, FfReluMaskClass<G, T>{gin, act_in, 0});
-    return;
+      ff_rows<G::C>(lc, kid, M, G::C, K, K, 4, rows, weights, ep);
+  } else {
+    const int M = n * G::H * G::W, K = G::K * G::K * G::CO;
+    const FfDgradWindow<G, T> rows{g};
+    const FfWeightT<G, TW> weights{w};
+    const FfReluMask<T> ep{gin, act_in, G::C};
+    if (t3_pays<T>(lc, M, G::C, K)) gemm_tc3<G::C>(lc, kid, M, G::C, K, K, 1, rows, weights, ep);
+    else ff_rows<G::C>(lc, kid, M, G::C, K, K, 1, rows, weights, ep);
   }
-  const int M = n * G::H * G::W, K = G::K * G::K * G::CO;
-  if (use_tc3(lc)) gemm_tc3(lc, kid, M, G::C, K, 1, ConvDgradOp<G, T>{g}, ConvWeightTOp<G, TW>{w}, ReluMaskEp<T>{gin, act_in, G::C});
-  else ff_rows<G::C>(lc, kid, M, G::C, K, K, 1, FfDgradWindow<G, T>{g}, FfWeightT<G, TW>{w}, FfReluMask<T>{gin, act_in, G::C});
 }
 template <class G, class TIn, class T>
 static void conv_wgrad(LaunchCtx& lc, int kid, const T* g, const TIn* x, int n, float scale, float* gw,
                        float* gb, float* scratch, GradSegments* segs) {
-  const int K = n * G::OH * G::OW;
-  if (!use_tc3(lc)) {
-    ff_wgrad<G::CO>(lc, kid, G::KK, G::CO, K, FfWindowT<G, TIn>{x}, FfCols<T>{g, G::CO}, scale, gw, gb, scratch, segs);
-    return;
-  }
-  const int M = G::CO, N = G::KK + 1;
-  const int splits = pick_splits(M, N, K);
-  gemm_tc3(lc, kid, M, N, K, splits, ColMajorOp<T>{g, G::CO}, ConvWindowTOp<G, TIn>{x}, PartialEp{scratch, M, N});
-  reduce_wgrad(lc, scratch, splits, M, 0, M, G::KK, scale, gw, gb);
+  ff_wgrad<G::CO>(lc, kid, G::KK, G::CO, n * G::OH * G::OW, FfWindowT<G, TIn>{x}, FfCols<T>{g, G::CO}, scale, gw, gb, scratch, segs);
 }
 template <class T, class TW>
 static void fc_dgrad(LaunchCtx& lc, int kid, const T* g, const TW* w, const T* act_in, T* gin, int n,
                      int IN, int F) {
-  if (use_tc3(lc)) gemm_tc3(lc, kid, n, IN, F, 1, RowMajorOp<T>{g, F}, ColMajorOp<TW>{w, IN}, ReluMaskEp<T>{gin, act_in, IN});
-  else ff_rows<64>(lc, kid, n, IN, F, F, 1, FfRows<T>{g, F}, FfCols<TW>{w, IN}, FfReluMask<T>{gin, act_in, IN});
+  const FfReluMask<T> ep{gin, act_in, IN};
+  if (t3_pays<T>(lc, n, IN, F)) gemm_tc3<64>(lc, kid, n, IN, F, F, 1, FfRows<T>{g, F}, FfCols<TW>{w, IN}, ep);
+  else ff_rows<64>(lc, kid, n, IN, F, F, 1, FfRows<T>{g, F}, FfCols<TW>{w, IN}, ep);
 }
 template <class T>
 static void fc_wgrad(LaunchCtx& lc, int kid, const T* g, const T* x, int n, int IN, int F, float* gw,
                      float* gb, float* scratch, GradSegments* segs) {
-  if (!use_tc3(lc)) {
-    ff_wgrad<64>(lc, kid, IN, F, n, FfCols<T>{x, IN}, FfCols<T>{g, F}, 1.f, gw, gb, scratch, segs);
-    return;
-  }
-  const int M = F, N = IN + 1, K = n;
-  const int splits = pick_splits(M, N, K);
-  gemm_tc3(lc, kid, M, N, K, splits, ColMajorOp<T>{g, F}, ColMajorOnesOp<T>{x, IN, IN}, PartialEp{scratch, M, N});
-  reduce_wgrad(lc, scratch, splits, M, 0, M, IN, 1.f, gw, gb);
+  ff_wgrad<64>(lc, kid, IN, F, n, FfCols<T>{x, IN}, FfCols<T>{g, F}, 1.f, gw, gb, scratch, segs);
 }
 
 template <class T, class TW>
@@ -226,14 +240,14 @@ static void backward_layer_t(LaunchCtx& lc, int arch, const NetDims& nd, const T
 }
 
 // Where layer l's partial sums start in the update's scratch; l = number of layers: the heads' region; one more: the end.
-// Every layer has a region of its own in both contractions: the CUDA-core one keeps its partial sums until
-// finish_gradients() has run, and the three-pass one, which adds each layer's up at once, may do so for one layer on the
-// side stream while the main stream works on another.  Both split alike, splits * (J + 1) * CO floats each.
+// Every layer has a region of its own, large enough for either contraction: partial sums stay until finish_gradients() has run.
 static size_t ff_scratch_offset(const NetDims& nd, int n, int l) {
   size_t off = 0;
   for (int q = 0; q < l && q <= nd.n_conv; ++q) {
     const LayerDims& d = nd.layer[q];
-    off += ff_wgrad_plan(q < nd.n_conv ? d.K * d.K * d.C : d.H * d.W * d.C, d.CO, n * d.OH * d.OW).total;
+    const int J = q < nd.n_conv ? d.K * d.K * d.C : d.H * d.W * d.C, K = n * d.OH * d.OW;
+    const size_t cuda = ff_wgrad_plan(J, d.CO, K, false).total, tensor = ff_wgrad_plan(J, d.CO, K, true).total;
+    off += cuda > tensor ? cuda : tensor;
   }
   if (l > nd.n_conv + 1) off += ff_heads_scratch_floats(nd, n);
   return off;
@@ -261,29 +275,12 @@ size_t simt_scratch_floats(int arch, const NetDims& nd, int n, int n_fwd) {
   // split-k partial sums of the fully connected layer's forward pass, which only ever sees n_fwd states at a time
   const LayerDims& f = nd.layer[nd.n_conv];
   const int IN = f.H * f.W * f.C;
-  const size_t fwd = (size_t)pick_splits(n_fwd, nd.F, IN) * n_fwd * nd.F;
+  const int cuda = pick_splits(n_fwd, nd.F, IN), tensor = t3_splits(n_fwd, nd.F, IN);
+  const size_t fwd = (size_t)(cuda > tensor ? cuda : tensor) * n_fwd * nd.F;
   return best > fwd ? best : fwd;
 }
 
 // ---- heads backward (tiny contractions over the A+1 head units) ------------------------------
-struct HeadGradOp {          // row = sample, k = head unit (policy logits then value)
-  static constexpr bool K_CONTIG = true;
-  const float* dz; const float* dV; int A;
-  __device__ __forceinline__ float operator()(int m, int k) const { return k < A ? dz[(size_t)m * A + k] : dV[m]; }
-};
-struct HeadGradTOp {         // row = head unit, k = sample
-  static constexpr bool K_CONTIG = false;
-  const float* dz; const float* dV; int A;
-  __device__ __forceinline__ float operator()(int u, int b) const { return u < A ? dz[(size_t)b * A + u] : dV[b]; }
-};
-template <class TW> struct HeadWeightOp {   // row = fc unit i, k = head unit
-  static constexpr bool K_CONTIG = false;
-  const TW* wpi; const TW* wv; int F, A;
-  __device__ __forceinline__ float operator()(int i, int k) const {
-    return k < A ? to_f(wpi[(size_t)k * F + i]) : to_f(wv[i]);
-  }
-};
-
 // Both heads in one kernel, for either storage type and either hidden size (the tensor-core path has one of its own for
 // 512 bf16 units): with dz[b][k] the loss gradient at output k of row b (the value is row k = A of the combined matrix),
 //   g_fc[b][i] = (h[b][i] > 0) * sum_k dz[b][k] W[k][i],   dW[k][i] = sum_b dz[b][k] h[b][i],   db[k] = sum_b dz[b][k].
@@ -364,17 +361,6 @@ template <class T, class TW>
 static void heads_backward_t(LaunchCtx& lc, const NetDims& nd, const TW* w, const T* h, int n,
                              const float* dz, const float* dV, T* gact_fc, float* grad, float* scratch, GradSegments* segs) {
   const int A = nd.A, F = nd.F;
-  if (use_tc3(lc)) {
-    gemm_tc3(lc, KID_HEADS_BWD, n, F, A + 1, 1, HeadGradOp{dz, dV, A}, HeadWeightOp<TW>{w + nd.pi_w, w + nd.v_w, F, A},
-              ReluMaskEp<T>{gact_fc, h, F});
-    const int splits = pick_splits(A + 1, F + 1, n);
-    float* part = scratch + ff_scratch_offset(nd, n, nd.n_conv + 1);
-    gemm_tc3(lc, KID_HEADS_BWD, A + 1, F + 1, n, splits, HeadGradTOp{dz, dV, A}, ColMajorOnesOp<T>{h, F, F},
-              PartialEp{part, A + 1, F + 1});
-    reduce_wgrad(lc, part, splits, A + 1, 0, A, F, 1.f, grad + nd.pi_w, grad + nd.pi_b);
-    reduce_wgrad(lc, part, splits, A + 1, A, 1, F, 1.f, grad + nd.v_w, grad + nd.v_b);
-    return;
-  }
   const int splits = pick_splits(A + 1, F + 1, n), rows_per = gemm_k_per_split(n, splits);
   float* part_w = scratch + ff_scratch_offset(nd, n, nd.n_conv + 1);
   float* part_b = part_w + (size_t)splits * A * F;

@@ -5,35 +5,6 @@
 
 namespace paac {
 
-constexpr int OPT_THREADS = 256;
-
-// pass 1: block b sums g^2 over its fixed slice of the parameter vector
-__global__ void __launch_bounds__(OPT_THREADS)
-sumsq_kernel(const float* __restrict__ g, size_t P, float* __restrict__ partials) {
-  pdl_entry();
-  __shared__ float sh[OPT_THREADS];
-  const size_t per = ((P + gridDim.x - 1) / gridDim.x + 3) / 4 * 4;
-  const size_t lo = (size_t)blockIdx.x * per, hi = lo + per < P ? lo + per : P;
-  float acc = 0.f;
-  if (lo < hi) {
-    // slice starts are multiples of 4 floats, so 16-byte loads are aligned
-    const size_t n4 = (hi - lo) / 4;
-    const float4* g4 = reinterpret_cast<const float4*>(g + lo);
-    for (size_t i = threadIdx.x; i < n4; i += OPT_THREADS) {
-      const float4 v = g4[i];
-      acc = fmaf(v.x, v.x, acc); acc = fmaf(v.y, v.y, acc); acc = fmaf(v.z, v.z, acc); acc = fmaf(v.w, v.w, acc);
-    }
-    for (size_t i = lo + n4 * 4 + threadIdx.x; i < hi; i += OPT_THREADS) acc = fmaf(g[i], g[i], acc);
-  }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = OPT_THREADS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) partials[blockIdx.x] = sh[0];
-}
-
 // Where four neighbouring parameters from element p on (outside the fully connected matrix) go in the regrouped images, as bf16 bits
 __device__ __forceinline__ void small_images(const WeightImages& img, size_t p, const uint16_t (&b)[4]) {
   if (p < img.w1_end) {
@@ -240,17 +211,11 @@ void launch_clip_rmsprop_images(LaunchCtx& lc, size_t P, float* theta, float* rm
 }
 
 void launch_clip_rmsprop(LaunchCtx& lc, size_t P, float* theta, float* rms, const float* grad,
-                         bf16* theta16, float lr, float rho, float eps, float clip, float* norm_partials,
+                         bf16* theta16, float lr, float rho, float eps, float clip, const float* norm_partials,
                          DeviceStats* stats, int ready_partials) {
-  int n_partials = ready_partials;
-  if (ready_partials <= 0) {
-    KernelScope scope(lc, KID_SUMSQ);
-    launch_kernel(lc, sumsq_kernel, NORM_BLOCKS, OPT_THREADS, 0, grad, P, norm_partials);
-    n_partials = NORM_BLOCKS;
-  }
   KernelScope scope(lc, KID_CLIP_RMSPROP);
   launch_kernel_overlapped(lc, clip_rmsprop_kernel, UPD_BLOCKS, UPD_THREADS, 0, P, theta, rms, grad, theta16, lr, rho, eps, clip,
-                                                              norm_partials, n_partials, stats);
+                                                              norm_partials, ready_partials, stats);
 }
 
 }  // namespace paac
