@@ -603,9 +603,9 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
                               c->grad, c->scratch + c->simt_scratch_off, &c->grad_segs, l, true, false);
       };
       if (l > 0) side.run(wgrad); else wgrad();
-      if (l == 2) {
-        // what has piled up so far (the heads, the fully connected layer, the third convolution) is most of the gradient:
-        // finished beside the rest of the chain
+      if (l == (L == 3 ? 1 : 2)) {
+        // what has piled up so far (all but the first layer of the larger network; the heads and the fully connected layer of the smaller one, whose
+        // second layer the chain would wait for) is most of the gradient: finished beside the rest of the chain
         auto finish = [&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2); };
         if (side.on) side.append(finish);
       }

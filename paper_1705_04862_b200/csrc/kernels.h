@@ -48,8 +48,8 @@ void launch_advance_step(LaunchCtx& lc, uint64_t* step_base, uint32_t by);
 // The weight-gradient kernels leave partial sums part[split][J][CO] (J = 1 for biases) in scratch regions of their own
 // and note them in a GradSegments list; finish_gradients() adds them up, splits in a fixed order, into the gradient
 // vector (dst[co * J + j], times scale) with one launch and empties the list.
-struct GradSegment { const float* part; float* dst; int splits, J, CO; float scale; int first_group, groups, mode; };
-struct GradSegments { GradSegment seg[12]; int n; int total_groups; };
+struct GradSegment { const float* part; float* dst; int splits, J, CO; float scale; int mode, view, row_shift, co_shift; };
+struct GradSegments { static constexpr int MOST = 12; GradSegment seg[MOST]; int first_group[MOST], n, total_groups; };
 // in_order: one running sum over the splits (the float path's); otherwise eight interleaved ones where there are many.
 // false: list full
 bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale, bool in_order = false);

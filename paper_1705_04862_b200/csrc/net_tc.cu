@@ -2125,123 +2125,176 @@ tc_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
   }
 }
 
-// One launch finishes every tensor-core weight gradient of an update: for each segment (a layer's weights, or
-// its bias with J = 1) dst[co * J + j] = scale * sum over splits of part[split][j][co], the splits added in a
-// fixed order.  The partial sums have co innermost and the gradient has j innermost, so every group of outputs
-// goes through a shared-memory tile: reads are whole 128-byte rows of co, writes whole runs of j.
-//   many splits: a group is FG_J j x 32 co; warp w adds the splits w, w + 8, ... for these j, the eight warps' sums
-//                are then added in warp order;
-//   few splits:  a group is 32 j x 32 co; warp w adds all splits, in order, for rows w, w + 8, w + 16, w + 24.
-//   many splits, in order (the float path): the warps bring FG_CHUNK splits of a group into shared memory and one thread
-//                per output adds them up one after the other.
-constexpr int FG_J = 2;          // rows of j per group of a many-split segment
-constexpr int FG_CHUNK = 128;    // splits at a time of a segment added in order
-enum { FG_FEW = 0, FG_MANY = 1, FG_IN_ORDER = 2 };
-__global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments segs, float* __restrict__ sumsq_partials) {
+// One launch finishes every weight gradient of an update: for each segment (a layer's weights, or its bias with J = 1)
+// dst[co * J + j] = scale * sum over splits of part[split][j][co], the splits added in a fixed order.  The partial sums have
+// co innermost and the gradient has j innermost, so every group of outputs turns in shared memory.  A thread reads four
+// neighbouring co at a time, and four such rows where there are few splits (a value at a time, 56 % of the issue slots were busy with
+// addresses: 15.8 us for the 47 MB that 32 environments leave beside the chain, now 11.3; with one row, a load per thread and split in
+// flight, 20.6).  J = 1 needs no turning: the vector is taken as rows of 32; and two j of 16 co are one row.
+//   few splits:  a group is FG_ROWS j x 32 co; a thread adds all splits of four times four, in order;
+//   many splits: a group is 4 j x 32 co and 8 running sums (splits w, w + 8, ...), added in order;
+//   odd widths (the heads' biases): the same, a value to a thread, one row;
+//   many splits, in order (the float path on the CUDA cores): the warps bring FG_CHUNK splits of FG_PAIR j into shared memory and one thread per
+//                output adds them up one after the other.
+constexpr int FG_PAIR_SHIFT = 1, FG_PAIR = 1 << FG_PAIR_SHIFT, FG_CHUNK = 128;      // rows of j of a segment added in order; splits at a time there
+constexpr int FG_ROW_SHIFT = 7, FG_ROWS = 1 << FG_ROW_SHIFT;                       // and of a few-split segment: a thread has four times as many loads in flight as splits
+constexpr int FG_AHEAD = 8;      // loads in flight per thread of a many-split segment
+constexpr int FG_LD = 36;        // floats from one j to the next in shared memory: 16-byte accesses, few bank conflicts
+enum { FG_FEW = 0, FG_MANY = 1, FG_IN_ORDER = 2, FG_ODD = 3 };
+enum { FG_TURNED = 0, FG_FLAT = 1, FG_PAIRS = 2 };      // [J][CO] as it is; a vector as rows of 32; two rows of 16 as one of 32
+// the splits first, first + step, ... of four values, `stride` floats apart
+__device__ __forceinline__ float4 add_splits(const float* src, int first, int splits, int step, size_t stride) {
+  float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float* p = src + (size_t)first * stride;
+  stride *= step;
+  for (int left = (splits - first + step - 1) / step; left > 0; left -= FG_AHEAD) {
+    float4 v[FG_AHEAD];
+#pragma unroll
+    for (int u = 0; u < FG_AHEAD; ++u) {
+      if (u < left) v[u] = __ldg(reinterpret_cast<const float4*>(p));
+      p += stride;
+    }
+#pragma unroll
+    for (int u = 0; u < FG_AHEAD; ++u)
+      if (u < left) { t.x += v[u].x; t.y += v[u].y; t.z += v[u].z; t.w += v[u].w; }
+  }
+  return t;
+}
+template <bool IN_ORDER>
+__global__ void __launch_bounds__(256, 3) tc_finalize_grads_kernel(const __grid_constant__ GradSegments segs, float* __restrict__ sumsq_partials) {
   pdl_entry();
-  __shared__ float sh[FG_CHUNK * FG_J * 32];
+  __shared__ __align__(16) float sh[IN_ORDER ? FG_CHUNK * FG_PAIR * 32 : FG_ROWS * FG_LD];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float ss = 0.f;                       // sum of squares of the gradient values this thread writes
   for (int grp = blockIdx.x; grp < segs.total_groups; grp += gridDim.x) {
     int si = 0;
-    while (si + 1 < segs.n && grp >= segs.seg[si + 1].first_group) ++si;
+#pragma unroll
+    for (int i = 1; i < GradSegments::MOST; ++i) si += grp >= segs.first_group[i];
     const GradSegment& sg = segs.seg[si];
-    const int local = grp - sg.first_group, co_tiles = (sg.CO + 31) / 32;
-    const int co0 = (local % co_tiles) * 32, J = sg.J, CO = sg.CO;
+    const int local = grp - segs.first_group[si], tile = local >> sg.co_shift;      // (a power of two of tiles of co)
+    const int co0 = (local - (tile << sg.co_shift)) * 32, J = sg.J, CO = sg.CO;
     const size_t total = (size_t)J * CO;
-    const bool co_ok = co0 + lane < CO;
-    if (sg.mode == FG_IN_ORDER) {
-      const int j0 = (local / co_tiles) * FG_J, j = j0 + (int)threadIdx.x / 32;
+    if (IN_ORDER && sg.mode == FG_IN_ORDER) {
+      const bool co_ok = co0 + lane < CO;
+      const int j0 = tile * FG_PAIR, j = j0 + (int)threadIdx.x / 32;
       const float* src = sg.part + (size_t)j0 * CO + co0 + lane;
       float t = 0.f;
       for (int p0 = 0; p0 < sg.splits; p0 += FG_CHUNK) {
         const int count = min(FG_CHUNK, sg.splits - p0);
         __syncthreads();
         constexpr int PER = FG_CHUNK / 8;
-        float v[PER][FG_J];
+        float v[PER][FG_PAIR];
 #pragma unroll
         for (int u = 0; u < PER; ++u)
 #pragma unroll
-          for (int q = 0; q < FG_J; ++q)
+          for (int q = 0; q < FG_PAIR; ++q)
             v[u][q] = (co_ok && j0 + q < J && warp + 8 * u < count) ? __ldg(src + (size_t)(p0 + warp + 8 * u) * total + (size_t)q * CO) : 0.f;
 #pragma unroll
         for (int u = 0; u < PER; ++u)
 #pragma unroll
-          for (int q = 0; q < FG_J; ++q) sh[((warp + 8 * u) * FG_J + q) * 32 + lane] = v[u][q];
+          for (int q = 0; q < FG_PAIR; ++q) sh[((warp + 8 * u) * FG_PAIR + q) * 32 + lane] = v[u][q];
         __syncthreads();
-        if (threadIdx.x < FG_J * 32) {
+        if (threadIdx.x < FG_PAIR * 32) {
           const float* column = sh + threadIdx.x;
           int p = 0;
           for (; p + 16 <= count; p += 16) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) t += column[(p + u) * FG_J * 32];
+            for (int u = 0; u < 16; ++u) t += column[(p + u) * FG_PAIR * 32];
           }
-          for (; p < count; ++p) t += column[p * FG_J * 32];
+          for (; p < count; ++p) t += column[p * FG_PAIR * 32];
         }
       }
-      if (threadIdx.x < FG_J * 32 && co_ok && j < J) {
+      if (threadIdx.x < FG_PAIR * 32 && co_ok && j < J) {
         const float v = t * sg.scale;
         sg.dst[(size_t)(co0 + lane) * J + j] = v;
         ss = fmaf(v, v, ss);
       }
       __syncthreads();
-    } else if (sg.mode == FG_MANY) {
-      // a group is FG_J j x 32 co: small, so that the many-split layers spread over all blocks of the grid; warp w
-      // adds the splits w, w + 8, ... with 32 loads in flight per thread (its latency, not the bandwidth, sets the
-      // pace of a group); the additions keep their order
-      constexpr int SPI = 32 / FG_J;                      // splits per iteration and warp
-      const int j0 = (local / co_tiles) * FG_J;
-      float acc[FG_J];
+    } else if (sg.mode == FG_FEW) {
+      const int j0 = tile * FG_ROWS, r = (int)threadIdx.x >> 3, q = (int)threadIdx.x & 7;
+      constexpr int PER = FG_ROWS / 32;
+      const float* src = sg.part + (size_t)(j0 + r) * CO + co0 + 4 * q;
+      float4 t[PER];
 #pragma unroll
-      for (int q = 0; q < FG_J; ++q) acc[q] = 0.f;
-      const float* src = sg.part + (size_t)j0 * CO + co0 + lane;
-      for (int p = warp; p < sg.splits; p += 8 * SPI) {
-        float v[SPI][FG_J];
+      for (int i = 0; i < PER; ++i) t[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int p = 0; p < sg.splits; p += 2) {
+        float4 v[2][PER];
 #pragma unroll
-        for (int u = 0; u < SPI; ++u)
+        for (int u = 0; u < 2; ++u)
 #pragma unroll
-          for (int q = 0; q < FG_J; ++q)
-            v[u][q] = (co_ok && j0 + q < J && p + 8 * u < sg.splits) ? __ldg(src + (size_t)(p + 8 * u) * total + (size_t)q * CO) : 0.f;
+          for (int i = 0; i < PER; ++i)
+            v[u][i] = p + u < sg.splits && j0 + r + 32 * i < J ? __ldg(reinterpret_cast<const float4*>(src + (size_t)(p + u) * total + (size_t)(32 * i) * CO))
+                                                               : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < SPI; ++u)
-          if (p + 8 * u < sg.splits) {
+        for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int q = 0; q < FG_J; ++q) acc[q] += v[u][q];
-          }
+          for (int i = 0; i < PER; ++i) { t[i].x += v[u][i].x; t[i].y += v[u][i].y; t[i].z += v[u][i].z; t[i].w += v[u][i].w; }
       }
 #pragma unroll
-      for (int q = 0; q < FG_J; ++q) sh[(warp * FG_J + q) * 33 + lane] = acc[q];
-      __syncthreads();
-      if (threadIdx.x < 32 * FG_J) {
-        const int c = threadIdx.x / FG_J, q = threadIdx.x % FG_J;   // consecutive threads write consecutive j
-        float t = 0.f;
+      for (int i = 0; i < PER; ++i) {
+        t[i] = make_float4(t[i].x * sg.scale, t[i].y * sg.scale, t[i].z * sg.scale, t[i].w * sg.scale);
+        ss = fmaf(t[i].x, t[i].x, ss); ss = fmaf(t[i].y, t[i].y, ss); ss = fmaf(t[i].z, t[i].z, ss); ss = fmaf(t[i].w, t[i].w, ss);
+        if (sg.view == FG_FLAT) {
+          if (j0 + r + 32 * i < J) *reinterpret_cast<float4*>(sg.dst + (size_t)(j0 + r + 32 * i) * 32 + 4 * q) = t[i];
+        } else {
+          *reinterpret_cast<float4*>(sh + (r + 32 * i) * FG_LD + 4 * q) = t[i];
+        }
+      }
+      if (sg.view != FG_FLAT) {
+        __syncthreads();
+        // a warp writes whole runs of j of a co at a time
 #pragma unroll
-        for (int w = 0; w < 8; ++w) t += sh[(w * FG_J + q) * 33 + c];
-        if (co0 + c < CO && j0 + q < J) { const float v = t * sg.scale; sg.dst[(size_t)(co0 + c) * J + j0 + q] = v; ss = fmaf(v, v, ss); }
+        for (int i = 0; i < PER; ++i) {
+          const int e = (int)threadIdx.x + 256 * i, c = e / (FG_ROWS / 4), j = e % (FG_ROWS / 4) * 4;
+          const float* column = sh + j * FG_LD + c;
+          float* dst = sg.dst + (size_t)(co0 + c) * J + j0 + j;
+          if (sg.view == FG_TURNED && J % 4 == 0) {
+            if (j0 + j < J) *reinterpret_cast<float4*>(dst) = make_float4(column[0], column[FG_LD], column[2 * FG_LD], column[3 * FG_LD]);
+          } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (j0 + j + u < J) (sg.view == FG_PAIRS ? sg.dst + (size_t)(c & 15) * (2 * J) + 2 * (j0 + j + u) + (c >> 4) : dst + u)[0] = column[u * FG_LD];
+          }
+        }
+        __syncthreads();
+      }
+    } else if (sg.mode == FG_MANY) {
+      const int shift = sg.row_shift, rows = 1 << shift, sums = 32 >> shift;
+      const int j0 = tile * rows, slot = (int)threadIdx.x >> 3, q = (int)threadIdx.x & 7, r = slot & (rows - 1);
+      static_assert(FG_ROWS >= 32 && FG_ROWS * FG_LD <= FG_CHUNK * FG_PAIR * 32, "32 threads' fours to a value; shared memory");
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j0 + r < J) t = add_splits(sg.part + (size_t)(j0 + r) * CO + co0 + 4 * q, slot >> shift, sg.splits, sums, total);
+      *reinterpret_cast<float4*>(sh + slot * FG_LD + 4 * q) = t;
+      __syncthreads();
+      if ((int)threadIdx.x < 32 * rows) {
+        // flat: neighbouring threads take neighbouring co; else neighbouring j
+        const bool flat = sg.view == FG_FLAT;
+        const int c = flat ? lane : (int)threadIdx.x >> shift, j = flat ? warp : (int)threadIdx.x & (rows - 1);
+        float v = 0.f;
+#pragma unroll 8
+        for (int w = 0; w < sums; ++w) v += sh[(w * rows + j) * FG_LD + c];
+        v *= sg.scale;
+        if (j0 + j < J) {
+          sg.dst[flat ? (size_t)(j0 + j) * 32 + c
+                      : (sg.view == FG_PAIRS ? (size_t)(c & 15) * (2 * J) + 2 * (j0 + j) + (c >> 4) : (size_t)(co0 + c) * J + j0 + j)] = v;
+          ss = fmaf(v, v, ss);
+        }
       }
       __syncthreads();
     } else {
-      const int j0 = (local / co_tiles) * 32;
-      float t[4] = {0.f, 0.f, 0.f, 0.f};
-      const float* src = sg.part + (size_t)(j0 + warp) * CO + co0 + lane;
-      bool ok[4];
-#pragma unroll
-      for (int rr = 0; rr < 4; ++rr) ok[rr] = co_ok && j0 + warp + 8 * rr < J;
-#pragma unroll 4
-      for (int p = 0; p < sg.splits; ++p) {
-        float v[4];
-#pragma unroll
-        for (int rr = 0; rr < 4; ++rr) v[rr] = ok[rr] ? __ldg(src + (size_t)p * total + (size_t)(8 * rr) * CO) : 0.f;
-#pragma unroll
-        for (int rr = 0; rr < 4; ++rr) t[rr] += v[rr];
-      }
-#pragma unroll
-      for (int rr = 0; rr < 4; ++rr) sh[(warp + 8 * rr) * 33 + lane] = t[rr];
+      const int j = tile;
+      float t = 0.f;
+      if (co0 + lane < CO)
+        for (int p = warp; p < sg.splits; p += 8) t += __ldg(sg.part + (size_t)p * total + (size_t)j * CO + co0 + lane);
+      sh[warp * 32 + lane] = t;
       __syncthreads();
+      if (warp == 0 && co0 + lane < CO) {
+        float v = 0.f;
 #pragma unroll
-      for (int rr = 0; rr < 4; ++rr) {
-        const int c = warp + 8 * rr;
-        if (co0 + c < CO && j0 + lane < J) { const float v = sh[lane * 33 + c] * sg.scale; sg.dst[(size_t)(co0 + c) * J + j0 + lane] = v; ss = fmaf(v, v, ss); }
+        for (int w = 0; w < 8; ++w) v += sh[w * 32 + lane];
+        v *= sg.scale;
+        sg.dst[(size_t)(co0 + lane) * J + j] = v;
+        ss = fmaf(v, v, ss);
       }
       __syncthreads();
     }
@@ -2262,14 +2315,20 @@ __global__ void __launch_bounds__(256) tc_finalize_grads_kernel(GradSegments seg
 }
 
 bool add_grad_segment(GradSegments* segs, const float* part, float* dst, int splits, int J, int CO, float scale, bool in_order) {
-  if (segs->n >= (int)(sizeof(segs->seg) / sizeof(segs->seg[0]))) return false;      // the caller reports a host failure
+  if (segs->n >= GradSegments::MOST) return false;      // the caller reports a host failure
   GradSegment& g = segs->seg[segs->n++];
+  const bool whole = CO % 32 == 0 && (J == 1 || (CO & (CO - 1)) == 0);       // tiles of 32 co, a power of two of them
+  const bool vectors = (whole || (CO == 16 && J % 2 == 0)) && ((uintptr_t)part & 15) == 0 && ((uintptr_t)dst & 15) == 0;
   g.part = part; g.dst = dst; g.splits = splits; g.J = J; g.CO = CO; g.scale = scale;
-  g.mode = splits <= 8 ? FG_FEW : (in_order ? FG_IN_ORDER : FG_MANY);
-  g.first_group = segs->total_groups;
-  const int rows = g.mode == FG_FEW ? 32 : FG_J;
-  g.groups = ((J + rows - 1) / rows) * ((CO + 31) / 32);
-  segs->total_groups += g.groups;
+  g.mode = splits > 8 && in_order ? FG_IN_ORDER : (!vectors ? FG_ODD : (splits <= 8 ? FG_FEW : FG_MANY));
+  g.view = FG_TURNED;
+  if (g.mode == FG_FEW || g.mode == FG_MANY) {
+    if (J == 1) { g.view = FG_FLAT; g.J = CO / 32; g.CO = 32; }
+    else if (CO == 16) { g.view = FG_PAIRS; g.J = J / 2; g.CO = 32; }
+  }
+  g.row_shift = g.mode == FG_FEW ? FG_ROW_SHIFT : (g.mode == FG_MANY ? 2 : (g.mode == FG_IN_ORDER ? FG_PAIR_SHIFT : 0));
+  g.co_shift = 0;
+  while (32 << g.co_shift < g.CO) ++g.co_shift;
   return true;
 }
 
@@ -2872,8 +2931,17 @@ int finish_gradients(LaunchCtx& lc, GradSegments* segs, float* sumsq_partials, i
   int blocks = 0;
   if (segs->n > 0) {
     KernelScope scope(lc, KID_WGRAD_REDUCE);
+    segs->total_groups = 0;
+    for (int i = 0; i < segs->n; ++i) {
+      GradSegment& g = segs->seg[i];
+      segs->first_group[i] = segs->total_groups;
+      segs->total_groups += (g.J + (1 << g.row_shift) - 1) >> g.row_shift << g.co_shift;
+    }
+    for (int i = segs->n; i < GradSegments::MOST; ++i) segs->first_group[i] = segs->total_groups;
     blocks = segs->total_groups < max_blocks ? segs->total_groups : max_blocks;
-    launch_kernel(lc, tc_finalize_grads_kernel, blocks, 256, 0, *segs, sumsq_partials);
+    bool in_order = false;
+    for (int i = 0; i < segs->n; ++i) in_order |= segs->seg[i].mode == FG_IN_ORDER;
+    launch_kernel(lc, in_order ? tc_finalize_grads_kernel<true> : tc_finalize_grads_kernel<false>, blocks, 256, 0, *segs, sumsq_partials);
   }
   segs->n = 0; segs->total_groups = 0;
   return blocks;
