@@ -32,6 +32,8 @@ __device__ __forceinline__ float4 widen4(uint2 halves) {
   return make_float4(__uint_as_float(halves.x << 16), __uint_as_float(halves.x & 0xFFFF0000u), __uint_as_float(halves.y << 16),
                      __uint_as_float(halves.y & 0xFFFF0000u));
 }
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const bf16* p) { return widen4(*reinterpret_cast<const uint2*>(p)); }
 __device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void store4(bf16* p, float4 v) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);

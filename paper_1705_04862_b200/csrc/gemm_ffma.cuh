@@ -38,8 +38,6 @@ __device__ __forceinline__ void widen(const uint4 v, const bf16*, float4 (&f)[2]
 __device__ __forceinline__ void widen(const uint4 v, const uint8_t*, float4 (&f)[4]) {
   f[0] = widen4(v.x); f[1] = widen4(v.y); f[2] = widen4(v.z); f[3] = widen4(v.w);
 }
-__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 load4(const bf16* p) { return widen4(*reinterpret_cast<const uint2*>(p)); }
 
 // A k block of R rows in shared memory: [R][BK + 4] or [BK][R + 4] (the padding keeps the reads below free of conflicts).
 template <class OP, int R, int BK> struct FfTile {

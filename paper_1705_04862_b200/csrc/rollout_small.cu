@@ -169,7 +169,6 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
   __shared__ EnvFrame s_frame;
   __shared__ int32_t s_action;
   __shared__ volatile uint32_t s_dead;
-  __shared__ uint32_t s_epoch;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = q.n, A = q.A;
   const bool conv = (int)blockIdx.x < n * C;
   const int e = blockIdx.x / C, rank = blockIdx.x % C;
@@ -193,59 +192,99 @@ rollout_small_kernel(RsArgs q, const TW* w1, const TW* w2, const TW* wfc, const 
     if (i >= own_lo && i < own_hi) state[i] = v;
     if (i >= row_lo * QUADS && i < row_hi * QUADS) frame[i] = v;
   };
-  if (conv && q.host.states != nullptr) {
-    // the whole state over the host link; a thread asks for all its words before it uses any
-    constexpr int MOST = (FRAME_WORDS / 4 + RS_THREADS - 1) / RS_THREADS;
-    const uint4* src = reinterpret_cast<const uint4*>(q.host.states) + (size_t)e * (FRAME_WORDS / 4);
-    uint4* state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
-    uint4 v[MOST];
+  // What stays for the rollout: both convolutions' weights as [k][channel], the weight tile, the head weights.  All are asked for before any is
+  // used, and what comes over the host link after them, so that one latency covers them all.  (A warp's lanes take a channel each, so
+  // that their values go to different banks; value by value in the order of the arrays, the stores of the second layer's weights alone met 32
+  // conflicts each: a launch took 8 us more; an iteration at 4 environments 121.7 -> 114.7 us, with whole states of 32 from outside 490 -> 439.)
+  constexpr int W1_PER = RC1::KK * RC1::CO / 4 / RS_THREADS, W2_PER = RC2::KK * RC2::CO / 4 / RS_THREADS, FC_PER = RS_COLS * RS_RUN / 4 / RS_THREADS, HEAD_PER = 32 * RS_F / 4 / RS_THREADS;
+  const uint32_t epoch = q.sync[0];
+  const uint64_t step0 = *q.step_base + q.t0;
+  float4 v1[W1_PER], v2[W2_PER], vf[FC_PER], vh[HEAD_PER];
+  float value_head = 0.f;
+  if (conv) {
 #pragma unroll
-    for (int u = 0; u < MOST; ++u)
-      if (part_lo + tid + u * RS_THREADS < part_hi) v[u] = src[part_lo + tid + u * RS_THREADS];
+    for (int u = 0; u < W1_PER; ++u) { const int i = tid + u * RS_THREADS; v1[u] = load4(w1 + i % RC1::CO * RC1::KK + i / RC1::CO * 4); }
 #pragma unroll
-    for (int u = 0; u < MOST; ++u)
-      if (part_lo + tid + u * RS_THREADS < part_hi) place(state, part_lo + tid + u * RS_THREADS, v[u]);
+    for (int u = 0; u < W2_PER; ++u) { const int i = tid + u * RS_THREADS; v2[u] = load4(w2 + i % RC2::CO * RC2::KK + i / RC2::CO * 4); }
+#pragma unroll
+    for (int u = 0; u < HEAD_PER; ++u) { const int i = tid + u * RS_THREADS; if (i < A * RS_F / 4) vh[u] = load4(wpi + 4 * i); }
+    if (tid < RS_F) value_head = to_f(wv[tid]);
   }
-  if (conv && q.host.newest != nullptr) {
-    // or the newest plane, sixteen pixels to a word, onto the stack of the state before
-    constexpr int MOST = (STACK_ITEMS + RS_THREADS - 1) / RS_THREADS;
-    const uint4* src = reinterpret_cast<const uint4*>(q.host.newest) + (size_t)e * STACK_ITEMS;
-    const uint4* prev = reinterpret_cast<const uint4*>(q.host.prev) + (size_t)e * (FRAME_WORDS / 4);
-    uint4* state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
-    const bool fresh = (q.host.fresh[e >> 5] >> (e & 31)) & 1u;
-    uint4 v[MOST];
+  if (fc) {
+#pragma unroll
+    for (int u = 0; u < FC_PER; ++u) {
+      const int i = tid + u * RS_THREADS, c = i / (RS_RUN / 4), k = i % (RS_RUN / 4) * 4;
+      vf[u] = k < len ? load4(wfc + (size_t)(col0 + c) * RS_IN + k0 + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  uint4* const state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
+  // the whole state over the host link, or the newest plane, sixteen pixels to a word
+  constexpr int MOST = (FRAME_WORDS / 4 + RS_THREADS - 1) / RS_THREADS, MOST_PLANE = (STACK_ITEMS + RS_THREADS - 1) / RS_THREADS;
+  static_assert(MOST_PLANE <= MOST, "the same registers");
+  uint4 in[MOST];
+  if (conv && q.host.states != nullptr) {
+    const uint4* src = reinterpret_cast<const uint4*>(q.host.states) + (size_t)e * (FRAME_WORDS / 4);
 #pragma unroll
     for (int u = 0; u < MOST; ++u)
-      if (part_lo / 4 + tid + u * RS_THREADS < (part_hi + 3) / 4) v[u] = src[part_lo / 4 + tid + u * RS_THREADS];
+      if (part_lo + tid + u * RS_THREADS < part_hi) in[u] = src[part_lo + tid + u * RS_THREADS];
+  } else if (conv && q.host.newest != nullptr) {
+    const uint4* src = reinterpret_cast<const uint4*>(q.host.newest) + (size_t)e * STACK_ITEMS;
 #pragma unroll
-    for (int u = 0; u < MOST; ++u) {
+    for (int u = 0; u < MOST_PLANE; ++u)
+      if (part_lo / 4 + tid + u * RS_THREADS < (part_hi + 3) / 4) in[u] = src[part_lo / 4 + tid + u * RS_THREADS];
+  } else if (conv) {
+#pragma unroll
+    for (int u = 0; u < MOST; ++u)
+      if (row_lo * QUADS + tid + u * RS_THREADS < row_hi * QUADS) in[u] = __ldcg(state + row_lo * QUADS + tid + u * RS_THREADS);
+  }
+  if (conv) {
+#pragma unroll
+    for (int u = 0; u < W1_PER; ++u) {
+      float* to = sm + RS_W1 + (tid + u * RS_THREADS) / RC1::CO * 4 * RC1::CO + (tid + u * RS_THREADS) % RC1::CO;
+      to[0] = v1[u].x; to[RC1::CO] = v1[u].y; to[2 * RC1::CO] = v1[u].z; to[3 * RC1::CO] = v1[u].w;
+    }
+#pragma unroll
+    for (int u = 0; u < W2_PER; ++u) {
+      float* to = sm + RS_W2 + (tid + u * RS_THREADS) / RC2::CO * 4 * RC2::CO + (tid + u * RS_THREADS) % RC2::CO;
+      to[0] = v2[u].x; to[RC2::CO] = v2[u].y; to[2 * RC2::CO] = v2[u].z; to[3 * RC2::CO] = v2[u].w;
+    }
+#pragma unroll
+    for (int u = 0; u < HEAD_PER; ++u)
+      if (tid + u * RS_THREADS < A * RS_F / 4) *reinterpret_cast<float4*>(sm + RS_HEADW + 4 * (tid + u * RS_THREADS)) = vh[u];
+    if (tid < RS_F) sm[RS_HEADW + A * RS_F + tid] = value_head;
+  }
+  if (fc) {
+#pragma unroll
+    for (int u = 0; u < FC_PER; ++u) {
+      const int i = tid + u * RS_THREADS;
+      *reinterpret_cast<float4*>(sm + RS_FCW + i / (RS_RUN / 4) * RS_FC_LD + i % (RS_RUN / 4) * 4) = vf[u];
+    }
+  }
+  if (conv && q.host.states != nullptr) {
+#pragma unroll
+    for (int u = 0; u < MOST; ++u)
+      if (part_lo + tid + u * RS_THREADS < part_hi) place(state, part_lo + tid + u * RS_THREADS, in[u]);
+  } else if (conv && q.host.newest != nullptr) {
+    // onto the stack of the state before
+    const uint4* prev = reinterpret_cast<const uint4*>(q.host.prev) + (size_t)e * (FRAME_WORDS / 4);
+    const bool fresh = (q.host.fresh[e >> 5] >> (e & 31)) & 1u;
+#pragma unroll
+    for (int u = 0; u < MOST_PLANE; ++u) {
       const int i = part_lo / 4 + tid + u * RS_THREADS;
       if (i < (part_hi + 3) / 4) {
         uint4 o[4];
-        stack_sixteen(v[u], fresh, prev + 4 * i, o);
+        stack_sixteen(in[u], fresh, prev + 4 * i, o);
 #pragma unroll
         for (int k = 0; k < 4; ++k) place(state, 4 * i + k, o[k]);
       }
     }
+  } else if (conv) {
+#pragma unroll
+    for (int u = 0; u < MOST; ++u)
+      if (row_lo * QUADS + tid + u * RS_THREADS < row_hi * QUADS) frame[row_lo * QUADS + tid + u * RS_THREADS] = in[u];
   }
-  // what stays for the rollout: both convolutions' weights as [k][channel], the head weights, the weight tile
-  if (conv) {
-    for (int i = tid; i < RC1::KK * RC1::CO; i += RS_THREADS) sm[RS_W1 + i % RC1::KK * RC1::CO + i / RC1::KK] = to_f(w1[i]);
-    for (int i = tid; i < RC2::KK * RC2::CO; i += RS_THREADS) sm[RS_W2 + i % RC2::KK * RC2::CO + i / RC2::KK] = to_f(w2[i]);
-    for (int i = tid; i < (A + 1) * RS_F; i += RS_THREADS) sm[RS_HEADW + i] = i < A * RS_F ? to_f(wpi[i]) : to_f(wv[i - A * RS_F]);
-    uint4* state = reinterpret_cast<uint4*>(const_cast<uint8_t*>(q.frames) + (size_t)e * FRAME_BYTES);
-    if (q.host.newest == nullptr && q.host.states == nullptr)
-      for (int i = row_lo * QUADS + tid; i < row_hi * QUADS; i += RS_THREADS) frame[i] = __ldcg(state + i);
-  }
-  if (fc)
-    for (int i = tid; i < RS_COLS * RS_RUN; i += RS_THREADS) {
-      const int c = i / RS_RUN, k = i % RS_RUN;
-      sm[RS_FCW + c * RS_FC_LD + k] = k < len ? to_f(wfc[(size_t)(col0 + c) * RS_IN + k0 + k]) : 0.f;
-    }
-  const uint64_t step0 = *q.step_base + q.t0;
-  if (tid == 0) { s_dead = 0u; s_epoch = q.sync[0]; }
+  if (tid == 0) s_dead = 0u;
   __syncthreads();
-  const uint32_t epoch = s_epoch;
 
   for (int t = 0; t < q.steps; ++t) {
     const size_t slot = (size_t)t * n;
