@@ -22,7 +22,7 @@
 // (12 with 4): first layer 4.8, second 4.0 (its weights, read from shared memory by every warp), waiting for the second map 1.2 and
 // the fully connected runs 3, waiting for their sums 1.0, heads, draw and transition 0.85.  With two barriers over the
 // device (1.3 us each, and a second round trip through L2 to read what they guard) instead of words, a rollout of five steps and the
-// bootstrap took 84 us with 4 states, 122 with 32 and 205 with 74; now 78, 119 and 202.
+// bootstrap took 84 us with 4 states, 122 with 32 and 205 with 74, with them 78, 119 and 202 (and 7 to 8 less since the set-up loads all at once).
 //
 // With environments outside, a step is one such launch too: each block fetches the part of the state that it needs (or of the newest
 // plane) over the host link and writes its share out; actions and values go straight into pinned memory.
