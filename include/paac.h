@@ -281,8 +281,9 @@ int paac_debug_read(paac_ctx* ctx, int which, void* dst /* host */, size_t bytes
  * PAAC_DBG_RMS and PAAC_DBG_COUNTERS on resume). Synchronises. */
 int paac_debug_write(paac_ctx* ctx, int which, const void* src /* host */, size_t bytes);
 
-/* Run-time options.  PAAC_OPT_CUDA_CORES_ONLY != 0 keeps the bf16 network off the tensor cores
- * (same rounding points, CUDA-core contractions): a second implementation to compare against.
+/* Run-time options.  PAAC_OPT_CUDA_CORES_ONLY != 0 keeps either network off the tensor cores, in either storage
+ * (same rounding points, CUDA-core contractions): a second implementation to compare against, and float learners whose
+ * gradients are chains of float multiply-adds throughout.  PAAC_OPT_FP32_TENSOR_CORES, if that is set too, comes first.
  * PAAC_OPT_TC_WGRAD_LAYERS: bit mask (bit l = layer l, conv1 = 0) of the layers whose weight gradient
  * runs on the tensor cores; the others use the CUDA-core contraction.  Default: all.
  * PAAC_OPT_CUDA_GRAPHS: != 0 (default) lets paac_rollout / paac_update record their kernel sequence into CUDA

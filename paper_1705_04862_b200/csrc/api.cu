@@ -77,7 +77,6 @@ struct paac_ctx {
   int plain_calls[GRAPH_KINDS][2];   // calls made with plain launches
   cudaGraphExec_t graph[GRAPH_KINDS][2];
   uint64_t graph_launches[GRAPH_KINDS][2];
-  bool simt_only;          // keep the bf16 network on the CUDA cores (cross-check of the tensor-core path)
   paac_ctx* next;          // the learners of this process (see Learners)
 
   // device buffers (all inside the workspace)
@@ -192,7 +191,7 @@ int cuda_status(paac_ctx* c) {
   return launches_ok && !c->lc.host_failure ? PAAC_OK : PAAC_ERR_CUDA;
 }
 
-bool use_tc(const paac_ctx* c) { return tc_supported(c->arch, c->prec) && !c->simt_only; }
+bool use_tc(const paac_ctx* c) { return tc_supported(c->arch, c->prec) && !c->lc.cuda_cores_only; }
 HeadMode head_mode(const paac_ctx* c) { return HeadMode{c->hp.algorithm, c->hp.epsilon}; }
 int pattern_actions(const paac_ctx* c) { return c->hp.environment == PAAC_ENV_PATTERN ? c->A : 0; }
 
@@ -743,7 +742,7 @@ uint64_t paac_launch_count(const paac_ctx* c) { return c ? c->lc.count : 0; }
 
 int paac_set_option(paac_ctx* c, int option, int value) {
   if (!c) return PAAC_ERR_ARG;
-  if (option == PAAC_OPT_CUDA_CORES_ONLY) { c->simt_only = value != 0; drop_graphs(c); return PAAC_OK; }
+  if (option == PAAC_OPT_CUDA_CORES_ONLY) { c->lc.cuda_cores_only = value != 0; drop_graphs(c); return PAAC_OK; }
   if (option == PAAC_OPT_TC_WGRAD_LAYERS) { c->tc_wgrad_mask = value & 0xF; drop_graphs(c); return PAAC_OK; }
   if (option == PAAC_OPT_CUDA_GRAPHS) { c->graphs_on = value != 0; drop_graphs(c); return PAAC_OK; }
   if (option == PAAC_OPT_DEPENDENT_LAUNCH) { pdl_enabled() = value != 0; drop_graphs(c); return PAAC_OK; }

@@ -247,6 +247,7 @@ struct LaunchCtx {
   bool serialize_next = true;         // the next launch takes plain stream order (no overlap with its predecessor)
   bool host_failure = false;          // a launch could not be prepared on the host (sticky; reported as PAAC_ERR_CUDA)
   bool fp32_tensor_cores = false;     // all of the float path's contractions go through the three-pass tensor-core kernel
+  bool cuda_cores_only = false;       // nothing goes to the tensor cores by itself, the bf16 network included (a second implementation to compare with)
   bool bf16_sums_on_tensor_cores = false;   // those of bf16 storage may, where it is the faster one (the larger network has kernels of its own)
   uint32_t* error_word = nullptr;     // device word the bounded waits of that kernel report to
   static constexpr int MAX_PENDING = 512;

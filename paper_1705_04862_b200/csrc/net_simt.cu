@@ -42,7 +42,7 @@ static int t3_splits(int M, int N, int K) {
 // sums in 64 bits, 2-norm: 1.2 to 1.5e-7 instead of 1.2 to 2.9e-7.
 // The forward pass stays on the CUDA cores, whose chains of multiply-adds are the same for every batch: sums as exact but in another order put
 // a unit or two per pass on the other side of the ReLU, and training then runs apart from there.
-template <class T> static bool t3_allowed(const LaunchCtx& lc) { return lc.error_word != nullptr && (sizeof(T) == 4 || lc.bf16_sums_on_tensor_cores); }
+template <class T> static bool t3_allowed(const LaunchCtx& lc) { return !lc.cuda_cores_only && lc.error_word != nullptr && (sizeof(T) == 4 || lc.bf16_sums_on_tensor_cores); }
 template <class T> static bool t3_pays(const LaunchCtx& lc, long long M, int N, int K) {
   if (lc.fp32_tensor_cores) return lc.error_word != nullptr;
   const long long blocks = (K + T3_BK - 1) / T3_BK, macs = M * N * K;

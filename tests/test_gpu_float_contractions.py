@@ -1,6 +1,7 @@
 """Data and weight gradients of the float path on the tensor cores (two TF32 pieces to a value), every layer from the oracle's own
 stored tensors: batches that fill less than a tile, k that ends inside a block of 32, and the sizes at which the library
 takes them by itself."""
+import numpy as np
 import pytest
 
 import paper_1705_04862_b200.binding as pb
@@ -24,3 +25,87 @@ def test_gradients_from_the_same_tensors(orc, arch, prec, n_e, t_max, n_actions,
         check_update(orc, o, g, TOL[prec], inject=True)
     assert g.error_word() == 0
     g.close()
+
+
+DATA, WEIGHTS = "gact", "weights"
+
+
+def contractions(arch, n):
+    """The gradients' contractions of a float learner over n states, as (kind, layer, outputs, k)."""
+    if arch == "nips":
+        return [(WEIGHTS, 2, 2592 * 256, n), (DATA, 2, n * 2592, 256), (WEIGHTS, 1, 256 * 32, 81 * n), (DATA, 1, n * 100 * 64, 128),
+                (WEIGHTS, 0, 256 * 16, 400 * n)]
+    return [(WEIGHTS, 3, 3136 * 512, n), (DATA, 3, n * 3136, 512), (WEIGHTS, 2, 576 * 64, 49 * n), (DATA, 2, n * 81 * 64, 576),
+            (WEIGHTS, 1, 512 * 64, 81 * n), (DATA, 1, n * 100 * 128, 256), (WEIGHTS, 0, 256 * 32, 400 * n)]
+
+
+def on_tensor_cores(kind, outputs, k):
+    """The rule of the dispatch for contractions nobody chose a path for."""
+    if kind == WEIGHTS:
+        return k >= 256 and outputs * k >= 64_000_000
+    return outputs * k >= max(80_000_000, 11_000_000 * -(-k // 32))
+
+
+def gradients(arch, prec, n_e, t_max, options, n_actions=6):
+    """Gradients of one update, layer by layer, all from the same rollout whatever the options of the update."""
+    g = pb.Paac(arch, n_e, t_max, n_actions, seed=9, precision=pb.BF16 if prec == "bf16" else pb.FP32, lr=0.0028, term_denom=50)
+    g.rollout()
+    for option, value in options.items():
+        g.set_option(option, value)
+    assert g.update()["status"] == 0 and g.error_word() == 0
+    L = 2 if arch == "nips" else 3
+    gact = [g.debug_read(pb.DBG_GACT0 + l).copy() for l in range(L + 1)]
+    grad, at = g.debug_read(pb.DBG_GRAD), 0
+    weights = []
+    for J, co in ((256, 16), (256, 32), (2592, 256)) if arch == "nips" else ((256, 32), (512, 64), (576, 64), (3136, 512)):
+        weights.append(grad[at:at + (J + 1) * co].copy())
+        at += (J + 1) * co
+    g.close()
+    return {"gact": gact, "weights": weights}
+
+
+AUTO, CORES_ONLY, TENSOR = {}, {pb.OPT_CUDA_CORES_ONLY: 1}, {pb.OPT_FP32_TENSOR_CORES: 1}
+
+
+@pytest.mark.parametrize("arch,prec,n", [("nips", "bf16", n) for n in (39, 40, 96, 97, 98, 255, 256)]
+                         + [("nips", "fp32", n) for n in (39, 40, 96, 97, 98, 132, 133, 255, 256)]
+                         + [("nature", "fp32", n) for n in (19, 20, 24, 25, 26, 27, 35, 36, 66, 67, 109, 110, 255, 256)])
+def test_which_contractions_go_to_the_tensor_cores(arch, prec, n):
+    """Just below and just above each line of the rule: what the library chooses by itself has the bits of the one contraction
+    or of the other, and with CUDA_CORES_ONLY none has those of the tensor cores."""
+    auto, cores, tensor = (gradients(arch, prec, n, 1, o) for o in (AUTO, CORES_ONLY, TENSOR))
+    compared = 0
+    for kind, l, outputs, k in contractions(arch, n):
+        at = l - 1 if kind == DATA else l
+        same_operand = np.array_equal(cores["gact"][l], tensor["gact"][l])
+        # (a data gradient in bf16 storage is rounded to eight bits, where the two contractions nearly always meet)
+        if same_operand and not (prec == "bf16" and kind == DATA):
+            assert not np.array_equal(cores[kind][at], tensor[kind][at]), (kind, l)
+        want = tensor if on_tensor_cores(kind, outputs, k) else cores
+        if np.array_equal(auto["gact"][l], want["gact"][l]):
+            assert np.array_equal(auto[kind][at], want[kind][at]), (kind, l)
+            compared += 1
+    assert compared >= 2
+
+
+@pytest.mark.parametrize("arch,hidden,width", [("nips", 256, 2592), ("nature", 512, 3136)])
+def test_cuda_cores_only_keeps_float_chains(arch, hidden, width):
+    """With CUDA_CORES_ONLY a data gradient of a float learner is one chain of fused multiply-adds over the hidden units, to the bit,
+    at a size whose contraction goes to the tensor cores otherwise."""
+    n = 160
+    g = pb.Paac(arch, n, 1, 6, seed=9, precision=pb.FP32, lr=0.0028, term_denom=50)
+    l = 2 if arch == "nips" else 3
+    at = {"nips": 257 * 16 + 257 * 32, "nature": 257 * 32 + 513 * 64 + 577 * 64}[arch]
+    w = g.params()[at:at + hidden * width].reshape(hidden, width).copy()
+    g.rollout()
+    g.set_option(pb.OPT_CUDA_CORES_ONLY, 1)
+    assert g.update()["status"] == 0
+    rows = slice(0, n, 23)
+    got = g.debug_read(pb.DBG_GACT0 + l - 1).reshape(n, width)[rows]
+    act = g.debug_read(pb.DBG_ACT0 + l - 1).reshape(n, width)[rows]
+    out = g.debug_read(pb.DBG_GACT0 + l).reshape(n, hidden)[rows].astype(np.float64)
+    g.close()
+    chain = np.zeros(got.shape, np.float32)
+    for k in range(hidden):       # the product is exact in 64 bits, and so nearly always is the sum
+        chain = (chain + out[:, k, None] * w[k].astype(np.float64)).astype(np.float32)
+    assert np.array_equal(got, np.where(act > 0, chain, np.float32(0)))
