@@ -616,11 +616,7 @@ template <int C_> struct RtKernel {
     cfg = cudaLaunchConfig_t{};
     cfg.gridDim = dim3(clusters * C); cfg.blockDim = dim3(RT_THREADS); cfg.dynamicSmemBytes = RtMem<C>::TOTAL;
     attr.id = cudaLaunchAttributeCooperative; attr.val.cooperative = 1;
-#ifdef NOCOOP
-    cfg.attrs = &attr; cfg.numAttrs = 0;
-#else
     cfg.attrs = &attr; cfg.numAttrs = 1;
-#endif
   }
   // Clusters that are resident at once (blocks that wait for one another have to be); 0 if they are too few for the fully
   // connected layer's tiles.
