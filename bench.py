@@ -59,7 +59,6 @@ def kernel_work(cfg):
     w["heads_bwd"] = ("tensor", 4.0 * (A + 1) * F * B, 1)
     w["env_step"] = ("hbm", n_e * (FRAME_BYTES + 6.0), T)
     w["clip_rmsprop"] = ("hbm", P * (22.0 if elt == 2 else 20.0), 1)
-    w["grad_sumsq"] = ("hbm", P * 4.0, 1)
     return w, P
 
 
@@ -403,7 +402,7 @@ def run_ours(args, cfg):
                                                       if pk.get("bf16_sustained") else None)
         sustained["iteration_tflops"] = (roll_flops + upd_flops) / (sustained["ms_per_step"] * 1e-3) / 1e12
     hbm_side = {}
-    for k in ("env_step", "clip_rmsprop", "grad_sumsq"):
+    for k in ("env_step", "clip_rmsprop"):
         if k in prof and prof[k][1]:
             gbs = work[k][1] / (prof[k][0] / K / work[k][2] * 1e-3) / 1e9
             hbm_side[k] = {"GB/s": gbs, "frac_of_%s_hbm" % pk["src"]: gbs / pk["hbm"]}
