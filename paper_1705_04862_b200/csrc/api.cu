@@ -604,9 +604,9 @@ int paac_update(paac_ctx* c, paac_update_stats* stats) {
       if (l > 0) side.run(wgrad); else wgrad();
       if (l == (L == 3 ? 1 : 2)) {
         // what has piled up so far (all but the first layer of the larger network; the heads and the fully connected layer of the smaller one, whose
-        // second layer the chain would wait for) is most of the gradient: finished beside the rest of the chain
-        auto finish = [&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2); };
-        if (side.on) side.append(finish);
+        // second layer the chain would wait for) is most of the gradient: finished beside the rest of the chain.  (In line too, in
+        // these two parts: the squared norm is added up block by block, and its bits are the same either way.)
+        side.append([&]() { ready = finish_gradients(c->lc, &c->grad_segs, c->norm_partials, NORM_BLOCKS / 2); });
       }
       if (chunked && l == 1) {
         // data gradient and first-layer weight gradient group by group
