@@ -22,6 +22,7 @@
 // and `done` that the stage may be filled again, so two barriers per stage are all.  Two blocks are resident per SM: one splits
 // while the other's multiplications run.  Every wait is bounded.
 #pragma once
+#include <cfloat>
 #include <type_traits>
 
 #include "gemm_ffma.cuh"
@@ -80,7 +81,8 @@ __device__ __forceinline__ void t3_tmem_ld(uint32_t taddr, uint32_t (&r)[8]) {
 }
 // Two values x = hi + lo in TF32 pieces.  hi is rounded to nearest by integer arithmetic (the conversion takes three instructions for one).
 // lo has up to twelve bits, of which the tensor cores read eleven: the factor brings what would be cut off up to a whole last place, so that lo
-// is rounded too.  A NaN may be lost in hi, not in lo; an infinity gives a NaN.
+// is rounded too.  A NaN may be lost in hi, not in lo; an infinity gives a NaN (see the
+// end of the kernel).
 __device__ __forceinline__ void split_tf32(float x, float y, uint32_t& xh, uint32_t& yh, uint32_t& xl, uint32_t& yl) {
   xh = (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u;
   yh = (__float_as_uint(y) + 0x1000u) & 0xFFFFE000u;
@@ -151,6 +153,11 @@ template <> __device__ __forceinline__ uint4 t3_lds<uint4>(uint32_t at) {
 template <> __device__ __forceinline__ uint2 t3_lds<uint2>(uint32_t at) {
   uint2 v;
   asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(at));
+  return v;
+}
+template <> __device__ __forceinline__ uint32_t t3_lds<uint32_t>(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at));
   return v;
 }
 template <> __device__ __forceinline__ float t3_lds<float>(uint32_t at) {
@@ -237,9 +244,10 @@ template <class OP, int R, bool K_CONTIG = OP::K_CONTIG> struct T3Raw {
   };
   template <int N> __device__ __forceinline__ static void read(const Reader& rd, uint32_t raw, float (&x)[N]) {
     if constexpr (N < V) {
-      static_assert(N == 4 && sizeof(T) <= 2, "half a piece");
-      const uint2 v = t3_lds<uint2>(raw + rd.at);
-      const float4 f = widen4(v);
+      static_assert(N == 4 && sizeof(T) <= 2, "part of a piece");
+      float4 f;
+      if constexpr (sizeof(T) == 2) f = widen4(t3_lds<uint2>(raw + rd.at));
+      else f = widen4(t3_lds<uint32_t>(raw + rd.at));
       x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
     } else {
 #pragma unroll
@@ -290,6 +298,12 @@ template <class OP, int R> struct T3Raw<OP, R, false> {
   }
 };
 __device__ __forceinline__ void t3_sync() { asm volatile("bar.sync 1, %0;" ::"n"(T3_NT) : "memory"); }      // the eight warps
+__device__ __forceinline__ bool t3_any(bool mine) {               // the same, and whether any thread says so
+  uint32_t any;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(any) : "r"(mine ? 1u : 0u), "n"(T3_NT) : "memory");
+  return any != 0u;
+}
 
 template <int BN, class LA, class LB, class EP>
 __global__ void __launch_bounds__(T3_THREADS, 2)
@@ -426,7 +440,39 @@ gemm_tc3_kernel(int M, int N, int K, int k_per_split, int splits, LA la, LB lb, 
     }
     if (alive && num_kb > 0) alive = collect(num_kb - 1);
     cp_async_wait<0>();
-    t3_sync();                       // the ring is free, and the instructions are through with the images
+    bool finite = true;
+#pragma unroll
+    for (int j = 0; j < C::COLS; ++j) finite = finite && fabsf(sum[j]) <= FLT_MAX;
+    if (t3_any(alive && !finite)) {  // (the ring is free, and the instructions are through with the images)
+      // An infinity, or a value that rounds to one, has no lo piece: where a sum is not finite, the tile is done again by chains of fused
+      // multiply-adds, as the CUDA cores would have done it.
+#pragma unroll
+      for (int j = 0; j < C::COLS; ++j) sum[j] = 0.f;
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (TABLE && (kb & 7) == 0) tabulate(kb >> 3);
+        t3_sync();                   // the table is in, and everyone is done with the block before
+        fetch(kb, raw_base);
+        cp_async_wait<0>();
+        t3_sync();
+#pragma unroll 1
+        for (int k = 0; k < T3_BK; k += 4) {
+          typename RawA::Reader from_a;
+          float x[4];
+          from_a.init(32 * quarter + lane, k);
+          RawA::read(from_a, raw_base, x);
+#pragma unroll
+          for (int j = 0; j < C::COLS; ++j) {
+            typename RawB::Reader from_b;
+            float y[4];
+            from_b.init(grp * C::COLS + j, k);
+            RawB::read(from_b, raw_base + RawA::BYTES, y);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sum[j] = fmaf(x[q], y[q], sum[j]);
+          }
+        }
+      }
+      t3_sync();
+    }
     float* out = reinterpret_cast<float*>(raws);
 #pragma unroll
     for (int j = 0; j < C::COLS; j += 4)

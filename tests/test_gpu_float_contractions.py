@@ -109,3 +109,66 @@ def test_cuda_cores_only_keeps_float_chains(arch, hidden, width):
     for k in range(hidden):       # the product is exact in 64 bits, and so nearly always is the sum
         chain = (chain + out[:, k, None] * w[k].astype(np.float64)).astype(np.float32)
     assert np.array_equal(got, np.where(act > 0, chain, np.float32(0)))
+
+
+def poisoned(arch, n_e, t_max, options, poison):
+    """The gradients of an update whose operands `poison` has changed: it gets the learner, the activations and the parameters."""
+    g = pb.Paac(arch, n_e, t_max, 6, seed=9, precision=pb.FP32, lr=0.0028, term_denom=50)
+    g.rollout()
+    for option, value in options.items():
+        g.set_option(option, value)
+    L = 2 if arch == "nips" else 3
+    act, theta = [g.debug_read(pb.DBG_ACT0 + l).copy() for l in range(L + 1)], g.params().copy()
+    poison(act, theta)
+    for l in range(L):
+        g.debug_write_act(l, act[l])
+    g.set_params(theta)
+    g.update()
+    out = {"gact": [g.debug_read(pb.DBG_GACT0 + l).copy() for l in range(L + 1)], "grad": g.debug_read(pb.DBG_GRAD).copy(), "act": act, "theta": theta}
+    assert g.error_word() == 0
+    g.close()
+    return out
+
+
+def assert_alike(got, want):
+    """The same values are infinite, with the same sign, or not numbers; the others agree to float rounding."""
+    finite = np.isfinite(want)
+    assert np.array_equal(finite, np.isfinite(got))
+    assert np.array_equal(got[~finite], want[~finite], equal_nan=True)
+    assert np.linalg.norm(got[finite].astype(np.float64) - want[finite]) <= 1e-6 * np.linalg.norm(want[finite].astype(np.float64))
+
+
+BIG = np.float32(3.4e38)          # rounds to infinity in fewer bits
+
+
+@pytest.mark.parametrize("arch,n_e,t_max", [("nips", 64, 4), ("nature", 86, 3)])
+def test_infinities_and_the_largest_values(arch, n_e, t_max):
+    """Infinite, absent and very large activations and weights give on the tensor cores what they give in a chain of multiply-adds."""
+    n, hidden, width = n_e * t_max, *((256, 2592) if arch == "nips" else (512, 3136))
+    L = 2 if arch == "nips" else 3
+    at = 257 * 16 + 257 * 32 if arch == "nips" else 257 * 32 + 513 * 64 + 577 * 64
+
+    def activations(act, theta):
+        for l, a in enumerate(act[:L]):
+            a[[5, a.size // 2, a.size - 9]] = np.inf, BIG, np.nan
+
+    def weights(act, theta):
+        theta[at + 77], theta[at + 9 * width + 1000], theta[at + 200 * width + width - 1] = np.inf, BIG, -np.inf
+
+    with np.errstate(invalid="ignore", over="ignore"):
+        for poison in (activations, weights):
+            got, want = poisoned(arch, n_e, t_max, AUTO, poison), poisoned(arch, n_e, t_max, CORES_ONLY, poison)
+            assert_alike(got["gact"][L - 1], want["gact"][L - 1])
+            # the fully connected layer once more from its own operands, in 64 bits
+            g = got["gact"][L].reshape(n, hidden).astype(np.float64)
+            x, w = got["act"][L - 1].reshape(n, width), got["theta"][at:at + hidden * width].reshape(hidden, width)
+            assert_alike(got["gact"][L - 1].reshape(n, width), np.where(x > 0, g @ w.astype(np.float64), 0).astype(np.float32))
+            weight_grad = got["grad"][at:at + hidden * width].reshape(hidden, width)
+            assert_alike(weight_grad, (g.T @ x.astype(np.float64)).astype(np.float32))
+            assert np.isfinite(weight_grad).all() == (poison is weights)
+            if poison is activations:
+                assert_alike(got["grad"], want["grad"])
+                assert np.isposinf(got["grad"]).any() and np.isneginf(got["grad"]).any()
+            else:
+                for l in range(L - 1):
+                    assert_alike(got["gact"][l], want["gact"][l])
