@@ -17,9 +17,9 @@ static int pick_splits(int M, int N, int K) {
   return gemm_k_splits(K, s);
 }
 
-// Shapes of the CUDA-core contraction for N columns (16, 32, or 64 and more).  At 128 states forward and 640 backward the
-// larger network's layers run at 9 to 14 and 13 to 20 TMAC/s of the 36 the multiply-add pipe could do, with 54 to 65 and 58 to
-// 82 % of the issue slots busy.  The wide shape (8 x 8 per lane for 64 columns, 8 x 4 below, where 8 x 8 leaves tiles of too
+// Shapes of the CUDA-core contraction for N columns (16, 32, or 64 and more).  At 128 states forward and 640 backward (where
+// nothing goes to the tensor cores, see below) the larger network's layers run at 9 to 14 and 13 to 20 TMAC/s of the 36 the multiply-add pipe
+// could do, with 54 to 65 and 58 to 82 % of the issue slots busy.  The wide shape (8 x 8 per lane for 64 columns, 8 x 4 below, where 8 x 8 leaves tiles of too
 // many rows) wins from two warps per scheduler on (1184 of them; 19.8 against 18.4 TMAC/s for the fully connected layer's
 // weight gradient), below that 4 x 4 (18.4 against 12.2 with one and a half), and 2 x 4 where even that leaves a scheduler
 // without a warp (592).  4 x 4 with 64 columns comes in blocks of two warps: the
@@ -35,11 +35,15 @@ static int t3_splits(int M, int N, int K) {
   if (s > by_k) s = by_k;
   return s < 1 ? 1 : gemm_k_splits(K, s, T3_BK);
 }
+// By itself only where its error against sums in 64 bits is no larger than the multiply-adds' chain's, in the 2-norm and over the largest value,
+// measured over both networks, 20 to 960 rows, before and after training.  (The pieces have 22 of a float's 24 bits.  That shows in elements with few
+// terms: root mean square of the error over the sum of the terms' sizes 0.5 to 1.1 times the chain's in data gradients and 0.5 to 1.8 times, 2 to 8.7e-8, in
+// weight gradients.  Who wants chains throughout sets PAAC_OPT_CUDA_CORES_ONLY.)
 // Data gradients, M rows.  A tile takes about a microsecond per block of 32 k, whatever the number of tiles up to two per SM, where the
 // CUDA cores take time with the multiply-adds: 11 M of them per block and 80 M in all is where the two meet.  (us, CUDA cores / tensor cores,
 // larger network: third layer, 18 blocks, 40 states 25 / 26, 64 states 29 / 25, 640 states 105 / 54; second layer, 8 blocks, 40 states 19 / 19, 80 states
-// 26 / 19, 640 states 126 / 67; fully connected layer, 16 blocks, 80 states 19 / 23, 120 states 25 / 23, 640 states 70 / 29.)  Errors against
-// sums in 64 bits, 2-norm: 1.2 to 1.5e-7 instead of 1.2 to 2.9e-7.
+// 26 / 19, 640 states 126 / 67; fully connected layer, 16 blocks, 80 states 19 / 23, 120 states 25 / 23, 640 states 70 / 29.)  Errors,
+// 2-norm: 1.2 to 1.5e-7 instead of 1.4 to 2.9e-7, 0.5 to 0.95 times the chain's.
 // The forward pass stays on the CUDA cores, whose chains of multiply-adds are the same for every batch: sums as exact but in another order put
 // a unit or two per pass on the other side of the ReLU, and training then runs apart from there.
 template <class T> static bool t3_allowed(const LaunchCtx& lc) { return !lc.cuda_cores_only && lc.error_word != nullptr && (sizeof(T) == 4 || lc.bf16_sums_on_tensor_cores); }
@@ -49,11 +53,13 @@ template <class T> static bool t3_pays(const LaunchCtx& lc, long long M, int N, 
   return t3_allowed<T>(lc) && macs >= blocks * 11000000 && macs >= 80000000;
 }
 // Weight gradients, whose k is split until the device is full: from 64 M multiply-adds on (first layer of the smaller network, 40 states 14 / 11 us,
-// 160 states 31 / 20, 960 states 152 / 66; second layer 80 states 13 / 11, 640 states 43 / 20).  The fully connected layer's sums over fewer than
-// 256 rows are more exact on the CUDA cores (160 rows: 1.08e-7 against 1.41e-7).
-template <class T> static bool t3_wgrad_pays(const LaunchCtx& lc, int J, int CO, int K) {
+// 160 states 31 / 20, 960 states 152 / 66; second layer 80 states 13 / 11, 640 states 43 / 20), and from as many rows on that the sums, not the operands,
+// make the error: 2-norm of a convolution's 0.2 to 0.95 times the chain's from 2048 rows on (40 states of the third layer, 1960 rows: 1.03
+// times), of the fully connected layer's 0.5 to 0.99 times from 512 on, in either storage (268 to 511 rows: 0.5 to 1.33 times).
+template <class T, class LA> static bool t3_wgrad_pays(const LaunchCtx& lc, int J, int CO, int K) {
   if (lc.fp32_tensor_cores) return lc.error_word != nullptr;
-  return t3_allowed<T>(lc) && K >= 256 && (long long)J * CO * K >= 64000000;
+  constexpr int LEAST = T3Table<LA>::use ? 2048 : 512;      // of a convolution's windows, or of the fully connected layer
+  return t3_allowed<T>(lc) && K >= LEAST && (long long)J * CO * K >= 64000000;
 }
 static size_t ff_heads_scratch_floats(const NetDims& nd, int n);
 static int ff_shape(int N, long long outputs) {              // outputs of all classes and splits
@@ -101,7 +107,7 @@ template <int CO_TILE, class LA, class LB>
 static void ff_wgrad(LaunchCtx& lc, int kid, int J, int CO, int K, LA window, LB grad_rows, float scale, float* gw, float* gb,
                      float* scratch, GradSegments* segs) {
   typedef typename LB::Elem T;
-  const bool tensor = t3_wgrad_pays<T>(lc, J, CO, K);
+  const bool tensor = t3_wgrad_pays<T, LA>(lc, J, CO, K);
   const FfWgradPlan p = ff_wgrad_plan(J, CO, K, tensor);
   FfPartialColsum ep;
   ep.part = scratch; ep.M = J; ep.N = CO; ep.colpart = scratch + p.part;

@@ -39,10 +39,10 @@ def contractions(arch, n):
             (WEIGHTS, 1, 512 * 64, 81 * n), (DATA, 1, n * 100 * 128, 256), (WEIGHTS, 0, 256 * 32, 400 * n)]
 
 
-def on_tensor_cores(kind, outputs, k):
+def on_tensor_cores(arch, kind, l, outputs, k):
     """The rule of the dispatch for contractions nobody chose a path for."""
     if kind == WEIGHTS:
-        return k >= 256 and outputs * k >= 64_000_000
+        return k >= (512 if l == (2 if arch == "nips" else 3) else 2048) and outputs * k >= 64_000_000
     return outputs * k >= max(80_000_000, 11_000_000 * -(-k // 32))
 
 
@@ -67,9 +67,9 @@ def gradients(arch, prec, n_e, t_max, options, n_actions=6):
 AUTO, CORES_ONLY, TENSOR = {}, {pb.OPT_CUDA_CORES_ONLY: 1}, {pb.OPT_FP32_TENSOR_CORES: 1}
 
 
-@pytest.mark.parametrize("arch,prec,n", [("nips", "bf16", n) for n in (39, 40, 96, 97, 98, 255, 256)]
-                         + [("nips", "fp32", n) for n in (39, 40, 96, 97, 98, 132, 133, 255, 256)]
-                         + [("nature", "fp32", n) for n in (19, 20, 24, 25, 26, 27, 35, 36, 66, 67, 109, 110, 255, 256)])
+@pytest.mark.parametrize("arch,prec,n", [("nips", "bf16", n) for n in (39, 40, 96, 97, 98, 511, 512)]
+                         + [("nips", "fp32", n) for n in (39, 40, 96, 97, 98, 132, 133, 511, 512)]
+                         + [("nature", "fp32", n) for n in (19, 20, 25, 26, 27, 41, 42, 66, 67, 109, 110, 511, 512)])
 def test_which_contractions_go_to_the_tensor_cores(arch, prec, n):
     """Just below and just above each line of the rule: what the library chooses by itself has the bits of the one contraction
     or of the other, and with CUDA_CORES_ONLY none has those of the tensor cores."""
@@ -81,7 +81,7 @@ def test_which_contractions_go_to_the_tensor_cores(arch, prec, n):
         # (a data gradient in bf16 storage is rounded to eight bits, where the two contractions nearly always meet)
         if same_operand and not (prec == "bf16" and kind == DATA):
             assert not np.array_equal(cores[kind][at], tensor[kind][at]), (kind, l)
-        want = tensor if on_tensor_cores(kind, outputs, k) else cores
+        want = tensor if on_tensor_cores(arch, kind, l, outputs, k) else cores
         if np.array_equal(auto["gact"][l], want["gact"][l]):
             assert np.array_equal(auto[kind][at], want[kind][at]), (kind, l)
             compared += 1
@@ -141,7 +141,7 @@ def assert_alike(got, want):
 BIG = np.float32(3.4e38)          # rounds to infinity in fewer bits
 
 
-@pytest.mark.parametrize("arch,n_e,t_max", [("nips", 64, 4), ("nature", 86, 3)])
+@pytest.mark.parametrize("arch,n_e,t_max", [("nips", 64, 8), ("nature", 86, 6)])
 def test_infinities_and_the_largest_values(arch, n_e, t_max):
     """Infinite, absent and very large activations and weights give on the tensor cores what they give in a chain of multiply-adds."""
     n, hidden, width = n_e * t_max, *((256, 2592) if arch == "nips" else (512, 3136))
