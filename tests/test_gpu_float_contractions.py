@@ -172,3 +172,27 @@ def test_infinities_and_the_largest_values(arch, n_e, t_max):
             else:
                 for l in range(L - 1):
                     assert_alike(got["gact"][l], want["gact"][l])
+
+
+def test_shape_sweep_cuda_cores_and_tensor_cores_agree():
+    """Thirty ragged shapes, both networks, both algorithms and environments: the update's gradients from one rollout by chains of multiply-adds
+    throughout and with every contraction on the tensor cores.  Each contraction is within 1e-6 of its own operands' sums in the 2-norm, and
+    at most four follow one another.  Nothing has the same bits, so there were two implementations."""
+    import random
+    rnd = random.Random(11)
+    combos = [(arch, n, t, a) for arch in ("nips", "nature") for n in (1, 2, 3, 5, 16, 37, 64, 100, 129, 255)
+              for t in (1, 2, 5, 7) for a in (2, 3, 5, 18, 19, 32)]
+    rnd.shuffle(combos)
+    for i, (arch, n_e, T, A) in enumerate(combos[:30]):
+        outs = []
+        for option in (pb.OPT_CUDA_CORES_ONLY, pb.OPT_FP32_TENSOR_CORES):
+            g = pb.Paac(arch, n_e, T, A, seed=5, precision=pb.FP32, lr=0.01, term_denom=50,
+                        algorithm=pb.ALGO_NSTEP_Q if i % 3 == 0 else pb.ALGO_A2C, environment=pb.ENV_PATTERN if i % 4 == 0 else pb.ENV_HASHED)
+            g.rollout()
+            g.set_option(option, 1)
+            assert g.update()["status"] == 0 and g.error_word() == 0, (arch, n_e, T, A)
+            outs.append([g.debug_read(pb.DBG_GACT0 + l).copy() for l in range(2 if arch == "nips" else 3)] + [g.debug_read(pb.DBG_GRAD).copy()])
+            g.close()
+        for x, y in zip(*outs):
+            d = np.linalg.norm(x.astype(np.float64) - y) / np.linalg.norm(x.astype(np.float64))
+            assert 0 < d <= 8e-6, (arch, n_e, T, A, d)
