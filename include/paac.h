@@ -300,7 +300,7 @@ int paac_debug_write(paac_ctx* ctx, int which, const void* src /* host */, size_
  * are added up in float; what is dropped is below 2^-21 of a product, so results stay within the 1e-4 tolerance of the
  * float path, free-running over ten updates included.  Default 0: the larger data and weight gradients of PAAC_FP32 on either
  * network and of PAAC_BF16 on the smaller one (whose values are their own first piece) do so, from the sizes on where it takes less time and their
- * error against sums in 64 bits is no larger, in the 2-norm and over the largest value, than that of a chain of float multiply-adds; a single element with few
+ * error against sums in 64 bits is no larger, in the 2-norm, than that of a chain of float multiply-adds; a single element with few
  * terms may be up to 2^-21 of their sizes off.  The forward passes, the smaller gradients and what PAAC_OPT_CUDA_CORES_ONLY
  * names are such chains, on the CUDA cores.
  * PAAC_OPT_UPDATE_CHUNKS: 1 (default) .. 4.  With more than one, the tensor-core update runs the second layer's data

@@ -35,15 +35,15 @@ static int t3_splits(int M, int N, int K) {
   if (s > by_k) s = by_k;
   return s < 1 ? 1 : gemm_k_splits(K, s, T3_BK);
 }
-// By itself only where its error against sums in 64 bits is no larger than the multiply-adds' chain's, in the 2-norm and over the largest value,
-// measured over both networks, 20 to 960 rows, before and after training.  (The pieces have 22 of a float's 24 bits.  That shows in elements with few
-// terms: root mean square of the error over the sum of the terms' sizes 0.5 to 1.1 times the chain's in data gradients and 0.5 to 1.8 times, 2 to 8.7e-8, in
+// By itself only where its error against sums in 64 bits is no larger, in the 2-norm, than that of the multiply-adds' chain, measured
+// over both networks, 20 to 960 rows, before and after training.  (The pieces have 22 of a float's 24 bits.  That shows in elements with few
+// terms: root mean square of the error over the sum of the terms' sizes 0.5 to 1.1 times the chain's in data gradients, 0.5 to 1.6 times in
 // weight gradients.  Who wants chains throughout sets PAAC_OPT_CUDA_CORES_ONLY.)
 // Data gradients, M rows.  A tile takes about a microsecond per block of 32 k, whatever the number of tiles up to two per SM, where the
 // CUDA cores take time with the multiply-adds: 11 M of them per block and 80 M in all is where the two meet.  (us, CUDA cores / tensor cores,
 // larger network: third layer, 18 blocks, 40 states 25 / 26, 64 states 29 / 25, 640 states 105 / 54; second layer, 8 blocks, 40 states 19 / 19, 80 states
 // 26 / 19, 640 states 126 / 67; fully connected layer, 16 blocks, 80 states 19 / 23, 120 states 25 / 23, 640 states 70 / 29.)  Errors,
-// 2-norm: 1.2 to 1.5e-7 instead of 1.4 to 2.9e-7, 0.5 to 0.95 times the chain's.
+// 2-norm: 1.2 to 1.5e-7 instead of 1.3 to 2.9e-7, 0.5 to 0.95 times the chain's.
 // The forward pass stays on the CUDA cores, whose chains of multiply-adds are the same for every batch: sums as exact but in another order put
 // a unit or two per pass on the other side of the ReLU, and training then runs apart from there.
 template <class T> static bool t3_allowed(const LaunchCtx& lc) { return !lc.cuda_cores_only && lc.error_word != nullptr && (sizeof(T) == 4 || lc.bf16_sums_on_tensor_cores); }

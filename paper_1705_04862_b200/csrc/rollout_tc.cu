@@ -277,7 +277,8 @@ rollout_tc_kernel(const __grid_constant__ RtArgs q) {
 
   // ---- what stays for the rollout ----
   // Everything by asynchronous copies, so that one latency covers all of it: with the small arrays loaded and stored by hand, one after
-  // the other, this took 2.7 us (a rollout at 32 environments 74.5 us; 150.0 -> 148.0 us an iteration, 341 -> 329 us with environments outside).
+  // the other, this took 2.7 us (a rollout at 32 environments 74.5 us; an iteration 150.0, now 148.0; with environments outside, six such launches,
+  // the iterations of one run differ by more).
   const uint32_t epoch = q.sync[0];
   if (tid == 0) {
     s_dead = 0u; s_linger = 0u;
